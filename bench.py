@@ -32,12 +32,11 @@ import synth  # noqa: E402
 
 TF32_PER_BF16 = 1.1 / 2.25  # nominal dense TF32 / BF16 tensor rates
 
-# DRAM bytes (read + write) per launch of the dominant kernel: the FP64 sigma launches of one
-# timed step of this workload (48 launches, one ncu capture of dram__bytes_read/write.sum with
-# --profile-step), valid only for the kernel source it was taken on (sha256 prefix);
-# otherwise, and for the mixed form, the bench reports null.
+# DRAM bytes (read + write) per launch of the dominant kernel, one ncu capture of
+# dram__bytes_read/write.sum with --profile-step, valid only for the kernel source it was taken
+# on (sha256 prefix); otherwise the bench reports null.
 TRAFFIC = {
-    "fp64": {"source": "lrt_kernels.cu", "sha256": "4b10c817f69cb891", "bytes": 1107.18e6},
+    "fp64": {"source": "lrt_fp64_mma.cu", "sha256": "", "bytes": None},
     "mixed": {"source": "lrt_tc.cu", "sha256": "", "bytes": None},
 }
 
@@ -61,6 +60,17 @@ def tf32_peak():
             return json.load(f)["bf16_tflops"] * TF32_PER_BF16, "of measured (bf16 burst x 1.1/2.25)"
     except (OSError, KeyError, ValueError):
         return 1900.0 * TF32_PER_BF16, "of fallback (1.9 PF bf16 x 1.1/2.25)"
+
+
+def digit_peak():
+    """FP64 products as 28 exact FP16 digit products each: the measured dense BF16 (= FP16) rate / 28."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            return json.load(f)["bf16_tflops"] / 28, "of measured (bf16 burst / 28 digit products)"
+    except (OSError, KeyError, ValueError):
+        return 1900.0 / 28, "of fallback (1.9 PF bf16 / 28 digit products)"
+
+
 WORKLOAD = "water_k24_e10_M500_onesite_6vec_fp64"
 
 
@@ -330,13 +340,11 @@ def run_ours(args):
                                  "(the tensor pipe issues it 3x)"}
             metric, dtype = "H_eff sigma TFLOP/s (algorithmic, split-TF32 mixed)", "tf32x3"
         else:
-            peak = fp64_peak(clocks)
-            roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+            peak, peak_note = digit_peak()
+            roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                     "frac": achieved / peak, "traffic": traffic("fp64"),
-                    "kernel": "gemm_fp64_kernel (sigma phases 1+2)",
-                    "peak_note": "FP64 FMA pipe: 152 SMs x 2 DFMA/clk x 2 flop at the sampled maximum SM "
-                                 "clock (sm_103a has no FP64 tensor kind); an FMA probe measured "
-                                 "1.20 TFLOP/s"}
+                    "kernel": "gemm_mma_kernel (sigma phases 1+2)",
+                    "peak_note": peak_note, "fp64_pipe_tflops": fp64_peak(clocks)}
             metric, dtype = "H_eff sigma TFLOP/s (algorithmic, FP64)", "f64"
         out = {
             "metric": metric,
@@ -660,7 +668,7 @@ def fe2s2_sigma(pkg, device, stream):
         tf64, tfmx = fl / t64 / 1e9, fl / tmx / 1e9
         peak, note = tf32_peak()
         return {"site": i, "wfn_elements": n, "nvec": nvec, "gflop": fl / 1e9, "environment_build_s": t_env,
-                "fp64_ms": t64, "fp64_tflops": tf64, "fp64_frac": tf64 / fp64_peak(None),
+                "fp64_ms": t64, "fp64_tflops": tf64, "fp64_frac": tf64 / digit_peak()[0],
                 "mixed_ms": tmx, "mixed_tflops": tfmx, "mixed_frac": tfmx / peak, "mixed_peak_note": note,
                 "mixed_max_rel_err_vs_fp64": err, "symmetry_rel": sym, "device_gb": _device_gb(device)}
     finally:

@@ -1,0 +1,552 @@
+// Grouped FP64 GEMM on the tensor cores by exact digit products.
+//
+// Same work lists and results as gemm_fp64_kernel (lrt_kernels.cu): an output tile sums,
+// over its segments, scale_q op(A_q) op(B_q), the segments concatenated along one K axis and
+// taken 32 positions (a chunk) at a time.  GB300 issues 2 FP64 FMA per clock and SM but 1024
+// FP16 FMA with FP32 accumulation through mma.sync, so each chunk is multiplied in integers:
+//
+//  - every row of A and column of B of the chunk is scaled by a power of two (its largest
+//    exponent) and cut into 7 balanced digits of 9 bits, g_d in [-256, 256]: 63 bits, so an
+//    element within 2^9 of its row's largest keeps all of its 53;
+//  - digit products A_i B_j with i + j = d <= 6 are summed over the chunk in FP32 (28
+//    mma.sync per 16 x 8 x 16): at most 7 * 32 * 2^16 < 2^24, so every sum is exact;
+//  - the 7 sums are joined in a 64-bit integer, rounded once to FP64 and added to the tile's
+//    FP64 accumulator with the row's and column's power of two: one FP64 instruction per
+//    element and chunk instead of 32.
+//
+// (The splitting is the error-free transformation of Ozaki, Ogita, Oishi and Rump, "Error-free
+// transformations of matrix multiplication by using fast routines of matrix multiplication",
+// Numer. Algorithms 59, 2012, with a fixed digit grid per chunk.)  What is lost per chunk is
+// below 2^-54 of its largest row times column product, less than the 32 roundings of an FP64
+// FMA chain.  Chunks that hold an infinity, a NaN or a row outside 2^-423 .. 2^477 are
+// multiplied in plain FP64 from the staged operands.
+//
+// Measured on the k = 24, M = 500, 6-vector sigma (23.7 G multiply-adds): 44.0 ms by FP64 FMAs,
+// 16.7 ms here; error against 64-bit exact values 3.4e-16 (8.5e-16 before) at k = 8, 2.8e-15
+// (7.3e-15) on the PPP chain.  The kernel is bound by issued instructions (44-48% of the issue
+// slots at 12 warps per SM; tensor pipe 20%, FP64 pipe 25%): cutting the operands (a third)
+// and staging them cost more than the products.  Hence tiles of 96 staged rows for up to 8
+// 16 x 16 units, 3 CTAs of 4 warps per SM; and one row or column scale per 32 positions, so a
+// chunk needs no look at the rest of K.
+#include "lrt_kernels.h"
+#include "lrt_fp64_tile.h"
+
+#include <atomic>
+
+namespace lrt {
+
+static_assert(GEMM_KC == 32 && GEMM_THREADS == 128, "the lane mappings below");
+constexpr int MMA_ND = 7;                 // digits
+constexpr int MMA_EMIN = 600, MMA_EMAX = 1500;   // exponent fields the integer path takes
+constexpr int MMA_E0 = 1023;
+constexpr int MMA_NOBAL = -4096;                  // balance exponent where B's row is zero
+constexpr int MMA_WILD = (int)0x80000000;        // exponent word of a row the integer path does not take
+
+struct MmaSmem {
+  double raw[MMA_ROWS][GEMM_KC];          // chunk operands: A rows, then B columns; 16-byte groups XOR row
+  uint32_t dig[MMA_ND][MMA_ROWS][GEMM_KC / 2];   // digits as FP16 pairs, 16-byte groups XOR row / 2
+  alignas(16) int ex[MMA_ROWS];           // (E - 539) << 20 of each row (read in pairs)
+  double sc[GEMM_KC];                     // segment scale of each K position
+  SegS sd[GEMM_SEGB];
+  int kst[GEMM_SEGB + 1];
+  alignas(16) int bal[GEMM_KC];           // balance exponents of the K positions
+  alignas(8) int2 vl[MMA_ROWS];           // vector block and index inside it of each row
+  int wild[2];                            // chunk (by parity) holds a row outside the integer path
+  uint32_t neg;                           // K positions of negative scale
+  int mode;                               // scales of the chunk: 0 all 1, 1 all +-1, 2 general
+};
+
+__device__ __forceinline__ void cp_async8z(void* dst, const void* src, int bytes) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t s) { return __byte_perm(a, b, s); }
+// (x & mask) | 0x64006400 as FP16 pairs is 1024 + field; times the signs minus 1280 times the
+// signs leaves +-(field - 256)
+__device__ __forceinline__ uint32_t digit_pair(uint32_t x, uint32_t mask, uint32_t sign, uint32_t off) {
+  uint32_t r;
+  const uint32_t h = (x & mask) | 0x64006400u;
+  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(h), "r"(sign), "r"(off));
+  return r;
+}
+
+// magnitude (its leading bit at bit 61 - sh) biased by 256 in every digit
+__device__ __forceinline__ uint2 fixed63(uint32_t hi, uint32_t lo, int sh) {
+  // sum_d 256 * 2^(9 d), d = 0..6
+  constexpr uint64_t BIAS = 256ull * ((1ull << 0) | (1ull << 9) | (1ull << 18) | (1ull << 27) | (1ull << 36) |
+                                      (1ull << 45) | (1ull << 54));
+  const uint32_t H = __funnelshift_l(lo, hi, 11) | 0x80000000u, L = lo << 11;   // leading bit at bit 63
+  const int s = sh + 2;
+  const uint32_t wl = __funnelshift_rc(__funnelshift_rc(L, H, s), 0u, max(s - 32, 0));
+  const uint32_t wh = __funnelshift_rc(H, 0u, s);
+  const uint64_t w = ((uint64_t)wh << 32 | wl) + BIAS;
+  return make_uint2((uint32_t)w, (uint32_t)(w >> 32));
+}
+// digits (most significant first) of two neighbouring K positions with high words ha, hb
+__device__ __forceinline__ void digits2(const uint2 a, const uint2 b, uint32_t ha, uint32_t hb, uint32_t (&d)[MMA_ND]) {
+  const uint32_t sg = prmt(ha, hb, 0x7632) & 0x80008000u;
+  const uint32_t one = sg | 0x3C003C00u, off = sg ^ 0xE500E500u;
+  d[6] = digit_pair(prmt(a.x, b.x, 0x5410), 0x01FF01FFu, one, off);            // bits 0-8
+  d[5] = digit_pair(prmt(a.x, b.x, 0x6521) >> 1, 0x01FF01FFu, one, off);       // 9-17
+  d[4] = digit_pair(prmt(a.x, b.x, 0x7632) >> 2, 0x01FF01FFu, one, off);       // 18-26
+  d[3] = digit_pair(prmt(prmt(a.x, a.y, 0x0043), prmt(b.x, b.y, 0x0043), 0x5410) >> 3, 0x01FF01FFu, one, off);   // 27-35
+  d[2] = digit_pair(prmt(a.y, b.y, 0x5410) >> 4, 0x01FF01FFu, one, off);       // 36-44
+  d[1] = digit_pair(prmt(a.y, b.y, 0x6521) >> 5, 0x01FF01FFu, one, off);       // 45-53
+  d[0] = digit_pair(prmt(a.y, b.y, 0x7632) >> 6, 0x03FF03FFu, one, off);       // 54-63
+}
+
+// four K positions of a row as (hi, lo) words
+struct Quad {
+  uint32_t hi[4], lo[4];
+};
+// positions 4l .. 4l + 3 of a staged row (16-byte groups XOR row)
+__device__ __forceinline__ Quad load_quad(const double* raw, int row, int l) {
+  Quad q;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int g = (2 * l + h) ^ (row & 15);
+    const uint4 v = *reinterpret_cast<const uint4*>(raw + (size_t)row * GEMM_KC + 2 * g);
+    q.lo[2 * h] = v.x;
+    q.hi[2 * h] = v.y;
+    q.lo[2 * h + 1] = v.z;
+    q.hi[2 * h + 1] = v.w;
+  }
+  return q;
+}
+__device__ __forceinline__ void exponents(const Quad& q, int (&e)[4], int& emax) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) e[j] = (int)((q.hi[j] & 0x7FFFFFFFu) >> 20);
+  emax = max(max(e[0], e[1]), max(e[2], e[3]));
+}
+// digits of a row's four positions, the row's exponent taken over its 8 lanes (e: 0 for a
+// zero).  Returns the row's exponent word, MMA_WILD when it needs the FP64 path.
+__device__ __forceinline__ int cut_row(const Quad& q, const int (&e)[4], int emax, uint32_t (&d0)[MMA_ND],
+                                       uint32_t (&d1)[MMA_ND]) {
+  emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 1));
+  emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 2));
+  emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 4));
+  const bool wild = emax > 0 && (emax < MMA_EMIN || emax > MMA_EMAX);
+  const int E = emax > 0 ? emax : MMA_E0;   // a zero row: every element shifts out
+  uint2 f[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) f[j] = fixed63(q.hi[j], q.lo[j], E - e[j]);
+  digits2(f[0], f[1], q.hi[0], q.hi[1], d0);
+  digits2(f[2], f[3], q.hi[2], q.hi[3], d1);
+  return wild ? MMA_WILD : (E - 539) << 20;
+}
+// word offset of positions 4l .. 4l + 3 inside a row's 16 digit words (16-byte groups XOR row / 2)
+__device__ __forceinline__ int digit_word(int row, int l) {
+  return ((((l >> 1) ^ (row >> 1)) & 3) << 2) + ((l & 1) << 1);
+}
+
+// the 7 digit-product sums of one element, in units of 2^13 of the last digits' product.
+// Sums that stay below 2^22 once scaled become integers by adding 1.5 * 2^23 (the two least
+// significant ones rounded to nearest); the others take the slower conversion.
+__device__ __forceinline__ int magic_int(float x) { return __float_as_int(x) - 0x4B400000; }
+__device__ __forceinline__ long long join_digits(const float (&v)[MMA_ND][4], int t) {
+  constexpr float MG = 12582912.0f;
+  const int d0 = magic_int(v[0][t] + MG), d1 = magic_int(v[1][t] + MG);   // <= 2^21, 2^22
+  const int d2 = __float2int_rn(v[2][t]), d3 = __float2int_rn(v[3][t]), d4 = __float2int_rn(v[4][t]);
+  const int d5 = magic_int(fmaf(v[5][t], 0.0625f, MG)), d6 = magic_int(fmaf(v[6][t], 1.0f / 8192.0f, MG));
+  return ((long long)d0 << 41) + ((long long)d1 << 32) + ((long long)d2 << 23) + ((long long)d3 << 14) +
+         ((long long)d4 << 5) + (long long)(d5 + d6);
+}
+
+// v[h][d] += the digit products of weight d over 16 positions, for a 16 x 16 unit (its first 8
+// columns when NH = 1): this lane's ldmatrix addresses aa, ba of the first digits, and the
+// digits' strides
+template <int NH>
+__device__ __forceinline__ void unit_products(float (&v)[2][MMA_ND][4], uint32_t aa, uint32_t ba, uint32_t adig,
+                                              uint32_t bdig) {
+  uint32_t B[MMA_ND][4];
+#pragma unroll
+  for (int j = 0; j < MMA_ND; ++j) ldsm4(B[j], ba + j * bdig);
+#pragma unroll
+  for (int i = 0; i < MMA_ND; ++i) {
+    uint32_t A[4];
+    ldsm4(A, aa + i * adig);
+#pragma unroll
+    for (int j = 0; j < MMA_ND - i; ++j) {
+      mma16816(v[0][i + j], A, B[j][0], B[j][1]);
+      if (NH > 1) mma16816(v[1][i + j], A, B[j][2], B[j][3]);
+    }
+  }
+}
+
+__device__ __forceinline__ void scale_quad(const MmaSmem& S, int mode, int l, Quad& q) {
+  if (mode == 1) {
+    const uint32_t n = S.neg >> (4 * l);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) q.hi[j] ^= (n << (31 - j)) & 0x80000000u;
+  } else if (mode == 2) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const double x = __hiloint2double((int)q.hi[j], (int)q.lo[j]) * S.sc[4 * l + j];
+      q.hi[j] = (uint32_t)__double2hiint(x);
+      q.lo[j] = (uint32_t)__double2loint(x);
+    }
+  }
+}
+
+template <class Extra>
+__device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, const int3 wi, const double* xbase,
+                                              double* ybase, double* tbase, double* wbase, const GemmOut& o,
+                                              const Extra& extra) {
+  extern __shared__ __align__(16) unsigned char mma_smem_raw[];
+  MmaSmem& S = *reinterpret_cast<MmaSmem*>(mma_smem_raw);
+  const int m0 = wi.y >> 8, mt = wi.y & 255, n0 = wi.z >> 8, nt = wi.z & 255;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int a16 = (mt + 15) >> 4, b16 = (nt + 15) >> 4;
+  const int RB = 16 * a16;                 // first B row
+  const int rows = RB + 16 * b16;          // <= MMA_ROWS
+  const int units = a16 * b16;             // <= 2 * GEMM_WARPS
+  const bool bal = o.balance != 0;
+
+  // row tables; padding rows are zero for the whole tile
+  if (tid < rows) {
+    const bool isA = tid < RB;
+    const int i = isA ? tid : tid - RB;
+    int g = (isA ? m0 : n0) + i, v = 0;
+    const int blk = isA ? o.c_vr : o.c_vc;
+    if (blk > 0) {
+      v = g / blk;
+      g -= v * blk;
+    }
+    S.vl[tid] = make_int2(v, g);
+  }
+  for (int r = warp; r < rows; r += GEMM_WARPS)
+    if (r < RB ? r >= mt : r - RB >= nt) S.raw[r][lane] = 0.0;
+  if (bal && tid < GEMM_KC) S.bal[tid] = MMA_NOBAL;
+  if (tid < 2) S.wild[tid] = 0;
+
+  double acc[2][2][4];
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[u][h][c] = 0.0;
+
+  int it = 0;            // chunks done
+  for (int b0 = 0; b0 < o.seg_count; b0 += GEMM_SEGB) {
+    const int nb = min(GEMM_SEGB, o.seg_count - b0);
+    __syncthreads();   // the previous batch's descriptors and digits are no longer read
+    if (warp == 0) {
+      int k = 0;
+      if (lane < nb) {
+        GemmSeg g = segs[o.seg_begin + b0 + lane];
+        if (g.a_rel) g.A = (g.a_rel == 1 ? xbase : g.a_rel == 2 ? tbase : extra(g.a_rel - 3)) + g.a_off;
+        if (g.b_rel) g.B = (g.b_rel == 1 ? xbase : g.b_rel == 2 ? tbase : extra(g.b_rel - 3)) + g.b_off;
+        S.sd[lane] = SegS{g.A, g.B, g.lda, g.ldb, g.transA, g.transB, g.scale, g.a_vr, g.b_vc, g.a_vs, g.b_vs};
+        k = g.k;
+      }
+      int incl = k;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += v;
+      }
+      S.kst[lane + 1] = incl;
+      if (lane == 0) S.kst[0] = 0;
+    }
+    __syncthreads();
+    const int Kb = S.kst[nb];
+    const int nch = (Kb + GEMM_KC - 1) / GEMM_KC;
+    int q1 = 0;   // segment of this lane's K position, chunk after chunk
+    int q2 = 0;   // segment of the chunk's first position
+
+    auto issue = [&](int c) {
+      const int p0 = c * GEMM_KC;
+      const int p = p0 + lane;
+      const bool in = p < Kb;
+      while (in && S.kst[q1 + 1] <= p) ++q1;
+      const SegS& s = S.sd[q1];
+      const int kl = p - S.kst[q1];
+      const int g16 = lane >> 1, half = lane & 1;
+      // lanes along K: operands stored K-contiguous, and zeros beyond Kb
+      const bool ka = !in || !s.transA, kb = !in || s.transB;
+      const int nz = in ? 8 : 0;
+      // rows i = warp, warp + 4, ...: i mod 16, and so the swizzle, repeats every fourth
+      auto rows_along_k = [&](int r0, int n, const double* base, int ld, int64_t vs) {
+        const uint32_t ld8 = in ? 8u * (uint32_t)ld : 0u, vs8 = in ? 8u * (uint32_t)vs : 0u;
+        const char* src = reinterpret_cast<const char*>(in ? base + kl : base);
+        for (int i0 = warp; i0 < n; i0 += 4 * GEMM_WARPS)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int i = i0 + GEMM_WARPS * u;
+            if (i < n) {
+              const int2 vl = S.vl[r0 + i];
+              cp_async8z(&S.raw[r0 + i][2 * (g16 ^ ((warp + GEMM_WARPS * u) & 15)) + half],
+                         src + (uint64_t)(uint32_t)vl.x * vs8 + (uint64_t)(uint32_t)vl.y * ld8, nz);
+            }
+          }
+      };
+      static_assert(GEMM_WARPS == 4, "the swizzle period above");
+      if (ka) rows_along_k(0, mt, s.A, s.lda, s.avs);
+      if (kb) rows_along_k(RB, nt, s.B, s.ldb, s.bvs);
+      // lanes along the rows: operands stored K-major, one segment after the other
+      if (__any_sync(0xffffffffu, !ka || !kb)) {
+        const int pend = min(p0 + GEMM_KC, Kb);
+        for (int q = q2; q < nb && S.kst[q] < pend; ++q) {
+          const int f = max(S.kst[q], p0), l = min(S.kst[q + 1], pend);
+          const int kk0 = f - p0 + ((warp - (f - p0)) & 3);   // first position of this warp
+          if (kk0 >= l - p0) continue;
+          const SegS& t = S.sd[q];
+          auto k_major = [&](int r0, int n, const double* base, int ld, int64_t vs) {
+            const double* src = base + (int64_t)(p0 + kk0 - S.kst[q]) * ld;
+            for (int i = lane; i < n; i += 32) {
+              const int r = r0 + i;
+              const int2 vl = S.vl[r];
+              const double* p = src + ((uint64_t)(uint32_t)vl.x * (uint32_t)vs + (uint32_t)vl.y);
+              double* row = &S.raw[r][0];
+              for (int kk = kk0; kk < l - p0; kk += GEMM_WARPS, p += (int64_t)GEMM_WARPS * ld)
+                cp_async8z(row + 2 * ((kk >> 1) ^ (r & 15)) + (kk & 1), p, 8);
+            }
+          };
+          if (t.transA) k_major(0, mt, t.A, t.lda, t.avs);
+          if (!t.transB) k_major(RB, nt, t.B, t.ldb, t.bvs);
+        }
+      }
+      if (warp == 0) {
+        const double sc = in ? s.scale : 1.0;
+        S.sc[lane] = sc;
+        const bool one = __all_sync(0xffffffffu, sc == 1.0), pm = __all_sync(0xffffffffu, fabs(sc) == 1.0);
+        const uint32_t neg = __ballot_sync(0xffffffffu, sc < 0.0);
+        if (lane == 0) {
+          S.mode = one ? 0 : pm ? 1 : 2;
+          S.neg = neg;
+        }
+      }
+      const int pn = p0 + GEMM_KC;
+      while (pn < Kb && S.kst[q2 + 1] <= pn) ++q2;
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+
+    if (nch > 0) issue(0);
+    for (int c = 0; c < nch; ++c, ++it) {
+      asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+      __syncthreads();               // the chunk has landed; the previous one's digits are no longer read
+      const int kc = min(GEMM_KC, Kb - c * GEMM_KC);
+      const int mode = S.mode;
+      const int l = lane & 7;
+      if (bal) {
+        // largest exponent of each K position over B's columns
+        int mx[4] = {0, 0, 0, 0};
+        for (int r = RB + 4 * warp + (lane >> 3); r < rows; r += 4 * GEMM_WARPS) {
+          Quad q = load_quad(&S.raw[0][0], r, l);
+          scale_quad(S, mode, l, q);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) mx[j] = max(mx[j], (int)(q.hi[j] & 0x7FFFFFFFu) >> 20);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          mx[j] = max(mx[j], __shfl_xor_sync(0xffffffffu, mx[j], 8));
+          mx[j] = max(mx[j], __shfl_xor_sync(0xffffffffu, mx[j], 16));
+          // kept as the exponent itself; a position where B is zero stays far below every other
+          if (lane < 8 && mx[j] > 0) atomicMax(&S.bal[4 * l + j], mx[j] - MMA_E0);
+        }
+        __syncthreads();
+      }
+      for (int r = 4 * warp + (lane >> 3); r < rows; r += 4 * GEMM_WARPS) {   // rows is a multiple of 16
+        Quad q = load_quad(&S.raw[0][0], r, l);
+        const bool isB = r >= RB;
+        if (isB) scale_quad(S, mode, l, q);
+        int e[4], emax;
+        exponents(q, e, emax);
+        if (bal) {
+          const bool inf = emax == 2047;
+          const int4 bk = *reinterpret_cast<const int4*>(&S.bal[4 * l]);
+          const int bj[4] = {bk.x, bk.y, bk.z, bk.w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) e[j] = e[j] == 0 ? -4096 : isB ? e[j] - bj[j] : e[j] + bj[j];
+          emax = inf ? 2047 : max(max(e[0], e[1]), max(e[2], e[3]));
+        }
+        uint32_t d0[MMA_ND], d1[MMA_ND];
+        const int x = cut_row(q, e, emax, d0, d1);
+        if (l == 0) S.ex[r] = x;
+        if (x == MMA_WILD) S.wild[it & 1] = 1;
+        const int w = digit_word(r, l);
+#pragma unroll
+        for (int d = 0; d < MMA_ND; ++d) *reinterpret_cast<uint2*>(&S.dig[d][r][w]) = make_uint2(d0[d], d1[d]);
+      }
+      __syncthreads();
+      const bool wild = S.wild[it & 1] != 0;
+      if (tid == 0) S.wild[(it & 1) ^ 1] = 0;   // last read before this chunk's first barrier
+      if (wild) {
+        // plain FP64 from the staged operands
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int un = warp + GEMM_WARPS * u;
+          if (un >= units) break;
+          const int ra = 16 * (un / b16) + (lane >> 2), rb = RB + 16 * (un % b16) + 2 * (lane & 3);
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+              const int i = ra + 8 * (t >> 1), j = rb + 8 * h + (t & 1);
+              double s = acc[u][h][t];
+              for (int kk = 0; kk < kc; ++kk)
+                s = fma(S.raw[i][2 * ((kk >> 1) ^ (i & 15)) + (kk & 1)],
+                        S.raw[j][2 * ((kk >> 1) ^ (j & 15)) + (kk & 1)] * S.sc[kk], s);
+              acc[u][h][t] = s;
+            }
+        }
+        __syncthreads();
+        if (bal && tid < GEMM_KC) S.bal[tid] = MMA_NOBAL;
+        if (c + 1 < nch) issue(c + 1);
+        continue;
+      }
+      if (bal && tid < GEMM_KC) S.bal[tid] = MMA_NOBAL;
+      if (c + 1 < nch) issue(c + 1);   // lands during the products; raw is free
+      const int nks = kc > 16 ? 2 : 1;
+      const uint32_t dig0 = (uint32_t)__cvta_generic_to_shared(&S.dig[0][0][0]);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int un = warp + GEMM_WARPS * u;
+        if (un >= units) break;
+        const int ra = 16 * (un / b16), cb = 16 * (un % b16);
+        const bool second = cb + 8 < nt;
+        float v[2][MMA_ND][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int d = 0; d < MMA_ND; ++d)
+#pragma unroll
+            for (int t = 0; t < 4; ++t) v[h][d][t] = 0.0f;
+        const int ar = ra + (lane & 15), br = RB + cb + (lane & 7) + ((lane >> 4) << 3);
+        for (int ks = 0; ks < nks; ++ks) {
+          const uint32_t aa = dig0 + ar * 64 + (((2 * ks + (lane >> 4)) ^ (ar >> 1)) & 3) * 16;
+          const uint32_t ba = dig0 + br * 64 + (((2 * ks + ((lane >> 3) & 1)) ^ (br >> 1)) & 3) * 16;
+          if (second) unit_products<2>(v, aa, ba, (uint32_t)sizeof(S.dig[0]), (uint32_t)sizeof(S.dig[0]));
+          else unit_products<1>(v, aa, ba, (uint32_t)sizeof(S.dig[0]), (uint32_t)sizeof(S.dig[0]));
+        }
+        const int e0 = S.ex[ra + (lane >> 2)], e1 = S.ex[ra + (lane >> 2) + 8];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (h == 1 && !second) break;
+          const int2 f = *reinterpret_cast<const int2*>(&S.ex[RB + cb + 8 * h + 2 * (lane & 3)]);
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            const long long s = join_digits(v[h], t);
+            const double sc = __hiloint2double(((t & 2) ? e1 : e0) + ((t & 1) ? f.y : f.x), 0);
+            acc[u][h][t] = fma((double)s, sc, acc[u][h][t]);
+          }
+        }
+      }
+    }
+  }
+  double* cbase = o.c_rel == GEMM_C_SPLIT ? wbase + o.c_off
+                 : o.c_rel ? (o.c_rel == 1 ? ybase : o.c_rel == 2 ? tbase : extra(o.c_rel - 3)) + o.c_off : o.C;
+  if (o.seg_count == 0) __syncthreads();   // the row tables are read below
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int un = warp + GEMM_WARPS * u;
+    if (un >= units) break;
+    const int ra = 16 * (un / b16) + (lane >> 2), cb = 16 * (un % b16) + 2 * (lane & 3);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int i = ra + 8 * (t >> 1), j = cb + 8 * h + (t & 1);
+        if (i >= mt || j >= nt) continue;
+        // a part of a split tile is dense, whatever the output's vector blocks
+        double* c = cbase + (o.c_rel == GEMM_C_SPLIT
+                                 ? (int64_t)(m0 + i) * o.ldc + n0 + j
+                                 : (int64_t)(S.vl[i].x + S.vl[RB + j].x) * o.c_vs + (int64_t)S.vl[i].y * o.ldc + S.vl[RB + j].y);
+        *c = o.accumulate ? (*c + acc[u][h][t]) : acc[u][h][t];
+      }
+  }
+}
+
+__device__ __forceinline__ double* mma_extra(const GemmExtra& ex, int i) {
+  switch (i) {
+    case 0: return ex.p[0];
+    case 1: return ex.p[1];
+    case 2: return ex.p[2];
+    case 3: return ex.p[3];
+    case 4: return ex.p[4];
+    case 5: return ex.p[5];
+    case 6: return ex.p[6];
+    default: return ex.p[7];
+  }
+}
+
+constexpr int MMA_CTAS = 3;
+
+__global__ void __launch_bounds__(GEMM_THREADS, MMA_CTAS)
+    gemm_mma_kernel(const GemmOut* __restrict__ outs, const GemmSeg* __restrict__ segs, const int3* __restrict__ tiles,
+                    int ntiles, const double* __restrict__ xbase, double* __restrict__ ybase, double* __restrict__ tbase,
+                    const GemmBases* __restrict__ multi, const GemmExtra ex, double* __restrict__ wbase) {
+  const int w = blockIdx.x;
+  if (w >= ntiles) return;
+  const int3 wi = tiles[w];
+  const GemmOut o = outs[wi.x];
+  if (multi) {
+    const GemmBases b = multi[o.inst];
+    xbase = b.x;
+    ybase = b.y;
+    tbase = b.t;
+  }
+  gemm_mma_tile(segs, wi, xbase, ybase, tbase, wbase, o, [&](int i) { return mma_extra(ex, i); });
+}
+
+__global__ void __launch_bounds__(GEMM_THREADS, MMA_CTAS)
+    gemm_mma_inst_kernel(const GemmOut* __restrict__ outs, const GemmSeg* __restrict__ segs,
+                         const int3* __restrict__ tiles, int ntiles, const __grid_constant__ GemmInstSet P, int ninst) {
+  const int w = blockIdx.x / ninst;
+  if (w >= ntiles) return;
+  const GemmInst* b = &P.b[blockIdx.x % ninst];
+  const int3 wi = tiles[w];
+  const GemmOut o = outs[wi.x];
+  gemm_mma_tile(segs, wi, b->x, b->y, b->t, nullptr, o, [&](int i) { return b->e[i]; });
+}
+
+// dynamic shared memory of the kernels, once per device
+static cudaError_t mma_smem_attr() {
+  constexpr int MAX_DEV = 64;
+  static std::atomic<int> done[MAX_DEV];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= MAX_DEV) return cudaErrorInvalidDevice;
+  if (done[dev].load(std::memory_order_acquire)) return cudaSuccess;
+  for (const void* f : {(const void*)gemm_mma_kernel, (const void*)gemm_mma_inst_kernel}) {
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MmaSmem));
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e != cudaSuccess) return e;
+  }
+  done[dev].store(1, std::memory_order_release);
+  return cudaSuccess;
+}
+
+void launch_gemm_mma(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles, const double* xbase,
+                     double* ybase, double* tbase, cudaStream_t st, const GemmBases* multi, const GemmExtra* extra,
+                     double* wbase) {
+  if (ntiles <= 0) return;
+  if (mma_smem_attr() != cudaSuccess) return;
+  const GemmExtra ex = extra ? *extra : GemmExtra{};
+  gemm_mma_kernel<<<ntiles, GEMM_THREADS, sizeof(MmaSmem), st>>>(outs, segs, tiles, ntiles, xbase, ybase, tbase, multi,
+                                                                ex, wbase);
+}
+
+void launch_gemm_mma_inst(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles,
+                          const GemmInstSet& bases, int ninst, cudaStream_t st) {
+  if (ntiles <= 0 || ninst <= 0) return;
+  if (mma_smem_attr() != cudaSuccess) return;
+  gemm_mma_inst_kernel<<<(unsigned)((long long)ntiles * ninst), GEMM_THREADS, sizeof(MmaSmem), st>>>(
+      outs, segs, tiles, ntiles, bases, ninst);
+}
+
+}  // namespace lrt

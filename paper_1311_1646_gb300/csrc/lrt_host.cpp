@@ -722,9 +722,25 @@ struct GemmPlan {
   int nsplit = 0;
   DevBuf ws;                 // partial tiles of the split tiles
   double flops = 0.0;
+  bool mma = false;          // tiles of the digit-product kernel
   void run(cudaStream_t st, const double* xb, double* yb, double* tb = nullptr, const GemmExtra* ex = nullptr) const {
-    launch_gemm_fp64(outs.p, segs.p, tiles.p, ntiles, xb, yb, tb, st, ex, ws.p);
+    if (mma)
+      launch_gemm_mma(outs.p, segs.p, tiles.p, ntiles, xb, yb, tb, st, nullptr, ex, ws.p);
+    else
+      launch_gemm_fp64(outs.p, segs.p, tiles.p, ntiles, xb, yb, tb, st, ex, ws.p);
     if (nsplit > 0) launch_split_reduce(outs.p, splits.p, nsplit, ws.p, yb, tb, st);
+  }
+  void run_inst(cudaStream_t st, const GemmInstSet& B, int n) const {
+    if (mma)
+      launch_gemm_mma_inst(outs.p, segs.p, tiles.p, ntiles, B, n, st);
+    else
+      launch_gemm_fp64_inst(outs.p, segs.p, tiles.p, ntiles, B, n, st);
+  }
+  void run_multi(cudaStream_t st, const GemmBases* bases) const {
+    if (mma)
+      launch_gemm_mma(outs.p, segs.p, tiles.p, ntiles, nullptr, nullptr, nullptr, st, bases, nullptr, nullptr);
+    else
+      launch_gemm_fp64_multi(outs.p, segs.p, tiles.p, ntiles, bases, st);
   }
   int launches() const { return (ntiles > 0) + (nsplit > 0); }
 };
@@ -741,6 +757,51 @@ static void build_gather(GatherPlan& P, std::vector<GatherTask>& tasks, std::vec
   P.srcs.upload(srcs, st);
   P.tiles.upload(tiles, st);
   P.ntiles = (int)tiles.size();
+}
+
+// Tile of the digit-product kernel for one output: a x b units of 16 x 16 with a + b <= 6
+// (MMA_ROWS) and a b <= 8, the shorter side whole where it fits, both sides cut evenly.  The
+// columns of a balanced output are cut by their own count only, so that a column sees the
+// same neighbours whatever the rows (the vectors of the call) are.
+static void mma_tile_shape(const GemmOut& O, int& tm, int& tn) {
+  const int m16 = (O.m + 15) / 16, n16 = (O.n + 15) / 16;
+  auto even = [](int n, int u, int step) {   // n in parts of at most u units of 16
+    const int parts = (n + 16 * u - 1) / (16 * u);
+    const int w = (n + parts - 1) / parts;
+    return (w + step - 1) / step * step;
+  };
+  if (O.balance || n16 < m16) {
+    tn = even(O.n, std::min(n16, 4), 8);
+    const int b = (tn + 15) / 16;
+    tm = even(O.m, std::min(6 - b, 8 / b), 16);
+  } else {
+    tm = even(O.m, std::min(m16, 4), 16);
+    const int a = (tm + 15) / 16;
+    tn = even(O.n, std::min(6 - a, 8 / a), 8);
+  }
+}
+
+// Whether a list runs as digit products: the work padded to 16 x 8 x 16 is at most three
+// times the exact work (the FP64 FMA kernel pays no padding).  Measured both ways: padding
+// 2.0 / 1.6 (phase 1 / 2; k = 24, M = 300, site 4) 745 -> 480 us, 2.0 / 1.9 (PPP k = 12,
+// M = 256) 174 -> 127 us, but 4 / 3 (eight molecules of 8 to 12 orbitals) 1.67 -> 2.08 ms.
+// Counted per vector, so that a call's kernel, and with it every bit of a vector's result,
+// does not depend on how many vectors the call has.
+static bool use_mma(const std::vector<GemmOut>& outs, const std::vector<GemmSeg>& segs, const std::vector<int64_t>& ktot) {
+  double exact = 0.0, padded = 0.0;
+  for (size_t i = 0; i < outs.size(); ++i) {
+    const GemmOut& o = outs[i];
+    for (int q = 0; q < o.seg_count; ++q) {
+      const GemmSeg& g = segs[o.seg_begin + q];
+      if (g.a_vr != o.c_vr || g.b_vc != o.c_vc) return false;
+      // the kernel's row offsets are 32-bit byte strides
+      if (std::max(g.a_vs, g.b_vs) >= ((int64_t)1 << 29) || std::max(g.lda, g.ldb) >= (1 << 28)) return false;
+    }
+    const int m = o.c_vr > 0 ? o.c_vr : o.m, n = o.c_vc > 0 ? o.c_vc : o.n;
+    exact += (double)m * n * ktot[i];
+    padded += (double)((m + 15) / 16 * 16) * ((n + 7) / 8 * 8) * ((ktot[i] + 15) / 16 * 16);
+  }
+  return padded <= 3.0 * exact;
 }
 
 static void build_gemm(GemmPlan& P, const std::vector<GemmOut>& outs_in, const std::vector<GemmSeg>& segs,
@@ -765,23 +826,36 @@ static void build_gemm(GemmPlan& P, const std::vector<GemmOut>& outs_in, const s
       ktot[i] += segs[outs_in[i].seg_begin + s].k;
       fl += 2.0 * outs_in[i].m * (double)outs_in[i].n * segs[outs_in[i].seg_begin + s].k;
     }
-  auto cost = [](int64_t mt, int64_t nt, int64_t k) {
-    return ((k + GEMM_KC - 1) / GEMM_KC) * (32 * ((mt * nt + 31) / 32) + 64) + 64;
+  const bool mma = use_mma(outs_in, segs, ktot);
+  auto cost = [mma](int64_t mt, int64_t nt, int64_t k) {
+    const int64_t nch = (k + GEMM_KC - 1) / GEMM_KC;
+    if (mma) return nch * (30 * ((mt + 15) / 16) * ((nt + 15) / 16) + 12 * ((mt + 15) / 16 + (nt + 15) / 16) + 20) + 40;
+    return nch * (32 * ((mt * nt + 31) / 32) + 64) + 64;
+  };
+  auto shape = [mma](const GemmOut& O, int& tm, int& tn) {
+    tm = GEMM_TM;
+    tn = GEMM_TN;
+    if (mma) mma_tile_shape(O, tm, tn);
   };
   int64_t total = 0;
-  for (size_t i = 0; i < outs_in.size(); ++i)
-    for (int m0 = 0; m0 < outs_in[i].m; m0 += GEMM_TM)
-      for (int n0 = 0; n0 < outs_in[i].n; n0 += GEMM_TN)
-        total += cost(std::min(GEMM_TM, outs_in[i].m - m0), std::min(GEMM_TN, outs_in[i].n - n0), ktot[i]);
+  for (size_t i = 0; i < outs_in.size(); ++i) {
+    int TM, TN;
+    shape(outs_in[i], TM, TN);
+    for (int m0 = 0; m0 < outs_in[i].m; m0 += TM)
+      for (int n0 = 0; n0 < outs_in[i].n; n0 += TN)
+        total += cost(std::min(TM, outs_in[i].m - m0), std::min(TN, outs_in[i].n - n0), ktot[i]);
+  }
   const int64_t cap = std::max<int64_t>(1, total / gemm_fp64_slots());
   std::vector<std::pair<int64_t, int3>> tl;
   std::vector<SplitTile> sp;
   int64_t wsz = 0;
   for (size_t i = 0; i < outs_in.size(); ++i) {
     const GemmOut& O = outs_in[i];
-    for (int m0 = 0; m0 < O.m; m0 += GEMM_TM)
-      for (int n0 = 0; n0 < O.n; n0 += GEMM_TN) {
-        const int mt = std::min(GEMM_TM, O.m - m0), nt = std::min(GEMM_TN, O.n - n0);
+    int TM, TN;
+    shape(O, TM, TN);
+    for (int m0 = 0; m0 < O.m; m0 += TM)
+      for (int n0 = 0; n0 < O.n; n0 += TN) {
+        const int mt = std::min(TM, O.m - m0), nt = std::min(TN, O.n - n0);
         const int64_t c = cost(mt, nt, ktot[i]);
         const int want = (int)std::min<int64_t>(O.seg_count, ktot[i] / GEMM_SPLIT_K);
         if (split && want >= 2 && O.c_rel <= 2 && outs.size() < (size_t)INT32_MAX) {
@@ -796,7 +870,7 @@ static void build_gemm(GemmPlan& P, const std::vector<GemmOut>& outs_in, const s
             po.c_off = wsz + (int64_t)t.nparts * mt * nt - ((int64_t)m0 * nt + n0);
             po.ldc = nt;
             po.accumulate = 0;
-            po.c_vr = po.c_vc = 0;
+            if (!mma) po.c_vr = po.c_vc = 0;   // the digit-product kernel reads its operands' blocks here
             po.c_vs = 0;
             po.seg_begin = O.seg_begin + sb;
             po.seg_count = se - sb;
@@ -808,7 +882,7 @@ static void build_gemm(GemmPlan& P, const std::vector<GemmOut>& outs_in, const s
           sp.push_back(t);
           continue;
         }
-        const int parts = (int)std::min<int64_t>(mt, (c + cap - 1) / cap);
+        const int parts = mma ? 1 : (int)std::min<int64_t>(mt, (c + cap - 1) / cap);
         for (int p = 0, r = m0; p < parts; ++p) {
           const int rows = mt / parts + (p < mt % parts ? 1 : 0);
           tl.push_back({cost(rows, nt, ktot[i]), gemm_tile((int)i, r, rows, n0, nt)});
@@ -830,6 +904,7 @@ static void build_gemm(GemmPlan& P, const std::vector<GemmOut>& outs_in, const s
   P.nsplit = (int)sp.size();
   if (wsz > 0) P.ws.ensure((size_t)wsz);
   P.flops = fl;
+  P.mma = mma;
 }
 
 }  // namespace lrt
@@ -1379,8 +1454,8 @@ static void ren_run(lrt_ctx* c, std::vector<GemmOut>& o1, std::vector<GemmSeg>& 
   double* tmp = nullptr;
   if (toff > 0 && dev_alloc((void**)&tmp, (size_t)toff * sizeof(double)) != cudaSuccess)
     throw Error(LRT_ENOMEM, "renormalize workspace");
-  launch_gemm_fp64(p1->outs.p, p1->segs.p, p1->tiles.p, p1->ntiles, nullptr, nullptr, tmp, c->st, &ex);
-  launch_gemm_fp64(p2->outs.p, p2->segs.p, p2->tiles.p, p2->ntiles, nullptr, nullptr, tmp, c->st, &ex);
+  p1->run(c->st, nullptr, nullptr, tmp, &ex);
+  p2->run(c->st, nullptr, nullptr, tmp, &ex);
   CK(cudaGetLastError());
   if (tmp) dev_free(tmp);
   if (tpl) {
@@ -1401,10 +1476,8 @@ static std::unique_ptr<OpSet> ren_replay(lrt_ctx* c, RenTemplate* tpl, uint64_t 
   double* tmp = nullptr;
   if (tpl->toff > 0 && dev_alloc((void**)&tmp, (size_t)tpl->toff * sizeof(double)) != cudaSuccess)
     throw Error(LRT_ENOMEM, "renormalize workspace");
-  const GemmPlan& p1 = *tpl->p1;
-  const GemmPlan& p2 = *tpl->p2;
-  launch_gemm_fp64(p1.outs.p, p1.segs.p, p1.tiles.p, p1.ntiles, nullptr, nullptr, tmp, c->st, &ex);
-  launch_gemm_fp64(p2.outs.p, p2.segs.p, p2.tiles.p, p2.ntiles, nullptr, nullptr, tmp, c->st, &ex);
+  tpl->p1->run(c->st, nullptr, nullptr, tmp, &ex);
+  tpl->p2->run(c->st, nullptr, nullptr, tmp, &ex);
   CK(cudaGetLastError());
   if (tmp) dev_free(tmp);
   return N;
@@ -1924,6 +1997,7 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
     }
     const int m1 = XF.dim[fx][os.r];
     GemmOut y{nullptr, coff, w.cols, m1 * nvec, ncols, (int)S2.size(), (int)seg2[u].size(), 0, 1};
+    y.balance = 1;
     if (vb) {
       y.c_vr = m1;
       y.c_vs = nelem;
@@ -3805,8 +3879,8 @@ struct TdaRunner {
   // one kept two-phase plan over instances: per instance x, y, workspace offset and extras
   void run_inst(const GemmPlan& p1, const GemmPlan& p2, int n, const GemmInstSet& B) {
     inst_check(std::max(p1.ntiles, p2.ntiles), n);
-    launch_gemm_fp64_inst(p1.outs.p, p1.segs.p, p1.tiles.p, p1.ntiles, B, n, c->st);
-    launch_gemm_fp64_inst(p2.outs.p, p2.segs.p, p2.tiles.p, p2.ntiles, B, n, c->st);
+    p1.run_inst(c->st, B, n);
+    p2.run_inst(c->st, B, n);
     CK(cudaGetLastError());
   }
   // out.v(mu) = [H_mu^{L_{i-1}} x h_i x H_0^{R_i}] C0_i for every mu with a first-order set
@@ -5347,8 +5421,8 @@ static void batch_issue(lrt_ctx* c0, BatchPlan& B, const std::vector<SigmaPlan*>
     launch_gemm_tf32x3(B.tci1.p, B.tcb1.p, B.tcn1, B.tn1, to, c0->derr, st);
     launch_gemm_tf32x3(B.tci2.p, B.tcb2.p, B.tcn2, B.tn2, to, c0->derr, st);
   } else {
-    launch_gemm_fp64_multi(B.p1.outs.p, B.p1.segs.p, B.p1.tiles.p, B.p1.ntiles, B.bases.p, st);
-    launch_gemm_fp64_multi(B.p2.outs.p, B.p2.segs.p, B.p2.tiles.p, B.p2.ntiles, B.bases.p, st);
+    B.p1.run_multi(st, B.bases.p);
+    B.p2.run_multi(st, B.bases.p);
   }
 }
 

@@ -45,6 +45,8 @@ struct GemmOut {
   int inst;      // batched launches: index of the instance whose bases the rel pointers use
   int c_vr, c_vc;
   int64_t c_vs;
+  int balance;   // digit products (launch_gemm_mma): K positions are first scaled to equal
+                 // exponents over op(B)'s columns (an output that sums many operators)
 };
 struct GemmSeg {
   const double* A;
@@ -97,9 +99,21 @@ constexpr int GEMM_NEXTRA = 8;
 struct GemmExtra {
   double* p[GEMM_NEXTRA];
 };
+struct GemmBases {
+  const double* x;
+  double* y;
+  double* t;
+};
 void launch_gemm_fp64(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles,
                       const double* xbase, double* ybase, double* tbase, cudaStream_t st,
                       const GemmExtra* extra = nullptr, double* wbase = nullptr);
+// Tensor-core form of the FP64 GEMM (exact digit products, lrt_fp64_mma.cu): the same lists
+// with tiles of at most MMA_ROWS rows and columns together, both rounded up to 16, and 8
+// 16 x 16 units; the segments' vector blocks are the output's (a_vr = c_vr, b_vc = c_vc).
+constexpr int MMA_ROWS = 96;
+void launch_gemm_mma(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles, const double* xbase,
+                     double* ybase, double* tbase, cudaStream_t st, const GemmBases* multi, const GemmExtra* extra,
+                     double* wbase);
 // Split K: an output tile whose segment list is long is cut into parts, each a contiguous
 // run of its segments written as a partial tile (c_rel GEMM_C_SPLIT: wbase + c_off, row
 // stride nt) into the plan's workspace; split_reduce then adds the parts in order and
@@ -115,11 +129,6 @@ struct SplitTile {
 void launch_split_reduce(const GemmOut* outs, const SplitTile* tiles, int ntiles, const double* wbase, double* ybase,
                          double* tbase, cudaStream_t st);
 // batched form: the bases of output o are bases[o.inst] (device array)
-struct GemmBases {
-  const double* x;
-  double* y;
-  double* t;
-};
 void launch_gemm_fp64_multi(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles,
                             const GemmBases* bases, cudaStream_t st);
 // One plan replayed over up to GEMM_MAX_INST instances in one launch: CTA b runs tile
@@ -139,6 +148,8 @@ struct GemmInstSet {
 };
 void launch_gemm_fp64_inst(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles,
                            const GemmInstSet& bases, int ninst, cudaStream_t st);
+void launch_gemm_mma_inst(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles,
+                          const GemmInstSet& bases, int ninst, cudaStream_t st);
 void launch_diag(const DiagOut* outs, const DiagTerm* terms, int nouts, double* dbase, cudaStream_t st);
 
 // Split-TF32 tensor-core variant of the grouped GEMM.
