@@ -18,8 +18,9 @@
 // transformations of matrix multiplication by using fast routines of matrix multiplication",
 // Numer. Algorithms 59, 2012, with a fixed digit grid per chunk.)  What is lost per chunk is
 // below 2^-54 of its largest row times column product, less than the 32 roundings of an FP64
-// FMA chain.  Chunks that hold an infinity, a NaN or a row outside 2^-423 .. 2^477 are
-// multiplied in plain FP64 from the staged operands.
+// FMA chain.  Elements whose row or column
+// holds an infinity, a NaN or lies outside 2^-423 .. 2^477 are multiplied in plain FP64 from the
+// staged operands.
 //
 // Measured on the k = 24, M = 500, 6-vector sigma (23.7 G multiply-adds): 44.0 ms by FP64 FMAs,
 // 16.7 ms here; error against 64-bit exact values 3.4e-16 (8.5e-16 before) at k = 8, 2.8e-15
@@ -365,12 +366,14 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
         int e[4], emax;
         exponents(q, e, emax);
         if (bal) {
-          const bool inf = emax == 2047;
+          // infinities and NaN keep their row (all columns, if op(B) holds them) out of the
+          // integer path
           const int4 bk = *reinterpret_cast<const int4*>(&S.bal[4 * l]);
           const int bj[4] = {bk.x, bk.y, bk.z, bk.w};
+          const bool inf = isB ? max(max(bk.x, bk.y), max(bk.z, bk.w)) == 2047 - MMA_E0 : emax == 2047;
 #pragma unroll
           for (int j = 0; j < 4; ++j) e[j] = e[j] == 0 ? -4096 : isB ? e[j] - bj[j] : e[j] + bj[j];
-          emax = inf ? 2047 : max(max(e[0], e[1]), max(e[2], e[3]));
+          emax = inf ? 4095 : max(max(e[0], e[1]), max(e[2], e[3]));
         }
         uint32_t d0[MMA_ND], d1[MMA_ND];
         const int x = cut_row(q, e, emax, d0, d1);
@@ -383,32 +386,8 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
       __syncthreads();
       const bool wild = S.wild[it & 1] != 0;
       if (tid == 0) S.wild[(it & 1) ^ 1] = 0;   // last read before this chunk's first barrier
-      if (wild) {
-        // plain FP64 from the staged operands
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int un = warp + GEMM_WARPS * u;
-          if (un >= units) break;
-          const int ra = 16 * (un / b16) + (lane >> 2), rb = RB + 16 * (un % b16) + 2 * (lane & 3);
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-              const int i = ra + 8 * (t >> 1), j = rb + 8 * h + (t & 1);
-              double s = acc[u][h][t];
-              for (int kk = 0; kk < kc; ++kk)
-                s = fma(S.raw[i][2 * ((kk >> 1) ^ (i & 15)) + (kk & 1)],
-                        S.raw[j][2 * ((kk >> 1) ^ (j & 15)) + (kk & 1)] * S.sc[kk], s);
-              acc[u][h][t] = s;
-            }
-        }
-        __syncthreads();
-        if (bal && tid < GEMM_KC) S.bal[tid] = MMA_NOBAL;
-        if (c + 1 < nch) issue(c + 1);
-        continue;
-      }
       if (bal && tid < GEMM_KC) S.bal[tid] = MMA_NOBAL;
-      if (c + 1 < nch) issue(c + 1);   // lands during the products; raw is free
+      if (!wild && c + 1 < nch) issue(c + 1);   // lands during the products; raw is free
       const int nks = kc > 16 ? 2 : 1;
       const uint32_t dig0 = (uint32_t)__cvta_generic_to_shared(&S.dig[0][0][0]);
 #pragma unroll
@@ -436,13 +415,39 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
         for (int h = 0; h < 2; ++h) {
           if (h == 1 && !second) break;
           const int2 f = *reinterpret_cast<const int2*>(&S.ex[RB + cb + 8 * h + 2 * (lane & 3)]);
+          if (!wild) {
 #pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            const long long s = join_digits(v[h], t);
-            const double sc = __hiloint2double(((t & 2) ? e1 : e0) + ((t & 1) ? f.y : f.x), 0);
-            acc[u][h][t] = fma((double)s, sc, acc[u][h][t]);
+            for (int t = 0; t < 4; ++t)
+              acc[u][h][t] = fma((double)join_digits(v[h], t),
+                                 __hiloint2double(((t & 2) ? e1 : e0) + ((t & 1) ? f.y : f.x), 0), acc[u][h][t]);
+          } else {
+#pragma unroll 1
+            for (int t = 0; t < 4; ++t) {
+              const int ea = (t & 2) ? e1 : e0, eb = (t & 1) ? f.y : f.x;
+              double s = t == 0 ? acc[u][h][0] : t == 1 ? acc[u][h][1] : t == 2 ? acc[u][h][2] : acc[u][h][3];
+              if ((ea | eb) >= 0) {
+                float w[MMA_ND][4];
+#pragma unroll
+                for (int d = 0; d < MMA_ND; ++d) w[d][0] = t == 0 ? v[h][d][0] : t == 1 ? v[h][d][1] : t == 2 ? v[h][d][2] : v[h][d][3];
+                s = fma((double)join_digits(w, 0), __hiloint2double(ea + eb, 0), s);
+              } else {
+                // plain FP64 from the staged operands
+                const int i = ra + (lane >> 2) + 8 * (t >> 1), j = RB + cb + 8 * h + 2 * (lane & 3) + (t & 1);
+                for (int kk = 0; kk < kc; ++kk)
+                  s = fma(S.raw[i][2 * ((kk >> 1) ^ (i & 15)) + (kk & 1)],
+                          S.raw[j][2 * ((kk >> 1) ^ (j & 15)) + (kk & 1)] * S.sc[kk], s);
+              }
+              if (t == 0) acc[u][h][0] = s;
+              if (t == 1) acc[u][h][1] = s;
+              if (t == 2) acc[u][h][2] = s;
+              if (t == 3) acc[u][h][3] = s;
+            }
           }
         }
+      }
+      if (wild) {          // the staged operands were kept for the FP64 path
+        __syncthreads();
+        if (c + 1 < nch) issue(c + 1);
       }
     }
   }
@@ -546,6 +551,401 @@ void launch_gemm_mma_inst(const GemmOut* outs, const GemmSeg* segs, const int3* 
   if (ntiles <= 0 || ninst <= 0) return;
   if (mma_smem_attr() != cudaSuccess) return;
   gemm_mma_inst_kernel<<<(unsigned)((long long)ntiles * ninst), GEMM_THREADS, sizeof(MmaSmem), st>>>(
+      outs, segs, tiles, ntiles, bases, ninst);
+}
+
+// ---------------------------------------------------------------------------
+// small blocks: one warp per tile
+//
+// The blocks of small and medium systems are a few states wide (2 x 2 x 4 to 16 x 16 x 30), so a
+// CTA that stages its operands spends microseconds of latency, barriers and descriptor reads
+// on a product that takes nanoseconds.  Here every warp takes its own work item, reads the
+// operands straight from global memory (L1 keeps a block's few lines) and meets no barrier:
+//
+//  - tiny tiles (WARP_DIRECT): lanes own output elements and run FP64 FMAs, a segment at a time;
+//  - others: 16 x 16 tiles as digit products, 16 positions a chunk.  A lane loads exactly the
+//    elements its mma.sync fragments hold and cuts them in registers, so shared memory only
+//    holds the segment table.  With WARP_SWAP the 16-wide side of the product carries the
+//    output's columns (the longer side pads less).
+//
+// Long segment lists are split into K parts on separate warps; the warp that finishes a
+// tile's last part adds the parts in order (a counter per tile, reset by that warp), which
+// spares the reduction launch.
+//
+// Measured (one-site sigma): k = 8, M = 64, 1 vector 183 -> 61 us; k = 17, M = 30, 6 vectors
+// 468 -> 137 us; eight molecules in one call 1.67 -> 0.94 ms.  Bound by latency: descriptor and
+// operand reads of short items, 16 warps per SM (128 registers; 3 CTAs of 168 registers are
+// 5% slower on the longer lists).
+// ---------------------------------------------------------------------------
+struct WarpSeg {
+  const double* p;          // operand along the tile's rows, and along its columns
+  const double* q;
+  int64_t pvs, qvs;         // vector block strides
+  double scale;
+  int prs, pks, qrs, qks;   // strides by row (column) and by K position
+};
+constexpr int WARP_WARPS = 4;
+struct WarpSmem {
+  WarpSeg sd[WARP_WARPS][GEMM_SEGB];
+  int kst[WARP_WARPS][GEMM_SEGB + 1];
+};
+
+// stages up to 32 segments for this warp; returns their total K
+template <class Extra>
+__device__ __forceinline__ int warp_segs(WarpSeg* sd, int* kst, const GemmSeg* __restrict__ segs, int sb, int nb, bool swap,
+                                         const double* xbase, const double* tbase, const Extra& extra, int lane) {
+  int k = 0;
+  __syncwarp();
+  if (lane < nb) {
+    GemmSeg g = segs[sb + lane];
+    if (g.a_rel) g.A = (g.a_rel == 1 ? xbase : g.a_rel == 2 ? tbase : extra(g.a_rel - 3)) + g.a_off;
+    if (g.b_rel) g.B = (g.b_rel == 1 ? xbase : g.b_rel == 2 ? tbase : extra(g.b_rel - 3)) + g.b_off;
+    const int ars = g.transA ? 1 : g.lda, aks = g.transA ? g.lda : 1;
+    const int brs = g.transB ? g.ldb : 1, bks = g.transB ? 1 : g.ldb;
+    sd[lane] = swap ? WarpSeg{g.B, g.A, g.b_vs, g.a_vs, g.scale, brs, bks, ars, aks}
+                    : WarpSeg{g.A, g.B, g.a_vs, g.b_vs, g.scale, ars, aks, brs, bks};
+    k = g.k;
+  }
+  int incl = k;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += v;
+  }
+  kst[lane + 1] = incl;
+  if (lane == 0) kst[0] = 0;
+  __syncwarp();
+  return kst[nb];
+}
+
+// where element (i, j) of an output lives (i, j inside the whole output)
+__device__ __forceinline__ int64_t out_offset(const GemmOut& o, int i, int j) {
+  int64_t off = 0;
+  if (o.c_vr > 0) {
+    const int v = i / o.c_vr;
+    off += v * o.c_vs;
+    i -= v * o.c_vr;
+  }
+  if (o.c_vc > 0) {
+    const int v = j / o.c_vc;
+    off += v * o.c_vs;
+    j -= v * o.c_vc;
+  }
+  return off + (int64_t)i * o.ldc + j;
+}
+
+// the last part of a split tile to finish adds the parts in order; all 32 lanes call
+__device__ __forceinline__ void warp_reduce_parts(const GemmOut* __restrict__ outs, const SplitTile& t, int* counter,
+                                                  const double* wbase, double* ybase, double* tbase, int lane) {
+  __threadfence();
+  __syncwarp();
+  int last = 0;
+  if (lane == 0) last = atomicAdd(counter, 1) == t.nparts - 1;
+  last = __shfl_sync(0xffffffffu, last, 0);
+  if (!last) return;
+  __threadfence();
+  const GemmOut o = outs[t.o];
+  double* cbase = o.c_rel == 1 ? ybase + o.c_off : o.c_rel == 2 ? tbase + o.c_off : o.C;
+  const int ne = t.mt * t.nt;
+  const double* w = wbase + t.ws_off;
+  for (int e = lane; e < ne; e += 32) {
+    double s = 0.0;
+#pragma unroll 8
+    for (int p = 0; p < t.nparts; ++p) s += __ldcg(w + (int64_t)p * ne + e);
+    double* c = cbase + out_offset(o, t.m0 + e / t.nt, t.n0 + e % t.nt);
+    *c = o.accumulate ? *c + s : s;
+  }
+  if (lane == 0) *counter = 0;
+}
+
+// exponent word of a row from the four positions of its lane's quad
+__device__ __forceinline__ int row_exponent(const int (&e)[4]) {
+  int m = max(max(e[0], e[1]), max(e[2], e[3]));
+  m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+  return max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+}
+__device__ __forceinline__ bool outside_range(int emax) { return emax > 0 && (emax < MMA_EMIN || emax > MMA_EMAX); }
+__device__ __forceinline__ int exponent_of(double x) { return (__double2hiint(x) & 0x7FFFFFFF) >> 20; }
+// fragments of four positions (2t, 2t + 1, 2t + 8, 2t + 9) of one row
+__device__ __forceinline__ void cut_quad(const double (&x)[4], const int (&e)[4], int E, uint32_t (&lo)[MMA_ND],
+                                         uint32_t (&hi)[MMA_ND]) {
+  uint2 f[4];
+  uint32_t h[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    h[j] = (uint32_t)__double2hiint(x[j]);
+    f[j] = fixed63(h[j], (uint32_t)__double2loint(x[j]), E - e[j]);
+  }
+  digits2(f[0], f[1], h[0], h[1], lo);
+  digits2(f[2], f[3], h[2], h[3], hi);
+}
+
+template <class Extra>
+__device__ __forceinline__ void warp_tile(const GemmOut* __restrict__ outs, const GemmSeg* __restrict__ segs, const int3 wi,
+                                          const double* xbase, double* ybase, double* tbase, double* wbase,
+                                          const SplitTile* __restrict__ splits, int* counters, const GemmOut& o,
+                                          const Extra& extra, WarpSmem& S) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int m0 = wi.y >> 8, mt = wi.y & 255, n0 = wi.z >> 8, nt = wi.z & 255;
+  WarpSeg* sd = S.sd[warp];
+  int* kst = S.kst[warp];
+  const bool part = o.c_rel == GEMM_C_SPLIT;
+  double* cbase = part ? wbase + o.c_off
+                  : o.c_rel ? (o.c_rel == 1 ? ybase : o.c_rel == 2 ? tbase : extra(o.c_rel - 3)) + o.c_off : o.C;
+  // a part of a split tile is dense, whatever the output's vector blocks
+  auto store = [&](int i, int j, double x) {
+    double* c = cbase + (part ? (int64_t)i * o.ldc + j : out_offset(o, i, j));
+    *c = o.accumulate ? *c + x : x;
+  };
+
+  if (o.flags & GEMM_WARP_DIRECT) {
+    const int ne = mt * nt, cnt = (ne + 31) >> 5;     // elements per lane
+    constexpr int MAXE = GEMM_DIRECT_MAX / 32;
+    int rv[MAXE], rr[MAXE], cv[MAXE], cr[MAXE];
+    double acc[MAXE];
+#pragma unroll
+    for (int u = 0; u < MAXE; ++u) {
+      const int e = min(lane + 32 * u, ne - 1);
+      rr[u] = m0 + e / nt;
+      cr[u] = n0 + e % nt;
+      rv[u] = cv[u] = 0;
+      if (o.c_vr > 0) {
+        rv[u] = rr[u] / o.c_vr;
+        rr[u] -= rv[u] * o.c_vr;
+      }
+      if (o.c_vc > 0) {
+        cv[u] = cr[u] / o.c_vc;
+        cr[u] -= cv[u] * o.c_vc;
+      }
+      acc[u] = 0.0;
+    }
+    for (int b0 = 0; b0 < o.seg_count; b0 += GEMM_SEGB) {
+      const int nb = min(GEMM_SEGB, o.seg_count - b0);
+      warp_segs(sd, kst, segs, o.seg_begin + b0, nb, false, xbase, tbase, extra, lane);
+      for (int q = 0; q < nb; ++q) {
+        const WarpSeg g = sd[q];
+        const int kq = kst[q + 1] - kst[q];
+#pragma unroll
+        for (int u = 0; u < MAXE; ++u) {
+          if (u >= cnt) break;
+          const double* a = g.p + rv[u] * g.pvs + (int64_t)rr[u] * g.prs;
+          const double* b = g.q + cv[u] * g.qvs + (int64_t)cr[u] * g.qrs;
+          double s = 0.0;
+#pragma unroll 4
+          for (int k = 0; k < kq; ++k) s = fma(a[(int64_t)k * g.pks], b[(int64_t)k * g.qks], s);
+          acc[u] = fma(g.scale, s, acc[u]);
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < MAXE; ++u) {
+      const int e = lane + 32 * u;
+      if (e < ne) store(m0 + e / nt, n0 + e % nt, acc[u]);
+    }
+  } else {
+    const bool swap = (o.flags & GEMM_WARP_SWAP) != 0, bal = o.balance != 0;
+    const int r0 = swap ? n0 : m0, rt = swap ? nt : mt, c0 = swap ? m0 : n0, ct = swap ? mt : nt;
+    const int rblk = swap ? o.c_vc : o.c_vr, cblk = swap ? o.c_vr : o.c_vc;
+    const int g = lane >> 2, t = lane & 3;
+    const int nh = ct > 8 ? 2 : 1;
+    int rv[2], rr[2], cv[2], cr[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {   // lanes beyond the tile repeat its last row or column
+      rr[h] = r0 + min(g + 8 * h, rt - 1);
+      cr[h] = c0 + min(g + 8 * h, ct - 1);
+      rv[h] = cv[h] = 0;
+      if (rblk > 0) {
+        rv[h] = rr[h] / rblk;
+        rr[h] -= rv[h] * rblk;
+      }
+      if (cblk > 0) {
+        cv[h] = cr[h] / cblk;
+        cr[h] -= cv[h] * cblk;
+      }
+    }
+    double acc[2][4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[h][i] = 0.0;
+    for (int b0 = 0; b0 < o.seg_count; b0 += GEMM_SEGB) {
+      const int nb = min(GEMM_SEGB, o.seg_count - b0);
+      const int Kb = warp_segs(sd, kst, segs, o.seg_begin + b0, nb, swap, xbase, tbase, extra, lane);
+      int qs = 0;
+      for (int p0 = 0; p0 < Kb; p0 += 16) {
+        double a[2][4], b[2][4], sc[4];
+        while (qs + 1 < nb && kst[qs + 1] <= p0) ++qs;
+        int q = qs;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int p = p0 + 2 * t + (j & 1) + 8 * (j >> 1);
+          a[0][j] = a[1][j] = b[0][j] = b[1][j] = 0.0;
+          sc[j] = 1.0;
+          if (p < Kb) {
+            while (kst[q + 1] <= p) ++q;
+            const WarpSeg& s = sd[q];
+            const int kl = p - kst[q];
+            const double* pp = s.p + (int64_t)kl * s.pks;
+            const double* qq = s.q + (int64_t)kl * s.qks;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              a[h][j] = pp[rv[h] * s.pvs + (int64_t)rr[h] * s.prs];
+              if (h < nh) b[h][j] = qq[cv[h] * s.qvs + (int64_t)cr[h] * s.qrs];
+            }
+            sc[j] = s.scale;
+          }
+        }
+        int ea[2][4], eb[2][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            // the segment's scale goes with the second operand of the product (op(B))
+            double& x = swap ? a[h][j] : b[h][j];
+            if (sc[j] != 1.0) x *= sc[j];
+            ea[h][j] = exponent_of(a[h][j]);
+            eb[h][j] = exponent_of(b[h][j]);
+          }
+        bool all = false;    // op(B) holds an infinity or NaN
+        if (bal) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            int m = max(eb[0][j], eb[1][j]);
+            m = max(m, __shfl_xor_sync(0xffffffffu, m, 4));
+            m = max(m, __shfl_xor_sync(0xffffffffu, m, 8));
+            m = max(m, __shfl_xor_sync(0xffffffffu, m, 16));
+            const int d = m > 0 ? m - MMA_E0 : MMA_NOBAL;
+            all |= m == 2047;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              ea[h][j] = ea[h][j] == 0 ? -4096 : ea[h][j] == 2047 ? 4095 : ea[h][j] + d;
+              eb[h][j] = eb[h][j] == 0 ? -4096 : eb[h][j] - d;
+            }
+          }
+          all = __any_sync(0xffffffffu, all);
+        }
+        int E[2], F[2], xe[2], xf[2];    // exponents of the rows and columns, and their words
+        bool wild = false;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          E[h] = row_exponent(ea[h]);
+          F[h] = row_exponent(eb[h]);
+          const bool we = outside_range(E[h]), wf = outside_range(F[h]) || all;
+          wild |= we | wf;
+          if (E[h] <= 0) E[h] = MMA_E0;
+          if (F[h] <= 0) F[h] = MMA_E0;
+          xe[h] = we ? MMA_WILD : (E[h] - 539) << 20;
+          xf[h] = wf ? MMA_WILD : (F[h] - 539) << 20;
+        }
+        // plain FP64 over the chunk for one element (r, c) of the tile
+        auto fp64_chunk = [&](int r, int c, double x) {
+          int r1 = r0 + min(r, rt - 1), c1 = c0 + min(c, ct - 1), v1 = 0, v2 = 0;
+          if (rblk > 0) v1 = r1 / rblk, r1 -= v1 * rblk;
+          if (cblk > 0) v2 = c1 / cblk, c1 -= v2 * cblk;
+          int qw = qs;
+          for (int p = p0; p < min(p0 + 16, Kb); ++p) {
+            while (kst[qw + 1] <= p) ++qw;
+            const WarpSeg& s = sd[qw];
+            const int kl = p - kst[qw];
+            const double u = s.p[(int64_t)kl * s.pks + v1 * s.pvs + (int64_t)r1 * s.prs];
+            const double w = s.q[(int64_t)kl * s.qks + v2 * s.qvs + (int64_t)c1 * s.qrs];
+            x = swap ? fma(w, u * s.scale, x) : fma(u, w * s.scale, x);
+          }
+          return x;
+        };
+        wild = __any_sync(0xffffffffu, wild);
+        uint32_t A0[MMA_ND], A1[MMA_ND], A2[MMA_ND], A3[MMA_ND];
+        cut_quad(a[0], ea[0], E[0], A0, A2);
+        cut_quad(a[1], ea[1], E[1], A1, A3);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (h >= nh) break;
+          uint32_t B0[MMA_ND], B1[MMA_ND];
+          cut_quad(b[h], eb[h], F[h], B0, B1);
+          float v[MMA_ND][4];
+#pragma unroll
+          for (int d = 0; d < MMA_ND; ++d)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[d][i] = 0.0f;
+#pragma unroll
+          for (int i = 0; i < MMA_ND; ++i) {
+            const uint32_t A[4] = {A0[i], A1[i], A2[i], A3[i]};
+#pragma unroll
+            for (int j = 0; j < MMA_ND - i; ++j) mma16816(v[i + j], A, B0[j], B1[j]);
+          }
+          // exponents of this lane's two columns, held by the lanes of those columns
+          const int f0 = __shfl_sync(0xffffffffu, xf[h], 8 * t), f1 = __shfl_sync(0xffffffffu, xf[h], 8 * t + 4);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int x = xe[i >> 1], f = (i & 1) ? f1 : f0;
+            if (!wild || (x | f) >= 0)
+              acc[h][i] = fma((double)join_digits(v, i), __hiloint2double(x + f, 0), acc[h][i]);
+            else
+              acc[h][i] = fp64_chunk(g + 8 * (i >> 1), 8 * h + 2 * t + (i & 1), acc[h][i]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int r = g + 8 * (i >> 1), c = 8 * h + 2 * t + (i & 1);
+        if (r < rt && c < ct) store(swap ? c0 + c : r0 + r, swap ? r0 + r : c0 + c, acc[h][i]);
+      }
+  }
+  if (part) warp_reduce_parts(outs, splits[o.split], counters + o.split, wbase, ybase, tbase, lane);
+}
+
+constexpr int WARP_CTAS = 4;
+
+__global__ void __launch_bounds__(32 * WARP_WARPS, WARP_CTAS)
+    gemm_warp_kernel(const GemmOut* __restrict__ outs, const GemmSeg* __restrict__ segs, const int3* __restrict__ tiles,
+                     int ntiles, const double* __restrict__ xbase, double* ybase, double* tbase,
+                     const GemmBases* __restrict__ multi, const GemmExtra ex, double* wbase,
+                     const SplitTile* __restrict__ splits, int* counters) {
+  __shared__ WarpSmem S;
+  const int w = blockIdx.x * WARP_WARPS + (threadIdx.x >> 5);
+  if (w >= ntiles) return;
+  const int3 wi = tiles[w];
+  const GemmOut o = outs[wi.x];
+  if (multi) {
+    const GemmBases b = multi[o.inst];
+    xbase = b.x;
+    ybase = b.y;
+    tbase = b.t;
+  }
+  warp_tile(outs, segs, wi, xbase, ybase, tbase, wbase, splits, counters, o, [&](int i) { return mma_extra(ex, i); }, S);
+}
+
+// instances interleave: the warps of a CTA take the same tile of neighbouring instances
+__global__ void __launch_bounds__(32 * WARP_WARPS, WARP_CTAS)
+    gemm_warp_inst_kernel(const GemmOut* __restrict__ outs, const GemmSeg* __restrict__ segs,
+                          const int3* __restrict__ tiles, int ntiles, const __grid_constant__ GemmInstSet P, int ninst) {
+  __shared__ WarpSmem S;
+  const unsigned w = blockIdx.x * WARP_WARPS + (threadIdx.x >> 5);
+  const int tile = (int)(w / ninst);
+  if (tile >= ntiles) return;
+  const GemmInst* b = &P.b[w % ninst];
+  const int3 wi = tiles[tile];
+  const GemmOut o = outs[wi.x];
+  warp_tile(outs, segs, wi, b->x, b->y, b->t, nullptr, nullptr, nullptr, o, [&](int i) { return b->e[i]; }, S);
+}
+
+void launch_gemm_warp(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles, const double* xbase,
+                      double* ybase, double* tbase, cudaStream_t st, const GemmBases* multi, const GemmExtra* extra,
+                      double* wbase, const SplitTile* splits, int* counters) {
+  if (ntiles <= 0) return;
+  const GemmExtra ex = extra ? *extra : GemmExtra{};
+  gemm_warp_kernel<<<(ntiles + WARP_WARPS - 1) / WARP_WARPS, 32 * WARP_WARPS, 0, st>>>(
+      outs, segs, tiles, ntiles, xbase, ybase, tbase, multi, ex, wbase, splits, counters);
+}
+
+void launch_gemm_warp_inst(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles,
+                           const GemmInstSet& bases, int ninst, cudaStream_t st) {
+  if (ntiles <= 0 || ninst <= 0) return;
+  const long long n = (long long)ntiles * ninst;
+  gemm_warp_inst_kernel<<<(unsigned)((n + WARP_WARPS - 1) / WARP_WARPS), 32 * WARP_WARPS, 0, st>>>(
       outs, segs, tiles, ntiles, bases, ninst);
 }
 

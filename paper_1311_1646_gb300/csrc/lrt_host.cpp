@@ -712,6 +712,9 @@ struct GatherPlan {
   void run(cudaStream_t st) const { launch_gather(tasks.p, srcs.p, tiles.p, ntiles, st); }
 };
 
+// kernel of a grouped GEMM: FP64 FMAs by CTA tiles, digit products by CTA tiles, one warp per tile
+enum class GemmKind { FP64, MMA, WARP };
+
 struct GemmPlan {
   DevArray<GemmOut> outs;    // the plan's outputs, then the K parts of split tiles
   DevArray<GemmSeg> segs;
@@ -722,27 +725,44 @@ struct GemmPlan {
   int nsplit = 0;
   DevBuf ws;                 // partial tiles of the split tiles
   double flops = 0.0;
-  bool mma = false;          // tiles of the digit-product kernel
+  GemmKind kind = GemmKind::FP64;
+  DevArray<int> counters;    // WARP: finished parts of every split tile (zero between launches)
   void run(cudaStream_t st, const double* xb, double* yb, double* tb = nullptr, const GemmExtra* ex = nullptr) const {
-    if (mma)
-      launch_gemm_mma(outs.p, segs.p, tiles.p, ntiles, xb, yb, tb, st, nullptr, ex, ws.p);
-    else
-      launch_gemm_fp64(outs.p, segs.p, tiles.p, ntiles, xb, yb, tb, st, ex, ws.p);
+    switch (kind) {
+      case GemmKind::WARP:
+        launch_gemm_warp(outs.p, segs.p, tiles.p, ntiles, xb, yb, tb, st, nullptr, ex, ws.p, splits.p, counters.p);
+        return;
+      case GemmKind::MMA:
+        launch_gemm_mma(outs.p, segs.p, tiles.p, ntiles, xb, yb, tb, st, nullptr, ex, ws.p);
+        break;
+      case GemmKind::FP64:
+        launch_gemm_fp64(outs.p, segs.p, tiles.p, ntiles, xb, yb, tb, st, ex, ws.p);
+        break;
+    }
     if (nsplit > 0) launch_split_reduce(outs.p, splits.p, nsplit, ws.p, yb, tb, st);
   }
   void run_inst(cudaStream_t st, const GemmInstSet& B, int n) const {
-    if (mma)
-      launch_gemm_mma_inst(outs.p, segs.p, tiles.p, ntiles, B, n, st);
-    else
-      launch_gemm_fp64_inst(outs.p, segs.p, tiles.p, ntiles, B, n, st);
+    switch (kind) {
+      case GemmKind::WARP: launch_gemm_warp_inst(outs.p, segs.p, tiles.p, ntiles, B, n, st); break;
+      case GemmKind::MMA: launch_gemm_mma_inst(outs.p, segs.p, tiles.p, ntiles, B, n, st); break;
+      case GemmKind::FP64: launch_gemm_fp64_inst(outs.p, segs.p, tiles.p, ntiles, B, n, st); break;
+    }
   }
   void run_multi(cudaStream_t st, const GemmBases* bases) const {
-    if (mma)
-      launch_gemm_mma(outs.p, segs.p, tiles.p, ntiles, nullptr, nullptr, nullptr, st, bases, nullptr, nullptr);
-    else
-      launch_gemm_fp64_multi(outs.p, segs.p, tiles.p, ntiles, bases, st);
+    switch (kind) {
+      case GemmKind::WARP:
+        launch_gemm_warp(outs.p, segs.p, tiles.p, ntiles, nullptr, nullptr, nullptr, st, bases, nullptr, ws.p,
+                         splits.p, counters.p);
+        break;
+      case GemmKind::MMA:
+        launch_gemm_mma(outs.p, segs.p, tiles.p, ntiles, nullptr, nullptr, nullptr, st, bases, nullptr, nullptr);
+        break;
+      case GemmKind::FP64:
+        launch_gemm_fp64_multi(outs.p, segs.p, tiles.p, ntiles, bases, st);
+        break;
+    }
   }
-  int launches() const { return (ntiles > 0) + (nsplit > 0); }
+  int launches() const { return (ntiles > 0) + (nsplit > 0 && kind != GemmKind::WARP); }
 };
 
 static void build_gather(GatherPlan& P, std::vector<GatherTask>& tasks, std::vector<GatherSrc>& srcs,
@@ -781,37 +801,70 @@ static void mma_tile_shape(const GemmOut& O, int& tm, int& tn) {
   }
 }
 
-// Whether a list runs as digit products: the work padded to 16 x 8 x 16 is at most three
-// times the exact work (the FP64 FMA kernel pays no padding).  Measured both ways: padding
-// 2.0 / 1.6 (phase 1 / 2; k = 24, M = 300, site 4) 745 -> 480 us, 2.0 / 1.9 (PPP k = 12,
-// M = 256) 174 -> 127 us, but 4 / 3 (eight molecules of 8 to 12 orbitals) 1.67 -> 2.08 ms.
-// Counted per vector, so that a call's kernel, and with it every bit of a vector's result,
-// does not depend on how many vectors the call has.
-static bool use_mma(const std::vector<GemmOut>& outs, const std::vector<GemmSeg>& segs, const std::vector<int64_t>& ktot) {
+// Kernel of a list.  CTA tiles of digit products for long lists (3e8 multiply-adds per vector
+// and more) of blocks that fill them (work padded to 16 x 8 x 16 at most 3 times the exact
+// work), one warp per tile elsewhere: a CTA shares the cut operands among its units, a warp
+// waits for nobody.  Both measured, CTA / warp (multiply-adds, padding of the two phases):
+// k = 24, M = 500, 6 vectors (2 x 1.9e9 per vector; 1.8, 1.1) 17.0 / 25.2 ms; the same chain at
+// M = 300, site 4 (1.3e8; 2.0, 1.6) 487 / 374 us; PPP k = 12, M = 256 (1.7e7; 2.0, 1.9) 129 / 93 us;
+// eight molecules of 8 to 12 orbitals (5e7; 4, 3) 1.94 / 0.94 ms; k = 8, M = 64 (1e6; 13, 5)
+// 135 / 61 us (183 by FP64 CTA tiles).  Counted per vector, so that a call's kernel, and with
+// it every bit of a vector's result, does not depend on how many vectors the call has.  FP64
+// CTA tiles are left for strides beyond 32 bits.
+static GemmKind gemm_kind(const std::vector<GemmOut>& outs, const std::vector<GemmSeg>& segs,
+                          const std::vector<int64_t>& ktot) {
   double exact = 0.0, padded = 0.0;
   for (size_t i = 0; i < outs.size(); ++i) {
     const GemmOut& o = outs[i];
     for (int q = 0; q < o.seg_count; ++q) {
       const GemmSeg& g = segs[o.seg_begin + q];
-      if (g.a_vr != o.c_vr || g.b_vc != o.c_vc) return false;
-      // the kernel's row offsets are 32-bit byte strides
-      if (std::max(g.a_vs, g.b_vs) >= ((int64_t)1 << 29) || std::max(g.lda, g.ldb) >= (1 << 28)) return false;
+      // one vector block per output, and 32-bit byte strides, are what those kernels take
+      if (g.a_vr != o.c_vr || g.b_vc != o.c_vc) return GemmKind::FP64;
+      if (std::max(g.a_vs, g.b_vs) >= ((int64_t)1 << 29) || std::max(g.lda, g.ldb) >= (1 << 28)) return GemmKind::FP64;
     }
     const int m = o.c_vr > 0 ? o.c_vr : o.m, n = o.c_vc > 0 ? o.c_vc : o.n;
     exact += (double)m * n * ktot[i];
     padded += (double)((m + 15) / 16 * 16) * ((n + 7) / 8 * 8) * ((ktot[i] + 15) / 16 * 16);
   }
-  return padded <= 3.0 * exact;
+  return exact >= 3e8 && padded <= 3.0 * exact ? GemmKind::MMA : GemmKind::WARP;
 }
 
+// Path and tile of one output in the warp kernel.  Direct FMAs cost about 0.5 clocks per
+// element and K position, digit products about 210 per 16 x 8 x 16: direct below 400
+// multiply-adds per 16 positions (counted per vector).
+static void warp_tile_shape(GemmOut& O, int64_t k, int& tm, int& tn) {
+  const int m = O.c_vr > 0 ? O.c_vr : O.m, n = O.c_vc > 0 ? O.c_vc : O.n;
+  auto even = [](int x, int most) {
+    const int parts = (x + most - 1) / most;
+    return (x + parts - 1) / parts;
+  };
+  O.flags = 0;
+  if ((int64_t)m * n * std::min<int64_t>(k, 16) < 400) {
+    O.flags = GEMM_WARP_DIRECT;
+    tn = even(O.n, GEMM_DIRECT_MAX);
+    tm = even(O.m, GEMM_DIRECT_MAX / tn);
+    return;
+  }
+  const int64_t plain = (int64_t)((O.m + 15) / 16) * ((O.n + 7) / 8), swapped = (int64_t)((O.n + 15) / 16) * ((O.m + 7) / 8);
+  if (!O.balance && swapped < plain) O.flags = GEMM_WARP_SWAP;   // a balanced output's column tiles are its own
+  tm = even(O.m, 16);
+  tn = even(O.n, 16);
+}
+
+// whether outputs may be split along K: never (lists replayed over instances, whose partial
+// tiles would need a workspace each), or only by the warp kernel (lists over several bases,
+// which the reduction launch does not know)
+enum class GemmSplit { NEVER, WARP, ALWAYS };
+
 static void build_gemm(GemmPlan& P, const std::vector<GemmOut>& outs_in, const std::vector<GemmSeg>& segs,
-                       cudaStream_t st, bool split = false) {
+                       cudaStream_t st, GemmSplit split = GemmSplit::NEVER) {
   // A tile costs its warps of outputs times its K chunks of DFMA issue, plus a fixed
   // cost per chunk.  Tiles far longer than an even share of the launch (an output with
   // many long K segments) would run on after all others finished.  With `split`, an
   // output that sums several segments (y or T outputs) and at least 2 GEMM_SPLIT_K of K
   // has each of its tiles cut along its segment list into K parts of about GEMM_SPLIT_K:
-  // each part a partial tile in the workspace, added in order by the reduction launch.
+  // each part a partial tile in the workspace, added in order by the reduction launch (by the
+  // last warp of the tile in the warp kernel, whose parts are shorter).
   // The parts depend on the output's own segments only, so an element is summed in the
   // same grouping whichever call (vector count, batch) the output belongs to.  Otherwise
   // tiles above an even share are cut into row slices.  Then the longest go first.  (Row
@@ -826,21 +879,24 @@ static void build_gemm(GemmPlan& P, const std::vector<GemmOut>& outs_in, const s
       ktot[i] += segs[outs_in[i].seg_begin + s].k;
       fl += 2.0 * outs_in[i].m * (double)outs_in[i].n * segs[outs_in[i].seg_begin + s].k;
     }
-  const bool mma = use_mma(outs_in, segs, ktot);
-  auto cost = [mma](int64_t mt, int64_t nt, int64_t k) {
+  const GemmKind kind = gemm_kind(outs_in, segs, ktot);
+  const bool mma = kind == GemmKind::MMA, warp = kind == GemmKind::WARP;
+  auto cost = [mma, warp](int64_t mt, int64_t nt, int64_t k) {
     const int64_t nch = (k + GEMM_KC - 1) / GEMM_KC;
+    if (warp) return k + 8;
     if (mma) return nch * (30 * ((mt + 15) / 16) * ((nt + 15) / 16) + 12 * ((mt + 15) / 16 + (nt + 15) / 16) + 20) + 40;
     return nch * (32 * ((mt * nt + 31) / 32) + 64) + 64;
   };
-  auto shape = [mma](const GemmOut& O, int& tm, int& tn) {
+  auto shape = [mma, warp](GemmOut& O, int64_t k, int& tm, int& tn) {
     tm = GEMM_TM;
     tn = GEMM_TN;
     if (mma) mma_tile_shape(O, tm, tn);
+    if (warp) warp_tile_shape(O, k, tm, tn);
   };
   int64_t total = 0;
-  for (size_t i = 0; i < outs_in.size(); ++i) {
+  for (size_t i = 0; i < outs_in.size() && kind == GemmKind::FP64; ++i) {
     int TM, TN;
-    shape(outs_in[i], TM, TN);
+    shape(outs[i], ktot[i], TM, TN);
     for (int m0 = 0; m0 < outs_in[i].m; m0 += TM)
       for (int n0 = 0; n0 < outs_in[i].n; n0 += TN)
         total += cost(std::min(TM, outs_in[i].m - m0), std::min(TN, outs_in[i].n - n0), ktot[i]);
@@ -850,15 +906,18 @@ static void build_gemm(GemmPlan& P, const std::vector<GemmOut>& outs_in, const s
   std::vector<SplitTile> sp;
   int64_t wsz = 0;
   for (size_t i = 0; i < outs_in.size(); ++i) {
-    const GemmOut& O = outs_in[i];
     int TM, TN;
-    shape(O, TM, TN);
+    shape(outs[i], ktot[i], TM, TN);
+    const GemmOut O = outs[i];
+    // K per part: the warp kernel, whose warps each walk their part alone, takes a sixteenth
+    // of the list between 96 and GEMM_SPLIT_K
+    const int64_t kpart = warp ? std::min<int64_t>(GEMM_SPLIT_K, std::max<int64_t>(96, ktot[i] / 16)) : GEMM_SPLIT_K;
     for (int m0 = 0; m0 < O.m; m0 += TM)
       for (int n0 = 0; n0 < O.n; n0 += TN) {
         const int mt = std::min(TM, O.m - m0), nt = std::min(TN, O.n - n0);
         const int64_t c = cost(mt, nt, ktot[i]);
-        const int want = (int)std::min<int64_t>(O.seg_count, ktot[i] / GEMM_SPLIT_K);
-        if (split && want >= 2 && O.c_rel <= 2 && outs.size() < (size_t)INT32_MAX) {
+        const int want = (int)std::min<int64_t>(O.seg_count, ktot[i] / kpart);
+        if ((split == GemmSplit::ALWAYS || (split == GemmSplit::WARP && warp)) && want >= 2 && O.c_rel <= 2 && outs.size() < (size_t)INT32_MAX) {
           // contiguous runs of the segment list, each about ktot / want of K
           SplitTile t{wsz, (int)i, 0, m0, mt, n0, nt};
           std::vector<int> kseg(O.seg_count);
@@ -870,7 +929,8 @@ static void build_gemm(GemmPlan& P, const std::vector<GemmOut>& outs_in, const s
             po.c_off = wsz + (int64_t)t.nparts * mt * nt - ((int64_t)m0 * nt + n0);
             po.ldc = nt;
             po.accumulate = 0;
-            if (!mma) po.c_vr = po.c_vc = 0;   // the digit-product kernel reads its operands' blocks here
+            if (kind == GemmKind::FP64) po.c_vr = po.c_vc = 0;   // the others read their operands' blocks here
+            po.split = (int)sp.size();
             po.c_vs = 0;
             po.seg_begin = O.seg_begin + sb;
             po.seg_count = se - sb;
@@ -882,7 +942,7 @@ static void build_gemm(GemmPlan& P, const std::vector<GemmOut>& outs_in, const s
           sp.push_back(t);
           continue;
         }
-        const int parts = mma ? 1 : (int)std::min<int64_t>(mt, (c + cap - 1) / cap);
+        const int parts = kind != GemmKind::FP64 ? 1 : (int)std::min<int64_t>(mt, (c + cap - 1) / cap);
         for (int p = 0, r = m0; p < parts; ++p) {
           const int rows = mt / parts + (p < mt % parts ? 1 : 0);
           tl.push_back({cost(rows, nt, ktot[i]), gemm_tile((int)i, r, rows, n0, nt)});
@@ -890,11 +950,22 @@ static void build_gemm(GemmPlan& P, const std::vector<GemmOut>& outs_in, const s
         }
       }
   }
-  std::stable_sort(tl.begin(), tl.end(), [](const std::pair<int64_t, int3>& a, const std::pair<int64_t, int3>& b) {
-    return a.first > b.first;
-  });
+  // longest first, to within an eighth of an octave, otherwise in list order (a counting sort:
+  // lists have up to a million tiles)
+  auto bucket = [](int64_t c) {
+    int e = 0;
+    while ((c >> e) > 1) ++e;
+    return 8 * e + (e >= 3 ? (int)(c >> (e - 3)) - 8 : 0);
+  };
+  std::vector<int> at(8 * 64 + 1, 0), key(tl.size());
+  for (size_t t = 0; t < tl.size(); ++t) ++at[511 - (key[t] = bucket(std::max<int64_t>(1, tl[t].first)))];
+  for (int b = 0, n = 0; b < 512; ++b) {
+    const int k = at[b];
+    at[b] = n;
+    n += k;
+  }
   std::vector<int3> tiles(tl.size());
-  for (size_t t = 0; t < tl.size(); ++t) tiles[t] = tl[t].second;
+  for (size_t t = 0; t < tl.size(); ++t) tiles[at[511 - key[t]]++] = tl[t].second;
   P.outs.upload(outs, st);
   P.segs.upload(segs, st);
   P.tiles.upload(tiles, st);
@@ -904,7 +975,8 @@ static void build_gemm(GemmPlan& P, const std::vector<GemmOut>& outs_in, const s
   P.nsplit = (int)sp.size();
   if (wsz > 0) P.ws.ensure((size_t)wsz);
   P.flops = fl;
-  P.mma = mma;
+  P.kind = kind;
+  if (warp && P.nsplit > 0) P.counters.upload(std::vector<int>(sp.size(), 0), st);
 }
 
 }  // namespace lrt
@@ -2015,7 +2087,8 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
     O2.push_back(y);
   }
   build_gemm(plan->p1, O1, S1, c->st);
-  build_gemm(plan->p2, O2, S2, c->st, !rel_ops);   // kept relative plans are replayed over instances
+  // kept relative plans are replayed over instances
+  build_gemm(plan->p2, O2, S2, c->st, rel_ops ? GemmSplit::NEVER : GemmSplit::ALWAYS);
   // tensor-core twin: phase-2 outputs, one per (y block, column group)
   plan->has_tc = tc;
   for (size_t w = 0; w < wb.size() && tc; ++w)
@@ -5405,7 +5478,7 @@ static void merge_fp64(GemmPlan& out, const std::vector<SigmaPlan*>& plans, bool
     }
     S.insert(S.end(), sg.begin(), sg.end());
   }
-  build_gemm(out, O, S, st);
+  build_gemm(out, O, S, st, GemmSplit::WARP);
 }
 
 // one batched call (the graph body): no host synchronization inside

@@ -47,7 +47,10 @@ struct GemmOut {
   int64_t c_vs;
   int balance;   // digit products (launch_gemm_mma): K positions are first scaled to equal
                  // exponents over op(B)'s columns (an output that sums many operators)
+  int flags;     // GEMM_WARP_* (launch_gemm_warp)
+  int split;     // launch_gemm_warp: the split tile a part (c_rel GEMM_C_SPLIT) belongs to
 };
+constexpr int GEMM_WARP_DIRECT = 1, GEMM_WARP_SWAP = 2;
 struct GemmSeg {
   const double* A;
   const double* B;
@@ -128,6 +131,13 @@ struct SplitTile {
 };
 void launch_split_reduce(const GemmOut* outs, const SplitTile* tiles, int ntiles, const double* wbase, double* ybase,
                          double* tbase, cudaStream_t st);
+// One warp per tile (small blocks, lrt_fp64_mma.cu): with GEMM_WARP_DIRECT at most
+// GEMM_DIRECT_MAX elements, else 16 x 16.  Parts of split tiles are added by the warp that
+// finishes last: one counter per split tile, zero before the first launch.
+constexpr int GEMM_DIRECT_MAX = 64;
+void launch_gemm_warp(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles, const double* xbase,
+                      double* ybase, double* tbase, cudaStream_t st, const GemmBases* multi, const GemmExtra* extra,
+                      double* wbase, const SplitTile* splits, int* counters);
 // batched form: the bases of output o are bases[o.inst] (device array)
 void launch_gemm_fp64_multi(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles,
                             const GemmBases* bases, cudaStream_t st);
@@ -150,6 +160,8 @@ void launch_gemm_fp64_inst(const GemmOut* outs, const GemmSeg* segs, const int3*
                            const GemmInstSet& bases, int ninst, cudaStream_t st);
 void launch_gemm_mma_inst(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles,
                           const GemmInstSet& bases, int ninst, cudaStream_t st);
+void launch_gemm_warp_inst(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles,
+                           const GemmInstSet& bases, int ninst, cudaStream_t st);
 void launch_diag(const DiagOut* outs, const DiagTerm* terms, int nouts, double* dbase, cudaStream_t st);
 
 // Split-TF32 tensor-core variant of the grouped GEMM.

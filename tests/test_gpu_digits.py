@@ -108,3 +108,24 @@ def test_extreme_exponents_and_infinities(pkg):
     assert np.array_equal(w[n:], y[n:])
     a.close()
     b.close()
+
+
+# blocks of 1 to 49 states: lanes with one and two elements, digit tiles in both orientations,
+# segment lists of one part and of many (their parts added by the last warp), and the CTA tiles
+@pytest.mark.parametrize("k,na,nb,M,i,nsite,nvec", [
+    (12, 1, 1, 3, 5, 1, 1), (9, 5, 4, 24, 4, 1, 7), (9, 4, 4, 60, 4, 2, 1), (8, 4, 4, 90, 3, 1, 4), (14, 2, 2, 140, 6, 1, 3)])
+def test_small_blocks_match_the_oracle(pkg, k, na, nb, M, i, nsite, nvec):
+    H = synth.ab_initio(k, na, nb, 90 + M)
+    m = synth.mixed_mps(k, na, nb, M, 91, center=i)
+    ctx = _context(pkg, k, na, nb, M, i, nsite, H.h, H.eri, m)
+    n, _ = ctx.wfn_layout(i, nsite)
+    x = synth.random_vector(nvec * n, 92)
+    y = _sigma(pkg, ctx, i, nsite, x, nvec)
+    ref = _oracle(H, m, i, nsite)
+    for v in (0, nvec - 1):
+        r = ref(x[v * n:(v + 1) * n])
+        assert np.abs(y[v * n:(v + 1) * n] - r).max() <= RTOL * np.abs(r).max(), v
+        assert np.array_equal(_sigma(pkg, ctx, i, nsite, x[v * n:(v + 1) * n], 1), y[v * n:(v + 1) * n])
+    # the parts' counters are back at zero: the same call again, the same bits
+    assert np.array_equal(_sigma(pkg, ctx, i, nsite, x, nvec), y)
+    ctx.close()
