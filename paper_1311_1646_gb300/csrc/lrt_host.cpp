@@ -1234,10 +1234,18 @@ static void reset_env(lrt_ctx* c) {
 // The plan of one enlargement (layout of the enlarged set and its gather tasks, with
 // addresses as offsets), reusable for any input set of the same layout and structure:
 // the TDA enlarges the first-order sets of every trial vector at a site, all alike.
+struct EnlPlan {
+  DevArray<unsigned char> blob;        // the tables, one upload
+  EnlTables t{};
+  DevArray<int3> items;
+  int nitems = 0;
+  void run(cudaStream_t st, double* d, const double* x, const double* xrev) const {
+    launch_enlarge(t, items.p, nitems, d, x, xrev, st);
+  }
+};
 struct EnlTemplate {
   std::unique_ptr<OpSet> proto;        // layout of the enlarged set, no data
-  std::unique_ptr<GatherPlan> gp;      // device task list: destinations relative to the new
-                                       // set, sources relative to X (rel 1) or Xrev (rel 2)
+  std::unique_ptr<EnlPlan> plan;       // device tables, all addresses relative to the launch's sets
   uint64_t sig = 0;
 };
 
@@ -1302,114 +1310,128 @@ static std::unique_ptr<OpSet> enlarge_set(lrt_ctx* c, const OpSet& X, const OpSe
   alloc_zero(*E, c->st);
   E->mask.assign(E->bra.size(), 0);
   const Fused& F = *E->fused;
+  const int nx = X.ns(), nxop = (int)X.keys.size(), ne = E->ns(), nop = (int)E->keys.size();
   auto terms = right ? blocking_terms(*E, sorbs, X.orbs, I) : blocking_terms(*E, X.orbs, sorbs, I);
 
-  std::vector<GatherTask> tasks;
-  std::vector<std::vector<GatherSrc>> tsrc;
-  std::vector<std::vector<std::pair<int64_t, char>>> tsrc_off;   // template: source offsets
-  std::unordered_map<const double*, int> task_of;
-  std::vector<Ref> refs;
-  for (size_t o = 0; o < E->keys.size(); ++o) {
-    std::map<std::pair<int, int>, Mat4> acc;
-    for (const Term& t : terms[o]) {
-      refs.clear();
-      Mat4 e4;
-      if (right) {
-        e4 = site.op(I, t.x.kind, t.x.p, t.x.q, t.x.t);
-        get_refs(X, I, t.y.kind, t.y.p, t.y.q, t.y.t, t.c, refs);
-      } else {
-        get_refs(X, I, t.x.kind, t.x.p, t.x.q, t.x.t, t.c, refs);
-        e4 = site.op(I, t.y.kind, t.y.p, t.y.q, t.y.t);
-      }
-      if (e4.zero()) continue;
-      for (const Ref& r : refs) acc[{r.op, r.t}].axpy(r.c, e4);
+  // distinct site operators and the references of every new operator
+  std::map<std::tuple<int, int, int, int>, int> site_of;   // -1: zero
+  std::vector<EnlSite> sites;
+  auto site_id = [&](const Spec& s) {
+    auto ins = site_of.emplace(std::make_tuple(s.kind, s.p, s.q, s.t), -1);
+    if (!ins.second) return ins.first->second;
+    const Mat4 m = site.op(I, s.kind, s.p, s.q, s.t);
+    if (m.zero()) return -1;
+    EnlSite g{};
+    for (int e = 0; e < 16; ++e) {
+      g.e[e] = m.m[e];
+      if (m.m[e] != 0.0) g.mask |= 1 << e;
     }
-    for (auto& kv : acc) {
-      const int j = kv.first.first, tr = kv.first.second;
-      const Mat4& e4 = kv.second;
-      if (e4.zero()) continue;
+    sites.push_back(g);
+    return ins.first->second = (int)sites.size() - 1;
+  };
+  std::vector<EnlRef> refs;
+  std::vector<int> rbeg(nop + 1, 0);
+  std::vector<std::array<int, 4>> fk_of(nx);   // fused label of sector s with site state n
+  for (int s = 0; s < nx; ++s)
+    for (int n = 0; n < 4; ++n)
+      fk_of[s][n] = right ? F.s.find(X.basis.a[s] - QNA[n], X.basis.b[s] - QNB[n])
+                          : F.s.find(X.basis.a[s] + QNA[n], X.basis.b[s] + QNB[n]);
+  std::vector<uint16_t> seen(2 * (size_t)nxop, 0);   // sub-blocks a reference reaches, per operator of X
+  std::vector<int> touched;
+  std::vector<Ref> rx;
+  for (int o = 0; o < nop; ++o) {
+    touched.clear();
+    for (const Term& t : terms[o]) {
+      const int g = site_id(right ? t.x : t.y);
+      if (g < 0) continue;
+      const Spec& sx = right ? t.y : t.x;
+      rx.clear();
+      get_refs(X, I, sx.kind, sx.p, sx.q, sx.t, t.c, rx);
+      for (const Ref& r : rx) {
+        const int id = 2 * r.op + r.t;
+        refs.push_back(EnlRef{id, g, r.c});
+        if (!seen[id]) touched.push_back(id);
+        seen[id] |= (uint16_t)sites[g].mask;
+      }
+    }
+    rbeg[o + 1] = (int)refs.size();
+    for (int id : touched) {
+      const int j = id >> 1, tr = id & 1;
+      const unsigned m = seen[id];
+      seen[id] = 0;
       const OpSet& XS = (tr && Xrev) ? *Xrev : X;
-      for (int s = 0; s < X.ns(); ++s) {
+      for (int s = 0; s < nx; ++s) {
         const int sb = X.bra_of(j, s);
         if (sb < 0 || !XS.block_nz(j, s)) continue;
         const int be = tr ? s : sb, ke = tr ? sb : s;
-        const double* src = XS.d + X.off_of(j, s);
-        const int ld = X.basis.d[s];
-        for (int n1 = 0; n1 < 4; ++n1)
-          for (int n0 = 0; n0 < 4; ++n0) {
-            const double e = e4(n1, n0);
-            if (e == 0.0) continue;
-            int fk, fb, sign;
-            if (right) {
-              fk = F.s.find(X.basis.a[ke] - QNA[n0], X.basis.b[ke] - QNB[n0]);
-              fb = F.s.find(X.basis.a[be] - QNA[n1], X.basis.b[be] - QNB[n1]);
-              sign = (X.par[j] && ((QNA[n0] + QNB[n0]) & 1)) ? -1 : 1;
-            } else {
-              fk = F.s.find(X.basis.a[ke] + QNA[n0], X.basis.b[ke] + QNB[n0]);
-              fb = F.s.find(X.basis.a[be] + QNA[n1], X.basis.b[be] + QNB[n1]);
-              const int sp = (QNA[n1] + QNB[n1] + QNA[n0] + QNB[n0]) & 1;
-              sign = (sp && ((X.basis.a[ke] + X.basis.b[ke]) & 1)) ? -1 : 1;
-            }
-            if (fk < 0 || fb < 0 || E->bra_of((int)o, fk) != fb)
-              throw Error(LRT_EINVAL, "internal: blocking term outside the operator's sector");
-            const int ldd = F.s.d[fk];
-            double* dst = E->d + E->off_of((int)o, fk) + (int64_t)F.off[fb][n1] * ldd + F.off[fk][n0];
-            auto it = task_of.find(dst);
-            int ti;
-            if (it == task_of.end()) {
-              ti = (int)tasks.size();
-              task_of[dst] = ti;
-              tasks.push_back(GatherTask{dst, ldd, X.basis.d[be], X.basis.d[ke], 0, 0});
-              tsrc.emplace_back();
-            } else {
-              ti = it->second;
-            }
-            tsrc[ti].push_back(GatherSrc{src, ld, tr, sign * e});
-            if (tpl) {
-              tsrc_off.resize(tsrc.size());
-              tsrc_off[ti].push_back({src - XS.d, (tr && Xrev) ? 1 : 0});
-            }
-            E->mask[(size_t)o * E->ns() + fk] |= (uint16_t)(1u << (4 * n1 + n0));
-            E->bnz[(size_t)o * E->ns() + fk] = 1;
-          }
+        for (unsigned w = m; w; w &= w - 1) {
+          const int bit = __builtin_ctz(w), n1 = bit >> 2, n0 = bit & 3;
+          const int fk = fk_of[ke][n0], fb = fk_of[be][n1];
+          if (fk < 0 || fb < 0 || E->bra_of(o, fk) != fb)
+            throw Error(LRT_EINVAL, "internal: blocking term outside the operator's sector");
+          E->mask[(size_t)o * ne + fk] |= (uint16_t)(1u << bit);
+        }
       }
     }
   }
-  std::vector<GatherSrc> srcs;
-  for (size_t i = 0; i < tasks.size(); ++i) {
-    tasks[i].src_begin = (int)srcs.size();
-    tasks[i].src_count = (int)tsrc[i].size();
-    srcs.insert(srcs.end(), tsrc[i].begin(), tsrc[i].end());
-  }
+  std::vector<int3> items;
+  for (int o = 0; o < nop; ++o)
+    for (int fk = 0; fk < ne; ++fk) {
+      const unsigned m = E->mask[(size_t)o * ne + fk];
+      if (!m) continue;
+      E->bnz[(size_t)o * ne + fk] = 1;
+      const int fb = E->bra_of(o, fk);
+      for (unsigned w = m; w; w &= w - 1) {
+        const int bit = __builtin_ctz(w);
+        const int64_t n = (int64_t)F.dim[fb][bit >> 2] * F.dim[fk][bit & 3];
+        if (n > INT32_MAX) throw Error(LRT_EINVAL, "enlargement: block too large");
+        for (int64_t e = 0; e < n; e += ENL_CHUNK) items.push_back(make_int3(o, 16 * fk + bit, (int)e));
+      }
+    }
   E->finish_nz();
-  if (tpl) {
-    // the same task list with addresses relative to the launch's bases, kept on the device
-    tpl->proto = layout_copy(*E);
-    tsrc_off.resize(tsrc.size());
-    std::vector<GatherSrc> rsrcs;
-    rsrcs.reserve(srcs.size());
-    for (size_t i = 0; i < tasks.size(); ++i) {
-      tasks[i].dst_off = tasks[i].dst - E->d;
-      tasks[i].dst = nullptr;
-      for (size_t j = 0; j < tsrc[i].size(); ++j) {
-        GatherSrc g = tsrc[i][j];
-        g.src = nullptr;
-        g.src_off = tsrc_off[i][j].first;
-        g.rel = tsrc_off[i][j].second ? 2 : 1;
-        rsrcs.push_back(g);
-      }
+
+  // one upload of all tables
+  auto plan = std::make_unique<EnlPlan>();
+  std::vector<EnlBlock> blk((size_t)nxop * nx);
+  for (int j = 0; j < nxop; ++j)
+    for (int s = 0; s < nx; ++s)
+      blk[(size_t)j * nx + s] = EnlBlock{X.off_of(j, s), X.bra_of(j, s),
+                                         (X.block_nz(j, s) ? 1 : 0) | (Xrev && Xrev->block_nz(j, s) ? 2 : 0)};
+  std::vector<int> xpar(nx), fsub(4 * (size_t)ne), foff(4 * (size_t)ne);
+  for (int s = 0; s < nx; ++s) xpar[s] = (X.basis.a[s] + X.basis.b[s]) & 1;
+  for (int f = 0; f < ne; ++f)
+    for (int n = 0; n < 4; ++n) {
+      fsub[4 * f + n] = F.sub[f][n];
+      foff[4 * f + n] = F.off[f][n];
     }
-    tpl->gp = std::make_unique<GatherPlan>();
-    build_gather(*tpl->gp, tasks, rsrcs, c->st);
-    launch_gather(tpl->gp->tasks.p, tpl->gp->srcs.p, tpl->gp->tiles.p, tpl->gp->ntiles, c->st, E->d, X.d,
-                  Xrev ? Xrev->d : nullptr);
-    CK(cudaGetLastError());
-    return E;
-  }
-  GatherPlan gp;
-  build_gather(gp, tasks, srcs, c->st);
-  gp.run(c->st);
+  std::vector<unsigned char> blob;
+  auto put = [&](const void* p, size_t bytes) {
+    const size_t at = (blob.size() + 15) / 16 * 16;
+    blob.resize(at + bytes);
+    if (bytes) std::memcpy(blob.data() + at, p, bytes);
+    return at;
+  };
+  const size_t a_refs = put(refs.data(), refs.size() * sizeof(EnlRef)), a_rbeg = put(rbeg.data(), rbeg.size() * sizeof(int));
+  const size_t a_blk = put(blk.data(), blk.size() * sizeof(EnlBlock)), a_sites = put(sites.data(), sites.size() * sizeof(EnlSite));
+  const size_t a_xdim = put(X.basis.d.data(), nx * sizeof(int)), a_xpar = put(xpar.data(), nx * sizeof(int));
+  const size_t a_opar = put(X.par.data(), nxop * sizeof(int)), a_fsub = put(fsub.data(), fsub.size() * sizeof(int));
+  const size_t a_foff = put(foff.data(), foff.size() * sizeof(int)), a_fdim = put(F.s.d.data(), ne * sizeof(int));
+  const size_t a_eoff = put(E->off.data(), E->off.size() * sizeof(int64_t)), a_ebra = put(E->bra.data(), E->bra.size() * sizeof(int));
+  plan->blob.upload(blob, c->st);
+  const unsigned char* B = plan->blob.p;
+  plan->t = EnlTables{(const EnlRef*)(B + a_refs), (const int*)(B + a_rbeg), (const EnlBlock*)(B + a_blk),
+                      (const EnlSite*)(B + a_sites), (const int*)(B + a_xdim), (const int*)(B + a_xpar),
+                      (const int*)(B + a_opar), (const int*)(B + a_fsub), (const int*)(B + a_foff),
+                      (const int*)(B + a_fdim), (const int64_t*)(B + a_eoff), (const int*)(B + a_ebra),
+                      nx, ne, right ? 1 : 0, 0};
+  plan->items.upload(items, c->st);
+  plan->nitems = (int)items.size();
+  plan->run(c->st, E->d, X.d, Xrev ? Xrev->d : nullptr);
   CK(cudaGetLastError());
+  if (tpl) {
+    tpl->proto = layout_copy(*E);
+    tpl->plan = std::move(plan);
+  }
   return E;
 }
 
@@ -1418,7 +1440,7 @@ static std::unique_ptr<OpSet> enlarge_set(lrt_ctx* c, const OpSet& X, const OpSe
 static std::unique_ptr<OpSet> enlarge_from(lrt_ctx* c, const EnlTemplate& t, const OpSet& X, const OpSet* Xrev) {
   auto E = layout_copy(*t.proto);
   alloc_zero(*E, c->st);
-  launch_gather(t.gp->tasks.p, t.gp->srcs.p, t.gp->tiles.p, t.gp->ntiles, c->st, E->d, X.d, Xrev ? Xrev->d : nullptr);
+  t.plan->run(c->st, E->d, X.d, Xrev ? Xrev->d : nullptr);
   CK(cudaGetLastError());
   return E;
 }
@@ -3913,10 +3935,10 @@ struct TdaRunner {
         out[mu] = enlarge_set(c, *X[mu], Xr[mu], i, right, &tmp);
       }
     }
-    const GatherPlan* gp = t.gp.get();
+    const EnlPlan* ep = t.plan.get();
     for (size_t j0 = 0; j0 < batch.size(); j0 += GEMM_MAX_INST) {
       const int n = (int)std::min<size_t>(GEMM_MAX_INST, batch.size() - j0);
-      inst_check(gp->ntiles, n);
+      inst_check(ep->nitems, n);
       GatherInstSet B{};
       for (int j = 0; j < n; ++j) {
         const int mu = batch[j0 + j];
@@ -3924,7 +3946,7 @@ struct TdaRunner {
         alloc_zero(*out[mu], c->st);
         B.b[j] = GatherBases{out[mu]->d, X[mu]->d, Xr[mu] ? Xr[mu]->d : nullptr};
       }
-      launch_gather_inst(gp->tasks.p, gp->srcs.p, gp->tiles.p, gp->ntiles, B, n, c->st);
+      launch_enlarge_inst(ep->t, ep->items.p, ep->nitems, B, n, c->st);
       CK(cudaGetLastError());
     }
     return out;

@@ -108,6 +108,146 @@ void launch_gather_inst(const GatherTask* tasks, const GatherSrc* srcs, const in
 }
 
 // ---------------------------------------------------------------------------
+// enlargement
+//
+// A sub-block of an enlarged operator sums up to a few hundred scaled source blocks (the
+// complementary operators of a cut combine every pair operator).  A host list of those sources
+// has millions of entries, one per sector, and took 50 ms to write and upload for a 1.5 ms
+// gather; the references that generate it do not depend on the sector.  So a warp takes up to
+// ENL_CHUNK elements of a sub-block, its lanes look up 32 references at a time (does the
+// reference have a block between these sectors, where, with which sign), and all lanes then
+// sum the blocks found, in reference order.  Sub-blocks of 16 elements and fewer spread the
+// references over the idle lanes.  One two-site sweep position at k = 12, M = 128: 92.7 -> 17.2 ms
+// (host list, upload and gather before; the rest is the sigma plan), TDA on PPP M = 128 240 ->
+// 153 ms.  Bound by the FP64 pipe (one FMA per source element) when the
+// blocks are large, by the reference reads when they are small.
+// ---------------------------------------------------------------------------
+constexpr int ENL_WARPS = 8;
+struct EnlSrc {
+  const double* p;
+  int rs, cs;          // strides of the block's rows and columns
+  double scale;
+};
+struct EnlSmem {
+  EnlSrc s[ENL_WARPS][32];
+};
+
+__device__ __forceinline__ void enlarge_item(const EnlTables& t, const int3 wi, double* __restrict__ d,
+                                             const double* __restrict__ x, const double* __restrict__ xrev, EnlSrc* S) {
+  const int lane = threadIdx.x & 31;
+  const int o = wi.x, fk = wi.y >> 4, n1 = (wi.y >> 2) & 3, n0 = wi.y & 3;
+  const int fb = t.ebra[o * t.nse + fk];
+  const int ke = t.fsub[4 * fk + n0], be = t.fsub[4 * fb + n1];
+  const int rows = t.xdim[be], cols = t.xdim[ke], n = rows * cols;
+  const int odd1 = (n1 == 1) | (n1 == 2), odd0 = (n0 == 1) | (n0 == 2);
+  // the sign that comes with an odd operator of X (site on the left) or with the site's own
+  const bool neg_odd = t.right && odd0, neg_all = !t.right && (odd1 ^ odd0) && t.xpar[ke];
+  // lanes: element wi.z + lane + 32 i, or (n <= 16) element lane mod n, every groups-th source
+  const int groups = n <= 16 ? 32 / n : 1;
+  const int e0 = groups > 1 ? lane % n : wi.z + lane, grp = groups > 1 ? lane / n : 0;
+  int rr[4], cc[4];
+  double acc[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int e = min(e0 + 32 * i, n - 1);
+    rr[i] = e / cols;
+    cc[i] = e - rr[i] * cols;
+    acc[i] = 0.0;
+  }
+  const int left = n - wi.z, cnt = groups > 1 ? 1 : min(4, (left + 31) >> 5);
+  const int r1 = t.rbeg[o + 1];
+  for (int r0 = t.rbeg[o]; r0 < r1; r0 += 32) {
+    bool ok = false;
+    EnlSrc src{};
+    if (r0 + lane < r1) {
+      const EnlRef r = t.refs[r0 + lane];
+      const EnlSite& g = t.sites[r.site];
+      if ((g.mask >> (4 * n1 + n0)) & 1) {
+        const int j = r.op >> 1, tr = r.op & 1;
+        const int s = tr ? be : ke;
+        const EnlBlock b = t.blk[j * t.ns + s];
+        const bool rev = tr && xrev;
+        if (b.bra == (tr ? ke : be) && (b.nz & (rev ? 2 : 1))) {
+          ok = true;
+          const int ld = t.xdim[s];
+          const bool neg = neg_all || (neg_odd && t.opar[j]);
+          src.p = (rev ? xrev : x) + b.off;
+          src.rs = tr ? 1 : ld;
+          src.cs = tr ? ld : 1;
+          src.scale = (neg ? -r.c : r.c) * g.e[4 * n1 + n0];
+        }
+      }
+    }
+    const uint32_t m = __ballot_sync(0xffffffffu, ok);
+    __syncwarp();                 // the previous sources are no longer read
+    if (ok) S[__popc(m & ((1u << lane) - 1))] = src;
+    __syncwarp();
+    const int ns = __popc(m);
+    if (cnt == 1) {
+#pragma unroll 4
+      for (int s = grp; s < ns; s += groups)
+        acc[0] = fma(S[s].scale, S[s].p[(int64_t)rr[0] * S[s].rs + (int64_t)cc[0] * S[s].cs], acc[0]);
+    } else {
+#pragma unroll 2
+      for (int s = 0; s < ns; ++s) {
+        const EnlSrc g = S[s];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (i < cnt) acc[i] = fma(g.scale, g.p[(int64_t)rr[i] * g.rs + (int64_t)cc[i] * g.cs], acc[i]);
+      }
+    }
+  }
+  const int ldd = t.fdim[fk];
+  double* dst = d + t.eoff[o * t.nse + fk] + (int64_t)t.foff[4 * fb + n1] * ldd + t.foff[4 * fk + n0];
+  if (groups > 1) {
+    double s = 0.0;               // the groups' sums, in order
+    for (int g = 0; g < groups; ++g) s += __shfl_sync(0xffffffffu, acc[0], g * n + e0);
+    if (lane < n) dst[(int64_t)rr[0] * ldd + cc[0]] = s;
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if (i < cnt && lane + 32 * i < left) dst[(int64_t)rr[i] * ldd + cc[i]] = acc[i];
+}
+
+__global__ void __launch_bounds__(32 * ENL_WARPS) enlarge_kernel(const EnlTables t, const int3* __restrict__ items,
+                                                                  int nitems, double* __restrict__ d,
+                                                                  const double* __restrict__ x,
+                                                                  const double* __restrict__ xrev) {
+  __shared__ EnlSmem S;
+  const int warp = threadIdx.x >> 5, w = blockIdx.x * ENL_WARPS + warp;
+  if (w >= nitems) return;
+  enlarge_item(t, items[w], d, x, xrev, S.s[warp]);
+}
+
+__global__ void __launch_bounds__(32 * ENL_WARPS) enlarge_inst_kernel(const EnlTables t, const int3* __restrict__ items,
+                                                                       int nitems, const __grid_constant__ GatherInstSet P,
+                                                                       int ninst) {
+  __shared__ EnlSmem S;
+  const int warp = threadIdx.x >> 5;
+  const unsigned w = blockIdx.x * ENL_WARPS + warp;
+  const int it = (int)(w / ninst);
+  if (it >= nitems) return;
+  const GatherBases* b = &P.b[w % ninst];
+  enlarge_item(t, items[it], b->d, b->s1, b->s2, S.s[warp]);
+}
+
+void launch_enlarge(const EnlTables& t, const int3* items, int nitems, double* d, const double* x, const double* xrev,
+                    cudaStream_t st) {
+  if (nitems <= 0) return;
+  enlarge_kernel<<<(nitems + ENL_WARPS - 1) / ENL_WARPS, 32 * ENL_WARPS, 0, st>>>(t, items, nitems, d, x, xrev);
+}
+
+void launch_enlarge_inst(const EnlTables& t, const int3* items, int nitems, const GatherInstSet& bases, int ninst,
+                         cudaStream_t st) {
+  // the caller checks 1 <= ninst <= 64 and nitems * ninst < 2^31
+  if (nitems <= 0 || ninst <= 0) return;
+  const long long n = (long long)nitems * ninst;
+  enlarge_inst_kernel<<<(unsigned)((n + ENL_WARPS - 1) / ENL_WARPS), 32 * ENL_WARPS, 0, st>>>(t, items, nitems, bases,
+                                                                                            ninst);
+}
+
+// ---------------------------------------------------------------------------
 // grouped FP64 GEMM with K-concatenated segments
 //
 // GB300 issues about 2 FP64 FMA per clock per SM, so the kernel is bound by the

@@ -82,7 +82,8 @@ void launch_gather(const GatherTask* tasks, const GatherSrc* srcs, const int3* t
                    cudaStream_t st, double* dbase = nullptr, const double* sbase1 = nullptr,
                    const double* sbase2 = nullptr);
 // one gather plan over up to GEMM_MAX_INST instances: CTA b runs work item b / ninst with
-// the bases of instance b % ninst (in the launch's parameter block)
+// the bases of instance b % ninst (in the
+// launch's parameter block); an enlargement's instances: the new set, X and its reverse set
 struct GatherBases {
   double* d;
   const double* s1;
@@ -93,6 +94,46 @@ struct GatherInstSet {
 };
 void launch_gather_inst(const GatherTask* tasks, const GatherSrc* srcs, const int3* tiles, int ntiles,
                         const GatherInstSet& bases, int ninst, cudaStream_t st);
+// Enlargement of an operator set by one site, its sources found on the device.  Operator o of
+// the new set is sum_r c_r X_{op_r} (x) site_r over refs[rbeg[o] .. rbeg[o + 1]) (site factor on
+// the left when `right`); its block of fused ket fk has sub-blocks (n1, n0), each the sum of the
+// references' blocks between the sectors behind n1 and n0.
+struct EnlRef {
+  int op;            // 2 * operator of X + transposed
+  int site;
+  double c;
+};
+struct EnlBlock {    // block (operator, ket sector) of X
+  int64_t off;
+  int bra;           // -1: none
+  int nz;            // not identically zero: bit 0 in X, bit 1 in the reverse set
+};
+struct EnlSite {
+  double e[16];      // e[4 * n1 + n0]
+  int mask, pad[3];  // its non-zeros
+};
+struct EnlTables {
+  const EnlRef* refs;
+  const int* rbeg;
+  const EnlBlock* blk;         // [operator * ns + ket]
+  const EnlSite* sites;
+  const int* xdim;             // per sector of X: states, parity of the electron count
+  const int* xpar;
+  const int* opar;             // per operator of X: parity
+  const int* fsub;             // [4 * fused + n]: sector behind sub-block n
+  const int* foff;             // and its offset
+  const int* fdim;
+  const int64_t* eoff;         // [operator * nse + ket] of the new set: block offset, bra
+  const int* ebra;
+  int ns, nse, right, pad;
+};
+constexpr int ENL_CHUNK = 128;   // elements per work item
+// items: (operator, 16 * fused ket + 4 * n1 + n0, first element); every element of an item's
+// chunk is written (the set's other sub-blocks are zero)
+void launch_enlarge(const EnlTables& t, const int3* items, int nitems, double* d, const double* x, const double* xrev,
+                    cudaStream_t st);
+void launch_enlarge_inst(const EnlTables& t, const int3* items, int nitems, const GatherInstSet& bases, int ninst,
+                         cudaStream_t st);
 // FP64 GEMM work items: output o, rows [m0, m0 + mt) and columns [n0, n0 + nt) of it,
 // mt <= GEMM_TM, nt <= GEMM_TN, packed as (o, (m0 << 8) | mt, (n0 << 8) | nt)
 inline int3 gemm_tile(int o, int m0, int mt, int n0, int nt) { return make_int3(o, (m0 << 8) | mt, (n0 << 8) | nt); }
