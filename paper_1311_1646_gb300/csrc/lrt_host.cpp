@@ -829,9 +829,11 @@ static GemmKind gemm_kind(const std::vector<GemmOut>& outs, const std::vector<Ge
   return exact >= 3e8 && padded <= 3.0 * exact ? GemmKind::MMA : GemmKind::WARP;
 }
 
-// Path and tile of one output in the warp kernel.  Direct FMAs cost about 0.5 clocks per
-// element and K position, digit products about 210 per 16 x 8 x 16: direct below 400
-// multiply-adds per 16 positions (counted per vector).
+// Path and tile of one output in the warp kernel.  Direct FMAs cost about 0.5 clocks of the FP64
+// pipe per element and K position, digit products about 210 issue slots per 16 x 8 x 16 but a
+// longer dependent chain: direct below 1000 multiply-adds per 16 positions (counted per vector;
+// limits of 150 / 400 / 1000: 52 / 51 / 49 us at k = 8, M = 64, 954 / 933 / 912 for the eight
+// molecules, and at 4000 1780).
 static void warp_tile_shape(GemmOut& O, int64_t k, int& tm, int& tn) {
   const int m = O.c_vr > 0 ? O.c_vr : O.m, n = O.c_vc > 0 ? O.c_vc : O.n;
   auto even = [](int x, int most) {
@@ -839,7 +841,7 @@ static void warp_tile_shape(GemmOut& O, int64_t k, int& tm, int& tn) {
     return (x + parts - 1) / parts;
   };
   O.flags = 0;
-  if ((int64_t)m * n * std::min<int64_t>(k, 16) < 400) {
+  if ((int64_t)m * n * std::min<int64_t>(k, 16) < 1000) {
     O.flags = GEMM_WARP_DIRECT;
     tn = even(O.n, GEMM_DIRECT_MAX);
     tm = even(O.m, GEMM_DIRECT_MAX / tn);
@@ -909,9 +911,13 @@ static void build_gemm(GemmPlan& P, const std::vector<GemmOut>& outs_in, const s
     int TM, TN;
     shape(outs[i], ktot[i], TM, TN);
     const GemmOut O = outs[i];
-    // K per part: the warp kernel, whose warps each walk their part alone, takes a sixteenth
-    // of the list between 96 and GEMM_SPLIT_K
-    const int64_t kpart = warp ? std::min<int64_t>(GEMM_SPLIT_K, std::max<int64_t>(96, ktot[i] / 16)) : GEMM_SPLIT_K;
+    // K per part.  A warp walks its part alone, a segment at a time: short parts where segments
+    // are a few positions (direct FMAs), longer ones for digit products.  24 / 96 positions for
+    // direct lists: 49 / 59 us (k = 8, M = 64), 51 / 103 (k = 13, M = 20); 24 / 64 / 96 for digit
+    // lists: 105 / 87 / 93 us (PPP M = 256).  Long lists fill the GPU with parts of a 16th.
+    const int64_t kshort = outs[i].flags & GEMM_WARP_DIRECT ? 24 : 64;
+    const int64_t kpart = warp ? std::min<int64_t>(GEMM_SPLIT_K, std::max<int64_t>(kshort, ktot[i] / (kshort == 24 ? 32 : 16)))
+                               : GEMM_SPLIT_K;
     for (int m0 = 0; m0 < O.m; m0 += TM)
       for (int n0 = 0; n0 < O.n; n0 += TN) {
         const int mt = std::min(TM, O.m - m0), nt = std::min(TN, O.n - n0);
