@@ -240,11 +240,16 @@ class Context:
                     "wfn_layout")
         return n.value, list(offs)[:nb.value]
 
+    def _wfn_size(self, site: int, nsite: int) -> int:
+        n = ctypes.c_int64()
+        self._check(self.lib.wfn_layout(self.h, site, nsite, ctypes.byref(n), None, None), "wfn_layout")
+        return n.value
+
     def renormalize(self, site: int, direction: int, precision: int = LRT_FP64):
         self._check(self.lib.renormalize(self.h, site, direction, precision), "renormalize")
 
     def sigma(self, site: int, nsite: int, x, y, nvec: int = 1, precision: int = LRT_FP64):
-        n, _ = self.wfn_layout(site, nsite)
+        n = self._wfn_size(site, nsite)
         self._check(self.lib.sigma(self.h, site, nsite, nvec, ctypes.c_void_p(_tensor_ptr(x, n * nvec)),
                                    ctypes.c_void_p(_tensor_ptr(y, n * nvec)), precision), "sigma")
 
@@ -254,12 +259,12 @@ class Context:
         synchronization).  Needs a plan prepared by an earlier sigma() call with the same
         (site, nsite, nvec); shares one static 32 MiB device array across all calls, so
         calls must not overlap on the GPU."""
-        n, _ = self.wfn_layout(site, nsite)
+        n = self._wfn_size(site, nsite)
         self._check(self.lib.sigma_noalloc(self.h, site, nsite, nvec, ctypes.c_void_p(_tensor_ptr(x, n * nvec)),
                                            ctypes.c_void_p(_tensor_ptr(y, n * nvec))), "sigma_noalloc")
 
     def heff_diag(self, site: int, nsite: int, d):
-        n, _ = self.wfn_layout(site, nsite)
+        n = self._wfn_size(site, nsite)
         self._check(self.lib.heff_diag(self.h, site, nsite, ctypes.c_void_p(_tensor_ptr(d, n))), "heff_diag")
 
     def sweep_gs(self, M_schedule, max_sweeps: int = 20, sweeps_per_M: int = 2, e_tol: float = 1e-10,
@@ -446,9 +451,9 @@ def sigma_batched(ctxs: list, sites: list, nsite: int, xs: list, ys: list, nvec:
         raise LrtError("sigma_batched: ctxs, sites, xs and ys must have the same non-zero length")
     hs = (ctypes.c_void_p * n)(*[c.h.value for c in ctxs])
     st = (ctypes.c_int * n)(*sites)
-    px = (ctypes.c_void_p * n)(*[_tensor_ptr(x, ctxs[j].wfn_layout(sites[j], nsite)[0] * nvec)
+    px = (ctypes.c_void_p * n)(*[_tensor_ptr(x, ctxs[j]._wfn_size(sites[j], nsite) * nvec)
                                  for j, x in enumerate(xs)])
-    py = (ctypes.c_void_p * n)(*[_tensor_ptr(y, ctxs[j].wfn_layout(sites[j], nsite)[0] * nvec)
+    py = (ctypes.c_void_p * n)(*[_tensor_ptr(y, ctxs[j]._wfn_size(sites[j], nsite) * nvec)
                                  for j, y in enumerate(ys)])
     ctxs[0]._check(ctxs[0].lib.sigma_batched(hs, n, st, nsite, nvec, px, py, precision), "sigma_batched")
 

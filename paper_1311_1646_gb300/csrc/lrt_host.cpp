@@ -858,7 +858,8 @@ static void warp_tile_shape(GemmOut& O, int64_t k, int& tm, int& tn) {
 // which the reduction launch does not know)
 enum class GemmSplit { NEVER, WARP, ALWAYS };
 
-static void build_gemm(GemmPlan& P, const std::vector<GemmOut>& outs_in, const std::vector<GemmSeg>& segs,
+// outs is worked on in place: the parts of split tiles are appended
+static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vector<GemmSeg>& segs,
                        cudaStream_t st, GemmSplit split = GemmSplit::NEVER) {
   // A tile costs its warps of outputs times its K chunks of DFMA issue, plus a fixed
   // cost per chunk.  Tiles far longer than an even share of the launch (an output with
@@ -873,15 +874,14 @@ static void build_gemm(GemmPlan& P, const std::vector<GemmOut>& outs_in, const s
   // slices of a quarter share were measured 2.5x slower on the k = 24 workload's phase 2:
   // every slice stages the whole K range of B for a few rows; a K part stages only its
   // own range.)
-  std::vector<GemmOut> outs = outs_in;
-  std::vector<int64_t> ktot(outs_in.size(), 0);
+  const size_t nout = outs.size();   // the parts of split tiles follow
+  std::vector<int64_t> ktot(nout, 0);
   double fl = 0.0;
-  for (size_t i = 0; i < outs_in.size(); ++i)
-    for (int s = 0; s < outs_in[i].seg_count; ++s) {
-      ktot[i] += segs[outs_in[i].seg_begin + s].k;
-      fl += 2.0 * outs_in[i].m * (double)outs_in[i].n * segs[outs_in[i].seg_begin + s].k;
-    }
-  const GemmKind kind = gemm_kind(outs_in, segs, ktot);
+  for (size_t i = 0; i < nout; ++i) {
+    for (int s = 0; s < outs[i].seg_count; ++s) ktot[i] += segs[outs[i].seg_begin + s].k;
+    fl += 2.0 * outs[i].m * (double)outs[i].n * (double)ktot[i];
+  }
+  const GemmKind kind = gemm_kind(outs, segs, ktot);
   const bool mma = kind == GemmKind::MMA, warp = kind == GemmKind::WARP;
   auto cost = [mma, warp](int64_t mt, int64_t nt, int64_t k) {
     const int64_t nch = (k + GEMM_KC - 1) / GEMM_KC;
@@ -896,18 +896,19 @@ static void build_gemm(GemmPlan& P, const std::vector<GemmOut>& outs_in, const s
     if (warp) warp_tile_shape(O, k, tm, tn);
   };
   int64_t total = 0;
-  for (size_t i = 0; i < outs_in.size() && kind == GemmKind::FP64; ++i) {
+  for (size_t i = 0; i < nout && kind == GemmKind::FP64; ++i) {
     int TM, TN;
     shape(outs[i], ktot[i], TM, TN);
-    for (int m0 = 0; m0 < outs_in[i].m; m0 += TM)
-      for (int n0 = 0; n0 < outs_in[i].n; n0 += TN)
-        total += cost(std::min(TM, outs_in[i].m - m0), std::min(TN, outs_in[i].n - n0), ktot[i]);
+    for (int m0 = 0; m0 < outs[i].m; m0 += TM)
+      for (int n0 = 0; n0 < outs[i].n; n0 += TN)
+        total += cost(std::min(TM, outs[i].m - m0), std::min(TN, outs[i].n - n0), ktot[i]);
   }
   const int64_t cap = std::max<int64_t>(1, total / gemm_fp64_slots());
   std::vector<std::pair<int64_t, int3>> tl;
   std::vector<SplitTile> sp;
   int64_t wsz = 0;
-  for (size_t i = 0; i < outs_in.size(); ++i) {
+  tl.reserve(nout + nout / 4);
+  for (size_t i = 0; i < nout; ++i) {
     int TM, TN;
     shape(outs[i], ktot[i], TM, TN);
     const GemmOut O = outs[i];
@@ -976,7 +977,7 @@ static void build_gemm(GemmPlan& P, const std::vector<GemmOut>& outs_in, const s
   P.segs.upload(segs, st);
   P.tiles.upload(tiles, st);
   P.ntiles = (int)tiles.size();
-  P.nbase = (int)outs_in.size();
+  P.nbase = (int)nout;
   P.splits.upload(sp, st);
   P.nsplit = (int)sp.size();
   if (wsz > 0) P.ws.ensure((size_t)wsz);
@@ -1111,6 +1112,35 @@ struct TcPlan {
   }
 };
 
+// Lists of a sigma plan under construction, kept by the context for the next plan.  At most
+// PLAN_SCRATCH_BYTES stay; freed with the context.
+struct Prod2 {                    // a phase-2 product
+  int64_t a_off;
+  const double* B;
+  double scale;
+  int out, lda, ldb, k;
+  short transB, ident, rev;       // B transposed; A rows from x; B in the reverse set
+};
+constexpr size_t PLAN_SCRATCH_BYTES = (size_t)256 << 20;
+struct PlanScratch {
+  std::vector<Prod2> prod2;
+  std::vector<GemmOut> o1;
+  std::vector<GemmSeg> s1, s2;
+  std::vector<char> s1rev;
+  void clear() {
+    prod2.clear();
+    o1.clear();
+    s1.clear();
+    s2.clear();
+    s1rev.clear();
+  }
+  void trim() {
+    if (prod2.capacity() * sizeof(Prod2) + o1.capacity() * sizeof(GemmOut) +
+            (s1.capacity() + s2.capacity()) * sizeof(GemmSeg) + s1rev.capacity() > PLAN_SCRATCH_BYTES)
+      *this = PlanScratch();
+  }
+};
+
 struct SigmaPlan {
   uint64_t serial = 0;      // unique per plan (batched launches detect rebuilt plans by it)
   bool has_tc = false;      // the tensor-core twin was planned
@@ -1170,6 +1200,7 @@ struct lrt_ctx {
   std::vector<lrt::SiteTensor> sites_r;   // right-canonical form, when given separately
   std::vector<std::unique_ptr<lrt::OpSet>> L, R, XL, YR;
   std::map<std::tuple<int, int, int>, std::unique_ptr<lrt::SigmaPlan>> plans;
+  lrt::PlanScratch scratch;
   lrt_sigma_stats last{};
   int last_sweeps = 0;
   std::vector<std::pair<double, int>> sweep_log;   // last sweep_tda: seconds and mixed flag per sweep
@@ -1782,17 +1813,25 @@ static uint16_t transpose_mask(uint16_t m) {
 // sets of first-order (transition) operator sets, read by transposed references.
 static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, const OpSet* Xrev, const OpSet& Y,
                                                   const OpSet* Yrev, int site, int nsite, int nvec, bool tc = true,
-                                                  bool rel_ops = false) {
+                                                  bool rel_ops = false, bool diag_only = false) {
   if (rel_ops && tc) throw Error(LRT_EINVAL, "internal: relative operator addresses are FP64 only");
   const Ints& I = c->I;
   const int k = c->k;
   const Fused& XF = *X.fused;
   const Fused* YF = (nsite == 2) ? Y.fused.get() : nullptr;
   const std::vector<WfnBlock> wb = wfn_blocks(c, site, nsite);
-  std::unordered_map<int, int> blk_of;   // label key -> wfn block
-  for (size_t i = 0; i < wb.size(); ++i) blk_of[Sectors::key(wb[i].label_a, wb[i].label_b)] = (int)i;
   int64_t nelem = 0;
   for (auto& w : wb) nelem = std::max(nelem, w.off + (int64_t)w.rows * w.cols);
+  // per sector of X: its wavefunction block and the sector of Y with the same label
+  std::vector<int> w_of(X.ns(), -1), y_of(X.ns(), -1);
+  {
+    Sectors lab;
+    for (const WfnBlock& w : wb) lab.add(w.label_a, w.label_b, 0);
+    for (int f = 0; f < X.ns(); ++f) {
+      w_of[f] = lab.find(X.basis.a[f], X.basis.b[f]);
+      y_of[f] = Y.basis.find(X.basis.a[f], X.basis.b[f]);
+    }
+  }
 
   std::vector<Term> terms;
   terms.push_back({1.0, {KH, -1, -1, 0}, {KI, -1, -1, 0}});
@@ -1809,29 +1848,32 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
   // every sub-block of y is an output (written even when no product reaches it)
   struct OutSub { int blk, r, mcol; };
   std::vector<OutSub> osub;
-  std::map<std::tuple<int, int, int>, int> out_of;
+  std::vector<int> out_of(16 * wb.size(), -1);   // [16 * block + 4 * row sub-block + column sub-block]
   for (size_t w = 0; w < wb.size(); ++w) {
     const int fx = XF.s.find(wb[w].label_a, wb[w].label_b);
     for (int r = 0; r < 4; ++r) {
       if (XF.dim[fx][r] == 0) continue;
       if (nsite == 1) {
-        out_of[{(int)w, r, 0}] = (int)osub.size();
+        out_of[16 * w + 4 * r] = (int)osub.size();
         osub.push_back({(int)w, r, 0});
       } else {
         const int fy = YF->s.find(wb[w].label_a, wb[w].label_b);
         for (int m = 0; m < 4; ++m) {
           if (YF->dim[fy][m] == 0) continue;
-          out_of[{(int)w, r, m}] = (int)osub.size();
+          out_of[16 * w + 4 * r + m] = (int)osub.size();
           osub.push_back({(int)w, r, m});
         }
       }
     }
   }
-  std::vector<std::vector<GemmSeg>> seg2(osub.size());
-  std::vector<std::vector<const OpSet*>> seg2set(osub.size());
-  std::vector<GemmOut> o1;
-  std::vector<GemmSeg> s1;
-  std::vector<const OpSet*> s1set;
+  // phase-2 products in the order they are found, sorted by output below; the lists live in the
+  // context's scratch (their pages are touched once, not at every plan)
+  PlanScratch& W = c->scratch;
+  W.clear();
+  std::vector<Prod2>& prod2 = W.prod2;
+  std::vector<GemmOut>& o1 = W.o1;
+  std::vector<GemmSeg>& s1 = W.s1;
+  std::vector<char>& s1rev = W.s1rev;   // the operator lives in the reverse set
   // Tensor-core twin: whole fused blocks instead of 4 x 4 sub-blocks (structurally
   // zero sub-blocks are stored zeros), so that the products fill the 128-row tiles.
   // Phase 1: per T block and right column group m, T_m = op(O_X) x_m; phase 2: per
@@ -1839,8 +1881,8 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
   TcPlan& tcp = plan->tc;
   std::map<std::tuple<int, int, int>, std::array<int, 4>> tc_T;   // T key -> TC matrix per m
   std::map<std::pair<int, int>, std::vector<TcPlanSeg>> tc_y;     // (y block, column group) -> products
-  struct TEntry { int64_t tp; uint16_t rows; };
-  std::map<std::tuple<int, int, int>, TEntry> tcache;   // (X op, trans, X ket fused) -> T
+  struct TEntry { int64_t tp; uint16_t rows; bool known; };
+  std::vector<TEntry> tcache(2 * X.keys.size() * (size_t)X.ns(), TEntry{-1, 0, false});   // (X op, trans, X ket fused) -> T
   int64_t toff = 0;
   std::vector<std::vector<DiagTerm>> dterm(wb.size());
   std::vector<Ref> rx, ry;
@@ -1865,14 +1907,10 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
           const int fb0 = X.bra_of(a.op, f);
           if (fb0 < 0 || !XS.block_nz(a.op, f)) continue;
           const int be = a.t ? f : fb0, ke = a.t ? fb0 : f;
-          auto ik = blk_of.find(Sectors::key(X.basis.a[ke], X.basis.b[ke]));
-          auto ib = blk_of.find(Sectors::key(X.basis.a[be], X.basis.b[be]));
-          if (ik == blk_of.end() || ib == blk_of.end()) continue;
-          const WfnBlock& wk = wb[ik->second];
-          const WfnBlock& wbb = wb[ib->second];
-          const int yk = Y.basis.find(wk.label_a, wk.label_b);
-          const int ybb = Y.basis.find(wbb.label_a, wbb.label_b);
-          if (yk < 0 || ybb < 0) continue;
+          const int ik = w_of[ke], ib = w_of[be], yk = y_of[ke], ybb = y_of[be];
+          if (ik < 0 || ib < 0 || yk < 0 || ybb < 0) continue;
+          const WfnBlock& wk = wb[ik];
+          const WfnBlock& wbb = wb[ib];
           const double* Bp;
           int transB, ldb;
           uint16_t ymask = 1;   // stored blocks: one dense sub-block
@@ -1894,17 +1932,28 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
           ++nprod;
           op_bytes += 8.0 * ((double)Y.basis.d[yk] * Y.basis.d[ybb]);
 
+          // ---- diagonal contribution
+          const bool ident = (a.op == Ikey);
+          if (be == ke && yk == ybb) {
+            DiagTerm d{};
+            d.x = ident ? nullptr : XS.d + X.off_of(a.op, f);
+            d.xs = X.basis.d[f] + 1;
+            d.y = Bp;
+            d.ys = Y.basis.d[yk] + 1;
+            d.scale = sc;
+            dterm[ik].push_back(d);
+          }
+          if (diag_only) continue;
+
           // ---- phase 1 (shared by every Y partner of this X block)
           uint16_t rows = 0;
           int64_t tp = -1;
-          const bool ident = (a.op == Ikey);
           if (ident) {
             for (int r = 0; r < 4; ++r)
               if (XF.dim[be][r]) rows |= (uint16_t)(1u << r);
           } else {
-            const auto key = std::make_tuple(a.op, a.t, f);
-            auto it = tcache.find(key);
-            if (it == tcache.end()) {
+            TEntry& te = tcache[(2 * (size_t)a.op + a.t) * X.ns() + f];
+            if (!te.known) {
               uint16_t mx = XS.mask[(size_t)a.op * X.ns() + f];
               if (a.t) mx = transpose_mask(mx);
               tp = toff;
@@ -1937,7 +1986,7 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
                   g.k = XF.dim[ke][cc];
                   g.scale = 1.0;
                   s1.push_back(g);
-                  s1set.push_back(&XS);
+                  s1rev.push_back(&XS != &X);
                   ++out.seg_count;
                   falg += 2.0 * XF.dim[be][r] * XF.dim[ke][cc] * wk.cols;
                 }
@@ -1955,12 +2004,12 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
                   tcp.out1.push_back(TcPlanOut{tm[m], 0, 0, wbb.rows, dim, (int)tcp.segs.size(), 1});
                   tcp.segs.push_back(TcPlanSeg{A, B, wk.rows, 1.0f});
                 }
-                tc_T[key] = tm;
+                tc_T[std::make_tuple(a.op, a.t, f)] = tm;
               }
-              tcache[key] = TEntry{tp, rows};
+              te = TEntry{tp, rows, true};
             } else {
-              tp = it->second.tp;
-              rows = it->second.rows;
+              tp = te.tp;
+              rows = te.rows;
             }
           }
           // ---- phase 2
@@ -1969,34 +2018,17 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
             const int64_t arow = ident ? wk.off + (int64_t)XF.off[ke][r] * wk.cols
                                        : tp + (int64_t)XF.off[be][r] * wk.cols;
             if (nsite == 1) {
-              GemmSeg g{};
-              g.a_rel = ident ? 1 : 0;
-              g.a_off = arow;
-              g.lda = wk.cols;
-              g.B = Bp;
-              g.ldb = ldb;
-              g.transB = transB;
-              g.k = wk.cols;
-              g.scale = sc;
-              seg2[out_of.at({ib->second, r, 0})].push_back(g);
-              seg2set[out_of.at({ib->second, r, 0})].push_back(&YS);
+              prod2.push_back(Prod2{arow, Bp, sc, out_of[16 * ib + 4 * r], wk.cols, ldb, wk.cols, (short)transB,
+                                    (short)ident, (short)(&YS != &Y)});
               falg += 2.0 * XF.dim[be][r] * wk.cols * wbb.cols;
             } else {
               for (int mp = 0; mp < 4; ++mp)
                 for (int m = 0; m < 4; ++m) {
                   if (!(ymask & (1u << (4 * mp + m)))) continue;
-                  GemmSeg g{};
-                  g.a_rel = ident ? 1 : 0;
-                  g.a_off = arow + YF->off[yk][m];
-                  g.lda = wk.cols;
-                  if (!bref.t) g.B = Bp + (int64_t)YF->off[ybb][mp] * ldb + YF->off[yk][m];
-                  else g.B = Bp + (int64_t)YF->off[yk][m] * ldb + YF->off[ybb][mp];
-                  g.ldb = ldb;
-                  g.transB = transB;
-                  g.k = YF->dim[yk][m];
-                  g.scale = sc;
-                  seg2[out_of.at({ib->second, r, mp})].push_back(g);
-                  seg2set[out_of.at({ib->second, r, mp})].push_back(&YS);
+                  const double* B = !bref.t ? Bp + (int64_t)YF->off[ybb][mp] * ldb + YF->off[yk][m]
+                                            : Bp + (int64_t)YF->off[yk][m] * ldb + YF->off[ybb][mp];
+                  prod2.push_back(Prod2{arow + YF->off[yk][m], B, sc, out_of[16 * ib + 4 * r + mp], wk.cols, ldb,
+                                        YF->dim[yk][m], (short)transB, (short)ident, (short)(&YS != &Y)});
                   falg += 2.0 * XF.dim[be][r] * YF->dim[yk][m] * YF->dim[ybb][mp];
                 }
             }
@@ -2006,7 +2038,7 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
             if (nsite == 1) {
               const int A = ident ? tcp.x(wk.off, wk.cols, 0, wk.rows, wk.cols) : (*tm)[0];
               const int B = tcp.op(Bp, ldb, bref.t ? 1 : 0, Y.basis.d[ybb], Y.basis.d[yk]);
-              tc_y[{ib->second, 0}].push_back(TcPlanSeg{A, B, wk.cols, (float)sc});
+              tc_y[{ib, 0}].push_back(TcPlanSeg{A, B, wk.cols, (float)sc});
             } else {
               for (int mp = 0; mp < 4; ++mp)
                 for (int m = 0; m < 4; ++m) {
@@ -2016,47 +2048,29 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
                   const double* src = !bref.t ? Bp + (int64_t)YF->off[ybb][mp] * ldb + YF->off[yk][m]
                                               : Bp + (int64_t)YF->off[yk][m] * ldb + YF->off[ybb][mp];
                   const int B = tcp.op(src, ldb, bref.t ? 1 : 0, YF->dim[ybb][mp], YF->dim[yk][m]);
-                  tc_y[{ib->second, mp}].push_back(TcPlanSeg{A, B, YF->dim[yk][m], (float)sc});
+                  tc_y[{ib, mp}].push_back(TcPlanSeg{A, B, YF->dim[yk][m], (float)sc});
                 }
             }
-          }
-          // ---- diagonal contribution
-          if (be == ke && yk == ybb) {
-            DiagTerm d{};
-            d.x = ident ? nullptr : XS.d + X.off_of(a.op, f);
-            d.xs = X.basis.d[f] + 1;
-            d.y = Bp;
-            d.ys = Y.basis.d[yk] + 1;
-            d.scale = sc;
-            dterm[ik->second].push_back(d);
           }
         }
       }
   }
   if (toff > 0 && dev_alloc((void**)&plan->tbuf, (size_t)toff * nvec * sizeof(double)) != cudaSuccess)
     throw Error(LRT_ENOMEM, "sigma workspace");
-  std::vector<GemmOut> O1, O2;
-  std::vector<GemmSeg> S1, S2;
+  std::vector<GemmOut> O2;
+  std::vector<GemmSeg>& S2 = W.s2;
   plan->tsize = toff * nvec;
   // operator pointers as offsets from the set they live in (extra bases 0..3)
-  auto set_rel = [&](const OpSet* S) { return S == &X ? 3 : S == Xrev ? 4 : S == &Y ? 5 : 6; };
   if (rel_ops) {
     plan->ex.p[0] = X.d;
     plan->ex.p[1] = Xrev ? Xrev->d : nullptr;
     plan->ex.p[2] = Y.d;
     plan->ex.p[3] = Yrev ? Yrev->d : nullptr;
     for (size_t q = 0; q < s1.size(); ++q) {
-      s1[q].a_off = s1[q].A - s1set[q]->d;
+      s1[q].a_off = s1[q].A - plan->ex.p[s1rev[q]];
       s1[q].A = nullptr;
-      s1[q].a_rel = set_rel(s1set[q]);
+      s1[q].a_rel = 3 + s1rev[q];
     }
-    for (size_t u = 0; u < seg2.size(); ++u)
-      for (size_t q = 0; q < seg2[u].size(); ++q) {
-        GemmSeg& g = seg2[u][q];
-        g.b_off = g.B - seg2set[u][q]->d;
-        g.B = nullptr;
-        g.b_rel = set_rel(seg2set[u][q]);
-      }
   }
   // The vectors of a call share every operator block: phase 1 (T = X x) places them side by
   // side along the columns of one output (x's block of vector v at + v * nelem, T of vector v
@@ -2064,26 +2078,22 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
   // vector v at + v * toff or + v * nelem, y of vector v at + v * nelem).  One output then
   // holds the same block product for every vector, which fills the GEMM's tiles.
   const bool vb = nvec > 1;
-  for (const GemmOut& x : o1) {
-    GemmOut y = x;
-    y.C = nullptr;
+  for (GemmOut& y : o1) {
     y.c_rel = 2;
-    y.seg_begin = (int)S1.size();
     if (vb) {
-      y.n = x.n * nvec;
-      y.c_vc = x.n;
+      const int n = y.n;
+      for (int q = 0; q < y.seg_count; ++q) {
+        s1[y.seg_begin + q].b_vc = n;
+        s1[y.seg_begin + q].b_vs = nelem;
+      }
+      y.n = n * nvec;
+      y.c_vc = n;
       y.c_vs = toff;
     }
-    for (int q = 0; q < x.seg_count; ++q) {
-      GemmSeg g = s1[x.seg_begin + q];
-      if (vb) {
-        g.b_vc = x.n;
-        g.b_vs = nelem;
-      }
-      S1.push_back(g);
-    }
-    O1.push_back(y);
   }
+  std::vector<int> at(osub.size() + 1, 0);   // first product of every output
+  for (const Prod2& p : prod2) ++at[p.out + 1];
+  for (size_t u = 0; u < osub.size(); ++u) at[u + 1] += at[u];
   for (size_t u = 0; u < osub.size(); ++u) {
     const OutSub& os = osub[u];
     const WfnBlock& w = wb[os.blk];
@@ -2096,27 +2106,38 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
       ncols = YF->dim[fy][os.mcol];
     }
     const int m1 = XF.dim[fx][os.r];
-    GemmOut y{nullptr, coff, w.cols, m1 * nvec, ncols, (int)S2.size(), (int)seg2[u].size(), 0, 1};
+    GemmOut y{nullptr, coff, w.cols, m1 * nvec, ncols, at[u], at[u + 1] - at[u], 0, 1};
     y.balance = 1;
     if (vb) {
       y.c_vr = m1;
       y.c_vs = nelem;
     }
-    for (size_t q = 0; q < seg2[u].size(); ++q) {
-      GemmSeg g = seg2[u][q];
-      const int64_t vs = g.a_rel ? nelem : toff;
-      if (!g.a_rel) g.a_rel = 2;
-      if (vb) {
-        g.a_vr = m1;
-        g.a_vs = vs;
-      }
-      S2.push_back(g);
-    }
     O2.push_back(y);
   }
-  build_gemm(plan->p1, O1, S1, c->st);
+  S2.resize(prod2.size());
+  for (const Prod2& p : prod2) {
+    GemmSeg& g = S2[at[p.out]++];
+    g.a_rel = p.ident ? 1 : 2;
+    g.a_off = p.a_off;
+    g.lda = p.lda;
+    g.ldb = p.ldb;
+    g.transB = p.transB;
+    g.k = p.k;
+    g.scale = p.scale;
+    if (rel_ops) {
+      g.b_off = p.B - plan->ex.p[2 + p.rev];
+      g.b_rel = 5 + p.rev;
+    } else {
+      g.B = p.B;
+    }
+    if (vb) {
+      g.a_vr = O2[p.out].c_vr;
+      g.a_vs = p.ident ? nelem : toff;
+    }
+  }
+  if (!diag_only) build_gemm(plan->p1, o1, s1, c->st);
   // kept relative plans are replayed over instances
-  build_gemm(plan->p2, O2, S2, c->st, rel_ops ? GemmSplit::NEVER : GemmSplit::ALWAYS);
+  if (!diag_only) build_gemm(plan->p2, O2, S2, c->st, rel_ops ? GemmSplit::NEVER : GemmSplit::ALWAYS);
   // tensor-core twin: phase-2 outputs, one per (y block, column group)
   plan->has_tc = tc;
   for (size_t w = 0; w < wb.size() && tc; ++w)
@@ -2148,10 +2169,11 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
   plan->op_bytes = op_bytes;
   plan->flops_alg = falg * nvec;
   CK(cudaStreamSynchronize(c->st));
+  W.trim();
   return plan;
 }
 
-static std::unique_ptr<SigmaPlan> plan_sigma(lrt_ctx* c, int site, int nsite, int nvec, bool tc) {
+static std::unique_ptr<SigmaPlan> plan_sigma(lrt_ctx* c, int site, int nsite, int nvec, bool tc, bool diag_only = false) {
   OpSet& X = enlarged(c, site, false);
   OpSet* Yp;
   if (nsite == 1) {
@@ -2160,7 +2182,7 @@ static std::unique_ptr<SigmaPlan> plan_sigma(lrt_ctx* c, int site, int nsite, in
   } else {
     Yp = &enlarged(c, site + 1, true);
   }
-  return plan_sigma_sets(c, X, nullptr, *Yp, nullptr, site, nsite, nvec, tc);
+  return plan_sigma_sets(c, X, nullptr, *Yp, nullptr, site, nsite, nvec, tc, false, diag_only);
 }
 
 // Work stream of one tensor-core launch over one or several plans (instances): tiles
@@ -2679,6 +2701,23 @@ static SigmaPlan* find_plan(lrt_ctx* c, int site, int nsite, int nvec) {
   return it == c->plans.end() ? nullptr : it->second.get();
 }
 
+// a plan of (site, nsite) for any number of vectors
+static SigmaPlan* any_plan(lrt_ctx* c, int site, int nsite) {
+  auto it = c->plans.lower_bound(std::make_tuple(site, nsite, 0));
+  return it != c->plans.end() && std::get<0>(it->first) == site && std::get<1>(it->first) == nsite ? it->second.get()
+                                                                                                  : nullptr;
+}
+
+// the diagonal of (site, nsite), which any plan of the position holds; without one, a plan of the
+// diagonal alone (kept as nvec 0)
+static SigmaPlan& get_diag_plan(lrt_ctx* c, int site, int nsite) {
+  if (SigmaPlan* p = any_plan(c, site, nsite)) return *p;
+  auto p = plan_sigma(c, site, nsite, 1, false, true);
+  SigmaPlan& ref = *p;
+  c->plans[std::make_tuple(site, nsite, 0)] = std::move(p);
+  return ref;
+}
+
 // the plan of (site, nsite, nvec); tc: with the tensor-core twin (replanned if missing)
 static SigmaPlan& get_plan(lrt_ctx* c, int site, int nsite, int nvec, bool tc = false) {
   auto key = std::make_tuple(site, nsite, nvec);
@@ -3167,7 +3206,7 @@ static SiteTensor new_site(lrt_ctx* c, int i) {
   return T;
 }
 
-static void run_gemms(lrt_ctx* c, const std::vector<GemmOut>& o, const std::vector<GemmSeg>& g) {
+static void run_gemms(lrt_ctx* c, std::vector<GemmOut>& o, const std::vector<GemmSeg>& g) {
   if (o.empty()) return;
   GemmPlan p;
   build_gemm(p, o, g, c->st);
@@ -5826,6 +5865,12 @@ int wfn_layout(lrt_t ctx, int site, int nsite, int64_t* nelem, int* nblocks, int
   return guard(ctx, [&] {
     if (!ctx->have_mps) throw Error(LRT_ESTATE, "wfn_layout: no MPS loaded");
     if (nsite < 1 || nsite > 2 || site < 0 || site + nsite > ctx->k) throw Error(LRT_EINVAL, "wfn_layout: bad site");
+    if (nelem && !nblocks && !block_offsets) {   // the size alone: any plan of the position holds it
+      if (const SigmaPlan* p = any_plan(ctx, site, nsite)) {
+        *nelem = p->nelem;
+        return;
+      }
+    }
     auto wb = wfn_blocks(ctx, site, nsite);
     int64_t n = 0;
     for (auto& w : wb) n = std::max(n, w.off + (int64_t)w.rows * w.cols);
@@ -5893,7 +5938,7 @@ int heff_diag(lrt_t ctx, int site, int nsite, double* d_dev) {
     if (!ctx->have_mps || !ctx->have_ham) throw Error(LRT_ESTATE, "heff_diag: op_build and mps_load first");
     if (nsite < 1 || nsite > 2 || site < 0 || site + nsite > ctx->k || !d_dev) throw Error(LRT_EINVAL, "heff_diag: bad arguments");
     if (!ctx->L[site]) throw Error(LRT_ESTATE, "heff_diag: left block missing");
-    SigmaPlan& p = get_plan(ctx, site, nsite, 1);
+    SigmaPlan& p = get_diag_plan(ctx, site, nsite);
     launch_diag(p.douts.p, p.dterms.p, p.ndiag, d_dev, ctx->st);
     CK(cudaGetLastError());
   });
