@@ -128,14 +128,16 @@ int wfn_layout(lrt_t ctx, int site, int nsite, int64_t* nelem, int* nblocks, int
  * `site`.  Left block 0 and right block k are the vacuum and always exist.
  * precision LRT_FP64, or LRT_MIXED: the enlarged operators are formed in FP64 and the
  * two grouped contractions O' = L^T (E L) run as split-TF32 tensor-core products with
- * FP32 accumulation per block product (the new operators are stored in FP64). */
+ * FP32 accumulation per block product (the new operators are stored in FP64); sets too
+ * small to gain from them are renormalized in FP64. */
 int renormalize(lrt_t ctx, int site, int dir, int precision);
 
 /* sigma = H_eff x (Eq. dmrg) for `nvec` wavefunctions stored back to back in the
  * wfn_layout order: nsite = 1 uses the left block of bond `site` and the right block
  * of bond site+1; nsite = 2 uses the left block of bond `site` and the right block of
  * bond site+2.  x_dev, y_dev: device pointers of nvec * nelem doubles; must not
- * overlap. */
+ * overlap.  precision LRT_MIXED allows split-TF32 tensor-core products (about seven digits);
+ * calls too small to gain from them run in FP64. */
 int sigma(lrt_t ctx, int site, int nsite, int nvec, const double* x_dev, double* y_dev,
           int precision);
 
@@ -300,8 +302,8 @@ int sweep_response(lrt_t ctx, lrt_t vctx, double omega, const lrt_resp_params* p
 int lrt_sweeps(lrt_t ctx, int* sweeps);
 /* lrt_sweep_log: the wall time of every sweep of the last sweep_tda on this context (the
  * start sweep first; each time from the sweep's start to the host synchronization that
- * ends it, so it includes all its device work) and whether its H_0 site products ran on
- * the tensor cores (1) or in FP64 (0).  Writes min(cap, n) entries to seconds and mixed
+ * ends it, so it includes all its device work) and whether its H_0 site products ran in the
+ * mixed form (1) or in FP64 (0).  Writes min(cap, n) entries to seconds and mixed
  * (host arrays of cap elements; NULL allowed when cap is 0) and the number of sweeps to *n. */
 int lrt_sweep_log(lrt_t ctx, int cap, double* seconds, int* mixed, int* n);
 /* sweep_tda_batched: the DMRG-TDA sweeps of Fig. alg:dmrgtda for n_inst independent

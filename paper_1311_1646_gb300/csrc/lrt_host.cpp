@@ -1157,6 +1157,7 @@ struct SigmaPlan {
   int n_terms = 0, n_products = 0;
   double op_bytes = 0.0;
   double flops_alg = 0.0;   // products of non-zero sub-blocks only
+  double macs1 = -1.0;      // phase1_macs of the position, once known
   // tensor-core twin of the two phases (host description; device streams built on
   // first mixed use): whole fused blocks, operands as TC matrices in three pools
   // (0: operator sub-matrices, 1: x-derived, per vector, 2: intermediates T, per vector)
@@ -1570,11 +1571,16 @@ static void ren_absolute(std::vector<GemmOut>& o1, std::vector<GemmSeg>& s1, std
   outs(o2);
 }
 
+static bool mixed_in_fp64(lrt_ctx* c, double macs, int nvec);
+
 // runs (and, given a template slot, keeps) a renormalization's two grouped GEMMs
 static void ren_run(lrt_ctx* c, std::vector<GemmOut>& o1, std::vector<GemmSeg>& s1, std::vector<GemmOut>& o2,
                     std::vector<GemmSeg>& s2, int64_t toff, const GemmExtra& ex, int prec, RenTemplate* tpl,
                     const OpSet& N, uint64_t sig) {
-  if (prec == LRT_MIXED) {
+  double macs = 0.0;
+  if (prec == LRT_MIXED)
+    for (const GemmOut& o : o1) macs += (double)o.m * o.n * s1[o.seg_begin].k;
+  if (prec == LRT_MIXED && !mixed_in_fp64(c, macs, 1)) {
     ren_absolute(o1, s1, o2, s2, ex);
     run_two_phase_tc(c, o1, s1, o2, s2);
     return;
@@ -2729,6 +2735,52 @@ static SigmaPlan& get_plan(lrt_ctx* c, int site, int nsite, int nvec, bool tc = 
   return ref;
 }
 
+// LRT_MIXED calls that run on the FP64 kernels: the split-TF32 kernel fills one persistent CTA per
+// SM with 128-row tiles and pays a host synchronization per call, which short lists of small
+// blocks do not repay, and the FP64 digit products are the more exact of the two.  Measured,
+// split-TF32 / FP64: two-site k = 13, M = 200, 3 vectors (1e8 multiply-adds of phase 1 per
+// vector) 3.89 / 1.52 ms; k = 24, M = 500, 6 vectors (1.9e9) 6.55 / 17.0 ms.  A pending
+// stall (lrt_set_wait_limit) is for the next tensor-core launch, so such a call keeps it.
+constexpr double MIXED_MIN_MACS = 2e8, MIXED_MIN_TOTAL = 7e8;   // phase 1, per vector / of the call
+static bool mixed_in_fp64(lrt_ctx* c, double macs, int nvec) {
+  return !c->tc_stall && macs < MIXED_MIN_MACS && macs * nvec < MIXED_MIN_TOTAL;
+}
+
+// multiply-adds of X psi over the non-zero sub-blocks of the enlarged left set, one vector
+static double phase1_macs(lrt_ctx* c, const OpSet& X, int site, int nsite) {
+  std::vector<double> cols(X.ns(), 0.0);
+  for (const WfnBlock& w : wfn_blocks(c, site, nsite)) {
+    const int f = X.basis.find(w.label_a, w.label_b);
+    if (f >= 0) cols[f] = w.cols;
+  }
+  const Fused& F = *X.fused;
+  double n = 0.0;
+  for (size_t o = 0; o < X.keys.size(); ++o)
+    for (int f = 0; f < X.ns(); ++f) {
+      const int fb = X.bra_of((int)o, f);
+      for (unsigned m = X.mask[o * X.ns() + f]; m; m &= m - 1) {
+        const int bit = __builtin_ctz(m);
+        n += (double)F.dim[fb][bit >> 2] * F.dim[f][bit & 3] * cols[f];
+      }
+    }
+  return n;
+}
+
+// the same, remembered by the position's plans
+static double position_macs(lrt_ctx* c, int site, int nsite) {
+  SigmaPlan* p = any_plan(c, site, nsite);
+  if (p && p->macs1 >= 0.0) return p->macs1;
+  const double m = phase1_macs(c, enlarged(c, site, false), site, nsite);
+  if (p) p->macs1 = m;
+  return m;
+}
+
+// the plan of a mixed sigma; tc: it runs on the split-TF32 kernels (and has their twin)
+static SigmaPlan& get_mixed_plan(lrt_ctx* c, int site, int nsite, int nvec, bool& tc) {
+  tc = !mixed_in_fp64(c, position_macs(c, site, nsite), nvec);
+  return get_plan(c, site, nsite, nvec, tc);
+}
+
 }  // namespace lrt
 
 // ===========================================================================
@@ -3758,9 +3810,11 @@ struct TdaRunner {
   // calls on whole blocks of `blk` vectors (the block-Davidson right-hand sides)
   void h0(int i, const SiteBatch& X, int nv, SiteBatch& Y) {
     auto& p = h0blk[{i, blk}];
-    if (!p) p = plan_sigma_sets(c, *c->XL[i], nullptr, *c->R[i + 1], nullptr, i, 1, blk, mixed);
-    if (mixed && !p->has_tc) p = plan_sigma_sets(c, *c->XL[i], nullptr, *c->R[i + 1], nullptr, i, 1, blk, true);
-    for (int v0 = 0; v0 < nv; v0 += blk) run_plan(*p, X.v(v0), Y.v(v0), blk, mixed);
+    const double macs = !mixed || (p && p->macs1 >= 0.0) ? (p ? p->macs1 : -1.0) : phase1_macs(c, *c->XL[i], i, 1);
+    const bool tc = mixed && !mixed_in_fp64(c, macs, blk);
+    if (!p || (tc && !p->has_tc)) p = plan_sigma_sets(c, *c->XL[i], nullptr, *c->R[i + 1], nullptr, i, 1, blk, tc);
+    p->macs1 = macs;
+    for (int v0 = 0; v0 < nv; v0 += blk) run_plan(*p, X.v(v0), Y.v(v0), blk, tc);
   }
 
   // ---- batched bond/site products: grouped GEMMs planned once per (kind, site, nv) with
@@ -5570,6 +5624,22 @@ static void sigma_batched_impl(lrt_ctx* const* ctxs, int n, const int* sites, in
                                const double* const* x, double* const* y, int precision) {
   lrt_ctx* c0 = ctxs[0];
   std::vector<SigmaPlan*> plans(n);
+  bool missing = false;
+  for (int j = 0; j < n; ++j) missing = missing || !ctxs[j] || !ctxs[j]->have_mps || !ctxs[j]->have_ham;
+  if (precision == LRT_MIXED && !missing) {
+    // all instances small: the call runs in FP64 (see mixed_in_fp64)
+    double macs = 0.0;
+    bool small = !c0->tc_stall;
+    for (int j = 0; j < n && small; ++j) {
+      lrt_ctx* c = ctxs[j];
+      if (sites[j] < 0 || sites[j] + nsite > c->k || !c->L[sites[j]]) break;   // refused below
+      PoolScope ps(&c->pool);
+      const double m = position_macs(c, sites[j], nsite);
+      macs += m;
+      small = mixed_in_fp64(c, m, nvec) && macs * nvec < MIXED_MIN_TOTAL;
+    }
+    if (small) precision = LRT_FP64;
+  }
   std::string key = std::to_string(nsite) + ":" + std::to_string(nvec) + ":" + std::to_string(precision);
   for (int j = 0; j < n; ++j) {
     lrt_ctx* c = ctxs[j];
@@ -5903,10 +5973,11 @@ int sigma(lrt_t ctx, int site, int nsite, int nvec, const double* x_dev, double*
       throw Error(LRT_EINVAL, "sigma: bad arguments");
     if (precision != LRT_FP64 && precision != LRT_MIXED) throw Error(LRT_EINVAL, "sigma: bad precision");
     if (!ctx->L[site]) throw Error(LRT_ESTATE, "sigma: left block of bond " + std::to_string(site) + " missing");
-    SigmaPlan& p = get_plan(ctx, site, nsite, nvec, precision == LRT_MIXED);
+    bool tc = false;
+    SigmaPlan& p = precision == LRT_MIXED ? get_mixed_plan(ctx, site, nsite, nvec, tc) : get_plan(ctx, site, nsite, nvec);
     if ((const double*)y_dev < x_dev + p.nelem * nvec && x_dev < (const double*)y_dev + p.nelem * nvec)
       throw Error(LRT_EINVAL, "sigma: x and y overlap");
-    if (precision == LRT_MIXED) {
+    if (tc) {
       run_tc(ctx, p, x_dev, y_dev, nvec);
     } else {
       p.p1.run(ctx->st, x_dev, y_dev, p.tbuf, &p.ex);

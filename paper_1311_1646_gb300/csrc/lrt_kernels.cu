@@ -510,40 +510,44 @@ void launch_gemm_fp64(const GemmOut* outs, const GemmSeg* segs, const int3* tile
                                                                   nullptr, ex, wbase);
 }
 
-// One CTA per split tile: each element sums its parts in part order (deterministic), then
-// lands where the tile's output puts it, vector blocking included, as in the GEMM epilogue.
+// 256 elements of a split tile per CTA: each sums its parts in part order (deterministic), eight
+// loads in flight, then lands where the tile's output puts it, vector blocking included, as in
+// the GEMM epilogue.  (One CTA for a whole tile of 100 parts: 385 us on the k = 24, M = 500
+// workload, most SMs idle at the end.)
 __global__ void __launch_bounds__(256) split_reduce_kernel(const GemmOut* __restrict__ outs,
                                                            const SplitTile* __restrict__ tiles,
                                                            const double* __restrict__ wbase,
                                                            double* __restrict__ ybase, double* __restrict__ tbase) {
   const SplitTile t = tiles[blockIdx.x];
+  const int ne = t.mt * t.nt;
+  const int e = blockIdx.y * blockDim.x + threadIdx.x;
+  if (e >= ne) return;
   const GemmOut o = outs[t.o];
   double* cbase = o.c_rel == 1 ? ybase + o.c_off : o.c_rel == 2 ? tbase + o.c_off : o.C;
-  const int ne = t.mt * t.nt;
-  const double* w = wbase + t.ws_off;
-  for (int e = threadIdx.x; e < ne; e += blockDim.x) {
-    double s = 0.0;
-    for (int p = 0; p < t.nparts; ++p) s += w[(int64_t)p * ne + e];
-    int r = t.m0 + e / t.nt, col = t.n0 + e % t.nt;
-    double* c = cbase;
-    if (o.c_vr > 0) {
-      const int v = r / o.c_vr;
-      c += (int64_t)v * o.c_vs;
-      r -= v * o.c_vr;
-    } else if (o.c_vc > 0) {
-      const int v = col / o.c_vc;
-      c += (int64_t)v * o.c_vs;
-      col -= v * o.c_vc;
-    }
-    c += (int64_t)r * o.ldc + col;
-    *c = o.accumulate ? (*c + s) : s;
+  const double* w = wbase + t.ws_off + e;
+  double s = 0.0;
+#pragma unroll 8
+  for (int p = 0; p < t.nparts; ++p) s += w[(int64_t)p * ne];
+  int r = t.m0 + e / t.nt, col = t.n0 + e % t.nt;
+  double* c = cbase;
+  if (o.c_vr > 0) {
+    const int v = r / o.c_vr;
+    c += (int64_t)v * o.c_vs;
+    r -= v * o.c_vr;
+  } else if (o.c_vc > 0) {
+    const int v = col / o.c_vc;
+    c += (int64_t)v * o.c_vs;
+    col -= v * o.c_vc;
   }
+  c += (int64_t)r * o.ldc + col;
+  *c = o.accumulate ? (*c + s) : s;
 }
 
 void launch_split_reduce(const GemmOut* outs, const SplitTile* tiles, int ntiles, const double* wbase, double* ybase,
                          double* tbase, cudaStream_t st) {
   if (ntiles <= 0) return;
-  split_reduce_kernel<<<ntiles, 256, 0, st>>>(outs, tiles, wbase, ybase, tbase);
+  constexpr int most = GEMM_TM * GEMM_TN > 8 * 256 ? GEMM_TM * GEMM_TN : 8 * 256;   // elements of a tile (either kernel)
+  split_reduce_kernel<<<dim3(ntiles, (most + 255) / 256), 256, 0, st>>>(outs, tiles, wbase, ybase, tbase);
 }
 
 void launch_gemm_fp64_inst(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles,
