@@ -164,6 +164,12 @@ __device__ __forceinline__ long long join_digits(const float (&v)[MMA_ND][4], in
          ((long long)d4 << 5) + (long long)(d5 + d6);
 }
 
+// x times the power of two with exponent word w (both inside the normal range), on the integer
+// pipe: a tile's first chunk needs no FP64 instruction
+__device__ __forceinline__ double scaled(double x, int w) {
+  return __hiloint2double(x != 0.0 ? __double2hiint(x) + w - (1023 << 20) : 0, __double2loint(x));
+}
+
 // v[h][d] += the digit products of weight d over 16 positions, for a 16 x 16 unit (its first 8
 // columns when NH = 1): this lane's ldmatrix addresses aa, ba of the first digits, and the
 // digits' strides
@@ -801,8 +807,12 @@ __device__ __forceinline__ void warp_tile(const GemmOut* __restrict__ outs, cons
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             // the segment's scale goes with the second operand of the product (op(B))
+            // (+-1, almost always: a sign, not a multiplication on the slow FP64 pipe)
             double& x = swap ? a[h][j] : b[h][j];
-            if (sc[j] != 1.0) x *= sc[j];
+            if (fabs(sc[j]) == 1.0)
+              x = __hiloint2double(__double2hiint(x) ^ (__double2hiint(sc[j]) & (int)0x80000000), __double2loint(x));
+            else
+              x *= sc[j];
             ea[h][j] = exponent_of(a[h][j]);
             eb[h][j] = exponent_of(b[h][j]);
           }
@@ -854,6 +864,7 @@ __device__ __forceinline__ void warp_tile(const GemmOut* __restrict__ outs, cons
           return x;
         };
         wild = __any_sync(0xffffffffu, wild);
+        const bool first = b0 == 0 && p0 == 0;
         uint32_t A0[MMA_ND], A1[MMA_ND], A2[MMA_ND], A3[MMA_ND];
         cut_quad(a[0], ea[0], E[0], A0, A2);
         cut_quad(a[1], ea[1], E[1], A1, A3);
@@ -878,7 +889,9 @@ __device__ __forceinline__ void warp_tile(const GemmOut* __restrict__ outs, cons
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const int x = xe[i >> 1], f = (i & 1) ? f1 : f0;
-            if (!wild || (x | f) >= 0)
+            if (first && !wild)
+              acc[h][i] = scaled((double)join_digits(v, i), x + f);
+            else if (!wild || (x | f) >= 0)
               acc[h][i] = fma((double)join_digits(v, i), __hiloint2double(x + f, 0), acc[h][i]);
             else
               acc[h][i] = fp64_chunk(g + 8 * (i >> 1), 8 * h + 2 * t + (i & 1), acc[h][i]);
