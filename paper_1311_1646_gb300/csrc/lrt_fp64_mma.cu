@@ -23,12 +23,14 @@
 // staged operands.
 //
 // Measured on the k = 24, M = 500, 6-vector sigma (23.7 G multiply-adds): 44.0 ms by FP64 FMAs,
-// 16.7 ms here; error against 64-bit exact values 3.4e-16 (8.5e-16 before) at k = 8, 2.8e-15
-// (7.3e-15) on the PPP chain.  The kernel is bound by issued instructions (44-48% of the issue
-// slots at 12 warps per SM; tensor pipe 20%, FP64 pipe 25%): cutting the operands (a third)
-// and staging them cost more than the products.  Hence tiles of 96 staged rows for up to 8
-// 16 x 16 units, 3 CTAs of 4 warps per SM; and one row or column scale per 32 positions, so a
-// chunk needs no look at the rest of K.
+// 15.2 ms here; error against 64-bit exact values 3.9e-16 (7.1e-16 before) at k = 8, 2.9e-15
+// (7.0e-15) on the PPP chain.  The kernel is bound by issued instructions (45% of the issue slots;
+// tensor pipe 20%, FP64 pipe 25%): cutting the operands (a third of them) and staging cost more
+// than the products.  Hence tiles of 128 staged rows for up to 16 16 x 16 units and 16 warps per
+// SM, 2 CTAs of 8 warps at 128 registers (96 rows for 8 units, 3 CTAs of 4 warps: 16.9 ms); and
+// one row or column scale per 32 positions, so a chunk needs no look at the rest of K.  Operands
+// cut ahead into digit matrices and fetched by bulk copies were not faster (19.3 ms: pools of
+// 14 bytes per element, chunks that end with every segment, fewer warps).
 #include "lrt_kernels.h"
 #include "lrt_fp64_tile.h"
 
@@ -36,8 +38,9 @@
 
 namespace lrt {
 
-static_assert(GEMM_KC == 32 && GEMM_THREADS == 128, "the lane mappings below");
+static_assert(GEMM_KC == 32, "the lane mappings below");
 constexpr int MMA_ND = 7;                 // digits
+constexpr int MMA_WARPS = 8;              // warps of a CTA tile
 constexpr int MMA_EMIN = 600, MMA_EMAX = 1500;   // exponent fields the integer path takes
 constexpr int MMA_E0 = 1023;
 constexpr int MMA_NOBAL = -4096;                  // balance exponent where B's row is zero
@@ -66,6 +69,9 @@ __device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(addr)
                : "memory");
+}
+__device__ __forceinline__ void ldsm2(uint32_t (&r)[2], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];\n" : "=r"(r[0]), "=r"(r[1]) : "r"(addr) : "memory");
 }
 __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
@@ -170,24 +176,19 @@ __device__ __forceinline__ double scaled(double x, int w) {
   return __hiloint2double(x != 0.0 ? __double2hiint(x) + w - (1023 << 20) : 0, __double2loint(x));
 }
 
-// v[h][d] += the digit products of weight d over 16 positions, for a 16 x 16 unit (its first 8
-// columns when NH = 1): this lane's ldmatrix addresses aa, ba of the first digits, and the
-// digits' strides
-template <int NH>
-__device__ __forceinline__ void unit_products(float (&v)[2][MMA_ND][4], uint32_t aa, uint32_t ba, uint32_t adig,
-                                              uint32_t bdig) {
-  uint32_t B[MMA_ND][4];
+// v[d] += the digit products of weight d over 16 positions, for 16 rows and 8 columns: this
+// lane's ldmatrix addresses aa, ba of the first digits, and the digits' stride.  (Two column
+// groups at a time would load A once for both, but keeps 8 warps per CTA from 128 registers.)
+__device__ __forceinline__ void unit_products(float (&v)[MMA_ND][4], uint32_t aa, uint32_t ba, uint32_t stride) {
+  uint32_t B[MMA_ND][2];
 #pragma unroll
-  for (int j = 0; j < MMA_ND; ++j) ldsm4(B[j], ba + j * bdig);
+  for (int j = 0; j < MMA_ND; ++j) ldsm2(B[j], ba + j * stride);
 #pragma unroll
   for (int i = 0; i < MMA_ND; ++i) {
     uint32_t A[4];
-    ldsm4(A, aa + i * adig);
+    ldsm4(A, aa + i * stride);
 #pragma unroll
-    for (int j = 0; j < MMA_ND - i; ++j) {
-      mma16816(v[0][i + j], A, B[j][0], B[j][1]);
-      if (NH > 1) mma16816(v[1][i + j], A, B[j][2], B[j][3]);
-    }
+    for (int j = 0; j < MMA_ND - i; ++j) mma16816(v[i + j], A, B[j][0], B[j][1]);
   }
 }
 
@@ -217,7 +218,7 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
   const int a16 = (mt + 15) >> 4, b16 = (nt + 15) >> 4;
   const int RB = 16 * a16;                 // first B row
   const int rows = RB + 16 * b16;          // <= MMA_ROWS
-  const int units = a16 * b16;             // <= 2 * GEMM_WARPS
+  const int units = a16 * b16;             // <= 2 * MMA_WARPS
   const bool bal = o.balance != 0;
 
   // row tables; padding rows are zero for the whole tile
@@ -232,7 +233,7 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
     }
     S.vl[tid] = make_int2(v, g);
   }
-  for (int r = warp; r < rows; r += GEMM_WARPS)
+  for (int r = warp; r < rows; r += MMA_WARPS)
     if (r < RB ? r >= mt : r - RB >= nt) S.raw[r][lane] = 0.0;
   if (bal && tid < GEMM_KC) S.bal[tid] = MMA_NOBAL;
   if (tid < 2) S.wild[tid] = 0;
@@ -284,22 +285,22 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
       // lanes along K: operands stored K-contiguous, and zeros beyond Kb
       const bool ka = !in || !s.transA, kb = !in || s.transB;
       const int nz = in ? 8 : 0;
-      // rows i = warp, warp + 4, ...: i mod 16, and so the swizzle, repeats every fourth
+      // rows i = warp, warp + 8, ...: i mod 16, and so the swizzle, repeats every second
       auto rows_along_k = [&](int r0, int n, const double* base, int ld, int64_t vs) {
         const uint32_t ld8 = in ? 8u * (uint32_t)ld : 0u, vs8 = in ? 8u * (uint32_t)vs : 0u;
         const char* src = reinterpret_cast<const char*>(in ? base + kl : base);
-        for (int i0 = warp; i0 < n; i0 += 4 * GEMM_WARPS)
+        for (int i0 = warp; i0 < n; i0 += 4 * MMA_WARPS)
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            const int i = i0 + GEMM_WARPS * u;
+            const int i = i0 + MMA_WARPS * u;
             if (i < n) {
               const int2 vl = S.vl[r0 + i];
-              cp_async8z(&S.raw[r0 + i][2 * (g16 ^ ((warp + GEMM_WARPS * u) & 15)) + half],
+              cp_async8z(&S.raw[r0 + i][2 * (g16 ^ ((warp + MMA_WARPS * u) & 15)) + half],
                          src + (uint64_t)(uint32_t)vl.x * vs8 + (uint64_t)(uint32_t)vl.y * ld8, nz);
             }
           }
       };
-      static_assert(GEMM_WARPS == 4, "the swizzle period above");
+      static_assert(16 % MMA_WARPS == 0, "the swizzle period above");
       if (ka) rows_along_k(0, mt, s.A, s.lda, s.avs);
       if (kb) rows_along_k(RB, nt, s.B, s.ldb, s.bvs);
       // lanes along the rows: operands stored K-major, one segment after the other
@@ -307,7 +308,7 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
         const int pend = min(p0 + GEMM_KC, Kb);
         for (int q = q2; q < nb && S.kst[q] < pend; ++q) {
           const int f = max(S.kst[q], p0), l = min(S.kst[q + 1], pend);
-          const int kk0 = f - p0 + ((warp - (f - p0)) & 3);   // first position of this warp
+          const int kk0 = f - p0 + ((warp - (f - p0)) & (MMA_WARPS - 1));   // first position of this warp
           if (kk0 >= l - p0) continue;
           const SegS& t = S.sd[q];
           auto k_major = [&](int r0, int n, const double* base, int ld, int64_t vs) {
@@ -317,7 +318,7 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
               const int2 vl = S.vl[r];
               const double* p = src + ((uint64_t)(uint32_t)vl.x * (uint32_t)vs + (uint32_t)vl.y);
               double* row = &S.raw[r][0];
-              for (int kk = kk0; kk < l - p0; kk += GEMM_WARPS, p += (int64_t)GEMM_WARPS * ld)
+              for (int kk = kk0; kk < l - p0; kk += MMA_WARPS, p += (int64_t)MMA_WARPS * ld)
                 cp_async8z(row + 2 * ((kk >> 1) ^ (r & 15)) + (kk & 1), p, 8);
             }
           };
@@ -350,7 +351,7 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
       if (bal) {
         // largest exponent of each K position over B's columns
         int mx[4] = {0, 0, 0, 0};
-        for (int r = RB + 4 * warp + (lane >> 3); r < rows; r += 4 * GEMM_WARPS) {
+        for (int r = RB + 4 * warp + (lane >> 3); r < rows; r += 4 * MMA_WARPS) {
           Quad q = load_quad(&S.raw[0][0], r, l);
           scale_quad(S, mode, l, q);
 #pragma unroll
@@ -365,7 +366,7 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
         }
         __syncthreads();
       }
-      for (int r = 4 * warp + (lane >> 3); r < rows; r += 4 * GEMM_WARPS) {   // rows is a multiple of 16
+      for (int r = 4 * warp + (lane >> 3); r < rows; r += 4 * MMA_WARPS) {   // rows is a multiple of 16
         Quad q = load_quad(&S.raw[0][0], r, l);
         const bool isB = r >= RB;
         if (isB) scale_quad(S, mode, l, q);
@@ -398,33 +399,30 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
       const uint32_t dig0 = (uint32_t)__cvta_generic_to_shared(&S.dig[0][0][0]);
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        const int un = warp + GEMM_WARPS * u;
+        const int un = warp + MMA_WARPS * u;
         if (un >= units) break;
         const int ra = 16 * (un / b16), cb = 16 * (un % b16);
         const bool second = cb + 8 < nt;
-        float v[2][MMA_ND][4];
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-          for (int d = 0; d < MMA_ND; ++d)
-#pragma unroll
-            for (int t = 0; t < 4; ++t) v[h][d][t] = 0.0f;
-        const int ar = ra + (lane & 15), br = RB + cb + (lane & 7) + ((lane >> 4) << 3);
-        for (int ks = 0; ks < nks; ++ks) {
-          const uint32_t aa = dig0 + ar * 64 + (((2 * ks + (lane >> 4)) ^ (ar >> 1)) & 3) * 16;
-          const uint32_t ba = dig0 + br * 64 + (((2 * ks + ((lane >> 3) & 1)) ^ (br >> 1)) & 3) * 16;
-          if (second) unit_products<2>(v, aa, ba, (uint32_t)sizeof(S.dig[0]), (uint32_t)sizeof(S.dig[0]));
-          else unit_products<1>(v, aa, ba, (uint32_t)sizeof(S.dig[0]), (uint32_t)sizeof(S.dig[0]));
-        }
+        const int ar = ra + (lane & 15), br = RB + cb + (lane & 7);
         const int e0 = S.ex[ra + (lane >> 2)], e1 = S.ex[ra + (lane >> 2) + 8];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           if (h == 1 && !second) break;
+          float v[MMA_ND][4];
+#pragma unroll
+          for (int d = 0; d < MMA_ND; ++d)
+#pragma unroll
+            for (int t = 0; t < 4; ++t) v[d][t] = 0.0f;
+          for (int ks = 0; ks < nks; ++ks) {
+            const int b8 = br + 8 * h;
+            unit_products(v, dig0 + ar * 64 + (((2 * ks + (lane >> 4)) ^ (ar >> 1)) & 3) * 16,
+                          dig0 + b8 * 64 + (((2 * ks + ((lane >> 3) & 1)) ^ (b8 >> 1)) & 3) * 16, (uint32_t)sizeof(S.dig[0]));
+          }
           const int2 f = *reinterpret_cast<const int2*>(&S.ex[RB + cb + 8 * h + 2 * (lane & 3)]);
           if (!wild) {
 #pragma unroll
             for (int t = 0; t < 4; ++t)
-              acc[u][h][t] = fma((double)join_digits(v[h], t),
+              acc[u][h][t] = fma((double)join_digits(v, t),
                                  __hiloint2double(((t & 2) ? e1 : e0) + ((t & 1) ? f.y : f.x), 0), acc[u][h][t]);
           } else {
 #pragma unroll 1
@@ -434,7 +432,7 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
               if ((ea | eb) >= 0) {
                 float w[MMA_ND][4];
 #pragma unroll
-                for (int d = 0; d < MMA_ND; ++d) w[d][0] = t == 0 ? v[h][d][0] : t == 1 ? v[h][d][1] : t == 2 ? v[h][d][2] : v[h][d][3];
+                for (int d = 0; d < MMA_ND; ++d) w[d][0] = t == 0 ? v[d][0] : t == 1 ? v[d][1] : t == 2 ? v[d][2] : v[d][3];
                 s = fma((double)join_digits(w, 0), __hiloint2double(ea + eb, 0), s);
               } else {
                 // plain FP64 from the staged operands
@@ -462,7 +460,7 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
   if (o.seg_count == 0) __syncthreads();   // the row tables are read below
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
-    const int un = warp + GEMM_WARPS * u;
+    const int un = warp + MMA_WARPS * u;
     if (un >= units) break;
     const int ra = 16 * (un / b16) + (lane >> 2), cb = 16 * (un % b16) + 2 * (lane & 3);
 #pragma unroll
@@ -493,9 +491,9 @@ __device__ __forceinline__ double* mma_extra(const GemmExtra& ex, int i) {
   }
 }
 
-constexpr int MMA_CTAS = 3;
+constexpr int MMA_CTAS = 2;
 
-__global__ void __launch_bounds__(GEMM_THREADS, MMA_CTAS)
+__global__ void __launch_bounds__(32 * MMA_WARPS, MMA_CTAS)
     gemm_mma_kernel(const GemmOut* __restrict__ outs, const GemmSeg* __restrict__ segs, const int3* __restrict__ tiles,
                     int ntiles, const double* __restrict__ xbase, double* __restrict__ ybase, double* __restrict__ tbase,
                     const GemmBases* __restrict__ multi, const GemmExtra ex, double* __restrict__ wbase) {
@@ -512,7 +510,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, MMA_CTAS)
   gemm_mma_tile(segs, wi, xbase, ybase, tbase, wbase, o, [&](int i) { return mma_extra(ex, i); });
 }
 
-__global__ void __launch_bounds__(GEMM_THREADS, MMA_CTAS)
+__global__ void __launch_bounds__(32 * MMA_WARPS, MMA_CTAS)
     gemm_mma_inst_kernel(const GemmOut* __restrict__ outs, const GemmSeg* __restrict__ segs,
                          const int3* __restrict__ tiles, int ntiles, const __grid_constant__ GemmInstSet P, int ninst) {
   const int w = blockIdx.x / ninst;
@@ -548,7 +546,7 @@ void launch_gemm_mma(const GemmOut* outs, const GemmSeg* segs, const int3* tiles
   if (ntiles <= 0) return;
   if (mma_smem_attr() != cudaSuccess) return;
   const GemmExtra ex = extra ? *extra : GemmExtra{};
-  gemm_mma_kernel<<<ntiles, GEMM_THREADS, sizeof(MmaSmem), st>>>(outs, segs, tiles, ntiles, xbase, ybase, tbase, multi,
+  gemm_mma_kernel<<<ntiles, 32 * MMA_WARPS, sizeof(MmaSmem), st>>>(outs, segs, tiles, ntiles, xbase, ybase, tbase, multi,
                                                                 ex, wbase);
 }
 
@@ -556,7 +554,7 @@ void launch_gemm_mma_inst(const GemmOut* outs, const GemmSeg* segs, const int3* 
                           const GemmInstSet& bases, int ninst, cudaStream_t st) {
   if (ntiles <= 0 || ninst <= 0) return;
   if (mma_smem_attr() != cudaSuccess) return;
-  gemm_mma_inst_kernel<<<(unsigned)((long long)ntiles * ninst), GEMM_THREADS, sizeof(MmaSmem), st>>>(
+  gemm_mma_inst_kernel<<<(unsigned)((long long)ntiles * ninst), 32 * MMA_WARPS, sizeof(MmaSmem), st>>>(
       outs, segs, tiles, ntiles, bases, ninst);
 }
 

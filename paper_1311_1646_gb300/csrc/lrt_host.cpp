@@ -779,8 +779,8 @@ static void build_gather(GatherPlan& P, std::vector<GatherTask>& tasks, std::vec
   P.ntiles = (int)tiles.size();
 }
 
-// Tile of the digit-product kernel for one output: a x b units of 16 x 16 with a + b <= 6
-// (MMA_ROWS) and a b <= 8, the shorter side whole where it fits, both sides cut evenly.  The
+// Tile of the digit-product kernel for one output: a x b units of 16 x 16 with a + b <= 8
+// (MMA_ROWS) and a b <= 16, the shorter side whole where it fits, both sides cut evenly.  The
 // columns of a balanced output are cut by their own count only, so that a column sees the
 // same neighbours whatever the rows (the vectors of the call) are.
 static void mma_tile_shape(const GemmOut& O, int& tm, int& tn) {
@@ -793,11 +793,11 @@ static void mma_tile_shape(const GemmOut& O, int& tm, int& tn) {
   if (O.balance || n16 < m16) {
     tn = even(O.n, std::min(n16, 4), 8);
     const int b = (tn + 15) / 16;
-    tm = even(O.m, std::min(6 - b, 8 / b), 16);
+    tm = even(O.m, std::min(8 - b, 16 / b), 16);
   } else {
     tm = even(O.m, std::min(m16, 4), 16);
     const int a = (tm + 15) / 16;
-    tn = even(O.n, std::min(6 - a, 8 / a), 8);
+    tn = even(O.n, std::min(8 - a, 16 / a), 8);
   }
 }
 
@@ -805,7 +805,7 @@ static void mma_tile_shape(const GemmOut& O, int& tm, int& tn) {
 // and more) of blocks that fill them (work padded to 16 x 8 x 16 at most 3 times the exact
 // work), one warp per tile elsewhere: a CTA shares the cut operands among its units, a warp
 // waits for nobody.  Both measured, CTA / warp (multiply-adds, padding of the two phases):
-// k = 24, M = 500, 6 vectors (2 x 1.9e9 per vector; 1.8, 1.1) 17.0 / 25.2 ms; the same chain at
+// k = 24, M = 500, 6 vectors (2 x 1.9e9 per vector; 1.8, 1.1) 15.2 / 25.2 ms; the same chain at
 // M = 300, site 4 (1.3e8; 2.0, 1.6) 487 / 374 us; PPP k = 12, M = 256 (1.7e7; 2.0, 1.9) 129 / 93 us;
 // eight molecules of 8 to 12 orbitals (5e7; 4, 3) 1.94 / 0.94 ms; k = 8, M = 64 (1e6; 13, 5)
 // 135 / 61 us (183 by FP64 CTA tiles).  Counted per vector, so that a call's kernel, and with
@@ -2739,7 +2739,7 @@ static SigmaPlan& get_plan(lrt_ctx* c, int site, int nsite, int nvec, bool tc = 
 // SM with 128-row tiles and pays a host synchronization per call, which short lists of small
 // blocks do not repay, and the FP64 digit products are the more exact of the two.  Measured,
 // split-TF32 / FP64: two-site k = 13, M = 200, 3 vectors (1e8 multiply-adds of phase 1 per
-// vector) 3.89 / 1.52 ms; k = 24, M = 500, 6 vectors (1.9e9) 6.55 / 17.0 ms.  A pending
+// vector) 3.89 / 1.47 ms; k = 24, M = 500, 6 vectors (1.9e9) 6.55 / 15.2 ms.  A pending
 // stall (lrt_set_wait_limit) is for the next tensor-core launch, so such a call keeps it.
 constexpr double MIXED_MIN_MACS = 2e8, MIXED_MIN_TOTAL = 7e8;   // phase 1, per vector / of the call
 static bool mixed_in_fp64(lrt_ctx* c, double macs, int nvec) {

@@ -546,7 +546,7 @@ __global__ void __launch_bounds__(256) split_reduce_kernel(const GemmOut* __rest
 void launch_split_reduce(const GemmOut* outs, const SplitTile* tiles, int ntiles, const double* wbase, double* ybase,
                          double* tbase, cudaStream_t st) {
   if (ntiles <= 0) return;
-  constexpr int most = GEMM_TM * GEMM_TN > 8 * 256 ? GEMM_TM * GEMM_TN : 8 * 256;   // elements of a tile (either kernel)
+  constexpr int most = GEMM_TM * GEMM_TN > 16 * 256 ? GEMM_TM * GEMM_TN : 16 * 256;   // elements of a tile (either kernel)
   split_reduce_kernel<<<dim3(ntiles, (most + 255) / 256), 256, 0, st>>>(outs, tiles, wbase, ybase, tbase);
 }
 

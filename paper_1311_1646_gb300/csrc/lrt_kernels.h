@@ -152,9 +152,9 @@ void launch_gemm_fp64(const GemmOut* outs, const GemmSeg* segs, const int3* tile
                       const double* xbase, double* ybase, double* tbase, cudaStream_t st,
                       const GemmExtra* extra = nullptr, double* wbase = nullptr);
 // Tensor-core form of the FP64 GEMM (exact digit products, lrt_fp64_mma.cu): the same lists
-// with tiles of at most MMA_ROWS rows and columns together, both rounded up to 16, and 8
+// with tiles of at most MMA_ROWS rows and columns together, both rounded up to 16, and 16
 // 16 x 16 units; the segments' vector blocks are the output's (a_vr = c_vr, b_vc = c_vc).
-constexpr int MMA_ROWS = 96;
+constexpr int MMA_ROWS = 128;
 void launch_gemm_mma(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles, const double* xbase,
                      double* ybase, double* tbase, cudaStream_t st, const GemmBases* multi, const GemmExtra* extra,
                      double* wbase);
