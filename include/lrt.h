@@ -365,7 +365,9 @@ int sigma_stats(lrt_t ctx, lrt_sigma_stats* out);
  *    make that first call during set-up, where the reservation is acceptable; later
  *    calls take no device memory.
  *  - Reuses the plan that a regular sigma() call with the same (site, nsite, nvec)
- *    prepared after the last renormalize(); without one it returns LRT_ESTATE.
+ *    prepared after the last renormalize(); without one it returns LRT_ESTATE, except
+ *    that a single-vector call after heff_diag() of the position prepares its plan itself
+ *    (that call allocates; while its stream is captured it returns LRT_ESTATE).
  *    A plan whose intermediates exceed the static array is rejected with LRT_EINVAL
  *    and a message giving both sizes.
  *  - The first call on each device resolves the array's device address

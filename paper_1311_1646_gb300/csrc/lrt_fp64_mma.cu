@@ -576,8 +576,8 @@ void launch_gemm_mma_inst(const GemmOut* outs, const GemmSeg* segs, const int3* 
 // tile's last part adds the parts in order (a counter per tile, reset by that warp), which
 // spares the reduction launch.
 //
-// Measured (one-site sigma): k = 8, M = 64, 1 vector 183 -> 61 us; k = 17, M = 30, 6 vectors
-// 468 -> 137 us; eight molecules in one call 1.67 -> 0.94 ms.  Bound by latency: descriptor and
+// Measured (one-site sigma): k = 8, M = 64, 1 vector 183 -> 51 us; k = 17, M = 30, 6 vectors
+// 468 -> 106 us; eight molecules in one call 1.67 -> 0.89 ms.  Bound by latency: descriptor and
 // operand reads of short items, 16 warps per SM (128 registers; 3 CTAs of 168 registers are
 // 5% slower on the longer lists).
 // ---------------------------------------------------------------------------

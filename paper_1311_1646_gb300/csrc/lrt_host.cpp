@@ -806,9 +806,10 @@ static void mma_tile_shape(const GemmOut& O, int& tm, int& tn) {
 // work), one warp per tile elsewhere: a CTA shares the cut operands among its units, a warp
 // waits for nobody.  Both measured, CTA / warp (multiply-adds, padding of the two phases):
 // k = 24, M = 500, 6 vectors (2 x 1.9e9 per vector; 1.8, 1.1) 15.2 / 25.2 ms; the same chain at
-// M = 300, site 4 (1.3e8; 2.0, 1.6) 487 / 374 us; PPP k = 12, M = 256 (1.7e7; 2.0, 1.9) 129 / 93 us;
-// eight molecules of 8 to 12 orbitals (5e7; 4, 3) 1.94 / 0.94 ms; k = 8, M = 64 (1e6; 13, 5)
-// 135 / 61 us (183 by FP64 CTA tiles).  Counted per vector, so that a call's kernel, and with
+// M = 300, site 4 (1.3e8; 2.0, 1.6) 628 / 354 us; two-site k = 13, M = 200, 3 vectors (1e8) 1.83 /
+// 1.46 ms; eight molecules of 8 to 12 orbitals (5e7; 4, 3) 1.32 / 0.88 ms; with earlier forms of
+// both, PPP k = 12, M = 256 (1.7e7; 2.0, 1.9) 129 / 93 us and k = 8, M = 64 (1e6; 13, 5) 135 / 61 us
+// (183 by FP64 CTA tiles).  Counted per vector, so that a call's kernel, and with
 // it every bit of a vector's result, does not depend on how many vectors the call has.  FP64
 // CTA tiles are left for strides beyond 32 bits.
 static GemmKind gemm_kind(const std::vector<GemmOut>& outs, const std::vector<GemmSeg>& segs,
@@ -1144,6 +1145,7 @@ struct PlanScratch {
 struct SigmaPlan {
   uint64_t serial = 0;      // unique per plan (batched launches detect rebuilt plans by it)
   bool has_tc = false;      // the tensor-core twin was planned
+  bool diag_used = false;   // heff_diag was answered from this plan
   GemmPlan p1, p2;
   // operator sets of a plan built with relative addresses (X, Xrev, Y, Yrev at extra
   // bases 0..3); a kept plan serves new sets of the same layout by changing these
@@ -2730,9 +2732,25 @@ static SigmaPlan& get_plan(lrt_ctx* c, int site, int nsite, int nvec, bool tc = 
   auto it = c->plans.find(key);
   if (it != c->plans.end() && (!tc || it->second->has_tc)) return *it->second;
   auto p = plan_sigma(c, site, nsite, nvec, tc);
+  if (it != c->plans.end()) p->diag_used = it->second->diag_used;
   SigmaPlan& ref = *p;
   c->plans[key] = std::move(p);
   return ref;
+}
+
+// the single-vector plan of sigma_noalloc where none is kept: after heff_diag of the position,
+// which answers from any plan, it is made here (never while the stream is captured)
+static SigmaPlan* plan_after_diag(lrt_ctx* c, int site, int nsite) {
+  for (auto it = c->plans.lower_bound(std::make_tuple(site, nsite, 0));
+       it != c->plans.end() && std::get<0>(it->first) == site && std::get<1>(it->first) == nsite; ++it) {
+    if (!it->second->diag_used) continue;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return nullptr;
+    CK(cudaSetDevice(c->dev));
+    PoolScope ps(&c->pool);
+    return &get_plan(c, site, nsite, 1);
+  }
+  return nullptr;
 }
 
 // LRT_MIXED calls that run on the FP64 kernels: the split-TF32 kernel fills one persistent CTA per
@@ -5785,6 +5803,7 @@ int sigma_launch_existing_plan(lrt_ctx* ctx, int site, int nsite, int nvec, cons
     if (nsite < 1 || nsite > 2 || site < 0 || nvec <= 0 || !x_dev || !y_dev || !workspace)
       throw Error(LRT_EINVAL, "sigma_noalloc: bad arguments");
     SigmaPlan* p = find_plan(ctx, site, nsite, nvec);
+    if (!p && nvec == 1) p = plan_after_diag(ctx, site, nsite);
     if (!p)
       throw Error(LRT_ESTATE, "sigma_noalloc: no prepared plan for this (site, nsite, nvec); call sigma() once "
                               "with the same arguments after the last renormalize()");
@@ -6010,6 +6029,7 @@ int heff_diag(lrt_t ctx, int site, int nsite, double* d_dev) {
     if (nsite < 1 || nsite > 2 || site < 0 || site + nsite > ctx->k || !d_dev) throw Error(LRT_EINVAL, "heff_diag: bad arguments");
     if (!ctx->L[site]) throw Error(LRT_ESTATE, "heff_diag: left block missing");
     SigmaPlan& p = get_diag_plan(ctx, site, nsite);
+    p.diag_used = true;
     launch_diag(p.douts.p, p.dterms.p, p.ndiag, d_dev, ctx->st);
     CK(cudaGetLastError());
   });

@@ -129,3 +129,27 @@ def test_small_blocks_match_the_oracle(pkg, k, na, nb, M, i, nsite, nvec):
     # the parts' counters are back at zero: the same call again, the same bits
     assert np.array_equal(_sigma(pkg, ctx, i, nsite, x, nvec), y)
     ctx.close()
+
+
+@pytest.mark.parametrize("first_nvec", [0, 3])
+def test_noalloc_single_vector_after_heff_diag(pkg, first_nvec):
+    """heff_diag answers from a plan of the diagonal alone or of another vector count; a
+    single-vector sigma_noalloc after it gives sigma()'s bits, one of 2 vectors is refused."""
+    cfg = synth.config(1)
+    H = cfg["ham"]
+    m = synth.mixed_mps(H.k, H.n_alpha, H.n_beta, cfg["M"], 77, center=3)
+    ctx = _context(pkg, H.k, H.n_alpha, H.n_beta, cfg["M"], 3, 1, H.h, H.eri, m)
+    n, _ = ctx.wfn_layout(3, 1)
+    if first_nvec:
+        _sigma(pkg, ctx, 3, 1, synth.random_vector(first_nvec * n, 4), first_nvec)
+    d = torch.empty(n, dtype=torch.float64, device="cuda:0")
+    ctx.heff_diag(3, 1, d)
+    x = synth.random_vector(2 * n, 5)
+    xd = torch.tensor(x, dtype=torch.float64, device="cuda:0")
+    yd = torch.full_like(xd, float("nan"))
+    with pytest.raises(pkg.LrtError, match="-6"):
+        ctx.sigma_noalloc(3, 1, xd, yd, nvec=2)
+    ctx.sigma_noalloc(3, 1, xd[:n], yd[:n])
+    torch.cuda.synchronize()
+    assert np.array_equal(yd[:n].cpu().numpy(), _sigma(pkg, ctx, 3, 1, x[:n], 1))
+    ctx.close()
