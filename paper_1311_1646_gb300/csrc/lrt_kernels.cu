@@ -888,14 +888,20 @@ void launch_reduced_acc(const double* D1, const double* D2, const double* D3, in
 // every thread applies two of them to 2 x 2 blocks of A, one to pairs of Z.  Sweeps stop when the
 // off-diagonal norm is below 1e-15 of the Frobenius norm, or after a fixed number.  One
 // rotation at a time, the chain of n (n - 1) / 2 rotations a sweep took 1.48 ms at n <= 24 (60%
-// of a ground-state run), 0.24 ms by disjoint rotations; bound by the FP64 pipe of one SM, hence
-// only the blocks on and above the diagonal and no work for rotations that are the identity.
+// of a ground-state run).  What is left is a serial chain of steps: the rotation (square root,
+// quotient, reciprocal square root), two barriers and the FP64 pipe of one SM.  Hence only the
+// blocks on and above the diagonal, no work for rotations that are the identity, a thread's
+// blocks found once and a step's pairs once by the thread that rotates them (n = 12 / 24: 233 /
+// 631 -> 178 / 472 us, the residual of a pair and the orthogonality 2 to 3 times smaller).
 constexpr int JACOBI_THREADS = 256;
+constexpr int JACOBI_NP = JACOBI_MAXN / 2;
+constexpr int JACOBI_ITEMS = (JACOBI_NP * (JACOBI_NP + 1) / 2 + JACOBI_MAXN * JACOBI_NP + JACOBI_THREADS - 1) / JACOBI_THREADS;
 __global__ void __launch_bounds__(JACOBI_THREADS) jacobi_kernel(double* __restrict__ Ag, int n, double* __restrict__ w,
                                                                 double* __restrict__ Zg) {
   __shared__ double A[JACOBI_MAXN][JACOBI_MAXN + 1];
   __shared__ double Z[JACOBI_MAXN][JACOBI_MAXN + 1];
-  __shared__ double cs[JACOBI_MAXN / 2], sn[JACOBI_MAXN / 2];
+  __shared__ double2 rot[JACOBI_NP];              // cosine and sine of a step's pairs
+  __shared__ int2 pair[JACOBI_NP];                // their indices, the smaller first
   __shared__ double red[2][JACOBI_THREADS / 32];
   __shared__ int order[JACOBI_MAXN];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -905,14 +911,26 @@ __global__ void __launch_bounds__(JACOBI_THREADS) jacobi_kernel(double* __restri
     A[i][j] = 0.5 * (Ag[i * n + j] + Ag[j * n + i]);
     Z[i][j] = (i == j) ? 1.0 : 0.0;
   }
+  // this thread's items, u | v << 8: rows of pair u times columns of pair v >= u of A, then
+  // (1 << 16 set) row u of Z times pair v; -1 none
+  int item[JACOBI_ITEMS];
+  const int na = np * (np + 1) / 2;
+#pragma unroll
+  for (int h = 0; h < JACOBI_ITEMS; ++h) {
+    const int e = tid + h * JACOBI_THREADS;
+    item[h] = -1;
+    if (e < na) {                                 // row u of the triangle starts at u np - u (u - 1) / 2
+      int u = 0, f = e;
+      while (f >= np - u) f -= np - u++;
+      item[h] = u | (u + f) << 8;
+    } else if (e < na + n * np) {
+      item[h] = (e - na) / np | (e - na) % np << 8 | 1 << 16;
+    }
+  }
+  // pair k of step r: player ne - 1 (k = 0) or (r + k) mod (ne - 1), against (r - k) mod (ne - 1)
+  const int m = ne - 1;
+  int pa = tid == 0 ? m : tid, pb = tid == 0 ? 0 : m - tid;
   __syncthreads();
-  // players of pair k in round r: ne - 1 stays, the others rotate
-  auto player = [&](int k, int r, int& p, int& q) {
-    const int m = ne - 1;
-    int a = k == 0 ? m : (r + k) % m, b = (r - k + m) % m;
-    p = min(a, b);
-    q = max(a, b);
-  };
   for (int sweep = 0; sweep < 60; ++sweep) {
     double off = 0.0, fro = 0.0;
     for (int e = tid; e < n * n; e += JACOBI_THREADS) {
@@ -938,47 +956,46 @@ __global__ void __launch_bounds__(JACOBI_THREADS) jacobi_kernel(double* __restri
     }
     // (a matrix with NaN or infinities ends after its 60 sweeps)
     if (off <= 1e-30 * fro) break;
-    for (int r = 0; r < ne - 1; ++r) {
+    for (int r = 0; r < m; ++r) {                 // m steps bring every pair back to its start
+      bool turns = false;
       if (tid < np) {
-        int p, q;
-        player(tid, r, p, q);
+        const int p = min(pa, pb), q = max(pa, pb);
         double c = 1.0, s = 0.0;
         if (q < n) {
           const double apq = A[p][q];
           // elements that together stay below a tenth of the stopping norm are left alone
           if (apq * apq * (double)(n * n) > 1e-31 * fro) {
-            const double tau = (A[q][q] - A[p][p]) / (2.0 * apq);
-            const double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-            c = 1.0 / sqrt(1.0 + t * t);
-            s = t * c;
+            // t = sgn(d / b) |b| / (|d| + sqrt(d^2 + b^2)), both scaled by a power of two to
+            // keep the squares in range
+            double d = A[q][q] - A[p][p], b = 2.0 * apq;
+            const bool neg = d != 0.0 && (d < 0.0) != (b < 0.0);
+            const int ex = min(max(__double2hiint(fmax(fabs(d), fabs(b))) >> 20, 1), 2045);
+            const double f = __hiloint2double((2046 - ex) << 20, 0);
+            d = fabs(d) * f;
+            b = fabs(b) * f;
+            const double t = b / (d + sqrt(d * d + b * b));
+            c = rsqrt(1.0 + t * t);
+            s = neg ? -t * c : t * c;
           }
         }
-        cs[tid] = c;
-        sn[tid] = s;
+        rot[tid] = make_double2(c, s);
+        pair[tid] = make_int2(p, q);
+        turns = s != 0.0;
+        if (tid > 0) pa = pa + 1 == m ? 0 : pa + 1;
+        pb = pb + 1 == m ? 0 : pb + 1;
       }
-      __syncthreads();
+      if (!__syncthreads_or(turns)) continue;
       // A <- J^T A J by 2 x 2 blocks (rows of pair u, columns of pair v >= u, mirrored), Z <- Z J
-      const int na = np * (np + 1) / 2;
-      for (int e = tid; e < na + n * np; e += JACOBI_THREADS) {
-        const bool isA = e < na;
-        int u, v;
-        if (isA) {                                 // row u of the triangle starts at u np - u (u - 1) / 2
-          u = 0;
-          int f = e;
-          while (f >= np - u) f -= np - u++;
-          v = u + f;
-        } else {
-          u = (e - na) / np;
-          v = (e - na) % np;
-        }
-        const double c = cs[v], s = sn[v];
-        if (s == 0.0 && !(isA && sn[u] != 0.0)) continue;
-        int p, q;
-        player(v, r, p, q);
-        if (isA) {
-          int i, j;
-          player(u, r, i, j);
-          const double cu = cs[u], su = sn[u];
+#pragma unroll
+      for (int h = 0; h < JACOBI_ITEMS; ++h) {
+        if (item[h] < 0) break;
+        const int u = item[h] & 255, v = item[h] >> 8 & 255;
+        const double c = rot[v].x, s = rot[v].y;
+        const int p = pair[v].x, q = pair[v].y;
+        if (item[h] < 1 << 16) {
+          const double cu = rot[u].x, su = rot[u].y;
+          if (s == 0.0 && su == 0.0) continue;
+          const int i = pair[u].x, j = pair[u].y;
           // rows or columns of the bye player (index n) do not exist
           const bool hi = j < n, hq = q < n;
           const double a00 = A[i][p], a01 = hq ? A[i][q] : 0.0, a10 = hi ? A[j][p] : 0.0, a11 = hi && hq ? A[j][q] : 0.0;
@@ -990,7 +1007,7 @@ __global__ void __launch_bounds__(JACOBI_THREADS) jacobi_kernel(double* __restri
           if (hq) A[i][q] = A[q][i] = d01;
           if (hi) A[j][p] = A[p][j] = d10;
           if (hi && hq) A[j][q] = A[q][j] = d11;
-        } else {
+        } else if (s != 0.0) {
           const double zp = Z[u][p], zq = Z[u][q];
           Z[u][p] = c * zp - s * zq;
           Z[u][q] = s * zp + c * zq;
