@@ -2822,17 +2822,13 @@ static double dev_dot(const double* a, const double* b, int64_t n, double* dtmp,
   return r;
 }
 
-static void upload_coef(double* dcoef, const std::vector<double>& c, cudaStream_t st) {
-  if (!c.empty()) CK(cudaMemcpyAsync(dcoef, c.data(), c.size() * sizeof(double), cudaMemcpyHostToDevice, st));
-}
-
 // Lowest eigenpair of H_eff at a two-site position; psi (device) is the start vector
 // and receives the eigenvector.  Returns the eigenvalue.
 static double davidson_site(lrt_ctx* c, int i, int nsite, double* psi, const lrt_gs_params& P, int* iters_out) {
   SigmaPlan& plan = get_plan(c, i, nsite, 1);
   const int64_t n = plan.nelem;
   const int maxs = std::max(2, std::min(P.dav_max_space, JACOBI_MAXN));
-  DevBuf V, AV, diag, r, t, u, au, small, coef, Hd, Wd, Zd;
+  DevBuf V, AV, diag, r, t, u, au, small, Hd, Wd, Zd;
   V.ensure((size_t)maxs * n);
   AV.ensure((size_t)maxs * n);
   diag.ensure(n);
@@ -2841,14 +2837,13 @@ static double davidson_site(lrt_ctx* c, int i, int nsite, double* psi, const lrt
   u.ensure(n);
   au.ensure(n);
   small.ensure(JACOBI_MAXN + 8);
-  coef.ensure(JACOBI_MAXN + 8);
-  Hd.ensure(JACOBI_MAXN * JACOBI_MAXN);
-  Wd.ensure(JACOBI_MAXN);
+  Hd.ensure(JACOBI_MAXN * JACOBI_MAXN);   // the subspace matrix, rows maxs apart
+  Wd.ensure(JACOBI_MAXN + 2);             // |t|^2, |r|^2, then its eigenvalues
+  double *t2 = Wd.p, *r2 = Wd.p + 1, *ev = Wd.p + 2;
   Zd.ensure(JACOBI_MAXN * JACOBI_MAXN);
   cudaStream_t st = c->st;
   launch_diag(plan.douts.p, plan.dterms.p, plan.ndiag, diag.p, st);
   CK(cudaMemcpyAsync(t.p, psi, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
-  std::vector<double> Hs((size_t)maxs * maxs, 0.0), hcol(maxs), w(maxs), Z((size_t)maxs * maxs);
   int m = 0;
   double theta = 0.0;
   int it = 0;
@@ -2856,57 +2851,32 @@ static double davidson_site(lrt_ctx* c, int i, int nsite, double* psi, const lrt
     // orthogonalize the new direction against the subspace (twice) and normalize
     for (int pass = 0; pass < 2 && m > 0; ++pass) {
       launch_dots(V.p, n, m, t.p, n, small.p, st);
-      std::vector<double> cc(m);
-      CK(cudaMemcpyAsync(cc.data(), small.p, m * sizeof(double), cudaMemcpyDeviceToHost, st));
-      CK(cudaStreamSynchronize(st));
-      for (double& x : cc) x = -x;
-      upload_coef(coef.p, cc, st);
-      launch_lincomb(V.p, n, m, coef.p, n, t.p, 1.0, st);
+      launch_lincomb(V.p, n, m, small.p, n, t.p, 1.0, st, -1.0);
     }
-    const double nt = std::sqrt(std::max(0.0, dev_dot(t.p, t.p, n, small.p, st)));
-    if (nt < 1e-14) break;
-    launch_lincomb(nullptr, n, 0, coef.p, n, t.p, 1.0 / nt, st);
-    CK(cudaMemcpyAsync(V.p + (size_t)m * n, t.p, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
+    launch_dots(t.p, n, 1, t.p, n, t2, st);
+    launch_dav_unit(t.p, t2, n, V.p + (size_t)m * n, st);
     plan.p1.run(st, V.p + (size_t)m * n, AV.p + (size_t)m * n, plan.tbuf, &plan.ex);
     plan.p2.run(st, V.p + (size_t)m * n, AV.p + (size_t)m * n, plan.tbuf, &plan.ex);
     launch_dots(V.p, n, m + 1, AV.p + (size_t)m * n, n, small.p, st);
-    CK(cudaMemcpyAsync(hcol.data(), small.p, (m + 1) * sizeof(double), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    for (int j = 0; j <= m; ++j) {
-      Hs[(size_t)j * maxs + m] = hcol[j];
-      Hs[(size_t)m * maxs + j] = hcol[j];
-    }
     ++m;
-    // subspace eigenproblem on the GPU
-    std::vector<double> Hc((size_t)m * m);
-    for (int a = 0; a < m; ++a)
-      for (int b = 0; b < m; ++b) Hc[(size_t)a * m + b] = Hs[(size_t)a * maxs + b];
-    CK(cudaMemcpyAsync(Hd.p, Hc.data(), Hc.size() * sizeof(double), cudaMemcpyHostToDevice, st));
-    launch_jacobi_eigh(Hd.p, m, Wd.p, Zd.p, st);
-    CK(cudaMemcpyAsync(w.data(), Wd.p, m * sizeof(double), cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(Z.data(), Zd.p, (size_t)m * m * sizeof(double), cudaMemcpyDeviceToHost, st));
+    // subspace eigenproblem, its lowest Ritz pair, residual and next direction on the GPU
+    launch_jacobi_eigh(Hd.p, m, ev, Zd.p, st, small.p, maxs);
+    launch_dav_ritz(V.p, AV.p, n, m, Zd.p, ev, t2, diag.p, n, u.p, au.p, r.p, t.p, st);
+    launch_dots(r.p, n, 1, r.p, n, r2, st);
+    double s[3];
+    CK(cudaMemcpyAsync(s, Wd.p, sizeof(s), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    theta = w[0];
-    std::vector<double> al(m);
-    for (int a = 0; a < m; ++a) al[a] = Z[(size_t)a * m + 0];
-    upload_coef(coef.p, al, st);
-    launch_lincomb(V.p, n, m, coef.p, n, u.p, 0.0, st);
-    launch_lincomb(AV.p, n, m, coef.p, n, au.p, 0.0, st);
-    CK(cudaMemcpyAsync(r.p, au.p, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    std::vector<double> mt = {-theta};
-    upload_coef(coef.p, mt, st);
-    launch_lincomb(u.p, n, 1, coef.p, n, r.p, 1.0, st);
-    const double rn = std::sqrt(std::max(0.0, dev_dot(r.p, r.p, n, small.p, st)));
+    if (std::sqrt(std::max(0.0, s[0])) < DAV_MIN_NORM) break;   // the last Ritz vector stays
+    theta = s[2];
+    const double rn = std::sqrt(std::max(0.0, s[1]));
     if (rn < P.dav_tol) {
       ++it;
       break;
     }
-    launch_precond(r.p, diag.p, theta, n, t.p, st);
     if (m == maxs) {   // restart with the Ritz vector
       CK(cudaMemcpyAsync(V.p, u.p, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
       CK(cudaMemcpyAsync(AV.p, au.p, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
-      std::fill(Hs.begin(), Hs.end(), 0.0);
-      Hs[0] = theta;
+      CK(cudaMemcpyAsync(Hd.p, ev, sizeof(double), cudaMemcpyDeviceToDevice, st));
       m = 1;
     }
   }

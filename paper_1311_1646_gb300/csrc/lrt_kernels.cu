@@ -679,35 +679,76 @@ void launch_pair_dots(const double* const* A, const double* const* B, int na, in
 }
 
 __global__ void __launch_bounds__(256) lincomb_kernel(const double* __restrict__ V, int64_t ld, int m,
-                                                      const double* __restrict__ coef, int64_t n,
+                                                      const double* __restrict__ coef, double sign, int64_t n,
                                                       double* __restrict__ out, double beta) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
     double acc = beta == 0.0 ? 0.0 : beta * out[e];
-    for (int j = 0; j < m; ++j) acc = fma(coef[j], V[j * ld + e], acc);
+    for (int j = 0; j < m; ++j) acc = fma(sign * coef[j], V[j * ld + e], acc);
     out[e] = acc;
   }
 }
 
 void launch_lincomb(const double* V, int64_t ld, int m, const double* coef, int64_t n, double* out, double beta,
-                    cudaStream_t st) {
+                    cudaStream_t st, double sign) {
   if (n <= 0) return;
   const int grid = (int)std::min<int64_t>((n + 255) / 256, 152 * 8);
-  lincomb_kernel<<<grid, 256, 0, st>>>(V, ld, m, coef, n, out, beta);
+  lincomb_kernel<<<grid, 256, 0, st>>>(V, ld, m, coef, sign, n, out, beta);
 }
 
-__global__ void __launch_bounds__(256) precond_kernel(const double* __restrict__ r, const double* __restrict__ d,
-                                                      double theta, int64_t n, double* __restrict__ t) {
+// Davidson: a direction's norm, Ritz pair and next direction stay on the device, so that an
+// iteration waits for the host once (to test convergence) and not six times: 373 -> 278 ms for a
+// ground-state sweep pair at k = 8, M = 64, whose vectors of a few thousand elements take
+// microseconds and a round trip 20.  A direction of norm below DAV_MIN_NORM ends the iteration:
+// the last Ritz vector is kept.
+__device__ __forceinline__ double dav_norm(double t2) { return sqrt(t2 > 0.0 ? t2 : 0.0); }
+
+// v = t / |t|
+__global__ void __launch_bounds__(256) dav_unit_kernel(const double* __restrict__ t, const double* __restrict__ t2,
+                                                       int64_t n, double* __restrict__ v) {
+  const double nt = dav_norm(*t2), f = nt < DAV_MIN_NORM ? 0.0 : 1.0 / nt;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
+    v[e] = f == 0.0 ? 0.0 : f * t[e];
+}
+
+void launch_dav_unit(const double* t, const double* t2, int64_t n, double* v, cudaStream_t st) {
+  if (n <= 0) return;
+  const int grid = (int)std::min<int64_t>((n + 255) / 256, 152 * 8);
+  dav_unit_kernel<<<grid, 256, 0, st>>>(t, t2, n, v);
+}
+
+// u = V z, au = AV z, r = au - theta u, t = -r / (d - theta) for the lowest pair (theta, z) of the
+// m-dimensional subspace
+__global__ void __launch_bounds__(256) dav_ritz_kernel(const double* __restrict__ V, const double* __restrict__ AV,
+                                                       int64_t ld, int m, const double* __restrict__ Z,
+                                                       const double* __restrict__ w, const double* __restrict__ t2,
+                                                       const double* __restrict__ d, int64_t n, double* __restrict__ u,
+                                                       double* __restrict__ au, double* __restrict__ r,
+                                                       double* __restrict__ t) {
+  if (dav_norm(*t2) < DAV_MIN_NORM) return;
+  const double theta = *w;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+    double x = 0.0, ax = 0.0;
+    for (int j = 0; j < m; ++j) {
+      const double z = Z[(int64_t)j * m];
+      x = fma(z, V[j * ld + e], x);
+      ax = fma(z, AV[j * ld + e], ax);
+    }
+    const double res = fma(-theta, x, ax);
     double den = d[e] - theta;
     if (fabs(den) < 1e-4) den = den < 0.0 ? -1e-4 : 1e-4;
-    t[e] = -r[e] / den;
+    u[e] = x;
+    au[e] = ax;
+    r[e] = res;
+    t[e] = -res / den;
   }
 }
 
-void launch_precond(const double* r, const double* d, double theta, int64_t n, double* t, cudaStream_t st) {
+void launch_dav_ritz(const double* V, const double* AV, int64_t ld, int m, const double* Z, const double* w,
+                     const double* t2, const double* d, int64_t n, double* u, double* au, double* r, double* t,
+                     cudaStream_t st) {
   if (n <= 0) return;
   const int grid = (int)std::min<int64_t>((n + 255) / 256, 152 * 8);
-  precond_kernel<<<grid, 256, 0, st>>>(r, d, theta, n, t);
+  dav_ritz_kernel<<<grid, 256, 0, st>>>(V, AV, ld, m, Z, w, t2, d, n, u, au, r, t);
 }
 
 // ---------------------------------------------------------------------------
@@ -893,10 +934,13 @@ void launch_reduced_acc(const double* D1, const double* D2, const double* D3, in
 // blocks on and above the diagonal, no work for rotations that are the identity, a thread's
 // blocks found once and a step's pairs once by the thread that rotates them (n = 12 / 24: 233 /
 // 631 -> 178 / 472 us, the residual of a pair and the orthogonality 2 to 3 times smaller).
+// The tangent in FP32, its element's rest kept, was 10% faster there but half as fast on matrices
+// of rank one: not kept.
 constexpr int JACOBI_THREADS = 256;
 constexpr int JACOBI_NP = JACOBI_MAXN / 2;
 constexpr int JACOBI_ITEMS = (JACOBI_NP * (JACOBI_NP + 1) / 2 + JACOBI_MAXN * JACOBI_NP + JACOBI_THREADS - 1) / JACOBI_THREADS;
-__global__ void __launch_bounds__(JACOBI_THREADS) jacobi_kernel(double* __restrict__ Ag, int n, double* __restrict__ w,
+__global__ void __launch_bounds__(JACOBI_THREADS) jacobi_kernel(double* __restrict__ Ag, int ld, int n,
+                                                                const double* __restrict__ col, double* __restrict__ w,
                                                                 double* __restrict__ Zg) {
   __shared__ double A[JACOBI_MAXN][JACOBI_MAXN + 1];
   __shared__ double Z[JACOBI_MAXN][JACOBI_MAXN + 1];
@@ -908,7 +952,11 @@ __global__ void __launch_bounds__(JACOBI_THREADS) jacobi_kernel(double* __restri
   const int ne = (n + 1) & ~1, np = ne / 2;       // an odd n gets a row that pairs with nobody
   for (int e = tid; e < n * n; e += JACOBI_THREADS) {
     const int i = e / n, j = e % n;
-    A[i][j] = 0.5 * (Ag[i * n + j] + Ag[j * n + i]);
+    if (col && max(i, j) == n - 1) {              // the new row and column
+      A[i][j] = Ag[i * ld + j] = col[min(i, j)];
+    } else {
+      A[i][j] = 0.5 * (Ag[i * ld + j] + Ag[j * ld + i]);
+    }
     Z[i][j] = (i == j) ? 1.0 : 0.0;
   }
   // this thread's items, u | v << 8: rows of pair u times columns of pair v >= u of A, then
@@ -1035,9 +1083,9 @@ __global__ void __launch_bounds__(JACOBI_THREADS) jacobi_kernel(double* __restri
   for (int i = tid; i < n; i += JACOBI_THREADS) w[i] = A[order[i]][order[i]];
 }
 
-void launch_jacobi_eigh(double* A, int n, double* w, double* Z, cudaStream_t st) {
+void launch_jacobi_eigh(double* A, int n, double* w, double* Z, cudaStream_t st, const double* col, int ld) {
   if (n <= 0) return;
-  jacobi_kernel<<<1, JACOBI_THREADS, 0, st>>>(A, n, w, Z);
+  jacobi_kernel<<<1, JACOBI_THREADS, 0, st>>>(A, ld > 0 ? ld : n, n, col, w, Z);
 }
 
 }  // namespace lrt

@@ -321,13 +321,22 @@ void launch_dots(const double* V, int64_t ld, int m, const double* w, int64_t n,
 // out[a * nb + b] = A[a] . B[b], a < na, b < nb (device arrays of device pointers, length n each)
 void launch_pair_dots(const double* const* A, const double* const* B, int na, int nb, int64_t n, double* out,
                       cudaStream_t st);
+// out = beta out + sign sum_j coef[j] V_j (coef on the device, sign +-1)
 void launch_lincomb(const double* V, int64_t ld, int m, const double* coef, int64_t n, double* out, double beta,
-                    cudaStream_t st);
-void launch_precond(const double* r, const double* d, double theta, int64_t n, double* t, cudaStream_t st);
+                    cudaStream_t st, double sign = 1.0);
+constexpr double DAV_MIN_NORM = 1e-14;   // a Davidson direction shorter than this ends the iteration
+// v = t / |t|, t2 = |t|^2 on the device; zero below DAV_MIN_NORM
+void launch_dav_unit(const double* t, const double* t2, int64_t n, double* v, cudaStream_t st);
+// lowest pair (w[0], column 0 of Z, m x m) of the subspace: u = V z, au = AV z, r = au - theta u,
+// t = -r / (d - theta); nothing is written if |t|^2 given in t2 is below DAV_MIN_NORM^2
+void launch_dav_ritz(const double* V, const double* AV, int64_t ld, int m, const double* Z, const double* w,
+                     const double* t2, const double* d, int64_t n, double* u, double* au, double* r, double* t,
+                     cudaStream_t st);
 // Eigen-decomposition of a small symmetric n x n matrix (n <= JACOBI_MAXN) by cyclic Jacobi
-// rotations in one CTA: A (row-major, overwritten) -> eigenvalues w (ascending) and
-// eigenvectors as the columns of Z (row-major n x n).
-void launch_jacobi_eigh(double* A, int n, double* w, double* Z, cudaStream_t st);
+// rotations in one CTA: A (row-major, rows ld or n apart) -> eigenvalues w (ascending) and
+// eigenvectors as the columns of Z (row-major n x n).  With col (n values on the device) the last
+// row and column of A are set to it first.
+void launch_jacobi_eigh(double* A, int n, double* w, double* Z, cudaStream_t st, const double* col = nullptr, int ld = 0);
 constexpr int JACOBI_MAXN = 48;
 
 // Batched forms for the sweeps of several trial vectors at once.  A batch holds nv
