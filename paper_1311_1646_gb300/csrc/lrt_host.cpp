@@ -5612,31 +5612,33 @@ static void sigma_batched_impl(lrt_ctx* const* ctxs, int n, const int* sites, in
                                const double* const* x, double* const* y, int precision) {
   lrt_ctx* c0 = ctxs[0];
   std::vector<SigmaPlan*> plans(n);
-  bool missing = false;
-  for (int j = 0; j < n; ++j) missing = missing || !ctxs[j] || !ctxs[j]->have_mps || !ctxs[j]->have_ham;
-  if (precision == LRT_MIXED && !missing) {
-    // all instances small: the call runs in FP64 (see mixed_in_fp64)
+  // every argument first: a refused call leaves all contexts (and the other devices) as they were
+  for (int j = 0; j < n; ++j) {
+    const lrt_ctx* c = ctxs[j];
+    if (!c) throw Error(LRT_EINVAL, "sigma_batched: NULL context");
+    if (c->dev != c0->dev) throw Error(LRT_EINVAL, "sigma_batched: contexts on different devices");
+    if (!c->have_mps || !c->have_ham) throw Error(LRT_ESTATE, "sigma_batched: op_build and mps_load first");
+    if (sites[j] < 0 || sites[j] + nsite > c->k || !c->L[sites[j]])
+      throw Error(LRT_ESTATE, "sigma_batched: environment of instance " + std::to_string(j) + " missing");
+    if (!c->R[sites[j] + nsite])
+      throw Error(LRT_ESTATE, "right block of bond " + std::to_string(sites[j] + nsite) + " not built");
+    if (!x[j] || !y[j]) throw Error(LRT_EINVAL, "sigma_batched: NULL vector");
+  }
+  if (precision == LRT_MIXED && !c0->tc_stall) {
+    // all instances small: the call runs in FP64 (see mixed_in_fp64; a pending stall is c0's)
     double macs = 0.0;
-    bool small = !c0->tc_stall;
+    bool small = true;
     for (int j = 0; j < n && small; ++j) {
-      lrt_ctx* c = ctxs[j];
-      if (sites[j] < 0 || sites[j] + nsite > c->k || !c->L[sites[j]]) break;   // refused below
-      PoolScope ps(&c->pool);
-      const double m = position_macs(c, sites[j], nsite);
+      PoolScope ps(&ctxs[j]->pool);
+      const double m = position_macs(ctxs[j], sites[j], nsite);
       macs += m;
-      small = mixed_in_fp64(c, m, nvec) && macs * nvec < MIXED_MIN_TOTAL;
+      small = m < MIXED_MIN_MACS && macs * nvec < MIXED_MIN_TOTAL;
     }
     if (small) precision = LRT_FP64;
   }
   std::string key = std::to_string(nsite) + ":" + std::to_string(nvec) + ":" + std::to_string(precision);
   for (int j = 0; j < n; ++j) {
     lrt_ctx* c = ctxs[j];
-    if (!c) throw Error(LRT_EINVAL, "sigma_batched: NULL context");
-    if (c->dev != c0->dev) throw Error(LRT_EINVAL, "sigma_batched: contexts on different devices");
-    if (!c->have_mps || !c->have_ham) throw Error(LRT_ESTATE, "sigma_batched: op_build and mps_load first");
-    if (sites[j] < 0 || sites[j] + nsite > c->k || !c->L[sites[j]])
-      throw Error(LRT_ESTATE, "sigma_batched: environment of instance " + std::to_string(j) + " missing");
-    if (!x[j] || !y[j]) throw Error(LRT_EINVAL, "sigma_batched: NULL vector");
     PoolScope ps(&c->pool);
     plans[j] = &get_plan(c, sites[j], nsite, nvec, precision == LRT_MIXED);
     key += ":" + std::to_string(c->id) + "/" + std::to_string(sites[j]);
