@@ -249,6 +249,16 @@ int sweep_tda(lrt_t ctx, int nroots, const lrt_tda_params* params, double* omega
  * first waits on a barrier that nothing completes, so that call ends through this path
  * after `seconds`; the hook clears itself with that launch.  Not part of the paper. */
 int lrt_set_wait_limit(lrt_t ctx, double seconds, int stall_next);
+/* lrt_set_kernels: test hook, the kernels of the context's later calls, whatever the rules on
+ * sizes say (kept plans are dropped).  list_kernel: the grouped FP64 products run on the FP64
+ * FMA tiles, the digit-product tiles of a CTA or those of a warp (FP64 FMA where such a kernel
+ * cannot take a list); mixed_always != 0: LRT_MIXED calls of any size run in split TF32.
+ * sigma_batched follows its first context.  lrt_kernel_launches: how many launches of the
+ * grouped-product kernels the context has issued, counts[4] = FP64 FMA, digits by CTA tiles,
+ * digits (and FMA) by warp tiles, split TF32. */
+enum { LRT_KERNEL_AUTO = 0, LRT_KERNEL_FP64 = 1, LRT_KERNEL_CTA = 2, LRT_KERNEL_WARP = 3 };
+int lrt_set_kernels(lrt_t ctx, int list_kernel, int mixed_always);
+int lrt_kernel_launches(lrt_t ctx, int64_t* counts);
 /* sweep_tda_density: sweep_tda, and for every root mu the one-particle transition density
  * gamma[mu * k * k + p * k + q] = <Psi^mu| sum_sigma a+_{p sigma} a_{q sigma} |Psi0> over spatial
  * orbitals p, q, with Psi^mu the root's normalized tangent vector (its overall sign is

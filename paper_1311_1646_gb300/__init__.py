@@ -19,10 +19,11 @@ LRT_FP64 = 0
 LRT_MIXED = 1
 LRT_CORR_SITE = 0
 LRT_CORR_SWEEP = 1
+KERNEL_AUTO, KERNEL_FP64, KERNEL_CTA, KERNEL_WARP = range(4)
 
 EXPORTS = ["lrt_create", "lrt_destroy", "lrt_last_error", "op_build", "mps_load", "wfn_layout",
            "renormalize", "sigma", "heff_diag", "sigma_stats", "sigma_noalloc", "sweep_gs",
-           "mps_save", "mps_get_bonds", "mps_get_site", "tda_load", "tda_prepare", "tda_stationarity", "sweep_tda", "sweep_tda_density", "sweep_response", "lrt_sweeps", "lrt_sweep_log", "lrt_set_wait_limit", "sigma_batched",
+           "mps_save", "mps_get_bonds", "mps_get_site", "tda_load", "tda_prepare", "tda_stationarity", "sweep_tda", "sweep_tda_density", "sweep_response", "lrt_sweeps", "lrt_sweep_log", "lrt_set_wait_limit", "lrt_set_kernels", "lrt_kernel_launches", "sigma_batched",
            "sweep_tda_batched"]
 
 _lib = None
@@ -116,6 +117,8 @@ def load(path: str | None = None) -> ctypes.CDLL:
     lib.lrt_sweep_log.argtypes = [vp, i, dp, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)]
     lib.sweep_response.argtypes = [vp, vp, d, ctypes.POINTER(RespParams), dp, dp, ctypes.POINTER(ctypes.c_int)]
     lib.lrt_set_wait_limit.argtypes = [vp, d, i]
+    lib.lrt_set_kernels.argtypes = [vp, i, i]
+    lib.lrt_kernel_launches.argtypes = [vp, ctypes.POINTER(ctypes.c_int64)]
     lib.sigma_batched.argtypes = [ctypes.POINTER(vp), i, ctypes.POINTER(ctypes.c_int), i, i,
                                   ctypes.POINTER(vp), ctypes.POINTER(vp), i]
     lib.sweep_tda.argtypes = [vp, i, ctypes.POINTER(TdaParams), dp, dp, dp]
@@ -304,6 +307,17 @@ class Context:
         nrm = ctypes.c_double()
         self._check(self.lib.tda_prepare(self.h, ctypes.byref(nrm)), "tda_prepare")
         return nrm.value
+
+    def set_kernels(self, list_kernel: int = KERNEL_AUTO, mixed_always: bool = False):
+        """Test hook: the kernel of the grouped FP64 products, and split TF32 for LRT_MIXED calls
+        of any size."""
+        self._check(self.lib.lrt_set_kernels(self.h, list_kernel, 1 if mixed_always else 0), "lrt_set_kernels")
+
+    def kernel_launches(self) -> list:
+        """Launches so far: [FP64 FMA, digits by CTA tiles, by warp tiles, split TF32]."""
+        c = (ctypes.c_int64 * 4)()
+        self._check(self.lib.lrt_kernel_launches(self.h, c), "lrt_kernel_launches")
+        return list(c)
 
     def set_wait_limit(self, seconds: float, stall_next: bool = False):
         """Limit of the tensor-core kernels' pipeline waits (0: the default); stall_next makes

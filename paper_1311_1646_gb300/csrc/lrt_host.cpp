@@ -714,6 +714,12 @@ struct GatherPlan {
 
 // kernel of a grouped GEMM: FP64 FMAs by CTA tiles, digit products by CTA tiles, one warp per tile
 enum class GemmKind { FP64, MMA, WARP };
+// a context's choice of kernels (test hook) and its launches of each: FP64, MMA, WARP, split TF32
+struct KernelChoice {
+  int forced = 0;              // 0: by the rules; 1 + GemmKind: that kernel wherever it takes the list
+  bool mixed_always = false;   // LRT_MIXED calls of any size run in split TF32
+  int64_t launches[4] = {0, 0, 0, 0};
+};
 
 struct GemmPlan {
   DevArray<GemmOut> outs;    // the plan's outputs, then the K parts of split tiles
@@ -727,7 +733,9 @@ struct GemmPlan {
   double flops = 0.0;
   GemmKind kind = GemmKind::FP64;
   DevArray<int> counters;    // WARP: finished parts of every split tile (zero between launches)
+  KernelChoice* choice = nullptr;   // of the context the list was built for
   void run(cudaStream_t st, const double* xb, double* yb, double* tb = nullptr, const GemmExtra* ex = nullptr) const {
+    count();
     switch (kind) {
       case GemmKind::WARP:
         launch_gemm_warp(outs.p, segs.p, tiles.p, ntiles, xb, yb, tb, st, nullptr, ex, ws.p, splits.p, counters.p);
@@ -741,7 +749,11 @@ struct GemmPlan {
     }
     if (nsplit > 0) launch_split_reduce(outs.p, splits.p, nsplit, ws.p, yb, tb, st);
   }
+  void count() const {
+    if (ntiles > 0) ++choice->launches[(int)kind];
+  }
   void run_inst(cudaStream_t st, const GemmInstSet& B, int n) const {
+    count();
     switch (kind) {
       case GemmKind::WARP: launch_gemm_warp_inst(outs.p, segs.p, tiles.p, ntiles, B, n, st); break;
       case GemmKind::MMA: launch_gemm_mma_inst(outs.p, segs.p, tiles.p, ntiles, B, n, st); break;
@@ -813,7 +825,7 @@ static void mma_tile_shape(const GemmOut& O, int& tm, int& tn) {
 // it every bit of a vector's result, does not depend on how many vectors the call has.  FP64
 // CTA tiles are left for strides beyond 32 bits.
 static GemmKind gemm_kind(const std::vector<GemmOut>& outs, const std::vector<GemmSeg>& segs,
-                          const std::vector<int64_t>& ktot) {
+                          const std::vector<int64_t>& ktot, int forced) {
   double exact = 0.0, padded = 0.0;
   for (size_t i = 0; i < outs.size(); ++i) {
     const GemmOut& o = outs[i];
@@ -827,6 +839,7 @@ static GemmKind gemm_kind(const std::vector<GemmOut>& outs, const std::vector<Ge
     exact += (double)m * n * ktot[i];
     padded += (double)((m + 15) / 16 * 16) * ((n + 7) / 8 * 8) * ((ktot[i] + 15) / 16 * 16);
   }
+  if (forced > 0) return (GemmKind)(forced - 1);
   return exact >= 3e8 && padded <= 3.0 * exact ? GemmKind::MMA : GemmKind::WARP;
 }
 
@@ -861,7 +874,7 @@ enum class GemmSplit { NEVER, WARP, ALWAYS };
 
 // outs is worked on in place: the parts of split tiles are appended
 static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vector<GemmSeg>& segs,
-                       cudaStream_t st, GemmSplit split = GemmSplit::NEVER) {
+                       cudaStream_t st, KernelChoice& choice, GemmSplit split = GemmSplit::NEVER) {
   // A tile costs its warps of outputs times its K chunks of DFMA issue, plus a fixed
   // cost per chunk.  Tiles far longer than an even share of the launch (an output with
   // many long K segments) would run on after all others finished.  With `split`, an
@@ -882,7 +895,7 @@ static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vecto
     for (int s = 0; s < outs[i].seg_count; ++s) ktot[i] += segs[outs[i].seg_begin + s].k;
     fl += 2.0 * outs[i].m * (double)outs[i].n * (double)ktot[i];
   }
-  const GemmKind kind = gemm_kind(outs, segs, ktot);
+  const GemmKind kind = gemm_kind(outs, segs, ktot, choice.forced);
   const bool mma = kind == GemmKind::MMA, warp = kind == GemmKind::WARP;
   auto cost = [mma, warp](int64_t mt, int64_t nt, int64_t k) {
     const int64_t nch = (k + GEMM_KC - 1) / GEMM_KC;
@@ -984,6 +997,7 @@ static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vecto
   if (wsz > 0) P.ws.ensure((size_t)wsz);
   P.flops = fl;
   P.kind = kind;
+  P.choice = &choice;
   if (warp && P.nsplit > 0) P.counters.upload(std::vector<int>(sp.size(), 0), st);
 }
 
@@ -1209,6 +1223,7 @@ struct lrt_ctx {
   std::vector<std::pair<double, int>> sweep_log;   // last sweep_tda: seconds and mixed flag per sweep
   uint64_t tc_wait_ns = 0;   // limit of the tensor-core pipeline waits (0: the default)
   int tc_stall = 0;          // test hook: the next tensor-core launch stalls on a wait
+  lrt::KernelChoice kernels;
   int* derr = nullptr;   // device flag set by a kernel whose bounded wait expired
   std::unique_ptr<lrt::TdaState> tda;
   // right-fused copy task lists per (bond, layout of site tensor and fused basis), relative
@@ -1588,8 +1603,8 @@ static void ren_run(lrt_ctx* c, std::vector<GemmOut>& o1, std::vector<GemmSeg>& 
     return;
   }
   auto p1 = std::make_unique<GemmPlan>(), p2 = std::make_unique<GemmPlan>();
-  build_gemm(*p1, o1, s1, c->st);
-  build_gemm(*p2, o2, s2, c->st);
+  build_gemm(*p1, o1, s1, c->st, c->kernels);
+  build_gemm(*p2, o2, s2, c->st, c->kernels);
   double* tmp = nullptr;
   if (toff > 0 && dev_alloc((void**)&tmp, (size_t)toff * sizeof(double)) != cudaSuccess)
     throw Error(LRT_ENOMEM, "renormalize workspace");
@@ -2143,9 +2158,9 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
       g.a_vs = p.ident ? nelem : toff;
     }
   }
-  if (!diag_only) build_gemm(plan->p1, o1, s1, c->st);
+  if (!diag_only) build_gemm(plan->p1, o1, s1, c->st, c->kernels);
   // kept relative plans are replayed over instances
-  if (!diag_only) build_gemm(plan->p2, O2, S2, c->st, rel_ops ? GemmSplit::NEVER : GemmSplit::ALWAYS);
+  if (!diag_only) build_gemm(plan->p2, O2, S2, c->st, c->kernels, rel_ops ? GemmSplit::NEVER : GemmSplit::ALWAYS);
   // tensor-core twin: phase-2 outputs, one per (y block, column group)
   plan->has_tc = tc;
   for (size_t w = 0; w < wb.size() && tc; ++w)
@@ -2617,6 +2632,7 @@ static void run_tc(lrt_ctx* ctx, SigmaPlan& p, const double* x_dev, double* y_de
   const TcOut to = tc_out(ctx, y_dev, nullptr);
   launch_gemm_tf32x3(p.tci1.p, p.tcb1.p, p.tcn1, p.tn1, to, ctx->derr, ctx->st);
   launch_gemm_tf32x3(p.tci2.p, p.tcb2.p, p.tcn2, p.tn2, to, ctx->derr, ctx->st);
+  ctx->kernels.launches[3] += 2;
   CK(cudaGetLastError());
   int flag = 0;
   CK(cudaMemcpyAsync(&flag, ctx->derr, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
@@ -2694,6 +2710,7 @@ static void run_two_phase_tc(lrt_ctx* c, const std::vector<GemmOut>& o1, const s
   const int t2 = tune_tc_stream(c, {TcSource{&tp, &tp.out2, phi, plo, 0, 0}}, 1, none, i2, b2, n2, false);
   launch_gemm_tf32x3(i1.p, b1.p, n1, t1, none, c->derr, c->st);
   launch_gemm_tf32x3(i2.p, b2.p, n2, t2, none, c->derr, c->st);
+  c->kernels.launches[3] += 2;
   CK(cudaGetLastError());
   int flag = 0;
   CK(cudaMemcpyAsync(&flag, c->derr, sizeof(int), cudaMemcpyDeviceToHost, c->st));
@@ -2761,7 +2778,7 @@ static SigmaPlan* plan_after_diag(lrt_ctx* c, int site, int nsite) {
 // stall (lrt_set_wait_limit) is for the next tensor-core launch, so such a call keeps it.
 constexpr double MIXED_MIN_MACS = 2e8, MIXED_MIN_TOTAL = 7e8;   // phase 1, per vector / of the call
 static bool mixed_in_fp64(lrt_ctx* c, double macs, int nvec) {
-  return !c->tc_stall && macs < MIXED_MIN_MACS && macs * nvec < MIXED_MIN_TOTAL;
+  return !c->tc_stall && !c->kernels.mixed_always && macs < MIXED_MIN_MACS && macs * nvec < MIXED_MIN_TOTAL;
 }
 
 // multiply-adds of X psi over the non-zero sub-blocks of the enlarged left set, one vector
@@ -2970,7 +2987,7 @@ static void form_theta(lrt_ctx* c, int i, double* psi, const std::vector<WfnBloc
     segs.push_back(GemmSeg{A.d + A.blk_off[q], rf.p + roff[q], 0, 0, mid.d[q], w.cols, mid.d[q], 0, 0, 0, 0, 1.0});
   }
   GemmPlan gp;
-  build_gemm(gp, outs, segs, c->st);
+  build_gemm(gp, outs, segs, c->st, c->kernels);
   gp.run(c->st, nullptr, nullptr);
   CK(cudaStreamSynchronize(c->st));
 }
@@ -3015,7 +3032,7 @@ static double decimate(lrt_ctx* c, int i, const double* psi, const std::vector<W
         segs.push_back(GemmSeg{psi + b.off, psi + b.off, 0, 0, b.cols, b.cols, b.rows, 1, 0, 0, 0, 1.0});
     }
     GemmPlan gp;
-    build_gemm(gp, outs, segs, st);
+    build_gemm(gp, outs, segs, st, c->kernels);
     gp.run(st, nullptr, nullptr);
   }
   // eigen-decomposition per sector (cuSOLVER, FP64 on the device)
@@ -3125,7 +3142,7 @@ static double decimate(lrt_ctx* c, int i, const double* psi, const std::vector<W
     build_gather(gp, gt, gs, st);
     gp.run(st);
     GemmPlan mp;
-    build_gemm(mp, outs, segs, st);
+    build_gemm(mp, outs, segs, st, c->kernels);
     mp.run(st, nullptr, nullptr);
   }
   // right-fused (d x fused_R) -> left-fused storage of site i+1
@@ -3249,7 +3266,7 @@ static SiteTensor new_site(lrt_ctx* c, int i) {
 static void run_gemms(lrt_ctx* c, std::vector<GemmOut>& o, const std::vector<GemmSeg>& g) {
   if (o.empty()) return;
   GemmPlan p;
-  build_gemm(p, o, g, c->st);
+  build_gemm(p, o, g, c->st, c->kernels);
   p.run(c->st, nullptr, nullptr);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(c->st));
@@ -3876,7 +3893,7 @@ struct TdaRunner {
       }
     }
     p = std::make_unique<GemmPlan>();
-    if (!o.empty()) build_gemm(*p, o, g, c->st);
+    if (!o.empty()) build_gemm(*p, o, g, c->st, c->kernels);
     return *p;
   }
   void run_bop(GemmPlan& p, const double* a, const double* b, double* out) {
@@ -5571,7 +5588,8 @@ static std::vector<T> download(const DevArray<T>& a, cudaStream_t st) {
   return h;
 }
 
-static void merge_fp64(GemmPlan& out, const std::vector<SigmaPlan*>& plans, bool phase2, cudaStream_t st) {
+static void merge_fp64(GemmPlan& out, const std::vector<SigmaPlan*>& plans, bool phase2, cudaStream_t st,
+                       KernelChoice& choice) {
   std::vector<GemmOut> O;
   std::vector<GemmSeg> S;
   for (size_t j = 0; j < plans.size(); ++j) {
@@ -5587,7 +5605,7 @@ static void merge_fp64(GemmPlan& out, const std::vector<SigmaPlan*>& plans, bool
     }
     S.insert(S.end(), sg.begin(), sg.end());
   }
-  build_gemm(out, O, S, st, GemmSplit::WARP);
+  build_gemm(out, O, S, st, choice, GemmSplit::WARP);
 }
 
 // one batched call (the graph body): no host synchronization inside
@@ -5624,7 +5642,7 @@ static void sigma_batched_impl(lrt_ctx* const* ctxs, int n, const int* sites, in
       throw Error(LRT_ESTATE, "right block of bond " + std::to_string(sites[j] + nsite) + " not built");
     if (!x[j] || !y[j]) throw Error(LRT_EINVAL, "sigma_batched: NULL vector");
   }
-  if (precision == LRT_MIXED && !c0->tc_stall) {
+  if (precision == LRT_MIXED && !c0->tc_stall && !c0->kernels.mixed_always) {
     // all instances small: the call runs in FP64 (see mixed_in_fp64; a pending stall is c0's)
     double macs = 0.0;
     bool small = true;
@@ -5676,8 +5694,8 @@ static void sigma_batched_impl(lrt_ctx* const* ctxs, int n, const int* sites, in
       B->tn2 = tune_tc_stream(c0, s2, nvec, scratch, B->tci2, B->tcb2, B->tcn2);
       CK(cudaStreamSynchronize(c0->st));
     } else {
-      merge_fp64(B->p1, plans, false, c0->st);
-      merge_fp64(B->p2, plans, true, c0->st);
+      merge_fp64(B->p1, plans, false, c0->st, c0->kernels);
+      merge_fp64(B->p2, plans, true, c0->st, c0->kernels);
     }
     CK(cudaStreamSynchronize(c0->st));
     slot = std::move(B);
@@ -5733,6 +5751,12 @@ static void sigma_batched_impl(lrt_ctx* const* ctxs, int n, const int* sites, in
     batch_issue(c0, B, plans, xv, nvec, c0->st);
   }
   CK(cudaGetLastError());
+  if (precision == LRT_MIXED) {
+    c0->kernels.launches[3] += 2;
+  } else {
+    B.p1.count();
+    B.p2.count();
+  }
   B.gx = xv;
   B.gy = yv;
   B.ran = true;
@@ -6192,6 +6216,23 @@ int lrt_set_wait_limit(lrt_t ctx, double seconds, int stall_next) {
     if (!(seconds >= 0.0) || seconds > 60.0) throw Error(LRT_EINVAL, "lrt_set_wait_limit: seconds in [0, 60]");
     ctx->tc_wait_ns = (uint64_t)(seconds * 1e9);
     ctx->tc_stall = stall_next ? 1 : 0;
+  });
+}
+
+int lrt_set_kernels(lrt_t ctx, int list_kernel, int mixed_always) {
+  return guard(ctx, [&] {
+    if (list_kernel < LRT_KERNEL_AUTO || list_kernel > LRT_KERNEL_WARP)
+      throw Error(LRT_EINVAL, "lrt_set_kernels: unknown kernel");
+    ctx->kernels.forced = list_kernel;
+    ctx->kernels.mixed_always = mixed_always != 0;
+    drop_plans(ctx);   // planned again under the new choice
+  });
+}
+
+int lrt_kernel_launches(lrt_t ctx, int64_t* counts) {
+  return guard(ctx, [&] {
+    if (!counts) throw Error(LRT_EINVAL, "lrt_kernel_launches: NULL output");
+    std::copy(ctx->kernels.launches, ctx->kernels.launches + 4, counts);
   });
 }
 
