@@ -714,6 +714,13 @@ struct GatherPlan {
 
 // kernel of a grouped GEMM: FP64 FMAs by CTA tiles, digit products by CTA tiles, one warp per tile
 enum class GemmKind { FP64, MMA, WARP };
+// Arithmetic of a list.  FMA: every element as accurate as an FMA chain, whatever its operands
+// span.  DIGITS (where it pays): the error of an element is relative to its row's largest times its
+// column's largest operand.  That serves H_eff x, whose operators are those of orthonormal bases,
+// and not products that carry Schmidt values or their inverses, whose small elements are divided
+// by Schmidt values later: with digit products in the tangent-space sweeps, the roots of one
+// sweep moved by 2e-9 (bonds damped to 1e-4) and 2e-8 (1e-6), with FMAs by 1e-14.
+enum class GemmMath { FMA, DIGITS };
 // a context's choice of kernels (test hook) and its launches of each: FP64, MMA, WARP, split TF32
 struct KernelChoice {
   int forced = 0;              // 0: by the rules; 1 + GemmKind: that kernel wherever it takes the list
@@ -813,8 +820,8 @@ static void mma_tile_shape(const GemmOut& O, int& tm, int& tn) {
   }
 }
 
-// Kernel of a list.  CTA tiles of digit products for long lists (3e8 multiply-adds per vector
-// and more) of blocks that fill them (work padded to 16 x 8 x 16 at most 3 times the exact
+// Kernel of a list.  DIGITS: CTA tiles of digit products for long lists (3e8 multiply-adds per
+// vector and more) of blocks that fill them (work padded to 16 x 8 x 16 at most 3 times the exact
 // work), one warp per tile elsewhere: a CTA shares the cut operands among its units, a warp
 // waits for nobody.  Both measured, CTA / warp (multiply-adds, padding of the two phases):
 // k = 24, M = 500, 6 vectors (2 x 1.9e9 per vector; 1.8, 1.1) 15.2 / 25.2 ms; the same chain at
@@ -822,10 +829,13 @@ static void mma_tile_shape(const GemmOut& O, int& tm, int& tn) {
 // 1.46 ms; eight molecules of 8 to 12 orbitals (5e7; 4, 3) 1.32 / 0.88 ms; with earlier forms of
 // both, PPP k = 12, M = 256 (1.7e7; 2.0, 1.9) 129 / 93 us and k = 8, M = 64 (1e6; 13, 5) 135 / 61 us
 // (183 by FP64 CTA tiles).  Counted per vector, so that a call's kernel, and with
-// it every bit of a vector's result, does not depend on how many vectors the call has.  FP64
-// CTA tiles are left for strides beyond 32 bits.
+// it every bit of a vector's result, does not depend on how many vectors the call has.
+// FMA: warp tiles of 64 elements straight from global memory up to 1e8 multiply-adds, CTA tiles
+// with staged operands above.  A renormalization's two launches, CTA / warp: 1.1e5 multiply-adds 24 /
+// 16 us, 1.2e7 138 / 69 (k = 12, M = 128), 5e7 292 / 193 and 1.4e8 499 / 539 (k = 14 and 16), 1.1e9 2.1 /
+// 2.9 ms (k = 24, M = 500).  CTA tiles also take strides beyond 32 bits.
 static GemmKind gemm_kind(const std::vector<GemmOut>& outs, const std::vector<GemmSeg>& segs,
-                          const std::vector<int64_t>& ktot, int forced) {
+                          const std::vector<int64_t>& ktot, GemmMath math, int forced) {
   double exact = 0.0, padded = 0.0;
   for (size_t i = 0; i < outs.size(); ++i) {
     const GemmOut& o = outs[i];
@@ -840,22 +850,23 @@ static GemmKind gemm_kind(const std::vector<GemmOut>& outs, const std::vector<Ge
     padded += (double)((m + 15) / 16 * 16) * ((n + 7) / 8 * 8) * ((ktot[i] + 15) / 16 * 16);
   }
   if (forced > 0) return (GemmKind)(forced - 1);
+  if (math == GemmMath::FMA) return exact >= 1e8 ? GemmKind::FP64 : GemmKind::WARP;
   return exact >= 3e8 && padded <= 3.0 * exact ? GemmKind::MMA : GemmKind::WARP;
 }
 
-// Path and tile of one output in the warp kernel.  Direct FMAs cost about 0.5 clocks of the FP64
-// pipe per element and K position, digit products about 210 issue slots per 16 x 8 x 16 but a
+// Path and tile of one output in the warp kernel (digits: the list may take them).  Direct FMAs
+// cost about 0.5 clocks of the FP64 pipe per element and K position, digit products about 210 issue slots per 16 x 8 x 16 but a
 // longer dependent chain: direct below 1000 multiply-adds per 16 positions (counted per vector;
 // limits of 150 / 400 / 1000: 52 / 51 / 49 us at k = 8, M = 64, 954 / 933 / 912 for the eight
 // molecules, and at 4000 1780).
-static void warp_tile_shape(GemmOut& O, int64_t k, int& tm, int& tn) {
+static void warp_tile_shape(GemmOut& O, int64_t k, bool digits, int& tm, int& tn) {
   const int m = O.c_vr > 0 ? O.c_vr : O.m, n = O.c_vc > 0 ? O.c_vc : O.n;
   auto even = [](int x, int most) {
     const int parts = (x + most - 1) / most;
     return (x + parts - 1) / parts;
   };
   O.flags = 0;
-  if ((int64_t)m * n * std::min<int64_t>(k, 16) < 1000) {
+  if (!digits || (int64_t)m * n * std::min<int64_t>(k, 16) < 1000) {
     O.flags = GEMM_WARP_DIRECT;
     tn = even(O.n, GEMM_DIRECT_MAX);
     tm = even(O.m, GEMM_DIRECT_MAX / tn);
@@ -874,7 +885,8 @@ enum class GemmSplit { NEVER, WARP, ALWAYS };
 
 // outs is worked on in place: the parts of split tiles are appended
 static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vector<GemmSeg>& segs,
-                       cudaStream_t st, KernelChoice& choice, GemmSplit split = GemmSplit::NEVER) {
+                       cudaStream_t st, KernelChoice& choice, GemmMath math = GemmMath::FMA,
+                       GemmSplit split = GemmSplit::NEVER) {
   // A tile costs its warps of outputs times its K chunks of DFMA issue, plus a fixed
   // cost per chunk.  Tiles far longer than an even share of the launch (an output with
   // many long K segments) would run on after all others finished.  With `split`, an
@@ -895,7 +907,8 @@ static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vecto
     for (int s = 0; s < outs[i].seg_count; ++s) ktot[i] += segs[outs[i].seg_begin + s].k;
     fl += 2.0 * outs[i].m * (double)outs[i].n * (double)ktot[i];
   }
-  const GemmKind kind = gemm_kind(outs, segs, ktot, choice.forced);
+  const GemmKind kind = gemm_kind(outs, segs, ktot, math, choice.forced);
+  const bool digits = math == GemmMath::DIGITS || choice.forced > 0;
   const bool mma = kind == GemmKind::MMA, warp = kind == GemmKind::WARP;
   auto cost = [mma, warp](int64_t mt, int64_t nt, int64_t k) {
     const int64_t nch = (k + GEMM_KC - 1) / GEMM_KC;
@@ -903,11 +916,11 @@ static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vecto
     if (mma) return nch * (30 * ((mt + 15) / 16) * ((nt + 15) / 16) + 12 * ((mt + 15) / 16 + (nt + 15) / 16) + 20) + 40;
     return nch * (32 * ((mt * nt + 31) / 32) + 64) + 64;
   };
-  auto shape = [mma, warp](GemmOut& O, int64_t k, int& tm, int& tn) {
+  auto shape = [mma, warp, digits](GemmOut& O, int64_t k, int& tm, int& tn) {
     tm = GEMM_TM;
     tn = GEMM_TN;
     if (mma) mma_tile_shape(O, tm, tn);
-    if (warp) warp_tile_shape(O, k, tm, tn);
+    if (warp) warp_tile_shape(O, k, digits, tm, tn);
   };
   int64_t total = 0;
   for (size_t i = 0; i < nout && kind == GemmKind::FP64; ++i) {
@@ -2158,9 +2171,10 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
       g.a_vs = p.ident ? nelem : toff;
     }
   }
-  if (!diag_only) build_gemm(plan->p1, o1, s1, c->st, c->kernels);
-  // kept relative plans are replayed over instances
-  if (!diag_only) build_gemm(plan->p2, O2, S2, c->st, c->kernels, rel_ops ? GemmSplit::NEVER : GemmSplit::ALWAYS);
+  // kept relative plans (first-order sets) are replayed over instances
+  const GemmMath math = rel_ops ? GemmMath::FMA : GemmMath::DIGITS;
+  if (!diag_only) build_gemm(plan->p1, o1, s1, c->st, c->kernels, math);
+  if (!diag_only) build_gemm(plan->p2, O2, S2, c->st, c->kernels, math, rel_ops ? GemmSplit::NEVER : GemmSplit::ALWAYS);
   // tensor-core twin: phase-2 outputs, one per (y block, column group)
   plan->has_tc = tc;
   for (size_t w = 0; w < wb.size() && tc; ++w)
@@ -5605,7 +5619,7 @@ static void merge_fp64(GemmPlan& out, const std::vector<SigmaPlan*>& plans, bool
     }
     S.insert(S.end(), sg.begin(), sg.end());
   }
-  build_gemm(out, O, S, st, choice, GemmSplit::WARP);
+  build_gemm(out, O, S, st, choice, GemmMath::DIGITS, GemmSplit::WARP);
 }
 
 // one batched call (the graph body): no host synchronization inside
