@@ -5,6 +5,11 @@
 // taken 32 positions (a chunk) at a time.  GB300 issues 2 FP64 FMA per clock and SM but 1024
 // FP16 FMA with FP32 accumulation through mma.sync, so each chunk is multiplied in integers:
 //
+//  - every K position is first given the exponent it has over one operand (its largest element
+//    among the tile's rows of A, or columns of B, there): that power of two moves to the other
+//    operand, so that a chunk may join operators of any size and operands that are graded in
+//    opposite directions along K.  The vectors of a call lie along the other operand, whose rows
+//    then do not see each other;
 //  - every row of A and column of B of the chunk is scaled by a power of two (its largest
 //    exponent) and cut into 7 balanced digits of 9 bits, g_d in [-256, 256]: 63 bits, so an
 //    element within 2^9 of its row's largest keeps all of its 53;
@@ -16,9 +21,13 @@
 //
 // (The splitting is the error-free transformation of Ozaki, Ogita, Oishi and Rump, "Error-free
 // transformations of matrix multiplication by using fast routines of matrix multiplication",
-// Numer. Algorithms 59, 2012, with a fixed digit grid per chunk.)  What is lost per chunk is
-// below 2^-54 of its largest row times column product, less than the 32 roundings of an FP64
-// FMA chain.  Elements whose row or column
+// Numer. Algorithms 59, 2012, with a fixed digit grid per chunk.)  What a chunk loses is
+// relative to its row's largest times its column's largest element (after the exponents above):
+// the dropped products (6 pairs of i + j = 7) are below 2^-53.4 of that, cut operands and the
+// join's rounding add up to 2^-52.4, and with digits of random sign it is about 2^-59.  That is
+// less than the 32 roundings of an FMA chain where the products of the row and column are of
+// one size, and more where all of them are far below the two largest elements: sums of small
+// products are not as accurate by themselves as an FMA chain's.  Elements whose row or column
 // holds an infinity, a NaN or lies outside 2^-423 .. 2^477 are multiplied in plain FP64 from the
 // staged operands.
 //
@@ -43,7 +52,7 @@ constexpr int MMA_ND = 7;                 // digits
 constexpr int MMA_WARPS = 8;              // warps of a CTA tile
 constexpr int MMA_EMIN = 600, MMA_EMAX = 1500;   // exponent fields the integer path takes
 constexpr int MMA_E0 = 1023;
-constexpr int MMA_NOBAL = -4096;                  // balance exponent where B's row is zero
+constexpr int MMA_NOBAL = -4096;                  // exponent of a K position where that operand is zero
 constexpr int MMA_WILD = (int)0x80000000;        // exponent word of a row the integer path does not take
 
 struct MmaSmem {
@@ -53,7 +62,7 @@ struct MmaSmem {
   double sc[GEMM_KC];                     // segment scale of each K position
   SegS sd[GEMM_SEGB];
   int kst[GEMM_SEGB + 1];
-  alignas(16) int bal[GEMM_KC];           // balance exponents of the K positions
+  alignas(16) int bal[GEMM_KC];           // exponents taken out of the K positions
   alignas(8) int2 vl[MMA_ROWS];           // vector block and index inside it of each row
   int wild[2];                            // chunk (by parity) holds a row outside the integer path
   uint32_t neg;                           // K positions of negative scale
@@ -219,7 +228,7 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
   const int RB = 16 * a16;                 // first B row
   const int rows = RB + 16 * b16;          // <= MMA_ROWS
   const int units = a16 * b16;             // <= 2 * MMA_WARPS
-  const bool bal = o.balance != 0;
+  const bool bal_a = o.balance_rows != 0;   // exponents of the K positions from op(A)'s rows, else op(B)'s columns
 
   // row tables; padding rows are zero for the whole tile
   if (tid < rows) {
@@ -235,7 +244,7 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
   }
   for (int r = warp; r < rows; r += MMA_WARPS)
     if (r < RB ? r >= mt : r - RB >= nt) S.raw[r][lane] = 0.0;
-  if (bal && tid < GEMM_KC) S.bal[tid] = MMA_NOBAL;
+  if (tid < GEMM_KC) S.bal[tid] = MMA_NOBAL;
   if (tid < 2) S.wild[tid] = 0;
 
   double acc[2][2][4];
@@ -348,12 +357,13 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
       const int kc = min(GEMM_KC, Kb - c * GEMM_KC);
       const int mode = S.mode;
       const int l = lane & 7;
-      if (bal) {
-        // largest exponent of each K position over B's columns
+      {
+        // largest exponent of each K position over the balanced side
         int mx[4] = {0, 0, 0, 0};
-        for (int r = RB + 4 * warp + (lane >> 3); r < rows; r += 4 * MMA_WARPS) {
+        const int r1 = bal_a ? RB : rows;
+        for (int r = (bal_a ? 0 : RB) + 4 * warp + (lane >> 3); r < r1; r += 4 * MMA_WARPS) {
           Quad q = load_quad(&S.raw[0][0], r, l);
-          scale_quad(S, mode, l, q);
+          if (!bal_a) scale_quad(S, mode, l, q);
 #pragma unroll
           for (int j = 0; j < 4; ++j) mx[j] = max(mx[j], (int)(q.hi[j] & 0x7FFFFFFFu) >> 20);
         }
@@ -361,7 +371,7 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
         for (int j = 0; j < 4; ++j) {
           mx[j] = max(mx[j], __shfl_xor_sync(0xffffffffu, mx[j], 8));
           mx[j] = max(mx[j], __shfl_xor_sync(0xffffffffu, mx[j], 16));
-          // kept as the exponent itself; a position where B is zero stays far below every other
+          // kept as the exponent itself; a position where that side is zero stays far below every other
           if (lane < 8 && mx[j] > 0) atomicMax(&S.bal[4 * l + j], mx[j] - MMA_E0);
         }
         __syncthreads();
@@ -372,16 +382,14 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
         if (isB) scale_quad(S, mode, l, q);
         int e[4], emax;
         exponents(q, e, emax);
-        if (bal) {
-          // infinities and NaN keep their row (all columns, if op(B) holds them) out of the
-          // integer path
-          const int4 bk = *reinterpret_cast<const int4*>(&S.bal[4 * l]);
-          const int bj[4] = {bk.x, bk.y, bk.z, bk.w};
-          const bool inf = isB ? max(max(bk.x, bk.y), max(bk.z, bk.w)) == 2047 - MMA_E0 : emax == 2047;
+        // infinities and NaN keep their row out of the integer path (all rows, on the balanced side)
+        const bool own = isB != bal_a;
+        const int4 bk = *reinterpret_cast<const int4*>(&S.bal[4 * l]);
+        const int bj[4] = {bk.x, bk.y, bk.z, bk.w};
+        const bool inf = own ? max(max(bk.x, bk.y), max(bk.z, bk.w)) == 2047 - MMA_E0 : emax == 2047;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) e[j] = e[j] == 0 ? -4096 : isB ? e[j] - bj[j] : e[j] + bj[j];
-          emax = inf ? 4095 : max(max(e[0], e[1]), max(e[2], e[3]));
-        }
+        for (int j = 0; j < 4; ++j) e[j] = e[j] == 0 ? -4096 : own ? e[j] - bj[j] : e[j] + bj[j];
+        emax = inf ? 4095 : max(max(e[0], e[1]), max(e[2], e[3]));
         uint32_t d0[MMA_ND], d1[MMA_ND];
         const int x = cut_row(q, e, emax, d0, d1);
         if (l == 0) S.ex[r] = x;
@@ -393,7 +401,7 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
       __syncthreads();
       const bool wild = S.wild[it & 1] != 0;
       if (tid == 0) S.wild[(it & 1) ^ 1] = 0;   // last read before this chunk's first barrier
-      if (bal && tid < GEMM_KC) S.bal[tid] = MMA_NOBAL;
+      if (tid < GEMM_KC) S.bal[tid] = MMA_NOBAL;
       if (!wild && c + 1 < nch) issue(c + 1);   // lands during the products; raw is free
       const int nks = kc > 16 ? 2 : 1;
       const uint32_t dig0 = (uint32_t)__cvta_generic_to_shared(&S.dig[0][0][0]);
@@ -747,7 +755,8 @@ __device__ __forceinline__ void warp_tile(const GemmOut* __restrict__ outs, cons
       if (e < ne) store(m0 + e / nt, n0 + e % nt, acc[u]);
     }
   } else {
-    const bool swap = (o.flags & GEMM_WARP_SWAP) != 0, bal = o.balance != 0;
+    const bool swap = (o.flags & GEMM_WARP_SWAP) != 0;
+    const bool bal_r = swap == (o.balance_rows == 0);   // exponents of the K positions from the tile's rows, else its columns
     const int r0 = swap ? n0 : m0, rt = swap ? nt : mt, c0 = swap ? m0 : n0, ct = swap ? mt : nt;
     const int rblk = swap ? o.c_vc : o.c_vr, cblk = swap ? o.c_vr : o.c_vc;
     const int g = lane >> 2, t = lane & 3;
@@ -814,31 +823,29 @@ __device__ __forceinline__ void warp_tile(const GemmOut* __restrict__ outs, cons
             ea[h][j] = exponent_of(a[h][j]);
             eb[h][j] = exponent_of(b[h][j]);
           }
-        bool all = false;    // op(B) holds an infinity or NaN
-        if (bal) {
+        bool all = false;    // the balanced side holds an infinity or NaN
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            int m = max(eb[0][j], eb[1][j]);
-            m = max(m, __shfl_xor_sync(0xffffffffu, m, 4));
-            m = max(m, __shfl_xor_sync(0xffffffffu, m, 8));
-            m = max(m, __shfl_xor_sync(0xffffffffu, m, 16));
-            const int d = m > 0 ? m - MMA_E0 : MMA_NOBAL;
-            all |= m == 2047;
+        for (int j = 0; j < 4; ++j) {
+          int m = bal_r ? max(ea[0][j], ea[1][j]) : max(eb[0][j], eb[1][j]);
+          m = max(m, __shfl_xor_sync(0xffffffffu, m, 4));
+          m = max(m, __shfl_xor_sync(0xffffffffu, m, 8));
+          m = max(m, __shfl_xor_sync(0xffffffffu, m, 16));
+          const int d = m > 0 ? m - MMA_E0 : MMA_NOBAL, da = bal_r ? -d : d;
+          all |= m == 2047;
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              ea[h][j] = ea[h][j] == 0 ? -4096 : ea[h][j] == 2047 ? 4095 : ea[h][j] + d;
-              eb[h][j] = eb[h][j] == 0 ? -4096 : eb[h][j] - d;
-            }
+          for (int h = 0; h < 2; ++h) {
+            ea[h][j] = ea[h][j] == 0 ? -4096 : ea[h][j] == 2047 ? 4095 : ea[h][j] + da;
+            eb[h][j] = eb[h][j] == 0 ? -4096 : eb[h][j] == 2047 ? 4095 : eb[h][j] - da;
           }
-          all = __any_sync(0xffffffffu, all);
         }
+        all = __any_sync(0xffffffffu, all);
         int E[2], F[2], xe[2], xf[2];    // exponents of the rows and columns, and their words
         bool wild = false;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           E[h] = row_exponent(ea[h]);
           F[h] = row_exponent(eb[h]);
-          const bool we = outside_range(E[h]), wf = outside_range(F[h]) || all;
+          const bool we = outside_range(E[h]) || (all && bal_r), wf = outside_range(F[h]) || (all && !bal_r);
           wild |= we | wf;
           if (E[h] <= 0) E[h] = MMA_E0;
           if (F[h] <= 0) F[h] = MMA_E0;

@@ -799,24 +799,23 @@ static void build_gather(GatherPlan& P, std::vector<GatherTask>& tasks, std::vec
 }
 
 // Tile of the digit-product kernel for one output: a x b units of 16 x 16 with a + b <= 8
-// (MMA_ROWS) and a b <= 16, the shorter side whole where it fits, both sides cut evenly.  The
-// columns of a balanced output are cut by their own count only, so that a column sees the
-// same neighbours whatever the rows (the vectors of the call) are.
+// (MMA_ROWS) and a b <= 16, both sides cut evenly.  The side that balances the K positions is cut
+// by its own count only, at most 4 units, so that its rows (columns) see the same neighbours
+// whatever the other side, the vectors of the call, is.
 static void mma_tile_shape(const GemmOut& O, int& tm, int& tn) {
-  const int m16 = (O.m + 15) / 16, n16 = (O.n + 15) / 16;
   auto even = [](int n, int u, int step) {   // n in parts of at most u units of 16
     const int parts = (n + 16 * u - 1) / (16 * u);
     const int w = (n + parts - 1) / parts;
     return (w + step - 1) / step * step;
   };
-  if (O.balance || n16 < m16) {
-    tn = even(O.n, std::min(n16, 4), 8);
-    const int b = (tn + 15) / 16;
-    tm = even(O.m, std::min(8 - b, 16 / b), 16);
-  } else {
-    tm = even(O.m, std::min(m16, 4), 16);
+  if (O.balance_rows) {
+    tm = even(O.m, 4, 16);
     const int a = (tm + 15) / 16;
     tn = even(O.n, std::min(8 - a, 16 / a), 8);
+  } else {
+    tn = even(O.n, 4, 8);
+    const int b = (tn + 15) / 16;
+    tm = even(O.m, std::min(8 - b, 16 / b), 16);
   }
 }
 
@@ -873,7 +872,7 @@ static void warp_tile_shape(GemmOut& O, int64_t k, bool digits, int& tm, int& tn
     return;
   }
   const int64_t plain = (int64_t)((O.m + 15) / 16) * ((O.n + 7) / 8), swapped = (int64_t)((O.n + 15) / 16) * ((O.m + 7) / 8);
-  if (!O.balance && swapped < plain) O.flags = GEMM_WARP_SWAP;   // a balanced output's column tiles are its own
+  if (swapped < plain) O.flags = GEMM_WARP_SWAP;
   tm = even(O.m, 16);
   tn = even(O.n, 16);
 }
@@ -2116,6 +2115,7 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
   const bool vb = nvec > 1;
   for (GemmOut& y : o1) {
     y.c_rel = 2;
+    y.balance_rows = 1;   // not by the columns, which hold the vectors
     if (vb) {
       const int n = y.n;
       for (int q = 0; q < y.seg_count; ++q) {
@@ -2143,7 +2143,6 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
     }
     const int m1 = XF.dim[fx][os.r];
     GemmOut y{nullptr, coff, w.cols, m1 * nvec, ncols, at[u], at[u + 1] - at[u], 0, 1};
-    y.balance = 1;
     if (vb) {
       y.c_vr = m1;
       y.c_vs = nelem;

@@ -45,8 +45,8 @@ struct GemmOut {
   int inst;      // batched launches: index of the instance whose bases the rel pointers use
   int c_vr, c_vc;
   int64_t c_vs;
-  int balance;   // digit products (launch_gemm_mma): K positions are first scaled to equal
-                 // exponents over op(B)'s columns (an output that sums many operators)
+  int balance_rows;   // digit products: the side whose exponents the K positions are scaled by,
+                      // op(A)'s rows (1) or op(B)'s columns (0)
   int flags;     // GEMM_WARP_* (launch_gemm_warp)
   int split;     // launch_gemm_warp: the split tile a part (c_rel GEMM_C_SPLIT) belongs to
 };

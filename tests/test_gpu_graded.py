@@ -62,3 +62,68 @@ def test_tda_with_small_schmidt_values_is_as_accurate_as_fma_products(pkg, M, sp
     assert abs(e1 - e0) <= 1e-12 * abs(e0)
     assert np.abs(w1 - w0).max() <= 1e-12 * abs(e0)
     assert np.abs(r1 / r0 - 1.0).max() <= 1e-12 * abs(e0)
+
+
+def _scaled_gauge(m, k, i, nsite, side, span, seed):
+    """The MPS with every state of the left (right) bases scaled by its own power of two, 1 to
+    2^-span: the renormalized operators of that side scale by row and column, exactly."""
+    rng = np.random.default_rng(seed)
+    S = []
+    for b, table in enumerate(m.bonds):
+        on = 0 < b <= i if side == "left" else i + nsite <= b < k
+        S.append({(qa, qb): 2.0 ** -(rng.integers(0, span + 1, size=d) if on else np.zeros(d)) for qa, qb, d in table})
+    sites = []
+    for j in range(k):
+        A = om.unpack_site(m.sites[j], m.bonds[j], m.bonds[j + 1])
+        if j < i:
+            A = {q: X / S[j][q[0]][:, None] * S[j + 1][q[2]][None, :] for q, X in A.items()}
+        elif j >= i + nsite:
+            A = {q: X * S[j][q[0]][:, None] / S[j + 1][q[2]][None, :] for q, X in A.items()}
+        sites.append(om.pack_site(A, m.bonds[j], m.bonds[j + 1]))
+    return S, sites
+
+
+def _wave_scale(m, S, i, nsite, n):
+    b = m.bonds
+    if nsite == 1:
+        w = {q: X * S[i][q[0]][:, None] * S[i + 1][q[-1]][None, :]
+             for q, X in om.unpack_site(np.ones(n), b[i], b[i + 1]).items()}
+        return om.pack_site(w, b[i], b[i + 1])
+    w = {q: X * S[i][q[0]][:, None] * S[i + 2][q[-1]][None, :]
+         for q, X in om.unpack_twosite(np.ones(n), b[i], b[i + 2]).items()}
+    return om.pack_twosite(w, b[i], b[i + 2])
+
+
+@pytest.mark.parametrize("kernel", [2, 3])
+@pytest.mark.parametrize("side", ["left", "right"])
+@pytest.mark.parametrize("k,na,nb,M,i,nsite", [(10, 2, 2, 131, 4, 1), (9, 4, 4, 60, 4, 2)])
+def test_sigma_in_a_graded_gauge(pkg, k, na, nb, M, i, nsite, side, kernel):
+    """Basis states scaled by 2^0 to 2^-30 and the vector by the inverse: along K one operand rises
+    as the other falls, by 2^60 on the two-sided operators.  Against the FMA tiles on the same
+    input, relative to the largest element, at the bar of every FP64 sigma; and several vectors
+    in one call give each vector's own bits."""
+    H = synth.ab_initio(k, na, nb, 7)
+    m = synth.mixed_mps(k, na, nb, M, 8, center=i)
+    S, sites = _scaled_gauge(m, k, i, nsite, side, 30, 1)
+    out = []
+    for kn in (KERNEL_FP64, kernel):
+        ctx = pkg.Context(0)
+        ctx.set_kernels(kn)
+        ctx.op_build(k, H.h, H.eri)
+        ctx.mps_load(k, na, nb, m.bonds, sites, i)
+        for b in range(i):
+            ctx.renormalize(b, +1)
+        for b in range(k - 1, i + nsite - 1, -1):
+            ctx.renormalize(b, -1)
+        n, _ = ctx.wfn_layout(i, nsite)
+        x = synth.random_vector(2 * n, 9) / np.tile(_wave_scale(m, S, i, nsite, n), 2)
+        xd = torch.tensor(x, dtype=torch.float64, device="cuda:0")
+        y, y1 = torch.empty_like(xd), torch.empty_like(xd)
+        ctx.sigma(i, nsite, xd, y, nvec=2)
+        ctx.sigma(i, nsite, xd[:n], y1[:n])
+        ctx.sigma(i, nsite, xd[n:], y1[n:])
+        torch.cuda.synchronize()
+        assert torch.equal(y, y1)
+        out.append(y.cpu().numpy())
+        ctx.close()
+    assert np.abs(out[1] - out[0]).max() <= 1e-12 * np.abs(out[0]).max()
