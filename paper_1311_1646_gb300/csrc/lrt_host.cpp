@@ -651,6 +651,7 @@ struct DevArray {
   size_t n = 0;
   DevArray() = default;
   DevArray(const DevArray&) = delete;
+  DevArray(DevArray&& o) noexcept { swap(o); }
   ~DevArray() {
     if (p) dev_free(p);
   }
@@ -3363,24 +3364,36 @@ static void t_lmul(lrt_ctx* c, int i, const BondMat& X, const SiteTensor& A, Sit
   run_gemms(c, o, g);
 }
 
-static void lam_mats(lrt_ctx* c, int b, const std::vector<double>& lam, double cut, BondMat& L, BondMat& Li) {
-  const Sectors& S = c->bonds[b];
-  bond_layout(S, L, c->st);
-  bond_layout(S, Li, c->st);
+// the Schmidt values of a bond and their inverses (zero at and below cut * largest), states in
+// sector order: products with them are elementwise (launch_diag_scale), exact to one rounding
+// each whatever the values span
+static void lam_diags(lrt_ctx* c, const std::vector<double>& lam, double cut, DevArray<double>& L, DevArray<double>& Li) {
   double smax = 0.0;
   for (double x : lam) smax = std::max(smax, x);
-  std::vector<double> hl(L.buf.n, 0.0), hi(L.buf.n, 0.0);
-  int64_t pos = 0;
+  std::vector<double> inv(lam.size());
+  for (size_t a = 0; a < lam.size(); ++a) inv[a] = (lam[a] > cut * smax) ? 1.0 / lam[a] : 0.0;
+  L.upload(lam, c->st);
+  Li.upload(inv, c->st);
+  CK(cudaStreamSynchronize(c->st));
+}
+
+// out = X diag(w) (rows false) or diag(w) X (rows true) for the D x D blocks of bond b
+static void scale_bond(lrt_ctx* c, int b, const BondMat& X, const std::vector<double>& w, bool rows, BondMat& out) {
+  const Sectors& S = c->bonds[b];
+  bond_layout(S, out, c->st);
+  std::vector<int> state;
+  int pos = 0;
   for (int q = 0; q < S.n(); ++q) {
-    for (int a = 0; a < S.d[q]; ++a) {
-      const double x = lam[pos + a];
-      hl[L.off[q] + (int64_t)a * S.d[q] + a] = x;
-      hi[L.off[q] + (int64_t)a * S.d[q] + a] = (x > cut * smax) ? 1.0 / x : 0.0;
-    }
+    for (int r = 0; r < S.d[q]; ++r)
+      for (int a = 0; a < S.d[q]; ++a) state.push_back(pos + (rows ? r : a));
     pos += S.d[q];
   }
-  CK(cudaMemcpyAsync(L.buf.p, hl.data(), hl.size() * sizeof(double), cudaMemcpyHostToDevice, c->st));
-  CK(cudaMemcpyAsync(Li.buf.p, hi.data(), hi.size() * sizeof(double), cudaMemcpyHostToDevice, c->st));
+  DevArray<double> dw;
+  DevArray<int> ds;
+  dw.upload(w, c->st);
+  ds.upload(state, c->st);
+  launch_diag_scale(X.buf.p, 0, dw.p, ds.p, 1, (int64_t)state.size(), out.buf.p, 0, false, c->st);
+  CK(cudaGetLastError());
   CK(cudaStreamSynchronize(c->st));
 }
 
@@ -3485,23 +3498,6 @@ static void run_gathers(lrt_ctx* c, std::vector<GatherTask>& t, std::vector<Gath
   CK(cudaStreamSynchronize(c->st));
 }
 
-// M = X diag(w) (X: D x D bond blocks; per sector the weights w in sector order)
-static void scale_cols(lrt_ctx* c, int b, const BondMat& X, const std::vector<double>& w, BondMat& out) {
-  BondMat Lm, Lmi;
-  lam_mats(c, b, w, 0.0, Lm, Lmi);
-  const Sectors& S = c->bonds[b];
-  bond_layout(S, out, c->st);
-  std::vector<GemmOut> o;
-  std::vector<GemmSeg> g;
-  for (int q = 0; q < S.n(); ++q) {
-    const int D = S.d[q];
-    if (D == 0) continue;
-    o.push_back(GemmOut{out.buf.p + out.off[q], 0, D, D, D, (int)g.size(), 1, 0, 0});
-    g.push_back(GemmSeg{X.buf.p + X.off[q], Lm.buf.p + Lm.off[q], 0, 0, D, D, D, 0, 0, 0, 0, 1.0});
-  }
-  run_gemms(c, o, g);
-}
-
 // centre psi at site i -> L_i and the new centre at site i+1
 static void gauge_shift_right(lrt_ctx* c, int i, const double* psi, SvdWork& W) {
   const Sectors& Rb = c->bonds[i + 1];
@@ -3558,7 +3554,7 @@ static void gauge_shift_right(lrt_ctx* c, int i, const double* psi, SvdWork& W) 
     }
     run_gathers(c, t2, s2);
   }
-  scale_cols(c, i + 1, UTt, lam, X);          // X^T = U_a diag(lam)  ->  X = diag(lam) U_a^T
+  scale_bond(c, i + 1, UTt, lam, false, X);          // X^T = U_a diag(lam)  ->  X = diag(lam) U_a^T
   BondMat Xs;
   bond_layout(Rb, Xs, c->st);
   {
@@ -3645,7 +3641,7 @@ static void gauge_shift_left(lrt_ctx* c, int i, const double* psi, SvdWork& W) {
     run_gathers(c, t2, s2);
   }
   BondMat US;
-  scale_cols(c, i, Y, lam, US);                 // U S of the right-fused SVD
+  scale_bond(c, i, Y, lam, false, US);                 // U S of the right-fused SVD
   SiteTensor prev = new_site(c, i - 1);
   t_rmul(c, i - 1, c->sites[i - 1], US, prev, false);
   c->sites[i] = std::move(R);
@@ -3772,7 +3768,8 @@ struct TdaRunner {
   lrt_ctx* c;
   int k;
   const lrt_tda_params& P;
-  std::vector<BondMat> lam, ilam;
+  std::vector<DevArray<double>> lam, ilam;
+  std::vector<DevArray<int>> lstate, rstate;   // left and right bond state of every element of a site
   std::vector<DevBuf> diag;
   std::vector<SiteTensor> lay;       // layout of every site (no data)
   std::vector<std::unique_ptr<SigmaPlan>> h0one;   // H_0^[i] plans for one vector
@@ -3792,7 +3789,7 @@ struct TdaRunner {
   void setup() {
     lam.resize(k + 1);
     ilam.resize(k + 1);
-    for (int b = 0; b <= k; ++b) lam_mats(c, b, c->tda->lam[b], P.pinv_cut, lam[b], ilam[b]);
+    for (int b = 0; b <= k; ++b) lam_diags(c, c->tda->lam[b], P.pinv_cut, lam[b], ilam[b]);
     // zeroth-order environments: left blocks from L0, right blocks from R0
     for (int b = 0; b + 1 < k; ++b) renorm_left(c, b);
     for (int b = k - 1; b >= 1; --b) renorm_right(c, b);
@@ -3802,9 +3799,12 @@ struct TdaRunner {
     }
     lay.resize(k);
     h0one.resize(k);
+    lstate.resize(k);
+    rstate.resize(k);
     diag.resize(k);
     for (int i = 0; i < k; ++i) {
       site_layout(lay[i], c->bonds[i], c->bonds[i + 1]);
+      site_states(i);
       h0one[i] = plan_sigma_sets(c, *c->XL[i], nullptr, *c->R[i + 1], nullptr, i, 1, 1, false);
       diag[i].ensure(std::max<int64_t>(h0one[i]->nelem, 1));
       launch_diag(h0one[i]->douts.p, h0one[i]->dterms.p, h0one[i]->ndiag, diag[i].p, c->st);
@@ -3812,6 +3812,26 @@ struct TdaRunner {
     SiteTensor y = new_site(c, 0);
     run_plan(*h0one[0], C0(0).d, y.d, 1, false);    // the reference energy is FP64
     E0 = t_dot(c, C0(0), y, tmp);
+  }
+
+  void site_states(int i) {
+    const Sectors &Lb = c->bonds[i], &Rb = c->bonds[i + 1];
+    std::vector<int> rpos(Rb.n() + 1, 0), l((size_t)lay[i].total), r((size_t)lay[i].total);
+    for (int q = 0; q < Rb.n(); ++q) rpos[q + 1] = rpos[q] + Rb.d[q];
+    for (int q = 0, lpos = 0; q < Lb.n(); lpos += Lb.d[q++])
+      for (int n = 0; n < 4; ++n) {
+        if (lay[i].sub_off[q][n] < 0) continue;
+        const int qr = lay[i].sub_qr[q][n], D = Rb.d[qr];
+        for (int a = 0; a < Lb.d[q]; ++a)
+          for (int b = 0; b < D; ++b) {
+            const size_t e = (size_t)lay[i].sub_off[q][n] + (size_t)a * D + b;
+            l[e] = lpos + a;
+            r[e] = rpos[qr] + b;
+          }
+      }
+    lstate[i].upload(l, c->st);
+    rstate[i].upload(r, c->st);
+    CK(cudaStreamSynchronize(c->st));
   }
 
   void run_plan(SigmaPlan& p, const double* x, double* y, int nvec, bool tc) {
@@ -3838,7 +3858,7 @@ struct TdaRunner {
   // ---- batched bond/site products: grouped GEMMs planned once per (kind, site, nv) with
   // every per-vector address relative to extra bases 0 (batched A), 1 (batched B) and 2
   // (output), replayed for new batches ----
-  enum { K_LC, K_RMUL, K_RMULB, K_RC, K_LMUL, K_LMULB };
+  enum { K_LC, K_RMULB, K_RC, K_LMULB };
   std::map<std::tuple<int, int, int, int, int, const void*>, std::unique_ptr<GemmPlan>> bops;
   GemmPlan& bop(int kind, int i, int nv, bool acc, double scale, const void* fixed, int64_t sa, int64_t sb,
                 int64_t so, const std::vector<int64_t>* boff) {
@@ -3850,7 +3870,7 @@ struct TdaRunner {
     const SiteTensor& L = lay[i];
     const int A0 = 3, B1 = 4, O2 = 5;
     for (int v = 0; v < nv; ++v) {
-      if (kind == K_LC || kind == K_RMUL || kind == K_RMULB) {
+      if (kind == K_LC || kind == K_RMULB) {
         // per right sector q of bond i+1
         const Sectors& R = c->bonds[i + 1];
         for (int q = 0; q < R.n(); ++q) {
@@ -3861,10 +3881,6 @@ struct TdaRunner {
             const SiteTensor& A = *(const SiteTensor*)fixed;
             o.push_back(GemmOut{nullptr, (*boff)[q] + v * so, D, D, D, (int)g.size(), 1, acc ? 1 : 0, O2, 0});
             g.push_back(GemmSeg{A.d + bo, nullptr, 0, bo + v * sb, D, D, rows, 1, 0, 0, B1, scale});
-          } else if (kind == K_RMUL) {   // out_v = A_v X     (X fixed bond matrices)
-            const BondMat& X = *(const BondMat*)fixed;
-            o.push_back(GemmOut{nullptr, bo + v * so, D, rows, D, (int)g.size(), 1, acc ? 1 : 0, O2, 0});
-            g.push_back(GemmSeg{nullptr, X.buf.p + X.off[q], bo + v * sa, 0, D, D, D, 0, 0, A0, 0, scale});
           } else {                       // out_v = A X_v     (A fixed, X batched)
             const SiteTensor& A = *(const SiteTensor*)fixed;
             o.push_back(GemmOut{nullptr, bo + v * so, D, rows, D, (int)g.size(), 1, acc ? 1 : 0, O2, 0});
@@ -3895,13 +3911,9 @@ struct TdaRunner {
             const int Dr = c->bonds[i + 1].d[L.sub_qr[q][n]];
             const int64_t so_ = L.sub_off[q][n];
             o.push_back(GemmOut{nullptr, so_ + v * so, Dr, D, Dr, (int)g.size(), 1, acc ? 1 : 0, O2, 0});
-            if (kind == K_LMUL) {        // out_v = X A_v   (X fixed bond matrices)
-              const BondMat& X = *(const BondMat*)fixed;
-              g.push_back(GemmSeg{X.buf.p + X.off[q], nullptr, 0, so_ + v * sb, D, Dr, D, 0, 0, 0, B1, scale});
-            } else {                     // out_v = X_v A   (A fixed, X batched)
-              const SiteTensor& A = *(const SiteTensor*)fixed;
-              g.push_back(GemmSeg{nullptr, A.d + so_, (*boff)[q] + v * sa, 0, D, Dr, D, 0, 0, A0, 0, scale});
-            }
+            // out_v = X_v A   (A fixed, X batched)
+            const SiteTensor& A = *(const SiteTensor*)fixed;
+            g.push_back(GemmSeg{nullptr, A.d + so_, (*boff)[q] + v * sa, 0, D, Dr, D, 0, 0, A0, 0, scale});
           }
       }
     }
@@ -3923,9 +3935,10 @@ struct TdaRunner {
     bond_batch(c, i + 1, X, nv);
     run_bop(bop(K_LC, i, nv, false, 1.0, &A, 0, B.stride, X.stride, &X.off), nullptr, B.buf.p, X.buf.p);
   }
-  // out_v (+)= s A_v X (X fixed on bond i+1)
-  void b_rmul(int i, const SiteBatch& A, int nv, const BondMat& X, SiteBatch& out, bool acc, double s = 1.0) {
-    run_bop(bop(K_RMUL, i, nv, acc, s, &X, A.stride, 0, out.stride, nullptr), A.buf.p, nullptr, out.buf.p);
+  // out_v (+)= A_v diag(w) (w on bond i+1)
+  void b_rmul(int i, const SiteBatch& A, int nv, const DevArray<double>& w, SiteBatch& out, bool acc) {
+    launch_diag_scale(A.buf.p, A.stride, w.p, rstate[i].p, nv, T(i), out.buf.p, out.stride, acc, c->st);
+    CK(cudaGetLastError());
   }
   // out_v (+)= s A X_v (A a fixed site-i tensor, X batched on bond i+1)
   void b_rmulb(int i, const SiteTensor& A, const BondBatch& X, int nv, SiteBatch& out, bool acc, double s = 1.0) {
@@ -3936,9 +3949,10 @@ struct TdaRunner {
     bond_batch(c, i, X, nv);
     run_bop(bop(K_RC, i, nv, false, 1.0, &B, A.stride, 0, X.stride, &X.off), A.buf.p, nullptr, X.buf.p);
   }
-  // out_v (+)= s X A_v (X fixed on bond i)
-  void b_lmul(int i, const BondMat& X, const SiteBatch& A, int nv, SiteBatch& out, bool acc, double s = 1.0) {
-    run_bop(bop(K_LMUL, i, nv, acc, s, &X, 0, A.stride, out.stride, nullptr), nullptr, A.buf.p, out.buf.p);
+  // out_v (+)= diag(w) A_v (w on bond i)
+  void b_lmul(int i, const DevArray<double>& w, const SiteBatch& A, int nv, SiteBatch& out, bool acc) {
+    launch_diag_scale(A.buf.p, A.stride, w.p, lstate[i].p, nv, T(i), out.buf.p, out.stride, acc, c->st);
+    CK(cudaGetLastError());
   }
   // out_v (+)= s X_v A (X batched on bond i, A a fixed site-i tensor)
   void b_lmulb(int i, const BondBatch& X, int nv, const SiteTensor& A, SiteBatch& out, bool acc, double s = 1.0) {
@@ -5531,18 +5545,7 @@ static void tda_prepare_impl(lrt_ctx* c, double* norm_out) {
         CK(cudaGetLastError());
         CK(cudaStreamSynchronize(st));
       }
-      // X_q = diag(lambda_q) VT_q
-      std::vector<GemmOut> o;
-      std::vector<GemmSeg> g;
-      BondMat Lm, Lmi;
-      lam_mats(c, i + 1, lam, 0.0, Lm, Lmi);
-      for (int q = 0; q < Rb.n(); ++q) {
-        const int D = Rb.d[q];
-        if (D == 0) continue;
-        o.push_back(GemmOut{X.buf.p + X.off[q], 0, D, D, D, (int)g.size(), 1, 0, 0});
-        g.push_back(GemmSeg{Lm.buf.p + Lm.off[q], VT.buf.p + VT.off[q], 0, 0, D, D, D, 0, 0, 0, 0, 1.0});
-      }
-      run_gemms(c, o, g);
+      scale_bond(c, i + 1, VT, lam, true, X);   // X_q = diag(lambda_q) VT_q
     }
   }
   c->sites = std::move(L0);

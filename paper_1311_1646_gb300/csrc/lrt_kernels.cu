@@ -774,6 +774,26 @@ void launch_rank1_batch(const double* w, int64_t ldw, const double* coef, double
   rank1_batch_kernel<<<dim3(vec_grid(n), nv), 256, 0, st>>>(w, ldw, coef, alpha, nv, V, ld, n);
 }
 
+// Products with diagonal matrices (Schmidt values, their inverses): one multiplication per
+// element, rounded once, however far the values span.  (As D x D products they cost D / 2 times
+// the operations of this bandwidth-bound pass.)
+__global__ void __launch_bounds__(256) diag_scale_kernel(const double* __restrict__ A, int64_t lda,
+                                                         const double* __restrict__ w, const int* __restrict__ state,
+                                                         int64_t n, double* __restrict__ out, int64_t ldo, bool acc) {
+  const double* a = A + (int64_t)blockIdx.y * lda;
+  double* o = out + (int64_t)blockIdx.y * ldo;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+    const double x = __dmul_rn(a[e], w[state[e]]);
+    o[e] = acc ? __dadd_rn(o[e], x) : x;
+  }
+}
+
+void launch_diag_scale(const double* A, int64_t lda, const double* w, const int* state, int nv, int64_t n, double* out,
+                       int64_t ldo, bool acc, cudaStream_t st) {
+  if (nv <= 0 || n <= 0) return;
+  diag_scale_kernel<<<dim3(vec_grid(n), nv), 256, 0, st>>>(A, lda, w, state, n, out, ldo, acc);
+}
+
 // one thread per element and up to ROT_MU outputs at a time: every old vector is read once
 // per group of ROT_MU new vectors
 constexpr int ROT_MU = 16;

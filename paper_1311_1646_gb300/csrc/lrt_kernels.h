@@ -324,6 +324,10 @@ void launch_pair_dots(const double* const* A, const double* const* B, int na, in
 // out = beta out + sign sum_j coef[j] V_j (coef on the device, sign +-1)
 void launch_lincomb(const double* V, int64_t ld, int m, const double* coef, int64_t n, double* out, double beta,
                     cudaStream_t st, double sign = 1.0);
+// out_v (+)= A_v times, element by element, w[state[e]]: products with the diagonal matrix of a
+// bond's Schmidt values (vectors lda, ldo apart)
+void launch_diag_scale(const double* A, int64_t lda, const double* w, const int* state, int nv, int64_t n, double* out,
+                       int64_t ldo, bool acc, cudaStream_t st);
 constexpr double DAV_MIN_NORM = 1e-14;   // a Davidson direction shorter than this ends the iteration
 // v = t / |t|, t2 = |t|^2 on the device; zero below DAV_MIN_NORM
 void launch_dav_unit(const double* t, const double* t2, int64_t n, double* v, cudaStream_t st);
