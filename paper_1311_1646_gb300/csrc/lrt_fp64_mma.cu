@@ -28,8 +28,8 @@
 // less than the 32 roundings of an FMA chain where the products of the row and column are of
 // one size, and more where all of them are far below the two largest elements: sums of small
 // products are not as accurate by themselves as an FMA chain's.  Elements whose row or column
-// holds an infinity, a NaN or lies outside 2^-423 .. 2^477 are multiplied in plain FP64 from the
-// staged operands.
+// holds an infinity, a NaN, subnormals alone or lies outside 2^-423 .. 2^477 are multiplied in
+// plain FP64 from the staged operands.
 //
 // Measured on the k = 24, M = 500, 6-vector sigma (23.7 G multiply-adds): 44.0 ms by FP64 FMAs,
 // 15.2 ms here; error against 64-bit exact values 3.9e-16 (7.1e-16 before) at k = 8, 2.9e-15
@@ -53,6 +53,7 @@ constexpr int MMA_WARPS = 8;              // warps of a CTA tile
 constexpr int MMA_EMIN = 600, MMA_EMAX = 1500;   // exponent fields the integer path takes
 constexpr int MMA_E0 = 1023;
 constexpr int MMA_NOBAL = -4096;                  // exponent of a K position where that operand is zero
+constexpr int MMA_NONE = -1100;                   // largest exponents of rows up to here: no product but zeros
 constexpr int MMA_WILD = (int)0x80000000;        // exponent word of a row the integer path does not take
 
 struct MmaSmem {
@@ -145,14 +146,18 @@ __device__ __forceinline__ void exponents(const Quad& q, int (&e)[4], int& emax)
   for (int j = 0; j < 4; ++j) e[j] = (int)((q.hi[j] & 0x7FFFFFFFu) >> 20);
   emax = max(max(e[0], e[1]), max(e[2], e[3]));
 }
-// digits of a row's four positions, the row's exponent taken over its 8 lanes (e: 0 for a
+// rows the integer path does not take, by their largest exponent (a subnormal's is 0 before the
+// K positions' exponents, a zero's -4096 after them)
+__device__ __forceinline__ bool outside_range(int emax) { return emax > MMA_NONE && (emax < MMA_EMIN || emax > MMA_EMAX); }
+__device__ __forceinline__ bool is_zero(uint32_t hi, uint32_t lo) { return ((hi & 0x7FFFFFFFu) | lo) == 0; }
+// digits of a row's four positions, the row's exponent taken over its 8 lanes (e: -4096 for a
 // zero).  Returns the row's exponent word, MMA_WILD when it needs the FP64 path.
 __device__ __forceinline__ int cut_row(const Quad& q, const int (&e)[4], int emax, uint32_t (&d0)[MMA_ND],
                                        uint32_t (&d1)[MMA_ND]) {
   emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 1));
   emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 2));
   emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 4));
-  const bool wild = emax > 0 && (emax < MMA_EMIN || emax > MMA_EMAX);
+  const bool wild = outside_range(emax);
   const int E = emax > 0 ? emax : MMA_E0;   // a zero row: every element shifts out
   uint2 f[4];
 #pragma unroll
@@ -388,7 +393,7 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
         const int bj[4] = {bk.x, bk.y, bk.z, bk.w};
         const bool inf = own ? max(max(bk.x, bk.y), max(bk.z, bk.w)) == 2047 - MMA_E0 : emax == 2047;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) e[j] = e[j] == 0 ? -4096 : own ? e[j] - bj[j] : e[j] + bj[j];
+        for (int j = 0; j < 4; ++j) e[j] = is_zero(q.hi[j], q.lo[j]) ? -4096 : own ? e[j] - bj[j] : e[j] + bj[j];
         emax = inf ? 4095 : max(max(e[0], e[1]), max(e[2], e[3]));
         uint32_t d0[MMA_ND], d1[MMA_ND];
         const int x = cut_row(q, e, emax, d0, d1);
@@ -676,7 +681,6 @@ __device__ __forceinline__ int row_exponent(const int (&e)[4]) {
   m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
   return max(m, __shfl_xor_sync(0xffffffffu, m, 2));
 }
-__device__ __forceinline__ bool outside_range(int emax) { return emax > 0 && (emax < MMA_EMIN || emax > MMA_EMAX); }
 __device__ __forceinline__ int exponent_of(double x) { return (__double2hiint(x) & 0x7FFFFFFF) >> 20; }
 // fragments of four positions (2t, 2t + 1, 2t + 8, 2t + 9) of one row
 __device__ __forceinline__ void cut_quad(const double (&x)[4], const int (&e)[4], int E, uint32_t (&lo)[MMA_ND],
@@ -834,8 +838,8 @@ __device__ __forceinline__ void warp_tile(const GemmOut* __restrict__ outs, cons
           all |= m == 2047;
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
-            ea[h][j] = ea[h][j] == 0 ? -4096 : ea[h][j] == 2047 ? 4095 : ea[h][j] + da;
-            eb[h][j] = eb[h][j] == 0 ? -4096 : eb[h][j] == 2047 ? 4095 : eb[h][j] - da;
+            ea[h][j] = is_zero(__double2hiint(a[h][j]), __double2loint(a[h][j])) ? -4096 : ea[h][j] == 2047 ? 4095 : ea[h][j] + da;
+            eb[h][j] = is_zero(__double2hiint(b[h][j]), __double2loint(b[h][j])) ? -4096 : eb[h][j] == 2047 ? 4095 : eb[h][j] - da;
           }
         }
         all = __any_sync(0xffffffffu, all);

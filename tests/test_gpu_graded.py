@@ -127,3 +127,36 @@ def test_sigma_in_a_graded_gauge(pkg, k, na, nb, M, i, nsite, side, kernel):
         out.append(y.cpu().numpy())
         ctx.close()
     assert np.abs(out[1] - out[0]).max() <= 1e-12 * np.abs(out[0]).max()
+
+
+@pytest.mark.parametrize("kernel", [2, 3])
+def test_subnormal_vectors_are_multiplied(pkg, kernel):
+    """A vector of subnormals only (46 bits and fewer) under a Hamiltonian of exponent 2^400: the
+    result is a normal number of about 40 bits, as from the FMA tiles (1e-11: the rounding of
+    subnormal intermediates to multiples of 2^-1074, a few of 2^-46 each)."""
+    k, na, nb, M, i = 10, 2, 2, 60, 4
+    H = synth.ab_initio(k, na, nb, 7)
+    m = synth.mixed_mps(k, na, nb, M, 8, center=i)
+    out = []
+    for kn in (KERNEL_FP64, kernel):
+        ctx = pkg.Context(0)
+        ctx.set_kernels(kn)
+        ctx.op_build(k, H.h * 2.0 ** 400, H.eri * 2.0 ** 400)
+        ctx.mps_load(k, na, nb, m.bonds, m.sites, i)
+        for b in range(i):
+            ctx.renormalize(b, +1)
+        for b in range(k - 1, i, -1):
+            ctx.renormalize(b, -1)
+        n, _ = ctx.wfn_layout(i, 1)
+        x = synth.random_vector(2 * n, 9)
+        x[:n] = np.round(x[:n] / np.abs(x[:n]).max() * 2.0 ** 46) * 2.0 ** -1000 * 2.0 ** -74
+        assert np.abs(x[:n]).max() < 2.0 ** -1022 and np.any(x[:n] != 0.0)
+        xd = torch.tensor(x, dtype=torch.float64, device="cuda:0")
+        y = torch.empty_like(xd)
+        ctx.sigma(i, 1, xd, y, nvec=2)
+        torch.cuda.synchronize()
+        out.append(y.cpu().numpy())
+        ctx.close()
+    for v in (slice(0, n), slice(n, 2 * n)):
+        assert np.abs(out[0][v]).max() > 0.0
+        assert np.abs(out[1][v] - out[0][v]).max() <= (1e-11 if v.start == 0 else 1e-12) * np.abs(out[0][v]).max()
