@@ -270,7 +270,7 @@ __device__ __forceinline__ void gemm_mma_tile(const GemmSeg* __restrict__ segs, 
         GemmSeg g = segs[o.seg_begin + b0 + lane];
         if (g.a_rel) g.A = (g.a_rel == 1 ? xbase : g.a_rel == 2 ? tbase : extra(g.a_rel - 3)) + g.a_off;
         if (g.b_rel) g.B = (g.b_rel == 1 ? xbase : g.b_rel == 2 ? tbase : extra(g.b_rel - 3)) + g.b_off;
-        S.sd[lane] = SegS{g.A, g.B, g.lda, g.ldb, g.transA, g.transB, g.scale, g.a_vr, g.b_vc, g.a_vs, g.b_vs};
+        S.sd[lane] = SegS{g.A, g.B, g.lda, g.ldb, g.transA, g.transB, g.scale, o.c_vr, o.c_vc, g.a_vs, g.b_vs};
         k = g.k;
       }
       int incl = k;

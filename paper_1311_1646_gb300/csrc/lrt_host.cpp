@@ -731,7 +731,7 @@ struct KernelChoice {
 
 struct GemmPlan {
   DevArray<GemmOut> outs;    // the plan's outputs, then the K parts of split tiles
-  DevArray<GemmSeg> segs;
+  std::shared_ptr<DevArray<GemmSeg>> segs;   // plans of one position share them, whatever their vectors
   DevArray<int3> tiles;      // FP64 kernel tiles
   int ntiles = 0;
   int nbase = 0;             // outputs before the K parts
@@ -746,13 +746,13 @@ struct GemmPlan {
     count();
     switch (kind) {
       case GemmKind::WARP:
-        launch_gemm_warp(outs.p, segs.p, tiles.p, ntiles, xb, yb, tb, st, nullptr, ex, ws.p, splits.p, counters.p);
+        launch_gemm_warp(outs.p, segs->p, tiles.p, ntiles, xb, yb, tb, st, nullptr, ex, ws.p, splits.p, counters.p);
         return;
       case GemmKind::MMA:
-        launch_gemm_mma(outs.p, segs.p, tiles.p, ntiles, xb, yb, tb, st, nullptr, ex, ws.p);
+        launch_gemm_mma(outs.p, segs->p, tiles.p, ntiles, xb, yb, tb, st, nullptr, ex, ws.p);
         break;
       case GemmKind::FP64:
-        launch_gemm_fp64(outs.p, segs.p, tiles.p, ntiles, xb, yb, tb, st, ex, ws.p);
+        launch_gemm_fp64(outs.p, segs->p, tiles.p, ntiles, xb, yb, tb, st, ex, ws.p);
         break;
     }
     if (nsplit > 0) launch_split_reduce(outs.p, splits.p, nsplit, ws.p, yb, tb, st);
@@ -763,22 +763,22 @@ struct GemmPlan {
   void run_inst(cudaStream_t st, const GemmInstSet& B, int n) const {
     count();
     switch (kind) {
-      case GemmKind::WARP: launch_gemm_warp_inst(outs.p, segs.p, tiles.p, ntiles, B, n, st); break;
-      case GemmKind::MMA: launch_gemm_mma_inst(outs.p, segs.p, tiles.p, ntiles, B, n, st); break;
-      case GemmKind::FP64: launch_gemm_fp64_inst(outs.p, segs.p, tiles.p, ntiles, B, n, st); break;
+      case GemmKind::WARP: launch_gemm_warp_inst(outs.p, segs->p, tiles.p, ntiles, B, n, st); break;
+      case GemmKind::MMA: launch_gemm_mma_inst(outs.p, segs->p, tiles.p, ntiles, B, n, st); break;
+      case GemmKind::FP64: launch_gemm_fp64_inst(outs.p, segs->p, tiles.p, ntiles, B, n, st); break;
     }
   }
   void run_multi(cudaStream_t st, const GemmBases* bases) const {
     switch (kind) {
       case GemmKind::WARP:
-        launch_gemm_warp(outs.p, segs.p, tiles.p, ntiles, nullptr, nullptr, nullptr, st, bases, nullptr, ws.p,
+        launch_gemm_warp(outs.p, segs->p, tiles.p, ntiles, nullptr, nullptr, nullptr, st, bases, nullptr, ws.p,
                          splits.p, counters.p);
         break;
       case GemmKind::MMA:
-        launch_gemm_mma(outs.p, segs.p, tiles.p, ntiles, nullptr, nullptr, nullptr, st, bases, nullptr, nullptr);
+        launch_gemm_mma(outs.p, segs->p, tiles.p, ntiles, nullptr, nullptr, nullptr, st, bases, nullptr, nullptr);
         break;
       case GemmKind::FP64:
-        launch_gemm_fp64_multi(outs.p, segs.p, tiles.p, ntiles, bases, st);
+        launch_gemm_fp64_multi(outs.p, segs->p, tiles.p, ntiles, bases, st);
         break;
     }
   }
@@ -841,9 +841,10 @@ static GemmKind gemm_kind(const std::vector<GemmOut>& outs, const std::vector<Ge
     const GemmOut& o = outs[i];
     for (int q = 0; q < o.seg_count; ++q) {
       const GemmSeg& g = segs[o.seg_begin + q];
-      // one vector block per output, and 32-bit byte strides, are what those kernels take
-      if (g.a_vr != o.c_vr || g.b_vc != o.c_vc) return GemmKind::FP64;
-      if (std::max(g.a_vs, g.b_vs) >= ((int64_t)1 << 29) || std::max(g.lda, g.ldb) >= (1 << 28)) return GemmKind::FP64;
+      // 32-bit byte strides are what those kernels take
+      if ((o.c_vr > 0 && g.a_vs >= (int64_t)1 << 29) || (o.c_vc > 0 && g.b_vs >= (int64_t)1 << 29) ||
+          std::max(g.lda, g.ldb) >= (1 << 28))
+        return GemmKind::FP64;
     }
     const int m = o.c_vr > 0 ? o.c_vr : o.m, n = o.c_vc > 0 ? o.c_vc : o.n;
     exact += (double)m * n * ktot[i];
@@ -883,7 +884,8 @@ static void warp_tile_shape(GemmOut& O, int64_t k, bool digits, int& tm, int& tn
 // which the reduction launch does not know)
 enum class GemmSplit { NEVER, WARP, ALWAYS };
 
-// outs is worked on in place: the parts of split tiles are appended
+// outs is worked on in place: the parts of split tiles are appended.  P.segs: the segments where
+// they are on the device already.
 static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vector<GemmSeg>& segs,
                        cudaStream_t st, KernelChoice& choice, GemmMath math = GemmMath::FMA,
                        GemmSplit split = GemmSplit::NEVER) {
@@ -963,7 +965,6 @@ static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vecto
             po.c_off = wsz + (int64_t)t.nparts * mt * nt - ((int64_t)m0 * nt + n0);
             po.ldc = nt;
             po.accumulate = 0;
-            if (kind == GemmKind::FP64) po.c_vr = po.c_vc = 0;   // the others read their operands' blocks here
             po.split = (int)sp.size();
             po.c_vs = 0;
             po.seg_begin = O.seg_begin + sb;
@@ -1001,7 +1002,10 @@ static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vecto
   std::vector<int3> tiles(tl.size());
   for (size_t t = 0; t < tl.size(); ++t) tiles[at[511 - key[t]]++] = tl[t].second;
   P.outs.upload(outs, st);
-  P.segs.upload(segs, st);
+  if (!P.segs) {
+    P.segs = std::make_shared<DevArray<GemmSeg>>();
+    P.segs->upload(segs, st);
+  }
   P.tiles.upload(tiles, st);
   P.ntiles = (int)tiles.size();
   P.nbase = (int)nout;
@@ -1152,34 +1156,43 @@ struct Prod2 {                    // a phase-2 product
 constexpr size_t PLAN_SCRATCH_BYTES = (size_t)256 << 20;
 struct PlanScratch {
   std::vector<Prod2> prod2;
-  std::vector<GemmOut> o1;
+  std::vector<GemmOut> o1, o2;
   std::vector<GemmSeg> s1, s2;
   std::vector<char> s1rev;
+  uint64_t lists = 0;      // SigmaPlan::lists of the plan these lists are of (0: of none)
   void clear() {
+    lists = 0;
     prod2.clear();
     o1.clear();
+    o2.clear();
     s1.clear();
     s2.clear();
     s1rev.clear();
   }
   void trim() {
-    if (prod2.capacity() * sizeof(Prod2) + o1.capacity() * sizeof(GemmOut) +
+    if (prod2.capacity() * sizeof(Prod2) + (o1.capacity() + o2.capacity()) * sizeof(GemmOut) +
             (s1.capacity() + s2.capacity()) * sizeof(GemmSeg) + s1rev.capacity() > PLAN_SCRATCH_BYTES)
       *this = PlanScratch();
   }
 };
 
+struct DiagList {
+  DevArray<DiagOut> outs;
+  DevArray<DiagTerm> terms;
+  int n = 0;
+  void run(double* d, cudaStream_t st) const { launch_diag(outs.p, terms.p, n, d, st); }
+};
+
 struct SigmaPlan {
   uint64_t serial = 0;      // unique per plan (batched launches detect rebuilt plans by it)
+  uint64_t lists = 0;       // serial of the plan its lists were written for (see plan_vectors)
   bool has_tc = false;      // the tensor-core twin was planned
-  bool diag_used = false;   // heff_diag was answered from this plan
+  int nvec = 1;
   GemmPlan p1, p2;
   // operator sets of a plan built with relative addresses (X, Xrev, Y, Yrev at extra
   // bases 0..3); a kept plan serves new sets of the same layout by changing these
   GemmExtra ex{};
-  DevArray<DiagOut> douts;
-  DevArray<DiagTerm> dterms;
-  int ndiag = 0;
+  std::shared_ptr<DiagList> diag;
   double* tbuf = nullptr;   // workspace of the phase-1 intermediates
   int64_t tsize = 0;        // its size in doubles
   int64_t nelem = 0;
@@ -1840,6 +1853,34 @@ static uint16_t transpose_mask(uint16_t m) {
   return r;
 }
 
+static std::atomic<uint64_t> next_serial{0};   // plans are built from several threads in sweep_tda_batched
+
+// The vectors of a call share every operator block: phase 1 (T = X x) places them side by
+// side along the columns of one output (x's block of vector v at + v * nelem, T of vector v
+// at + v * toff), phase 2 (y = sum T Y^T) stacks them along the rows (the T or x rows of
+// vector v at + v * toff or + v * nelem, y of vector v at + v * nelem).  One output then
+// holds the same block product for every vector, which fills the GEMM's tiles.  o1, o2: the
+// n1, n2 outputs of the phases for any number of vectors (K parts behind them), set to nvec.
+static void set_vectors(std::vector<GemmOut>& o1, size_t n1, std::vector<GemmOut>& o2, size_t n2, int nvec,
+                        int64_t nelem, int64_t toff) {
+  o1.resize(n1);
+  o2.resize(n2);
+  for (GemmOut& y : o1) {
+    const int n = y.c_vc > 0 ? y.c_vc : y.n;
+    y.c_rel = 2;
+    y.balance_rows = 1;   // not by the columns, which hold the vectors
+    y.n = n * nvec;
+    y.c_vc = nvec > 1 ? n : 0;
+    y.c_vs = nvec > 1 ? toff : 0;
+  }
+  for (GemmOut& y : o2) {
+    const int m = y.c_vr > 0 ? y.c_vr : y.m;
+    y.m = m * nvec;
+    y.c_vr = nvec > 1 ? m : 0;
+    y.c_vs = nvec > 1 ? nelem : 0;
+  }
+}
+
 // Products are formed at sub-block granularity so that zero sub-blocks of the
 // enlarged operators are never multiplied:
 //   phase 1: T[t](rows n') = sum_{n : X_t(n',n) != 0} X_t(n',n) psi_Q(rows n)
@@ -1849,7 +1890,7 @@ static uint16_t transpose_mask(uint16_t m) {
 // sets of first-order (transition) operator sets, read by transposed references.
 static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, const OpSet* Xrev, const OpSet& Y,
                                                   const OpSet* Yrev, int site, int nsite, int nvec, bool tc = true,
-                                                  bool rel_ops = false, bool diag_only = false) {
+                                                  bool rel_ops = false) {
   if (rel_ops && tc) throw Error(LRT_EINVAL, "internal: relative operator addresses are FP64 only");
   const Ints& I = c->I;
   const int k = c->k;
@@ -1876,8 +1917,8 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
   if (I.e_core != 0.0) terms.push_back({I.e_core, {KI, -1, -1, 0}, {KI, -1, -1, 0}});
 
   auto plan = std::make_unique<SigmaPlan>();
-  static std::atomic<uint64_t> next_serial{0};   // plans are built from several threads in sweep_tda_batched
-  plan->serial = ++next_serial;
+  plan->serial = plan->lists = ++next_serial;
+  plan->nvec = nvec;
   plan->nelem = nelem;
   plan->n_terms = (int)terms.size();
 
@@ -1979,7 +2020,6 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
             d.scale = sc;
             dterm[ik].push_back(d);
           }
-          if (diag_only) continue;
 
           // ---- phase 1 (shared by every Y partner of this X block)
           uint16_t rows = 0;
@@ -2093,7 +2133,7 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
   }
   if (toff > 0 && dev_alloc((void**)&plan->tbuf, (size_t)toff * nvec * sizeof(double)) != cudaSuccess)
     throw Error(LRT_ENOMEM, "sigma workspace");
-  std::vector<GemmOut> O2;
+  std::vector<GemmOut>& O2 = W.o2;
   std::vector<GemmSeg>& S2 = W.s2;
   plan->tsize = toff * nvec;
   // operator pointers as offsets from the set they live in (extra bases 0..3)
@@ -2106,26 +2146,6 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
       s1[q].a_off = s1[q].A - plan->ex.p[s1rev[q]];
       s1[q].A = nullptr;
       s1[q].a_rel = 3 + s1rev[q];
-    }
-  }
-  // The vectors of a call share every operator block: phase 1 (T = X x) places them side by
-  // side along the columns of one output (x's block of vector v at + v * nelem, T of vector v
-  // at + v * toff), phase 2 (y = sum T Y^T) stacks them along the rows (the T or x rows of
-  // vector v at + v * toff or + v * nelem, y of vector v at + v * nelem).  One output then
-  // holds the same block product for every vector, which fills the GEMM's tiles.
-  const bool vb = nvec > 1;
-  for (GemmOut& y : o1) {
-    y.c_rel = 2;
-    y.balance_rows = 1;   // not by the columns, which hold the vectors
-    if (vb) {
-      const int n = y.n;
-      for (int q = 0; q < y.seg_count; ++q) {
-        s1[y.seg_begin + q].b_vc = n;
-        s1[y.seg_begin + q].b_vs = nelem;
-      }
-      y.n = n * nvec;
-      y.c_vc = n;
-      y.c_vs = toff;
     }
   }
   std::vector<int> at(osub.size() + 1, 0);   // first product of every output
@@ -2142,13 +2162,7 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
       coff += YF->off[fy][os.mcol];
       ncols = YF->dim[fy][os.mcol];
     }
-    const int m1 = XF.dim[fx][os.r];
-    GemmOut y{nullptr, coff, w.cols, m1 * nvec, ncols, at[u], at[u + 1] - at[u], 0, 1};
-    if (vb) {
-      y.c_vr = m1;
-      y.c_vs = nelem;
-    }
-    O2.push_back(y);
+    O2.push_back(GemmOut{nullptr, coff, w.cols, XF.dim[fx][os.r], ncols, at[u], at[u + 1] - at[u], 0, 1});
   }
   S2.resize(prod2.size());
   for (const Prod2& p : prod2) {
@@ -2166,15 +2180,14 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
     } else {
       g.B = p.B;
     }
-    if (vb) {
-      g.a_vr = O2[p.out].c_vr;
-      g.a_vs = p.ident ? nelem : toff;
-    }
+    g.a_vs = p.ident ? nelem : toff;
   }
+  for (GemmSeg& g : s1) g.b_vs = nelem;
+  set_vectors(o1, o1.size(), O2, O2.size(), nvec, nelem, toff);
   // kept relative plans (first-order sets) are replayed over instances
   const GemmMath math = rel_ops ? GemmMath::FMA : GemmMath::DIGITS;
-  if (!diag_only) build_gemm(plan->p1, o1, s1, c->st, c->kernels, math);
-  if (!diag_only) build_gemm(plan->p2, O2, S2, c->st, c->kernels, math, rel_ops ? GemmSplit::NEVER : GemmSplit::ALWAYS);
+  build_gemm(plan->p1, o1, s1, c->st, c->kernels, math);
+  build_gemm(plan->p2, O2, S2, c->st, c->kernels, math, rel_ops ? GemmSplit::NEVER : GemmSplit::ALWAYS);
   // tensor-core twin: phase-2 outputs, one per (y block, column group)
   plan->has_tc = tc;
   for (size_t w = 0; w < wb.size() && tc; ++w)
@@ -2199,18 +2212,52 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
     dout.push_back(DiagOut{wb[w].off, wb[w].rows, wb[w].cols, (int)dts.size(), (int)dterm[w].size()});
     dts.insert(dts.end(), dterm[w].begin(), dterm[w].end());
   }
-  plan->douts.upload(dout, c->st);
-  plan->dterms.upload(dts, c->st);
-  plan->ndiag = (int)dout.size();
+  plan->diag = std::make_shared<DiagList>();
+  plan->diag->outs.upload(dout, c->st);
+  plan->diag->terms.upload(dts, c->st);
+  plan->diag->n = (int)dout.size();
   plan->n_products = nprod;
   plan->op_bytes = op_bytes;
   plan->flops_alg = falg * nvec;
   CK(cudaStreamSynchronize(c->st));
+  if (!rel_ops) W.lists = plan->lists;
   W.trim();
   return plan;
 }
 
-static std::unique_ptr<SigmaPlan> plan_sigma(lrt_ctx* c, int site, int nsite, int nvec, bool tc, bool diag_only = false) {
+// The FP64 plan of a position for another number of vectors, from the lists of plan P while the
+// scratch still holds them: P's segments and diagonal, and outputs, tiles and a workspace of its
+// own (null when the lists are gone).  Walking the terms again and writing and uploading the
+// segments is most of a plan: heff_diag and then sigma of 4 vectors at k = 16, M = 384: 37 ms
+// for two whole plans, PLACEHOLDER.
+static std::unique_ptr<SigmaPlan> plan_vectors(lrt_ctx* c, const SigmaPlan& P, int nvec) {
+  PlanScratch& W = c->scratch;
+  if (W.lists == 0 || W.lists != P.lists) return nullptr;
+  auto plan = std::make_unique<SigmaPlan>();
+  plan->serial = ++next_serial;
+  plan->lists = P.lists;
+  plan->nvec = nvec;
+  plan->diag = P.diag;
+  plan->nelem = P.nelem;
+  plan->n_terms = P.n_terms;
+  plan->n_products = P.n_products;
+  plan->op_bytes = P.op_bytes;
+  plan->flops_alg = P.flops_alg / P.nvec * nvec;
+  plan->macs1 = P.macs1;
+  const int64_t toff = P.tsize / P.nvec;
+  plan->tsize = toff * nvec;
+  if (toff > 0 && dev_alloc((void**)&plan->tbuf, (size_t)plan->tsize * sizeof(double)) != cudaSuccess)
+    throw Error(LRT_ENOMEM, "sigma workspace");
+  plan->p1.segs = P.p1.segs;
+  plan->p2.segs = P.p2.segs;
+  set_vectors(W.o1, (size_t)P.p1.nbase, W.o2, (size_t)P.p2.nbase, nvec, P.nelem, toff);
+  build_gemm(plan->p1, W.o1, W.s1, c->st, c->kernels, GemmMath::DIGITS);
+  build_gemm(plan->p2, W.o2, W.s2, c->st, c->kernels, GemmMath::DIGITS, GemmSplit::ALWAYS);
+  CK(cudaStreamSynchronize(c->st));
+  return plan;
+}
+
+static std::unique_ptr<SigmaPlan> plan_sigma(lrt_ctx* c, int site, int nsite, int nvec, bool tc) {
   OpSet& X = enlarged(c, site, false);
   OpSet* Yp;
   if (nsite == 1) {
@@ -2219,7 +2266,7 @@ static std::unique_ptr<SigmaPlan> plan_sigma(lrt_ctx* c, int site, int nsite, in
   } else {
     Yp = &enlarged(c, site + 1, true);
   }
-  return plan_sigma_sets(c, X, nullptr, *Yp, nullptr, site, nsite, nvec, tc, false, diag_only);
+  return plan_sigma_sets(c, X, nullptr, *Yp, nullptr, site, nsite, nvec, tc);
 }
 
 // Work stream of one tensor-core launch over one or several plans (instances): tiles
@@ -2747,41 +2794,19 @@ static SigmaPlan* any_plan(lrt_ctx* c, int site, int nsite) {
                                                                                                   : nullptr;
 }
 
-// the diagonal of (site, nsite), which any plan of the position holds; without one, a plan of the
-// diagonal alone (kept as nvec 0)
-static SigmaPlan& get_diag_plan(lrt_ctx* c, int site, int nsite) {
-  if (SigmaPlan* p = any_plan(c, site, nsite)) return *p;
-  auto p = plan_sigma(c, site, nsite, 1, false, true);
-  SigmaPlan& ref = *p;
-  c->plans[std::make_tuple(site, nsite, 0)] = std::move(p);
-  return ref;
-}
-
 // the plan of (site, nsite, nvec); tc: with the tensor-core twin (replanned if missing)
 static SigmaPlan& get_plan(lrt_ctx* c, int site, int nsite, int nvec, bool tc = false) {
   auto key = std::make_tuple(site, nsite, nvec);
   auto it = c->plans.find(key);
   if (it != c->plans.end() && (!tc || it->second->has_tc)) return *it->second;
-  auto p = plan_sigma(c, site, nsite, nvec, tc);
-  if (it != c->plans.end()) p->diag_used = it->second->diag_used;
+  std::unique_ptr<SigmaPlan> p;
+  for (auto q = c->plans.lower_bound(std::make_tuple(site, nsite, 0));
+       !p && !tc && q != c->plans.end() && std::get<0>(q->first) == site && std::get<1>(q->first) == nsite; ++q)
+    p = plan_vectors(c, *q->second, nvec);
+  if (!p) p = plan_sigma(c, site, nsite, nvec, tc);
   SigmaPlan& ref = *p;
   c->plans[key] = std::move(p);
   return ref;
-}
-
-// the single-vector plan of sigma_noalloc where none is kept: after heff_diag of the position,
-// which answers from any plan, it is made here (never while the stream is captured)
-static SigmaPlan* plan_after_diag(lrt_ctx* c, int site, int nsite) {
-  for (auto it = c->plans.lower_bound(std::make_tuple(site, nsite, 0));
-       it != c->plans.end() && std::get<0>(it->first) == site && std::get<1>(it->first) == nsite; ++it) {
-    if (!it->second->diag_used) continue;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(c->st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return nullptr;
-    CK(cudaSetDevice(c->dev));
-    PoolScope ps(&c->pool);
-    return &get_plan(c, site, nsite, 1);
-  }
-  return nullptr;
 }
 
 // LRT_MIXED calls that run on the FP64 kernels: the split-TF32 kernel fills one persistent CTA per
@@ -2873,7 +2898,7 @@ static double davidson_site(lrt_ctx* c, int i, int nsite, double* psi, const lrt
   double *t2 = Wd.p, *r2 = Wd.p + 1, *ev = Wd.p + 2;
   Zd.ensure(JACOBI_MAXN * JACOBI_MAXN);
   cudaStream_t st = c->st;
-  launch_diag(plan.douts.p, plan.dterms.p, plan.ndiag, diag.p, st);
+  plan.diag->run(diag.p, st);
   CK(cudaMemcpyAsync(t.p, psi, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
   int m = 0;
   double theta = 0.0;
@@ -3807,7 +3832,7 @@ struct TdaRunner {
       site_states(i);
       h0one[i] = plan_sigma_sets(c, *c->XL[i], nullptr, *c->R[i + 1], nullptr, i, 1, 1, false);
       diag[i].ensure(std::max<int64_t>(h0one[i]->nelem, 1));
-      launch_diag(h0one[i]->douts.p, h0one[i]->dterms.p, h0one[i]->ndiag, diag[i].p, c->st);
+      h0one[i]->diag->run(diag[i].p, c->st);
     }
     SiteTensor y = new_site(c, 0);
     run_plan(*h0one[0], C0(0).d, y.d, 1, false);    // the reference energy is FP64
@@ -5612,7 +5637,7 @@ static void merge_fp64(GemmPlan& out, const std::vector<SigmaPlan*>& plans, bool
     const GemmPlan& g = phase2 ? plans[j]->p2 : plans[j]->p1;
     std::vector<GemmOut> o = download(g.outs, st);
     o.resize(g.nbase);   // not the K parts of split tiles: the merged plan tiles anew
-    std::vector<GemmSeg> sg = download(g.segs, st);
+    std::vector<GemmSeg> sg = download(*g.segs, st);
     const int sb = (int)S.size();
     for (GemmOut x : o) {
       x.seg_begin += sb;
@@ -5815,7 +5840,6 @@ int sigma_launch_existing_plan(lrt_ctx* ctx, int site, int nsite, int nvec, cons
     if (nsite < 1 || nsite > 2 || site < 0 || nvec <= 0 || !x_dev || !y_dev || !workspace)
       throw Error(LRT_EINVAL, "sigma_noalloc: bad arguments");
     SigmaPlan* p = find_plan(ctx, site, nsite, nvec);
-    if (!p && nvec == 1) p = plan_after_diag(ctx, site, nsite);
     if (!p)
       throw Error(LRT_ESTATE, "sigma_noalloc: no prepared plan for this (site, nsite, nvec); call sigma() once "
                               "with the same arguments after the last renormalize()");
@@ -6040,9 +6064,8 @@ int heff_diag(lrt_t ctx, int site, int nsite, double* d_dev) {
     if (!ctx->have_mps || !ctx->have_ham) throw Error(LRT_ESTATE, "heff_diag: op_build and mps_load first");
     if (nsite < 1 || nsite > 2 || site < 0 || site + nsite > ctx->k || !d_dev) throw Error(LRT_EINVAL, "heff_diag: bad arguments");
     if (!ctx->L[site]) throw Error(LRT_ESTATE, "heff_diag: left block missing");
-    SigmaPlan& p = get_diag_plan(ctx, site, nsite);
-    p.diag_used = true;
-    launch_diag(p.douts.p, p.dterms.p, p.ndiag, d_dev, ctx->st);
+    SigmaPlan& p = get_plan(ctx, site, nsite, 1);
+    p.diag->run(d_dev, ctx->st);
     CK(cudaGetLastError());
   });
 }

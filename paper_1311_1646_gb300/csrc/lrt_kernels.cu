@@ -343,7 +343,7 @@ __device__ __forceinline__ void gemm_fp64_tile(const GemmOut* __restrict__ outs,
         GemmSeg g = segs[o.seg_begin + b0 + lane];
         if (g.a_rel) g.A = (g.a_rel == 1 ? xbase : g.a_rel == 2 ? tbase : extra(g.a_rel - 3)) + g.a_off;
         if (g.b_rel) g.B = (g.b_rel == 1 ? xbase : g.b_rel == 2 ? tbase : extra(g.b_rel - 3)) + g.b_off;
-        S.sd[lane] = SegS{g.A, g.B, g.lda, g.ldb, g.transA, g.transB, g.scale, g.a_vr, g.b_vc, g.a_vs, g.b_vs};
+        S.sd[lane] = SegS{g.A, g.B, g.lda, g.ldb, g.transA, g.transB, g.scale, o.c_vr, o.c_vc, g.a_vs, g.b_vs};
         k = g.k;
       }
       int incl = k;   // inclusive prefix of k over the lanes
@@ -412,7 +412,9 @@ __device__ __forceinline__ void gemm_fp64_tile(const GemmOut* __restrict__ outs,
     if (j >= cnt) break;
     int r = m0 + (int)(rc[j] >> 16), col = n0 + (int)(rc[j] & 0xFFFFu);
     double* c = cbase;
-    if (o.c_vr > 0) {            // row blocks of the vectors
+    if (o.c_rel == GEMM_C_SPLIT) {
+      // a part of a split tile is dense, whatever the output's vector blocks
+    } else if (o.c_vr > 0) {     // row blocks of the vectors
       const int v = r / o.c_vr;
       c += (int64_t)v * o.c_vs;
       r -= v * o.c_vr;

@@ -32,8 +32,8 @@ struct GatherSrc {
 // of the same layout.
 // Vector blocking (several trial vectors in one output): with c_vr > 0 the output's rows
 // come in blocks of c_vr, block v at C + v * c_vs; with c_vc > 0 its columns come in blocks
-// of c_vc, block v at C + v * c_vs.  A segment's A rows (a_vr, a_vs) and B columns (b_vc,
-// b_vs) are blocked the same way.  Zero: an ordinary dense operand.
+// of c_vc, block v at C + v * c_vs.  A segment's A rows then come in blocks of c_vr, a_vs
+// apart, its B columns in blocks of c_vc, b_vs apart.  Zero: ordinary dense operands.
 struct GemmOut {
   double* C;
   int64_t c_off;
@@ -60,7 +60,6 @@ struct GemmSeg {
   int transA, transB;
   int a_rel, b_rel;
   double scale;
-  int a_vr, b_vc;
   int64_t a_vs, b_vs;
 };
 
@@ -153,7 +152,7 @@ void launch_gemm_fp64(const GemmOut* outs, const GemmSeg* segs, const int3* tile
                       const GemmExtra* extra = nullptr, double* wbase = nullptr);
 // Tensor-core form of the FP64 GEMM (exact digit products, lrt_fp64_mma.cu): the same lists
 // with tiles of at most MMA_ROWS rows and columns together, both rounded up to 16, and 16
-// 16 x 16 units; the segments' vector blocks are the output's (a_vr = c_vr, b_vc = c_vc).
+// 16 x 16 units.
 constexpr int MMA_ROWS = 128;
 void launch_gemm_mma(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles, const double* xbase,
                      double* ybase, double* tbase, cudaStream_t st, const GemmBases* multi, const GemmExtra* extra,
