@@ -722,8 +722,34 @@ enum class GemmKind { FP64, MMA, WARP };
 // by Schmidt values later: with digit products in the tangent-space sweeps, the roots of one
 // sweep moved by 2e-9 (bonds damped to 1e-4) and 2e-8 (1e-6), with FMAs by 1e-14.
 enum class GemmMath { FMA, DIGITS };
+// Arrays that build_gemm works in, kept by the context so that their pages are touched once: a
+// position of k = 16, M = 384 has half a million tiles in its two plans.  At most
+// TILE_BUFFER_BYTES stay.
+constexpr size_t TILE_BUFFER_BYTES = (size_t)64 << 20;
+struct TileBuffers {
+  std::vector<int64_t> ktot;   // K of every output
+  std::vector<int> key;        // of every tile: its place in the order of costs
+  std::vector<int3> list;
+  void clear() {
+    key.clear();
+    list.clear();
+  }
+  void add(int64_t cost, int3 tile) {
+    // to within an eighth of an octave
+    const uint64_t c = (uint64_t)std::max<int64_t>(1, cost);
+    const int e = 63 - __builtin_clzll(c);
+    key.push_back(8 * e + (e >= 3 ? (int)(c >> (e - 3)) - 8 : 0));
+    list.push_back(tile);
+  }
+  void trim() {
+    if (ktot.capacity() * sizeof(int64_t) + key.capacity() * sizeof(int) +
+            list.capacity() * sizeof(int3) > TILE_BUFFER_BYTES)
+      *this = TileBuffers();
+  }
+};
 // a context's choice of kernels (test hook) and its launches of each: FP64, MMA, WARP, split TF32
 struct KernelChoice {
+  TileBuffers buf;
   int forced = 0;              // 0: by the rules; 1 + GemmKind: that kernel wherever it takes the list
   bool mixed_always = false;   // LRT_MIXED calls of any size run in split TF32
   int64_t launches[4] = {0, 0, 0, 0};
@@ -903,7 +929,10 @@ static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vecto
   // every slice stages the whole K range of B for a few rows; a K part stages only its
   // own range.)
   const size_t nout = outs.size();   // the parts of split tiles follow
-  std::vector<int64_t> ktot(nout, 0);
+  TileBuffers& buf = choice.buf;
+  buf.clear();
+  std::vector<int64_t>& ktot = buf.ktot;
+  ktot.assign(nout, 0);
   double fl = 0.0;
   for (size_t i = 0; i < nout; ++i) {
     for (int s = 0; s < outs[i].seg_count; ++s) ktot[i] += segs[outs[i].seg_begin + s].k;
@@ -933,10 +962,8 @@ static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vecto
         total += cost(std::min(TM, outs[i].m - m0), std::min(TN, outs[i].n - n0), ktot[i]);
   }
   const int64_t cap = std::max<int64_t>(1, total / gemm_fp64_slots());
-  std::vector<std::pair<int64_t, int3>> tl;
   std::vector<SplitTile> sp;
   int64_t wsz = 0;
-  tl.reserve(nout + nout / 4);
   for (size_t i = 0; i < nout; ++i) {
     int TM, TN;
     shape(outs[i], ktot[i], TM, TN);
@@ -970,7 +997,7 @@ static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vecto
             po.seg_begin = O.seg_begin + sb;
             po.seg_count = se - sb;
             outs.push_back(po);
-            tl.push_back({cost(mt, nt, kp), gemm_tile((int)outs.size() - 1, m0, mt, n0, nt)});
+            buf.add(cost(mt, nt, kp), gemm_tile((int)outs.size() - 1, m0, mt, n0, nt));
             ++t.nparts;
           });
           wsz += (int64_t)t.nparts * mt * nt;
@@ -980,27 +1007,21 @@ static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vecto
         const int parts = kind != GemmKind::FP64 ? 1 : (int)std::min<int64_t>(mt, (c + cap - 1) / cap);
         for (int p = 0, r = m0; p < parts; ++p) {
           const int rows = mt / parts + (p < mt % parts ? 1 : 0);
-          tl.push_back({cost(rows, nt, ktot[i]), gemm_tile((int)i, r, rows, n0, nt)});
+          buf.add(cost(rows, nt, ktot[i]), gemm_tile((int)i, r, rows, n0, nt));
           r += rows;
         }
       }
   }
-  // longest first, to within an eighth of an octave, otherwise in list order (a counting sort:
-  // lists have up to a million tiles)
-  auto bucket = [](int64_t c) {
-    int e = 0;
-    while ((c >> e) > 1) ++e;
-    return 8 * e + (e >= 3 ? (int)(c >> (e - 3)) - 8 : 0);
-  };
-  std::vector<int> at(8 * 64 + 1, 0), key(tl.size());
-  for (size_t t = 0; t < tl.size(); ++t) ++at[511 - (key[t] = bucket(std::max<int64_t>(1, tl[t].first)))];
+  // longest first, otherwise in list order (a counting sort: lists have up to a million tiles)
+  std::array<int, 513> at{};
+  for (int k : buf.key) ++at[511 - k];
   for (int b = 0, n = 0; b < 512; ++b) {
     const int k = at[b];
     at[b] = n;
     n += k;
   }
-  std::vector<int3> tiles(tl.size());
-  for (size_t t = 0; t < tl.size(); ++t) tiles[at[511 - key[t]]++] = tl[t].second;
+  std::vector<int3> tiles(buf.list.size());
+  for (size_t t = 0; t < tiles.size(); ++t) tiles[at[511 - buf.key[t]]++] = buf.list[t];
   P.outs.upload(outs, st);
   if (!P.segs) {
     P.segs = std::make_shared<DevArray<GemmSeg>>();
@@ -1013,6 +1034,7 @@ static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vecto
   P.nsplit = (int)sp.size();
   if (wsz > 0) P.ws.ensure((size_t)wsz);
   P.flops = fl;
+  buf.trim();
   P.kind = kind;
   P.choice = &choice;
   if (warp && P.nsplit > 0) P.counters.upload(std::vector<int>(sp.size(), 0), st);
@@ -2227,9 +2249,9 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
 
 // The FP64 plan of a position for another number of vectors, from the lists of plan P while the
 // scratch still holds them: P's segments and diagonal, and outputs, tiles and a workspace of its
-// own (null when the lists are gone).  Walking the terms again and writing and uploading the
-// segments is most of a plan: heff_diag and then sigma of 4 vectors at k = 16, M = 384: 37 ms
-// for two whole plans, PLACEHOLDER.
+// own (null when the lists are gone).  Walking the terms and writing the segments is half of a
+// plan.  A sweep position with heff_diag and sigma of 4 vectors at k = 16, M = 384: 39 ms with two
+// whole plans, 24 this way.
 static std::unique_ptr<SigmaPlan> plan_vectors(lrt_ctx* c, const SigmaPlan& P, int nvec) {
   PlanScratch& W = c->scratch;
   if (W.lists == 0 || W.lists != P.lists) return nullptr;
