@@ -1970,6 +1970,11 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
   PlanScratch& W = c->scratch;
   W.clear();
   std::vector<Prod2>& prod2 = W.prod2;
+  auto output = [&](int w, int r, int m) {
+    const int u = out_of[16 * w + 4 * r + m];
+    if (u < 0) throw Error(LRT_EINVAL, "internal: block product outside the wavefunction's sub-blocks");
+    return u;
+  };
   std::vector<GemmOut>& o1 = W.o1;
   std::vector<GemmSeg>& s1 = W.s1;
   std::vector<char>& s1rev = W.s1rev;   // the operator lives in the reverse set
@@ -2116,7 +2121,7 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
             const int64_t arow = ident ? wk.off + (int64_t)XF.off[ke][r] * wk.cols
                                        : tp + (int64_t)XF.off[be][r] * wk.cols;
             if (nsite == 1) {
-              prod2.push_back(Prod2{arow, Bp, sc, out_of[16 * ib + 4 * r], wk.cols, ldb, wk.cols, (short)transB,
+              prod2.push_back(Prod2{arow, Bp, sc, output(ib, r, 0), wk.cols, ldb, wk.cols, (short)transB,
                                     (short)ident, (short)(&YS != &Y)});
               falg += 2.0 * XF.dim[be][r] * wk.cols * wbb.cols;
             } else {
@@ -2125,7 +2130,7 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
                   if (!(ymask & (1u << (4 * mp + m)))) continue;
                   const double* B = !bref.t ? Bp + (int64_t)YF->off[ybb][mp] * ldb + YF->off[yk][m]
                                             : Bp + (int64_t)YF->off[yk][m] * ldb + YF->off[ybb][mp];
-                  prod2.push_back(Prod2{arow + YF->off[yk][m], B, sc, out_of[16 * ib + 4 * r + mp], wk.cols, ldb,
+                  prod2.push_back(Prod2{arow + YF->off[yk][m], B, sc, output(ib, r, mp), wk.cols, ldb,
                                         YF->dim[yk][m], (short)transB, (short)ident, (short)(&YS != &Y)});
                   falg += 2.0 * XF.dim[be][r] * YF->dim[yk][m] * YF->dim[ybb][mp];
                 }
