@@ -534,22 +534,22 @@ __global__ void __launch_bounds__(32 * MMA_WARPS, MMA_CTAS)
   gemm_mma_tile(segs, wi, b->x, b->y, b->t, nullptr, o, [&](int i) { return b->e[i]; });
 }
 
-// dynamic shared memory of the kernels, once per device
+// dynamic shared memory of the kernels, once per device (beyond MAX_DEV devices, at every launch)
 static cudaError_t mma_smem_attr() {
   constexpr int MAX_DEV = 64;
   static std::atomic<int> done[MAX_DEV];
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= MAX_DEV) return cudaErrorInvalidDevice;
-  if (done[dev].load(std::memory_order_acquire)) return cudaSuccess;
+  const bool kept = dev >= 0 && dev < MAX_DEV;
+  if (kept && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
   for (const void* f : {(const void*)gemm_mma_kernel, (const void*)gemm_mma_inst_kernel}) {
     e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MmaSmem));
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
   }
-  done[dev].store(1, std::memory_order_release);
+  if (kept) done[dev].store(1, std::memory_order_release);
   return cudaSuccess;
 }
 
