@@ -795,18 +795,20 @@ struct GemmPlan {
     }
   }
   void run_multi(cudaStream_t st, const GemmBases* bases) const {
+    if (ntiles == 0) return;
     switch (kind) {
       case GemmKind::WARP:
         launch_gemm_warp(outs.p, segs->p, tiles.p, ntiles, nullptr, nullptr, nullptr, st, bases, nullptr, ws.p,
                          splits.p, counters.p);
-        break;
+        return;
       case GemmKind::MMA:
-        launch_gemm_mma(outs.p, segs->p, tiles.p, ntiles, nullptr, nullptr, nullptr, st, bases, nullptr, nullptr);
+        launch_gemm_mma(outs.p, segs->p, tiles.p, ntiles, nullptr, nullptr, nullptr, st, bases, nullptr, ws.p);
         break;
       case GemmKind::FP64:
-        launch_gemm_fp64_multi(outs.p, segs->p, tiles.p, ntiles, bases, st);
+        launch_gemm_fp64_multi(outs.p, segs->p, tiles.p, ntiles, bases, ws.p, st);
         break;
     }
+    if (nsplit > 0) launch_split_reduce(outs.p, splits.p, nsplit, ws.p, nullptr, nullptr, st, bases);
   }
   int launches() const { return (ntiles > 0) + (nsplit > 0 && kind != GemmKind::WARP); }
 };
@@ -905,16 +907,13 @@ static void warp_tile_shape(GemmOut& O, int64_t k, bool digits, int& tm, int& tn
   tn = even(O.n, 16);
 }
 
-// whether outputs may be split along K: never (lists replayed over instances, whose partial
-// tiles would need a workspace each), or only by the warp kernel (lists over several bases,
-// which the reduction launch does not know)
-enum class GemmSplit { NEVER, WARP, ALWAYS };
-
 // outs is worked on in place: the parts of split tiles are appended.  P.segs: the segments where
-// they are on the device already.
+// they are on the device already.  split: outputs may be cut along K (not in lists replayed over
+// instances, whose partial tiles would need a workspace each).  like: the kernel to use, for
+// lists merged from others.
 static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vector<GemmSeg>& segs,
                        cudaStream_t st, KernelChoice& choice, GemmMath math = GemmMath::FMA,
-                       GemmSplit split = GemmSplit::NEVER) {
+                       bool split = false, const GemmKind* like = nullptr) {
   // A tile costs its warps of outputs times its K chunks of DFMA issue, plus a fixed
   // cost per chunk.  Tiles far longer than an even share of the launch (an output with
   // many long K segments) would run on after all others finished.  With `split`, an
@@ -938,7 +937,7 @@ static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vecto
     for (int s = 0; s < outs[i].seg_count; ++s) ktot[i] += segs[outs[i].seg_begin + s].k;
     fl += 2.0 * outs[i].m * (double)outs[i].n * (double)ktot[i];
   }
-  const GemmKind kind = gemm_kind(outs, segs, ktot, math, choice.forced);
+  const GemmKind kind = like ? *like : gemm_kind(outs, segs, ktot, math, choice.forced);
   const bool digits = math == GemmMath::DIGITS || choice.forced > 0;
   const bool mma = kind == GemmKind::MMA, warp = kind == GemmKind::WARP;
   auto cost = [mma, warp](int64_t mt, int64_t nt, int64_t k) {
@@ -980,7 +979,7 @@ static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vecto
         const int mt = std::min(TM, O.m - m0), nt = std::min(TN, O.n - n0);
         const int64_t c = cost(mt, nt, ktot[i]);
         const int want = (int)std::min<int64_t>(O.seg_count, ktot[i] / kpart);
-        if ((split == GemmSplit::ALWAYS || (split == GemmSplit::WARP && warp)) && want >= 2 && O.c_rel <= 2 && outs.size() < (size_t)INT32_MAX) {
+        if (split && want >= 2 && O.c_rel <= 2 && outs.size() < (size_t)INT32_MAX) {
           // contiguous runs of the segment list, each about ktot / want of K
           SplitTile t{wsz, (int)i, 0, m0, mt, n0, nt};
           std::vector<int> kseg(O.seg_count);
@@ -2214,7 +2213,7 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
   // kept relative plans (first-order sets) are replayed over instances
   const GemmMath math = rel_ops ? GemmMath::FMA : GemmMath::DIGITS;
   build_gemm(plan->p1, o1, s1, c->st, c->kernels, math);
-  build_gemm(plan->p2, O2, S2, c->st, c->kernels, math, rel_ops ? GemmSplit::NEVER : GemmSplit::ALWAYS);
+  build_gemm(plan->p2, O2, S2, c->st, c->kernels, math, !rel_ops);
   // tensor-core twin: phase-2 outputs, one per (y block, column group)
   plan->has_tc = tc;
   for (size_t w = 0; w < wb.size() && tc; ++w)
@@ -2279,7 +2278,7 @@ static std::unique_ptr<SigmaPlan> plan_vectors(lrt_ctx* c, const SigmaPlan& P, i
   plan->p2.segs = P.p2.segs;
   set_vectors(W.o1, (size_t)P.p1.nbase, W.o2, (size_t)P.p2.nbase, nvec, P.nelem, toff);
   build_gemm(plan->p1, W.o1, W.s1, c->st, c->kernels, GemmMath::DIGITS);
-  build_gemm(plan->p2, W.o2, W.s2, c->st, c->kernels, GemmMath::DIGITS, GemmSplit::ALWAYS);
+  build_gemm(plan->p2, W.o2, W.s2, c->st, c->kernels, GemmMath::DIGITS, true);
   CK(cudaStreamSynchronize(c->st));
   return plan;
 }
@@ -5626,8 +5625,8 @@ struct BatchPlan {
   std::vector<uint64_t> ids, serials;   // instances and the plans this batch was built from
   int precision = LRT_FP64;
   double flops = 0.0;
-  // FP64: merged task lists, bases (x, y, T) per instance
-  GemmPlan p1, p2;
+  // FP64: merged task lists, one per GemmKind, and bases (x, y, T) per instance
+  std::array<GemmPlan, 3> p1, p2;
   DevArray<GemmBases> bases;
   std::vector<GemmBases> hbases;
   // split-TF32: merged work streams, y per instance
@@ -5656,12 +5655,15 @@ static std::vector<T> download(const DevArray<T>& a, cudaStream_t st) {
   return h;
 }
 
-static void merge_fp64(GemmPlan& out, const std::vector<SigmaPlan*>& plans, bool phase2, cudaStream_t st,
+// the lists of one phase that run on `kind`, every instance's on its own kernel and in its own
+// K parts: an instance's result is that of its own call, whatever the others are
+static void merge_fp64(GemmPlan& out, const std::vector<SigmaPlan*>& plans, bool phase2, GemmKind kind, cudaStream_t st,
                        KernelChoice& choice) {
   std::vector<GemmOut> O;
   std::vector<GemmSeg> S;
   for (size_t j = 0; j < plans.size(); ++j) {
     const GemmPlan& g = phase2 ? plans[j]->p2 : plans[j]->p1;
+    if (g.kind != kind) continue;
     std::vector<GemmOut> o = download(g.outs, st);
     o.resize(g.nbase);   // not the K parts of split tiles: the merged plan tiles anew
     std::vector<GemmSeg> sg = download(*g.segs, st);
@@ -5673,7 +5675,7 @@ static void merge_fp64(GemmPlan& out, const std::vector<SigmaPlan*>& plans, bool
     }
     S.insert(S.end(), sg.begin(), sg.end());
   }
-  build_gemm(out, O, S, st, choice, GemmMath::DIGITS, GemmSplit::WARP);
+  if (!O.empty()) build_gemm(out, O, S, st, choice, GemmMath::DIGITS, phase2, &kind);
 }
 
 // one batched call (the graph body): no host synchronization inside
@@ -5689,8 +5691,8 @@ static void batch_issue(lrt_ctx* c0, BatchPlan& B, const std::vector<SigmaPlan*>
     launch_gemm_tf32x3(B.tci1.p, B.tcb1.p, B.tcn1, B.tn1, to, c0->derr, st);
     launch_gemm_tf32x3(B.tci2.p, B.tcb2.p, B.tcn2, B.tn2, to, c0->derr, st);
   } else {
-    B.p1.run_multi(st, B.bases.p);
-    B.p2.run_multi(st, B.bases.p);
+    for (const GemmPlan& p : B.p1) p.run_multi(st, B.bases.p);
+    for (const GemmPlan& p : B.p2) p.run_multi(st, B.bases.p);
   }
 }
 
@@ -5762,8 +5764,10 @@ static void sigma_batched_impl(lrt_ctx* const* ctxs, int n, const int* sites, in
       B->tn2 = tune_tc_stream(c0, s2, nvec, scratch, B->tci2, B->tcb2, B->tcn2);
       CK(cudaStreamSynchronize(c0->st));
     } else {
-      merge_fp64(B->p1, plans, false, c0->st, c0->kernels);
-      merge_fp64(B->p2, plans, true, c0->st, c0->kernels);
+      for (int q = 0; q < 3; ++q) {
+        merge_fp64(B->p1[q], plans, false, (GemmKind)q, c0->st, c0->kernels);
+        merge_fp64(B->p2[q], plans, true, (GemmKind)q, c0->st, c0->kernels);
+      }
     }
     CK(cudaStreamSynchronize(c0->st));
     slot = std::move(B);
@@ -5822,8 +5826,8 @@ static void sigma_batched_impl(lrt_ctx* const* ctxs, int n, const int* sites, in
   if (precision == LRT_MIXED) {
     c0->kernels.launches[3] += 2;
   } else {
-    B.p1.count();
-    B.p2.count();
+    for (const GemmPlan& p : B.p1) p.count();
+    for (const GemmPlan& p : B.p2) p.count();
   }
   B.gx = xv;
   B.gy = yv;
@@ -5839,7 +5843,8 @@ static void sigma_batched_impl(lrt_ctx* const* ctxs, int n, const int* sites, in
   }
   c0->last.flops = B.flops;
   c0->last.flops_issued = 0.0;
-  c0->last.launches = 2;
+  c0->last.launches = precision == LRT_MIXED ? 2 : 0;
+  for (int q = 0; q < 3; ++q) c0->last.launches += B.p1[q].launches() + B.p2[q].launches();
   c0->last.n_terms = 0;
   c0->last.n_products = 0;
   c0->last.op_bytes = 0.0;

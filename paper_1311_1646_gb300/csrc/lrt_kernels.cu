@@ -519,12 +519,17 @@ void launch_gemm_fp64(const GemmOut* outs, const GemmSeg* segs, const int3* tile
 __global__ void __launch_bounds__(256) split_reduce_kernel(const GemmOut* __restrict__ outs,
                                                            const SplitTile* __restrict__ tiles,
                                                            const double* __restrict__ wbase,
-                                                           double* __restrict__ ybase, double* __restrict__ tbase) {
+                                                           double* __restrict__ ybase, double* __restrict__ tbase,
+                                                           const GemmBases* __restrict__ multi) {
   const SplitTile t = tiles[blockIdx.x];
   const int ne = t.mt * t.nt;
   const int e = blockIdx.y * blockDim.x + threadIdx.x;
   if (e >= ne) return;
   const GemmOut o = outs[t.o];
+  if (multi) {
+    ybase = multi[o.inst].y;
+    tbase = multi[o.inst].t;
+  }
   double* cbase = o.c_rel == 1 ? ybase + o.c_off : o.c_rel == 2 ? tbase + o.c_off : o.C;
   const double* w = wbase + t.ws_off + e;
   double s = 0.0;
@@ -546,10 +551,10 @@ __global__ void __launch_bounds__(256) split_reduce_kernel(const GemmOut* __rest
 }
 
 void launch_split_reduce(const GemmOut* outs, const SplitTile* tiles, int ntiles, const double* wbase, double* ybase,
-                         double* tbase, cudaStream_t st) {
+                         double* tbase, cudaStream_t st, const GemmBases* multi) {
   if (ntiles <= 0) return;
   constexpr int most = GEMM_TM * GEMM_TN > 16 * 256 ? GEMM_TM * GEMM_TN : 16 * 256;   // elements of a tile (either kernel)
-  split_reduce_kernel<<<dim3(ntiles, (most + 255) / 256), 256, 0, st>>>(outs, tiles, wbase, ybase, tbase);
+  split_reduce_kernel<<<dim3(ntiles, (most + 255) / 256), 256, 0, st>>>(outs, tiles, wbase, ybase, tbase, multi);
 }
 
 void launch_gemm_fp64_inst(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles,
@@ -562,11 +567,11 @@ void launch_gemm_fp64_inst(const GemmOut* outs, const GemmSeg* segs, const int3*
 }
 
 void launch_gemm_fp64_multi(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles,
-                            const GemmBases* bases, cudaStream_t st) {
+                            const GemmBases* bases, double* wbase, cudaStream_t st) {
   if (ntiles <= 0) return;
   if (gemm_fp64_smem_attr() != cudaSuccess) return;
   gemm_fp64_kernel<<<ntiles, GEMM_THREADS, sizeof(GemmSmem), st>>>(outs, segs, tiles, ntiles, nullptr, nullptr,
-                                                                  nullptr, bases, GemmExtra{}, nullptr);
+                                                                  nullptr, bases, GemmExtra{}, wbase);
 }
 
 // ---------------------------------------------------------------------------

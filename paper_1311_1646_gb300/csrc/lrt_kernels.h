@@ -170,7 +170,7 @@ struct SplitTile {
   int m0, mt, n0, nt;
 };
 void launch_split_reduce(const GemmOut* outs, const SplitTile* tiles, int ntiles, const double* wbase, double* ybase,
-                         double* tbase, cudaStream_t st);
+                         double* tbase, cudaStream_t st, const GemmBases* multi = nullptr);
 // One warp per tile (small blocks, lrt_fp64_mma.cu): with GEMM_WARP_DIRECT at most
 // GEMM_DIRECT_MAX elements, else 16 x 16.  Parts of split tiles are added by the warp that
 // finishes last: one counter per split tile, zero before the first launch.
@@ -180,7 +180,7 @@ void launch_gemm_warp(const GemmOut* outs, const GemmSeg* segs, const int3* tile
                       double* wbase, const SplitTile* splits, int* counters);
 // batched form: the bases of output o are bases[o.inst] (device array)
 void launch_gemm_fp64_multi(const GemmOut* outs, const GemmSeg* segs, const int3* tiles, int ntiles,
-                            const GemmBases* bases, cudaStream_t st);
+                            const GemmBases* bases, double* wbase, cudaStream_t st);
 // One plan replayed over up to GEMM_MAX_INST instances in one launch: CTA b runs tile
 // b / ninst of instance b % ninst, every base (x, y, t and the extra bases) taken from
 // that instance's entry.  The entries travel in the launch's parameter block (no upload,

@@ -53,3 +53,39 @@ def test_a_refused_batch_leaves_the_contexts_untouched(pkg, precision):
     assert free1 == free0
     for c in ctxs:
         c.close()
+
+
+@pytest.mark.parametrize("nsite", [1, 2])
+@pytest.mark.parametrize("kernels", [(1, 2, 3), (3, 0, 2), (2, 2, 2), (0, 0, 0)])
+def test_an_instance_of_a_batch_has_the_bits_of_its_own_call(pkg, kernels, nsite):
+    """Whatever the other molecules are: each instance keeps its own kernel and K parts, on long
+    segment lists (split) and short ones, through the first call and the replayed graph."""
+    ctxs, xs, ys, want, sites = [], [], [], [], []
+    for j, (k, na, nb, M) in enumerate([(8, 4, 4, 64), (10, 2, 2, 131), (9, 4, 4, 60)]):
+        H = synth.ab_initio(k, na, nb, 70 + j)
+        i = k // 2 - 1
+        m = synth.mixed_mps(k, na, nb, M, 71 + j, center=i)
+        c = pkg.Context(0)
+        c.set_kernels(kernels[j])
+        c.op_build(k, H.h, H.eri)
+        c.mps_load(k, na, nb, m.bonds, m.sites, i)
+        for b in range(i):
+            c.renormalize(b, +1)
+        for b in range(k - 1, i + nsite - 1, -1):
+            c.renormalize(b, -1)
+        n, _ = c.wfn_layout(i, nsite)
+        xs.append(torch.tensor(synth.random_vector(3 * n, 72 + j), dtype=torch.float64, device="cuda:0"))
+        ys.append(torch.empty_like(xs[-1]))
+        want.append(torch.empty_like(xs[-1]))
+        c.sigma(i, nsite, xs[-1], want[-1], nvec=3)
+        ctxs.append(c)
+        sites.append(i)
+    for _ in range(3):
+        for y in ys:
+            y.fill_(float("nan"))
+        pkg.sigma_batched(ctxs, sites, nsite, xs, ys, nvec=3)
+        torch.cuda.synchronize()
+        for j in range(3):
+            assert torch.equal(ys[j], want[j]), j
+    for c in ctxs:
+        c.close()
