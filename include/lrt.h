@@ -137,7 +137,7 @@ int renormalize(lrt_t ctx, int site, int dir, int precision);
  * of bond site+1; nsite = 2 uses the left block of bond `site` and the right block of
  * bond site+2.  x_dev, y_dev: device pointers of nvec * nelem doubles; must not
  * overlap.  precision LRT_MIXED allows split-TF32 tensor-core products (about seven digits);
- * calls too small to gain from them run in FP64. */
+ * positions too small to gain from them, whatever nvec is, run in FP64. */
 int sigma(lrt_t ctx, int site, int nsite, int nvec, const double* x_dev, double* y_dev,
           int precision);
 

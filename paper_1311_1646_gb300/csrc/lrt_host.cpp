@@ -1220,7 +1220,7 @@ struct SigmaPlan {
   int n_terms = 0, n_products = 0;
   double op_bytes = 0.0;
   double flops_alg = 0.0;   // products of non-zero sub-blocks only
-  double macs1 = -1.0;      // phase1_macs of the position, once known
+  double work1 = -1.0;      // phase1_work of the position, once known
   // tensor-core twin of the two phases (host description; device streams built on
   // first mixed use): whole fused blocks, operands as TC matrices in three pools
   // (0: operator sub-matrices, 1: x-derived, per vector, 2: intermediates T, per vector)
@@ -1635,7 +1635,10 @@ static void ren_absolute(std::vector<GemmOut>& o1, std::vector<GemmSeg>& s1, std
   outs(o2);
 }
 
-static bool mixed_in_fp64(lrt_ctx* c, double macs, int nvec);
+// An LRT_MIXED renormalization runs on the FP64 kernels below MIXED_REN_MACS multiply-adds of its first
+// phase: the split-TF32 form packs and plans its operands on the host.  Split TF32 / FP64, ms: 0.77 /
+// 0.13 (1e5), 3.7 / 0.86 (5e7), 14.5 / 3.0 (4e8), 20.2 / 7.7 (2e9), 20.9 / 41 (1.6e10, k = 24, M = 1000).
+constexpr double MIXED_REN_MACS = 6e9;
 
 // runs (and, given a template slot, keeps) a renormalization's two grouped GEMMs
 static void ren_run(lrt_ctx* c, std::vector<GemmOut>& o1, std::vector<GemmSeg>& s1, std::vector<GemmOut>& o2,
@@ -1644,7 +1647,7 @@ static void ren_run(lrt_ctx* c, std::vector<GemmOut>& o1, std::vector<GemmSeg>& 
   double macs = 0.0;
   if (prec == LRT_MIXED)
     for (const GemmOut& o : o1) macs += (double)o.m * o.n * s1[o.seg_begin].k;
-  if (prec == LRT_MIXED && !mixed_in_fp64(c, macs, 1)) {
+  if (prec == LRT_MIXED && (macs >= MIXED_REN_MACS || c->tc_stall || c->kernels.mixed_always)) {
     ren_absolute(o1, s1, o2, s2, ex);
     run_two_phase_tc(c, o1, s1, o2, s2);
     return;
@@ -2269,7 +2272,7 @@ static std::unique_ptr<SigmaPlan> plan_vectors(lrt_ctx* c, const SigmaPlan& P, i
   plan->n_products = P.n_products;
   plan->op_bytes = P.op_bytes;
   plan->flops_alg = P.flops_alg / P.nvec * nvec;
-  plan->macs1 = P.macs1;
+  plan->work1 = P.work1;
   const int64_t toff = P.tsize / P.nvec;
   plan->tsize = toff * nvec;
   if (toff > 0 && dev_alloc((void**)&plan->tbuf, (size_t)plan->tsize * sizeof(double)) != cudaSuccess)
@@ -2277,8 +2280,10 @@ static std::unique_ptr<SigmaPlan> plan_vectors(lrt_ctx* c, const SigmaPlan& P, i
   plan->p1.segs = P.p1.segs;
   plan->p2.segs = P.p2.segs;
   set_vectors(W.o1, (size_t)P.p1.nbase, W.o2, (size_t)P.p2.nbase, nvec, P.nelem, toff);
-  build_gemm(plan->p1, W.o1, W.s1, c->st, c->kernels, GemmMath::DIGITS);
-  build_gemm(plan->p2, W.o2, W.s2, c->st, c->kernels, GemmMath::DIGITS, true);
+  // the kernels are P's too, unless a vector stride is beyond what one of them takes
+  const bool same = std::max(P.nelem, toff) < (int64_t)1 << 29;
+  build_gemm(plan->p1, W.o1, W.s1, c->st, c->kernels, GemmMath::DIGITS, false, same ? &P.p1.kind : nullptr);
+  build_gemm(plan->p2, W.o2, W.s2, c->st, c->kernels, GemmMath::DIGITS, true, same ? &P.p2.kind : nullptr);
   CK(cudaStreamSynchronize(c->st));
   return plan;
 }
@@ -2836,48 +2841,65 @@ static SigmaPlan& get_plan(lrt_ctx* c, int site, int nsite, int nvec, bool tc = 
 }
 
 // LRT_MIXED calls that run on the FP64 kernels: the split-TF32 kernel fills one persistent CTA per
-// SM with 128-row tiles and pays a host synchronization per call, which short lists of small
-// blocks do not repay, and the FP64 digit products are the more exact of the two.  Measured,
-// split-TF32 / FP64: two-site k = 13, M = 200, 3 vectors (1e8 multiply-adds of phase 1 per
-// vector) 3.89 / 1.47 ms; k = 24, M = 500, 6 vectors (1.9e9) 6.55 / 15.2 ms.  A pending
-// stall (lrt_set_wait_limit) is for the next tensor-core launch, so such a call keeps it.
-constexpr double MIXED_MIN_MACS = 2e8, MIXED_MIN_TOTAL = 7e8;   // phase 1, per vector / of the call
-static bool mixed_in_fp64(lrt_ctx* c, double macs, int nvec) {
-  return !c->tc_stall && !c->kernels.mixed_always && macs < MIXED_MIN_MACS && macs * nvec < MIXED_MIN_TOTAL;
+// SM with tiles of 128 rows and 32 K positions, packs its operands and waits for the host once
+// per call.  Small blocks do not repay that, and FP64 is the more exact.  What counts is the work
+// of the first phase discounted by the square of its padding to 16 x 8 x 16.  Split TF32 / FP64, ms,
+// for 1 and 6 vectors, by that work (x 1e6):
+//   0.4  k = 10, M = 150, one site  0.41 / 0.12  0.68 / 0.28
+//   2.4  k = 13, M = 200, two sites 1.9 / 0.67   3.7 / 2.8
+//   5.0  k = 14, M = 300, one site  0.82 / 0.45  2.0 / 1.6
+//   7.8  k = 16, M = 384, one site  1.1 / 0.97   3.5 / 3.8
+//   17   k = 24, M = 300, site 4    0.53 / 0.36  0.95 / 1.6
+//   24   k = 11, M = 300, one site  0.42 / 0.47  0.55 / 1.9
+//   25   k = 12, M = 256, two sites 1.4 / 1.7    4.2 / 4.9
+//   100  k = 24, M = 400, one site  2.6 / 4.4    5.3 / 11.1
+//   260  k = 24, M = 500, one site  3.2 / 5.6    6.6 / 16.3
+// It is the position's, so that a vector's precision depends neither on the other vectors of
+// the call nor on the other molecules of a batch.  A pending stall (lrt_set_wait_limit) is for the
+// next tensor-core launch, so such a call keeps it.
+constexpr double MIXED_MIN_WORK = 1.15e7;
+static double tile_work(double macs, double padded) { return padded > 0.0 ? macs * (macs / padded) * (macs / padded) : 0.0; }
+static bool mixed_in_fp64(lrt_ctx* c, double work) {
+  return !c->tc_stall && !c->kernels.mixed_always && work < MIXED_MIN_WORK;
 }
 
-// multiply-adds of X psi over the non-zero sub-blocks of the enlarged left set, one vector
-static double phase1_macs(lrt_ctx* c, const OpSet& X, int site, int nsite) {
-  std::vector<double> cols(X.ns(), 0.0);
+// tile_work of X psi over the non-zero sub-blocks of the enlarged left set, one vector
+static double phase1_work(lrt_ctx* c, const OpSet& X, int site, int nsite) {
+  std::vector<int> cols(X.ns(), 0);
   for (const WfnBlock& w : wfn_blocks(c, site, nsite)) {
     const int f = X.basis.find(w.label_a, w.label_b);
     if (f >= 0) cols[f] = w.cols;
   }
   const Fused& F = *X.fused;
-  double n = 0.0;
+  double macs = 0.0, padded = 0.0;
   for (size_t o = 0; o < X.keys.size(); ++o)
     for (int f = 0; f < X.ns(); ++f) {
+      const unsigned m = X.mask[o * X.ns() + f];
+      if (!m || cols[f] == 0) continue;
       const int fb = X.bra_of((int)o, f);
-      for (unsigned m = X.mask[o * X.ns() + f]; m; m &= m - 1) {
-        const int bit = __builtin_ctz(m);
-        n += (double)F.dim[fb][bit >> 2] * F.dim[f][bit & 3] * cols[f];
+      for (int r = 0; r < 4; ++r) {
+        int k = 0;
+        for (int q = 0; q < 4; ++q)
+          if (m >> (4 * r + q) & 1) k += F.dim[f][q];
+        macs += (double)F.dim[fb][r] * k * cols[f];
+        padded += (double)((F.dim[fb][r] + 15) / 16 * 16) * ((k + 15) / 16 * 16) * ((cols[f] + 7) / 8 * 8);
       }
     }
-  return n;
+  return tile_work(macs, padded);
 }
 
 // the same, remembered by the position's plans
-static double position_macs(lrt_ctx* c, int site, int nsite) {
+static double position_work(lrt_ctx* c, int site, int nsite) {
   SigmaPlan* p = any_plan(c, site, nsite);
-  if (p && p->macs1 >= 0.0) return p->macs1;
-  const double m = phase1_macs(c, enlarged(c, site, false), site, nsite);
-  if (p) p->macs1 = m;
-  return m;
+  if (p && p->work1 >= 0.0) return p->work1;
+  const double w = phase1_work(c, enlarged(c, site, false), site, nsite);
+  if (p) p->work1 = w;
+  return w;
 }
 
 // the plan of a mixed sigma; tc: it runs on the split-TF32 kernels (and has their twin)
 static SigmaPlan& get_mixed_plan(lrt_ctx* c, int site, int nsite, int nvec, bool& tc) {
-  tc = !mixed_in_fp64(c, position_macs(c, site, nsite), nvec);
+  tc = !mixed_in_fp64(c, position_work(c, site, nsite));
   return get_plan(c, site, nsite, nvec, tc);
 }
 
@@ -3899,10 +3921,10 @@ struct TdaRunner {
   // calls on whole blocks of `blk` vectors (the block-Davidson right-hand sides)
   void h0(int i, const SiteBatch& X, int nv, SiteBatch& Y) {
     auto& p = h0blk[{i, blk}];
-    const double macs = !mixed || (p && p->macs1 >= 0.0) ? (p ? p->macs1 : -1.0) : phase1_macs(c, *c->XL[i], i, 1);
-    const bool tc = mixed && !mixed_in_fp64(c, macs, blk);
+    const double work = !mixed || (p && p->work1 >= 0.0) ? (p ? p->work1 : -1.0) : phase1_work(c, *c->XL[i], i, 1);
+    const bool tc = mixed && !mixed_in_fp64(c, work);
     if (!p || (tc && !p->has_tc)) p = plan_sigma_sets(c, *c->XL[i], nullptr, *c->R[i + 1], nullptr, i, 1, blk, tc);
-    p->macs1 = macs;
+    p->work1 = work;
     for (int v0 = 0; v0 < nv; v0 += blk) run_plan(*p, X.v(v0), Y.v(v0), blk, tc);
   }
 
@@ -5623,7 +5645,8 @@ namespace lrt {
 
 struct BatchPlan {
   std::vector<uint64_t> ids, serials;   // instances and the plans this batch was built from
-  int precision = LRT_FP64;
+  std::vector<char> tc;                 // instances in split TF32, the others in FP64
+  int ntc = 0;
   double flops = 0.0;
   // FP64: merged task lists, one per GemmKind, and bases (x, y, T) per instance
   std::array<GemmPlan, 3> p1, p2;
@@ -5657,13 +5680,13 @@ static std::vector<T> download(const DevArray<T>& a, cudaStream_t st) {
 
 // the lists of one phase that run on `kind`, every instance's on its own kernel and in its own
 // K parts: an instance's result is that of its own call, whatever the others are
-static void merge_fp64(GemmPlan& out, const std::vector<SigmaPlan*>& plans, bool phase2, GemmKind kind, cudaStream_t st,
-                       KernelChoice& choice) {
+static void merge_fp64(GemmPlan& out, const std::vector<SigmaPlan*>& plans, const std::vector<char>& tc, bool phase2,
+                       GemmKind kind, cudaStream_t st, KernelChoice& choice) {
   std::vector<GemmOut> O;
   std::vector<GemmSeg> S;
   for (size_t j = 0; j < plans.size(); ++j) {
     const GemmPlan& g = phase2 ? plans[j]->p2 : plans[j]->p1;
-    if (g.kind != kind) continue;
+    if (tc[j] || g.kind != kind) continue;
     std::vector<GemmOut> o = download(g.outs, st);
     o.resize(g.nbase);   // not the K parts of split tiles: the merged plan tiles anew
     std::vector<GemmSeg> sg = download(*g.segs, st);
@@ -5681,8 +5704,9 @@ static void merge_fp64(GemmPlan& out, const std::vector<SigmaPlan*>& plans, bool
 // one batched call (the graph body): no host synchronization inside
 static void batch_issue(lrt_ctx* c0, BatchPlan& B, const std::vector<SigmaPlan*>& plans,
                         const std::vector<const double*>& x, int nvec, cudaStream_t st) {
-  if (B.precision == LRT_MIXED) {
+  if (B.ntc > 0) {
     for (size_t j = 0; j < plans.size(); ++j) {
+      if (!B.tc[j]) continue;
       SigmaPlan& p = *plans[j];
       launch_tc_pack(p.xpack.p, (int)p.tc.pack1.size(), x[j], p.nelem, p.pool_hi[1], p.pool_lo[1],
                      p.tc.pool_size[1], nvec, st);
@@ -5690,10 +5714,9 @@ static void batch_issue(lrt_ctx* c0, BatchPlan& B, const std::vector<SigmaPlan*>
     const TcOut to = tc_out(c0, nullptr, B.ys.p);
     launch_gemm_tf32x3(B.tci1.p, B.tcb1.p, B.tcn1, B.tn1, to, c0->derr, st);
     launch_gemm_tf32x3(B.tci2.p, B.tcb2.p, B.tcn2, B.tn2, to, c0->derr, st);
-  } else {
-    for (const GemmPlan& p : B.p1) p.run_multi(st, B.bases.p);
-    for (const GemmPlan& p : B.p2) p.run_multi(st, B.bases.p);
   }
+  for (const GemmPlan& p : B.p1) p.run_multi(st, B.bases.p);
+  for (const GemmPlan& p : B.p2) p.run_multi(st, B.bases.p);
 }
 
 static void sigma_batched_impl(lrt_ctx* const* ctxs, int n, const int* sites, int nsite, int nvec,
@@ -5712,24 +5735,20 @@ static void sigma_batched_impl(lrt_ctx* const* ctxs, int n, const int* sites, in
       throw Error(LRT_ESTATE, "right block of bond " + std::to_string(sites[j] + nsite) + " not built");
     if (!x[j] || !y[j]) throw Error(LRT_EINVAL, "sigma_batched: NULL vector");
   }
-  if (precision == LRT_MIXED && !c0->tc_stall && !c0->kernels.mixed_always) {
-    // all instances small: the call runs in FP64 (see mixed_in_fp64; a pending stall is c0's)
-    double macs = 0.0;
-    bool small = true;
-    for (int j = 0; j < n && small; ++j) {
-      PoolScope ps(&ctxs[j]->pool);
-      const double m = position_macs(ctxs[j], sites[j], nsite);
-      macs += m;
-      small = m < MIXED_MIN_MACS && macs * nvec < MIXED_MIN_TOTAL;
-    }
-    if (small) precision = LRT_FP64;
+  // the instances that run in split TF32 (a pending stall is c0's)
+  std::vector<char> tc(n, 0);
+  int ntc = 0;
+  for (int j = 0; j < n && precision == LRT_MIXED; ++j) {
+    PoolScope ps(&ctxs[j]->pool);
+    tc[j] = c0->tc_stall || c0->kernels.mixed_always || position_work(ctxs[j], sites[j], nsite) >= MIXED_MIN_WORK;
+    ntc += tc[j];
   }
   std::string key = std::to_string(nsite) + ":" + std::to_string(nvec) + ":" + std::to_string(precision);
   for (int j = 0; j < n; ++j) {
     lrt_ctx* c = ctxs[j];
     PoolScope ps(&c->pool);
-    plans[j] = &get_plan(c, sites[j], nsite, nvec, precision == LRT_MIXED);
-    key += ":" + std::to_string(c->id) + "/" + std::to_string(sites[j]);
+    plans[j] = &get_plan(c, sites[j], nsite, nvec, tc[j]);
+    key += ":" + std::to_string(c->id) + "/" + std::to_string(sites[j]) + (tc[j] ? "t" : "");
   }
   auto& slot = c0->batches[key];
   bool fresh = false;
@@ -5738,15 +5757,17 @@ static void sigma_batched_impl(lrt_ctx* const* ctxs, int n, const int* sites, in
   }
   if (!slot || fresh) {
     auto B = std::make_unique<BatchPlan>();
-    B->precision = precision;
+    B->tc = tc;
+    B->ntc = ntc;
     for (int j = 0; j < n; ++j) {
       B->ids.push_back(ctxs[j]->id);
       B->serials.push_back(plans[j]->serial);
       B->flops += plans[j]->flops_alg;
     }
-    if (precision == LRT_MIXED) {
+    if (ntc > 0) {
       std::vector<TcSource> s1, s2;
       for (int j = 0; j < n; ++j) {
+        if (!tc[j]) continue;
         PoolScope ps(&ctxs[j]->pool);
         prepare_tc(ctxs[j], *plans[j], nvec);
         SigmaPlan& p = *plans[j];
@@ -5763,17 +5784,18 @@ static void sigma_batched_impl(lrt_ctx* const* ctxs, int n, const int* sites, in
       B->tn1 = tune_tc_stream(c0, s1, nvec, scratch, B->tci1, B->tcb1, B->tcn1);
       B->tn2 = tune_tc_stream(c0, s2, nvec, scratch, B->tci2, B->tcb2, B->tcn2);
       CK(cudaStreamSynchronize(c0->st));
-    } else {
+    }
+    if (ntc < n) {
       for (int q = 0; q < 3; ++q) {
-        merge_fp64(B->p1[q], plans, false, (GemmKind)q, c0->st, c0->kernels);
-        merge_fp64(B->p2[q], plans, true, (GemmKind)q, c0->st, c0->kernels);
+        merge_fp64(B->p1[q], plans, tc, false, (GemmKind)q, c0->st, c0->kernels);
+        merge_fp64(B->p2[q], plans, tc, true, (GemmKind)q, c0->st, c0->kernels);
       }
     }
     CK(cudaStreamSynchronize(c0->st));
     slot = std::move(B);
   }
   BatchPlan& B = *slot;
-  if (precision == LRT_MIXED && !c0->derr) {
+  if (ntc > 0 && !c0->derr) {
     if (dev_alloc((void**)&c0->derr, sizeof(int)) != cudaSuccess) throw Error(LRT_ENOMEM, "error flag");
     CK(cudaMemsetAsync(c0->derr, 0, sizeof(int), c0->st));
   }
@@ -5789,10 +5811,11 @@ static void sigma_batched_impl(lrt_ctx* const* ctxs, int n, const int* sites, in
   }
   const bool same = B.ran && xv == B.gx && yv == B.gy;
   if (!same) {
-    if (precision == LRT_MIXED) {
+    if (ntc > 0) {
       B.hys = yv;
       B.ys.upload(B.hys, c0->st);
-    } else {
+    }
+    if (ntc < n) {
       B.hbases.resize(n);
       for (int j = 0; j < n; ++j) B.hbases[j] = GemmBases{x[j], y[j], plans[j]->tbuf};
       B.bases.upload(B.hbases, c0->st);
@@ -5823,16 +5846,13 @@ static void sigma_batched_impl(lrt_ctx* const* ctxs, int n, const int* sites, in
     batch_issue(c0, B, plans, xv, nvec, c0->st);
   }
   CK(cudaGetLastError());
-  if (precision == LRT_MIXED) {
-    c0->kernels.launches[3] += 2;
-  } else {
-    for (const GemmPlan& p : B.p1) p.count();
-    for (const GemmPlan& p : B.p2) p.count();
-  }
+  if (ntc > 0) c0->kernels.launches[3] += 2;
+  for (const GemmPlan& p : B.p1) p.count();
+  for (const GemmPlan& p : B.p2) p.count();
   B.gx = xv;
   B.gy = yv;
   B.ran = true;
-  if (precision == LRT_MIXED) {
+  if (ntc > 0) {
     int flag = 0;
     CK(cudaMemcpyAsync(&flag, c0->derr, sizeof(int), cudaMemcpyDeviceToHost, c0->st));
     CK(cudaStreamSynchronize(c0->st));
@@ -5843,7 +5863,7 @@ static void sigma_batched_impl(lrt_ctx* const* ctxs, int n, const int* sites, in
   }
   c0->last.flops = B.flops;
   c0->last.flops_issued = 0.0;
-  c0->last.launches = precision == LRT_MIXED ? 2 : 0;
+  c0->last.launches = ntc > 0 ? 2 : 0;
   for (int q = 0; q < 3; ++q) c0->last.launches += B.p1[q].launches() + B.p2[q].launches();
   c0->last.n_terms = 0;
   c0->last.n_products = 0;

@@ -89,3 +89,43 @@ def test_an_instance_of_a_batch_has_the_bits_of_its_own_call(pkg, kernels, nsite
             assert torch.equal(ys[j], want[j]), j
     for c in ctxs:
         c.close()
+
+
+def test_precision_of_a_mixed_call_is_the_positions_own(pkg):
+    """A position that takes split TF32 and one that does not: each as in its own call, in a batch of
+    both and for one vector or several."""
+    ctxs, xs, ys, sites, want = [], [], [], [], []
+    for j, (k, na, nb, M, i) in enumerate([(8, 4, 4, 64, 3), (11, 3, 3, 300, 5)]):
+        H = synth.ab_initio(k, na, nb, 80 + j)
+        m = synth.mixed_mps(k, na, nb, M, 81 + j, center=i)
+        c = pkg.Context(0)
+        c.op_build(k, H.h, H.eri)
+        c.mps_load(k, na, nb, m.bonds, m.sites, i)
+        for b in range(i):
+            c.renormalize(b, +1)
+        for b in range(k - 1, i, -1):
+            c.renormalize(b, -1)
+        n, _ = c.wfn_layout(i, 1)
+        x = torch.tensor(synth.random_vector(4 * n, 82 + j), dtype=torch.float64, device="cuda:0")
+        y64, y = torch.empty_like(x), torch.empty_like(x)
+        c.sigma(i, 1, x, y64, nvec=4)
+        for nvec in (1, 4):
+            before = c.kernel_launches()
+            c.sigma(i, 1, x, y, nvec=nvec, precision=pkg.LRT_MIXED)
+            after = c.kernel_launches()
+            torch.cuda.synchronize()
+            assert (after[3] > before[3]) == (j == 1), (j, nvec)
+            assert torch.equal(y[:nvec * n], y64[:nvec * n]) == (j == 0)
+        ctxs.append(c)
+        xs.append(x)
+        ys.append(torch.empty_like(x))
+        sites.append(i)
+        want.append(y64)
+    for _ in range(3):
+        pkg.sigma_batched(ctxs, sites, 1, xs, ys, nvec=4, precision=pkg.LRT_MIXED)
+        torch.cuda.synchronize()
+        assert torch.equal(ys[0], want[0])
+        e = (ys[1] - want[1]).abs().max().item()
+        assert 0.0 < e <= 1e-5 * want[1].abs().max().item()
+    for c in ctxs:
+        c.close()
