@@ -717,10 +717,12 @@ struct GatherPlan {
 enum class GemmKind { FP64, MMA, WARP };
 // Arithmetic of a list.  FMA: every element as accurate as an FMA chain, whatever its operands
 // span.  DIGITS (where it pays): the error of an element is relative to its row's largest times its
-// column's largest operand.  That serves H_eff x, whose operators are those of orthonormal bases,
-// and not products that carry Schmidt values or their inverses, whose small elements are divided
-// by Schmidt values later: with digit products in the tangent-space sweeps, the roots of one
-// sweep moved by 2e-9 (bonds damped to 1e-4) and 2e-8 (1e-6), with FMAs by 1e-14.
+// column's largest operand, once the K positions are scaled by one side (GemmOut::balance_rows).
+// Lists take digits where that is what the result needs: H_eff x, with operators of orthonormal
+// bases, and the first-order sets and products, whose grading by Schmidt values lies along one
+// index and where the scaled side is chosen by it (RenOrder).  With the other side, the roots of
+// one tangent-space sweep moved by 1e-11 (bonds damped to 1e-4) and 4e-10 (1e-6), without any by
+// 2e-9 and 2e-8, and with the right one by 1e-14, as under a last-bit change of the input.
 enum class GemmMath { FMA, DIGITS };
 // Arrays that build_gemm works in, kept by the context so that their pages are touched once: a
 // position of k = 16, M = 384 has half a million tiles in its two plans.  At most
@@ -1635,6 +1637,14 @@ static void ren_absolute(std::vector<GemmOut>& o1, std::vector<GemmSeg>& s1, std
   outs(o2);
 }
 
+// What a renormalization makes: a zeroth-order set (FP64 FMAs), or a first-order set whose KET or
+// BRA index is the first-order one, of a tensor C Lambda^-1 (Lambda^-1 C on the right).  Its
+// columns (rows) grow as 1 / lambda, so their accuracy has to be their own: what is summed
+// over K, graded by the previous bond's 1 / lambda in one factor and by lambda in the other
+// (Lambda_i^-1 L_i = R_i Lambda_{i+1}^-1), is scaled by the factor on the other side, op(A)'s rows for
+// KET and op(B)'s columns for BRA, in both phases.  An element's error is then 2^-52 times its
+// column's (row's) largest sum of products.
+enum class RenOrder { ZEROTH, KET, BRA };
 // An LRT_MIXED renormalization runs on the FP64 kernels below MIXED_REN_MACS multiply-adds of its first
 // phase: the split-TF32 form packs and plans its operands on the host.  Split TF32 / FP64, ms: 0.77 /
 // 0.13 (1e5), 3.7 / 0.86 (5e7), 14.5 / 3.0 (4e8), 20.2 / 7.7 (2e9), 20.9 / 41 (1.6e10, k = 24, M = 1000).
@@ -1643,7 +1653,7 @@ constexpr double MIXED_REN_MACS = 6e9;
 // runs (and, given a template slot, keeps) a renormalization's two grouped GEMMs
 static void ren_run(lrt_ctx* c, std::vector<GemmOut>& o1, std::vector<GemmSeg>& s1, std::vector<GemmOut>& o2,
                     std::vector<GemmSeg>& s2, int64_t toff, const GemmExtra& ex, int prec, RenTemplate* tpl,
-                    const OpSet& N, uint64_t sig) {
+                    const OpSet& N, uint64_t sig, RenOrder order) {
   double macs = 0.0;
   if (prec == LRT_MIXED)
     for (const GemmOut& o : o1) macs += (double)o.m * o.n * s1[o.seg_begin].k;
@@ -1653,8 +1663,13 @@ static void ren_run(lrt_ctx* c, std::vector<GemmOut>& o1, std::vector<GemmSeg>& 
     return;
   }
   auto p1 = std::make_unique<GemmPlan>(), p2 = std::make_unique<GemmPlan>();
-  build_gemm(*p1, o1, s1, c->st, c->kernels);
-  build_gemm(*p2, o2, s2, c->st, c->kernels);
+  if (order == RenOrder::KET) {
+    for (GemmOut& o : o1) o.balance_rows = 1;
+    for (GemmOut& o : o2) o.balance_rows = 1;
+  }
+  const GemmMath math = order == RenOrder::ZEROTH ? GemmMath::FMA : GemmMath::DIGITS;
+  build_gemm(*p1, o1, s1, c->st, c->kernels, math);
+  build_gemm(*p2, o2, s2, c->st, c->kernels, math);
   double* tmp = nullptr;
   if (toff > 0 && dev_alloc((void**)&tmp, (size_t)toff * sizeof(double)) != cudaSuccess)
     throw Error(LRT_ENOMEM, "renormalize workspace");
@@ -1690,7 +1705,8 @@ static std::unique_ptr<OpSet> ren_replay(lrt_ctx* c, RenTemplate* tpl, uint64_t 
 // left block of bond b+1 = sum_t bra_t^T E_t ket_t over the enlarged left block of bond b
 // (prec LRT_MIXED: the two grouped GEMMs as split-TF32 tensor-core products)
 static std::unique_ptr<OpSet> renorm_left_terms(lrt_ctx* c, int b, const std::vector<RenTerm>& terms,
-                                                int prec = LRT_FP64, RenTemplate* tpl = nullptr) {
+                                                int prec = LRT_FP64, RenTemplate* tpl = nullptr,
+                                                RenOrder order = RenOrder::ZEROTH) {
   if (terms.empty() || (int)terms.size() > REN_MAX_TERMS) throw Error(LRT_EINVAL, "renormalize: 1 or 2 terms");
   GemmExtra ex{};
   for (size_t t = 0; t < terms.size(); ++t) {
@@ -1744,13 +1760,14 @@ static std::unique_ptr<OpSet> renorm_left_terms(lrt_ctx* c, int b, const std::ve
       }
     }
   N->finish_nz();
-  ren_run(c, o1, s1, o2, s2, toff, ex, prec, tpl, *N, sig);
+  ren_run(c, o1, s1, o2, s2, toff, ex, prec, tpl, *N, sig, order);
   return N;
 }
 
 // right block of bond b = sum_t R_bra,t [E_t] R_ket,t^T over the enlarged right block site b (+) R
 static std::unique_ptr<OpSet> renorm_right_terms(lrt_ctx* c, int b, const std::vector<RenTerm>& terms,
-                                                 int prec = LRT_FP64, RenTemplate* tpl = nullptr) {
+                                                 int prec = LRT_FP64, RenTemplate* tpl = nullptr,
+                                                RenOrder order = RenOrder::ZEROTH) {
   if (terms.empty() || (int)terms.size() > REN_MAX_TERMS) throw Error(LRT_EINVAL, "renormalize: 1 or 2 terms");
   const OpSet& E0 = *terms[0].E;
   const Fused& F = *E0.fused;
@@ -1812,7 +1829,7 @@ static std::unique_ptr<OpSet> renorm_right_terms(lrt_ctx* c, int b, const std::v
       }
     }
   N->finish_nz();
-  ren_run(c, o1, s1, o2, s2, toff, ex, prec, tpl, *N, sig);
+  ren_run(c, o1, s1, o2, s2, toff, ex, prec, tpl, *N, sig, order);
   return N;
 }
 
@@ -2213,10 +2230,9 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
   }
   for (GemmSeg& g : s1) g.b_vs = nelem;
   set_vectors(o1, o1.size(), O2, O2.size(), nvec, nelem, toff);
-  // kept relative plans (first-order sets) are replayed over instances
-  const GemmMath math = rel_ops ? GemmMath::FMA : GemmMath::DIGITS;
-  build_gemm(plan->p1, o1, s1, c->st, c->kernels, math);
-  build_gemm(plan->p2, O2, S2, c->st, c->kernels, math, !rel_ops);
+  build_gemm(plan->p1, o1, s1, c->st, c->kernels, GemmMath::DIGITS);
+  // kept relative plans (first-order sets) are replayed over instances: no K parts
+  build_gemm(plan->p2, O2, S2, c->st, c->kernels, GemmMath::DIGITS, !rel_ops);
   // tensor-core twin: phase-2 outputs, one per (y block, column group)
   plan->has_tc = tc;
   for (size_t w = 0; w < wb.size() && tc; ++w)
@@ -3990,6 +4006,8 @@ struct TdaRunner {
           }
       }
     }
+    // (digit products, by the test hook alone: columns that carry Schmidt values keep their accuracy)
+    for (GemmOut& x : o) x.balance_rows = kind == K_LC || kind == K_RMULB;
     p = std::make_unique<GemmPlan>();
     if (!o.empty()) build_gemm(*p, o, g, c->st, c->kernels);
     return *p;
@@ -4277,6 +4295,7 @@ struct TdaRunner {
     std::deque<SiteView> views;   // site tensors borrowing the batch's slots (not movable)
     for (int mu = 0; mu < nv; ++mu) views.emplace_back(lay[i], L1.v(mu));
     for (int dir = 0; dir < 2; ++dir) {
+      const RenOrder order = dir == 0 ? RenOrder::KET : RenOrder::BRA;
       std::vector<std::vector<RenTerm>> terms(nv);
       std::vector<std::vector<double*>> kets(nv), bras(nv);
       for (int mu = 0; mu < nv; ++mu) {
@@ -4302,9 +4321,9 @@ struct TdaRunner {
             sig0 = sig;
             batch.push_back(mu);
           } else if (batch.empty() && !(tp->p1 && tp->sig == sig)) {
-            out[mu] = renorm_left_terms(c, i, terms[mu], LRT_FP64, tp);   // builds the template
+            out[mu] = renorm_left_terms(c, i, terms[mu], LRT_FP64, tp, order);   // builds the template
           } else {
-            out[mu] = renorm_left_terms(c, i, terms[mu], LRT_FP64, nullptr);
+            out[mu] = renorm_left_terms(c, i, terms[mu], LRT_FP64, nullptr, order);
           }
         }
         ren_batch(tp, terms, batch, kets, bras, out);
@@ -4360,6 +4379,7 @@ struct TdaRunner {
       CK(cudaGetLastError());
     }
     for (int dir = 0; dir < 2; ++dir) {
+      const RenOrder order = dir == 0 ? RenOrder::KET : RenOrder::BRA;
       std::vector<std::vector<RenTerm>> terms(nv);
       std::vector<std::vector<double*>> kets(nv), bras(nv);
       for (int mu = 0; mu < nv; ++mu) {
@@ -4387,9 +4407,9 @@ struct TdaRunner {
             sig0 = sig;
             batch.push_back(mu);
           } else if (batch.empty() && !(tp->p1 && tp->sig == sig)) {
-            out[mu] = renorm_right_terms(c, i, terms[mu], LRT_FP64, tp);   // builds the template
+            out[mu] = renorm_right_terms(c, i, terms[mu], LRT_FP64, tp, order);   // builds the template
           } else {
-            out[mu] = renorm_right_terms(c, i, terms[mu], LRT_FP64, nullptr);
+            out[mu] = renorm_right_terms(c, i, terms[mu], LRT_FP64, nullptr, order);
           }
         }
         ren_batch(tp, terms, batch, kets, bras, out);

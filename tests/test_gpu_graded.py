@@ -48,8 +48,9 @@ def _tda(pkg, H, ref, n, kernel, **kw):
     return out
 
 
+@pytest.mark.parametrize("kernel", [0, 2, 3])
 @pytest.mark.parametrize("M,span", [(40, 4), (64, 4), (40, 6), (64, 6)])
-def test_tda_with_small_schmidt_values_is_as_accurate_as_fma_products(pkg, M, span):
+def test_tda_with_small_schmidt_values_is_as_accurate_as_fma_products(pkg, M, span, kernel):
     """One tangent-space sweep after the start sweep, on Schmidt values down to below 1e-6: the
     products with Lambda^-1 magnify every error that is relative to a row's or column's largest
     element only.  Products accurate element by element leave the roots of the two arithmetics
@@ -58,7 +59,7 @@ def test_tda_with_small_schmidt_values_is_as_accurate_as_fma_products(pkg, M, sp
     ref = _graded_reference(8, 4, 4, M, 3, span)
     assert min(x.min() for b in range(H.k + 1) for x in ref[3][b].values()) < 1e-6
     w0, r0, e0 = _tda(pkg, H, ref, 2, KERNEL_FP64, max_iter=1, eps=1e-30)
-    w1, r1, e1 = _tda(pkg, H, ref, 2, 0, max_iter=1, eps=1e-30)
+    w1, r1, e1 = _tda(pkg, H, ref, 2, kernel, max_iter=1, eps=1e-30)
     assert abs(e1 - e0) <= 1e-12 * abs(e0)
     assert np.abs(w1 - w0).max() <= 1e-12 * abs(e0)
     assert np.abs(r1 / r0 - 1.0).max() <= 1e-12 * abs(e0)
