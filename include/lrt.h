@@ -52,7 +52,7 @@ extern "C" {
 #define LRT_ETIMEOUT (-5) /* a bounded device wait expired */
 #define LRT_ESTATE (-6)   /* call order: a required object has not been built */
 
-#define LRT_FP64 0        /* all products in binary64 on the CUDA cores */
+#define LRT_FP64 0        /* binary64 products: FMAs, or exact digit products on the tensor cores */
 #define LRT_MIXED 1       /* split-TF32 tensor-core products, FP32 accumulation */
 
 typedef struct lrt_ctx* lrt_t;
@@ -141,7 +141,8 @@ int renormalize(lrt_t ctx, int site, int dir, int precision);
 int sigma(lrt_t ctx, int site, int nsite, int nvec, const double* x_dev, double* y_dev,
           int precision);
 
-/* Diagonal of H_eff (the preconditioner of Eq. error) in the same layout as sigma. */
+/* Diagonal of H_eff (the preconditioner of Eq. error) in the same layout as sigma.  Prepares the
+ * single-vector plan of the position. */
 int heff_diag(lrt_t ctx, int site, int nsite, double* d_dev);
 
 /* Ground state by two-site DMRG sweeps (Eq. dmrg solved by Davidson at every
@@ -197,8 +198,8 @@ typedef struct {
   uint64_t seed;      /* initial trial vectors projected by Q^C: SplitMix64 Gaussians of this
                          seed, or (seed 0) at every site the unit vector on the root's rank
                          among the lowest diagonal elements of H_0 where |C0| < 1/2 */
-  int precision;      /* LRT_FP64, or LRT_MIXED: the site products H_0 C run as split-TF32
-                         tensor-core products until every root's sum |r|^2 is below
+  int precision;      /* LRT_FP64, or LRT_MIXED: the site products H_0 C run in sigma's mixed
+                         form (split-TF32 where the position is large enough) until every root's sum |r|^2 is below
                          refine_tol (or two thirds of max_iter have passed), then the sweeps
                          continue in FP64 to eps (the FP64 residual correction); with
                          max_iter >= 2 the results come from FP64 sweeps.  The first-order
@@ -375,9 +376,8 @@ int sigma_stats(lrt_t ctx, lrt_sigma_stats* out);
  *    make that first call during set-up, where the reservation is acceptable; later
  *    calls take no device memory.
  *  - Reuses the plan that a regular sigma() call with the same (site, nsite, nvec)
- *    prepared after the last renormalize(); without one it returns LRT_ESTATE, except
- *    that a single-vector call after heff_diag() of the position prepares its plan itself
- *    (that call allocates; while its stream is captured it returns LRT_ESTATE).
+ *    prepared after the last renormalize(); heff_diag() of the position prepares the
+ *    single-vector one too.  Without a plan it returns LRT_ESTATE.
  *    A plan whose intermediates exceed the static array is rejected with LRT_EINVAL
  *    and a message giving both sizes.
  *  - The first call on each device resolves the array's device address

@@ -32,14 +32,16 @@
 // plain FP64 from the staged operands.
 //
 // Measured on the k = 24, M = 500, 6-vector sigma (23.7 G multiply-adds): 44.0 ms by FP64 FMAs,
-// 15.2 ms here; error against 64-bit exact values 3.9e-16 (7.1e-16 before) at k = 8, 2.9e-15
-// (7.0e-15) on the PPP chain.  The kernel is bound by issued instructions (45% of the issue slots;
-// tensor pipe 20%, FP64 pipe 25%): cutting the operands (a third of them) and staging cost more
-// than the products.  Hence tiles of 128 staged rows for up to 16 16 x 16 units and 16 warps per
-// SM, 2 CTAs of 8 warps at 128 registers (96 rows for 8 units, 3 CTAs of 4 warps: 16.9 ms); and
-// one row or column scale per 32 positions, so a chunk needs no look at the rest of K.  Operands
-// cut ahead into digit matrices and fetched by bulk copies were not faster (19.3 ms: pools of
-// 14 bytes per element, chunks that end with every segment, fewer warps).
+// 16.3 ms here (15.2 with the exponents taken out of the K positions of phase 2 alone: one more
+// pass over the staged operand and one more barrier per chunk); error against 64-bit exact values
+// 3.7e-16 (8.3e-16 by FMAs) at k = 8, 3.5e-15 (7.3e-15) on the PPP chain.  The kernel is bound by
+// issued instructions (48% of the issue slots; tensor pipe 20%, FP64 pipe 24%): cutting the
+// operands (a third of them) and staging cost more than the products.  Hence tiles of 128 staged
+// rows for up to 16 16 x 16 units and 16 warps per SM, 2 CTAs of 8 warps at 128 registers (96 rows
+// for 8 units, 3 CTAs of 4 warps: 16.9 ms where this split took 15.2); and one row or column scale
+// per 32 positions, so a chunk needs no look at the rest of K.  Operands cut ahead into digit
+// matrices and fetched by bulk copies were not faster (19.3 ms then: pools of 14 bytes per
+// element, chunks that end with every segment, fewer warps).
 #include "lrt_kernels.h"
 #include "lrt_fp64_tile.h"
 
@@ -589,10 +591,11 @@ void launch_gemm_mma_inst(const GemmOut* outs, const GemmSeg* segs, const int3* 
 // tile's last part adds the parts in order (a counter per tile, reset by that warp), which
 // spares the reduction launch.
 //
-// Measured (one-site sigma): k = 8, M = 64, 1 vector 183 -> 51 us; k = 17, M = 30, 6 vectors
-// 468 -> 106 us; eight molecules in one call 1.67 -> 0.89 ms.  Bound by latency: descriptor and
-// operand reads of short items, 16 warps per SM (128 registers; 3 CTAs of 168 registers are
-// 5% slower on the longer lists).
+// Measured (one-site sigma, FP64 FMA tiles of a CTA -> here): k = 8, M = 64, 1 vector 183 -> 51 us;
+// k = 17, M = 30, 6 vectors 468 -> 106 us; eight molecules in one call 1.67 -> 0.90 ms.  Bound by
+// latency: descriptor and operand reads of short items, 16 warps per SM (128 registers; 3 CTAs of
+// 168 registers are 5% slower on the longer lists).  Lists of FMA arithmetic (GemmMath) run
+// whole on the direct path.
 // ---------------------------------------------------------------------------
 struct WarpSeg {
   const double* p;          // operand along the tile's rows, and along its columns

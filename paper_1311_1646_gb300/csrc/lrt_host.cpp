@@ -853,13 +853,22 @@ static void mma_tile_shape(const GemmOut& O, int& tm, int& tn) {
 // Kernel of a list.  DIGITS: CTA tiles of digit products for long lists (3e8 multiply-adds per
 // vector and more) of blocks that fill them (work padded to 16 x 8 x 16 at most 3 times the exact
 // work), one warp per tile elsewhere: a CTA shares the cut operands among its units, a warp
-// waits for nobody.  Both measured, CTA / warp (multiply-adds, padding of the two phases):
-// k = 24, M = 500, 6 vectors (2 x 1.9e9 per vector; 1.8, 1.1) 15.2 / 25.2 ms; the same chain at
-// M = 300, site 4 (1.3e8; 2.0, 1.6) 628 / 354 us; two-site k = 13, M = 200, 3 vectors (1e8) 1.83 /
-// 1.46 ms; eight molecules of 8 to 12 orbitals (5e7; 4, 3) 1.32 / 0.88 ms; with earlier forms of
-// both, PPP k = 12, M = 256 (1.7e7; 2.0, 1.9) 129 / 93 us and k = 8, M = 64 (1e6; 13, 5) 135 / 61 us
-// (183 by FP64 CTA tiles).  Counted per vector, so that a call's kernel, and with
-// it every bit of a vector's result, does not depend on how many vectors the call has.
+// waits for nobody.  Sigma with every list on CTA / warp tiles, ms, for 1, 3 and 6 vectors, by the
+// two phases' multiply-adds (x 1e8) and padding:
+//   0.9 1.5  4.4 2.9  k = 13, M = 200, two sites  1.7 / 0.67   2.2 / 1.5   3.4 / 2.8
+//   1.3 0.8  2.0 1.6  k = 24, M = 300, site 4     0.67 / 0.36  0.94 / 0.89 1.4 / 1.6
+//   2.0 1.6  3.7 2.1  k = 16, M = 384, one site   2.7 / 0.97   3.1 / 2.2   4.1 / 3.8
+//   2.4 4.8  2.3 1.9  k = 12, M = 256, two sites  2.1 / 1.1    3.1 / 2.9   5.0 / 5.5
+//   3.6 7.4  2.5 1.7  k = 14, M = 300, two sites  3.5 / 1.8    5.1 / 4.5   8.0 / 8.4
+//   4.2 4.4  3.1 1.9  k = 24, M = 300, one site   3.1 / 1.9    4.3 / 4.1   6.6 / 7.4
+//   5.6 5.4  1.8 1.4  k = 14, M = 400, one site   1.2 / 1.5    2.3 / 3.6   4.1 / 6.7
+//   6.4 13   3.6 3.3  k = 24, M = 300, two sites  7.7 / 4.6    12 / 10     19 / 19
+//   8.0 17   2.7 2.1  k = 16, M = 384, two sites  6.5 / 4.2    9.9 / 11    16 / 19
+//   9.7 10   2.3 1.6  k = 24, M = 400, one site   4.4 / 3.3    6.9 / 7.4   11 / 14
+//   19 20    2.0 1.5  k = 24, M = 500, one site   5.6 / 5.4    9.6 / 13    16 / 24
+// One vector favours the warps up to six times the line, six vectors the CTA tiles from half of it.
+// Counted per vector, so that a call's kernel, and with it every bit of a vector's result, does
+// not depend on how many vectors the call has.
 // FMA: warp tiles of 64 elements straight from global memory up to 1e8 multiply-adds, CTA tiles
 // with staged operands above.  A renormalization's two launches, CTA / warp: 1.1e5 multiply-adds 24 /
 // 16 us, 1.2e7 138 / 69 (k = 12, M = 128), 5e7 292 / 193 and 1.4e8 499 / 539 (k = 14 and 16), 1.1e9 2.1 /
@@ -886,10 +895,10 @@ static GemmKind gemm_kind(const std::vector<GemmOut>& outs, const std::vector<Ge
 }
 
 // Path and tile of one output in the warp kernel (digits: the list may take them).  Direct FMAs
-// cost about 0.5 clocks of the FP64 pipe per element and K position, digit products about 210 issue slots per 16 x 8 x 16 but a
-// longer dependent chain: direct below 1000 multiply-adds per 16 positions (counted per vector;
-// limits of 150 / 400 / 1000: 52 / 51 / 49 us at k = 8, M = 64, 954 / 933 / 912 for the eight
-// molecules, and at 4000 1780).
+// cost about 0.5 clocks of the FP64 pipe per element and K position, digit products about 210
+// issue slots per 16 x 8 x 16 but a longer dependent chain: direct below 1000 multiply-adds per 16
+// positions (counted per vector; limits of 150 / 400 / 1000: 52 / 51 / 49 us at k = 8, M = 64, 954 /
+// 933 / 912 for the eight molecules, and at 4000 1780).
 static void warp_tile_shape(GemmOut& O, int64_t k, bool digits, int& tm, int& tn) {
   const int m = O.c_vr > 0 ? O.c_vr : O.m, n = O.c_vc > 0 ? O.c_vc : O.n;
   auto even = [](int x, int most) {
