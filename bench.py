@@ -33,24 +33,25 @@ import synth  # noqa: E402
 TF32_PER_BF16 = 1.1 / 2.25  # nominal dense TF32 / BF16 tensor rates
 
 # DRAM bytes (read + write) per launch of the dominant kernel, one ncu capture of
-# dram__bytes_read/write.sum with --profile-step, valid only for the kernel source it was taken
-# on (sha256 prefix); otherwise the bench reports null.
-TRAFFIC = {
-    "fp64": {"source": "lrt_fp64_mma.cu", "sha256": "", "bytes": None},
-    "mixed": {"source": "lrt_tc.cu", "sha256": "", "bytes": None},
-}
+# dram__bytes_read/write.sum over the sigma launches of one step (--profile-step: 29 of
+# gemm_mma_kernel; the other 19, near the chain's ends, are gemm_warp_kernel's at 57 MB each),
+# valid only for the kernel source it was taken on (sha256 prefix); otherwise, and for the
+# mixed form, the bench reports null.
+TRAFFIC = {"fp64": {"source": "lrt_fp64_mma.cu", "sha256": "c01ee0d65db15e93", "bytes": 1410.96e6}}
 
 
 def traffic(precision):
     import hashlib
-    t = TRAFFIC[precision]
+    t = TRAFFIC.get(precision)
+    if t is None:
+        return None
     path = os.path.join(ROOT, "paper_1311_1646_gb300", "csrc", t["source"])
     try:
         with open(path, "rb") as f:
             h = hashlib.sha256(f.read()).hexdigest()[:16]
     except OSError:
         return None
-    return t["bytes"] if t["bytes"] and h == t["sha256"] else None
+    return t["bytes"] if h == t["sha256"] else None
 
 
 def tf32_peak():
@@ -343,7 +344,7 @@ def run_ours(args):
             peak, peak_note = digit_peak()
             roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                     "frac": achieved / peak, "traffic": traffic("fp64"),
-                    "kernel": "gemm_mma_kernel (sigma phases 1+2)",
+                    "kernel": "gemm_mma_kernel (sigma phases 1+2; gemm_warp_kernel near the chain's ends)",
                     "peak_note": peak_note, "fp64_pipe_tflops": fp64_peak(clocks)}
             metric, dtype = "H_eff sigma TFLOP/s (algorithmic, FP64)", "f64"
         out = {
@@ -434,7 +435,7 @@ def _tda_converged(pkg, device, cfg_idx, schedule, eps, max_iter):
         "note": "ground state on the GPU: two-site sweeps with M = %s, then one-site sweeps "
                 "(reference_gradient2 = sum_i |Q^C (H_0^[i] - E0) C0_i|^2); TDA: sweep_tda to sum "
                 "|Q^C r|^2 < eps for every root, thick restart (2 n kept, subspace 32), sweep "
-                "correction, diagonal-damped random start; mixed: tensor-core H_0 site products "
+                "correction, diagonal-damped random start; mixed: H_0 site products in mixed form "
                 "until sum |r|^2 < 1e-6, then FP64 sweeps to eps" % schedule}
 
 
@@ -464,9 +465,9 @@ def _tda_sweep_times(pkg, device, cfg_idx=3, iters=3):
         finally:
             t.close()
         out[name] = {"total_s": dt, "setup_s": dt - sum(x for x, _ in log), "sweep_s": [x for x, _ in log],
-                     "tensor_core_sweep": [f for _, f in log]}
+                     "mixed_form_sweep": [f for _, f in log]}
     fp, mx = out["fp64"], out["mixed"]
-    both = [j for j in range(1, min(len(fp["sweep_s"]), len(mx["sweep_s"]))) if mx["tensor_core_sweep"][j]]
+    both = [j for j in range(1, min(len(fp["sweep_s"]), len(mx["sweep_s"]))) if mx["mixed_form_sweep"][j]]
     if both:
         a = sum(fp["sweep_s"][j] for j in both)
         b = sum(mx["sweep_s"][j] for j in both)
