@@ -728,8 +728,18 @@ enum class GemmMath { FMA, DIGITS };
 // position of k = 16, M = 384 has half a million tiles in its two plans.  At most
 // TILE_BUFFER_BYTES stay.
 constexpr size_t TILE_BUFFER_BYTES = (size_t)64 << 20;
-struct TileBuffers {
+struct ListSums {              // what the planner needs of a list's segments
   std::vector<int64_t> ktot;   // K of every output
+  int max_ld = 0;              // largest leading dimension and vector stride
+  int64_t max_vs = 0;
+  void clear() {
+    ktot.clear();
+    max_ld = 0;
+    max_vs = 0;
+  }
+};
+struct TileBuffers {
+  ListSums sums;
   std::vector<int> key;        // of every tile: its place in the order of costs
   std::vector<int3> list;
   void clear() {
@@ -744,7 +754,7 @@ struct TileBuffers {
     list.push_back(tile);
   }
   void trim() {
-    if (ktot.capacity() * sizeof(int64_t) + key.capacity() * sizeof(int) +
+    if (sums.ktot.capacity() * sizeof(int64_t) + key.capacity() * sizeof(int) +
             list.capacity() * sizeof(int3) > TILE_BUFFER_BYTES)
       *this = TileBuffers();
   }
@@ -873,21 +883,17 @@ static void mma_tile_shape(const GemmOut& O, int& tm, int& tn) {
 // with staged operands above.  A renormalization's two launches, CTA / warp: 1.1e5 multiply-adds 24 /
 // 16 us, 1.2e7 138 / 69 (k = 12, M = 128), 5e7 292 / 193 and 1.4e8 499 / 539 (k = 14 and 16), 1.1e9 2.1 /
 // 2.9 ms (k = 24, M = 500).  CTA tiles also take strides beyond 32 bits.
-static GemmKind gemm_kind(const std::vector<GemmOut>& outs, const std::vector<GemmSeg>& segs,
-                          const std::vector<int64_t>& ktot, GemmMath math, int forced) {
+static GemmKind gemm_kind(const std::vector<GemmOut>& outs, const ListSums& sums, GemmMath math, int forced) {
+  // 32-bit byte strides are what the digit and warp kernels take
+  if (sums.max_ld >= (1 << 28)) return GemmKind::FP64;
   double exact = 0.0, padded = 0.0;
   for (size_t i = 0; i < outs.size(); ++i) {
     const GemmOut& o = outs[i];
-    for (int q = 0; q < o.seg_count; ++q) {
-      const GemmSeg& g = segs[o.seg_begin + q];
-      // 32-bit byte strides are what those kernels take
-      if ((o.c_vr > 0 && g.a_vs >= (int64_t)1 << 29) || (o.c_vc > 0 && g.b_vs >= (int64_t)1 << 29) ||
-          std::max(g.lda, g.ldb) >= (1 << 28))
-        return GemmKind::FP64;
-    }
+    if ((o.c_vr > 0 || o.c_vc > 0) && sums.max_vs >= (int64_t)1 << 29) return GemmKind::FP64;
     const int m = o.c_vr > 0 ? o.c_vr : o.m, n = o.c_vc > 0 ? o.c_vc : o.n;
-    exact += (double)m * n * ktot[i];
-    padded += (double)((m + 15) / 16 * 16) * ((n + 7) / 8 * 8) * ((ktot[i] + 15) / 16 * 16);
+    const int64_t k = sums.ktot[i];
+    exact += (double)m * n * k;
+    padded += (double)((m + 15) / 16 * 16) * ((n + 7) / 8 * 8) * ((k + 15) / 16 * 16);
   }
   if (forced > 0) return (GemmKind)(forced - 1);
   if (math == GemmMath::FMA) return exact >= 1e8 ? GemmKind::FP64 : GemmKind::WARP;
@@ -921,10 +927,10 @@ static void warp_tile_shape(GemmOut& O, int64_t k, bool digits, int& tm, int& tn
 // outs is worked on in place: the parts of split tiles are appended.  P.segs: the segments where
 // they are on the device already.  split: outputs may be cut along K (not in lists replayed over
 // instances, whose partial tiles would need a workspace each).  like: the kernel to use, for
-// lists merged from others.
+// lists merged from others.  known: the list's sums, where its writer kept them.
 static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vector<GemmSeg>& segs,
                        cudaStream_t st, KernelChoice& choice, GemmMath math = GemmMath::FMA,
-                       bool split = false, const GemmKind* like = nullptr) {
+                       bool split = false, const GemmKind* like = nullptr, const ListSums* known = nullptr) {
   // A tile costs its warps of outputs times its K chunks of DFMA issue, plus a fixed
   // cost per chunk.  Tiles far longer than an even share of the launch (an output with
   // many long K segments) would run on after all others finished.  With `split`, an
@@ -941,14 +947,23 @@ static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vecto
   const size_t nout = outs.size();   // the parts of split tiles follow
   TileBuffers& buf = choice.buf;
   buf.clear();
-  std::vector<int64_t>& ktot = buf.ktot;
-  ktot.assign(nout, 0);
-  double fl = 0.0;
-  for (size_t i = 0; i < nout; ++i) {
-    for (int s = 0; s < outs[i].seg_count; ++s) ktot[i] += segs[outs[i].seg_begin + s].k;
-    fl += 2.0 * outs[i].m * (double)outs[i].n * (double)ktot[i];
+  if (!known) {
+    ListSums& sums = buf.sums;
+    sums.clear();
+    sums.ktot.assign(nout, 0);
+    for (size_t i = 0; i < nout; ++i)
+      for (int q = 0; q < outs[i].seg_count; ++q) {
+        const GemmSeg& g = segs[outs[i].seg_begin + q];
+        sums.ktot[i] += g.k;
+        sums.max_ld = std::max(sums.max_ld, std::max(g.lda, g.ldb));
+        sums.max_vs = std::max(sums.max_vs, std::max(g.a_vs, g.b_vs));
+      }
+    known = &sums;
   }
-  const GemmKind kind = like ? *like : gemm_kind(outs, segs, ktot, math, choice.forced);
+  const std::vector<int64_t>& ktot = known->ktot;
+  double fl = 0.0;
+  for (size_t i = 0; i < nout; ++i) fl += 2.0 * outs[i].m * (double)outs[i].n * (double)ktot[i];
+  const GemmKind kind = like ? *like : gemm_kind(outs, *known, math, choice.forced);
   const bool digits = math == GemmMath::DIGITS || choice.forced > 0;
   const bool mma = kind == GemmKind::MMA, warp = kind == GemmKind::WARP;
   auto cost = [mma, warp](int64_t mt, int64_t nt, int64_t k) {
@@ -977,7 +992,7 @@ static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vecto
   for (size_t i = 0; i < nout; ++i) {
     int TM, TN;
     shape(outs[i], ktot[i], TM, TN);
-    const GemmOut O = outs[i];
+    const int om = outs[i].m, on = outs[i].n, nseg = outs[i].seg_count, c_rel = outs[i].c_rel;
     // K per part.  A warp walks its part alone, a segment at a time: short parts where segments
     // are a few positions (direct FMAs), longer ones for digit products.  24 / 96 positions for
     // direct lists: 49 / 59 us (k = 8, M = 64), 51 / 103 (k = 13, M = 20); 24 / 64 / 96 for digit
@@ -985,12 +1000,13 @@ static void build_gemm(GemmPlan& P, std::vector<GemmOut>& outs, const std::vecto
     const int64_t kshort = outs[i].flags & GEMM_WARP_DIRECT ? 24 : 64;
     const int64_t kpart = warp ? std::min<int64_t>(GEMM_SPLIT_K, std::max<int64_t>(kshort, ktot[i] / (kshort == 24 ? 32 : 16)))
                                : GEMM_SPLIT_K;
-    for (int m0 = 0; m0 < O.m; m0 += TM)
-      for (int n0 = 0; n0 < O.n; n0 += TN) {
-        const int mt = std::min(TM, O.m - m0), nt = std::min(TN, O.n - n0);
+    for (int m0 = 0; m0 < om; m0 += TM)
+      for (int n0 = 0; n0 < on; n0 += TN) {
+        const int mt = std::min(TM, om - m0), nt = std::min(TN, on - n0);
         const int64_t c = cost(mt, nt, ktot[i]);
-        const int want = (int)std::min<int64_t>(O.seg_count, ktot[i] / kpart);
-        if (split && want >= 2 && O.c_rel <= 2 && outs.size() < (size_t)INT32_MAX) {
+        const int want = (int)std::min<int64_t>(nseg, ktot[i] / kpart);
+        if (split && want >= 2 && c_rel <= 2 && outs.size() < (size_t)INT32_MAX) {
+          const GemmOut O = outs[i];
           // contiguous runs of the segment list, each about ktot / want of K
           SplitTile t{wsz, (int)i, 0, m0, mt, n0, nt};
           std::vector<int> kseg(O.seg_count);
@@ -1191,9 +1207,12 @@ struct PlanScratch {
   std::vector<GemmOut> o1, o2;
   std::vector<GemmSeg> s1, s2;
   std::vector<char> s1rev;
+  ListSums sum1, sum2;
   uint64_t lists = 0;      // SigmaPlan::lists of the plan these lists are of (0: of none)
   void clear() {
     lists = 0;
+    sum1.clear();
+    sum2.clear();
     prod2.clear();
     o1.clear();
     o2.clear();
@@ -1203,7 +1222,8 @@ struct PlanScratch {
   }
   void trim() {
     if (prod2.capacity() * sizeof(Prod2) + (o1.capacity() + o2.capacity()) * sizeof(GemmOut) +
-            (s1.capacity() + s2.capacity()) * sizeof(GemmSeg) + s1rev.capacity() > PLAN_SCRATCH_BYTES)
+            (s1.capacity() + s2.capacity()) * sizeof(GemmSeg) + s1rev.capacity() +
+            (sum1.ktot.capacity() + sum2.ktot.capacity()) * sizeof(int64_t) > PLAN_SCRATCH_BYTES)
       *this = PlanScratch();
   }
 };
@@ -2100,6 +2120,7 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
                 rows |= (uint16_t)(1u << r);
                 GemmOut out{nullptr, tp + (int64_t)XF.off[be][r] * wk.cols, wk.cols, XF.dim[be][r], wk.cols,
                             (int)s1.size(), 0, 0, 0};
+                int kout = 0;
                 for (int cc = 0; cc < 4; ++cc) {
                   if (!(mx & (1u << (4 * r + cc)))) continue;
                   GemmSeg g{};
@@ -2116,12 +2137,16 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
                   g.ldb = wk.cols;
                   g.k = XF.dim[ke][cc];
                   g.scale = 1.0;
+                  g.b_vs = nelem;
+                  kout += g.k;
+                  W.sum1.max_ld = std::max(W.sum1.max_ld, std::max(ld, wk.cols));
                   s1.push_back(g);
                   s1rev.push_back(&XS != &X);
                   ++out.seg_count;
                   falg += 2.0 * XF.dim[be][r] * XF.dim[ke][cc] * wk.cols;
                 }
                 o1.push_back(out);
+                W.sum1.ktot.push_back(kout);
               }
               if (tc && rows) {
                 const int A = tcp.op(base, ld, a.t ? 1 : 0, wbb.rows, wk.rows);
@@ -2220,7 +2245,10 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
     O2.push_back(GemmOut{nullptr, coff, w.cols, XF.dim[fx][os.r], ncols, at[u], at[u + 1] - at[u], 0, 1});
   }
   S2.resize(prod2.size());
+  W.sum2.ktot.assign(O2.size(), 0);
   for (const Prod2& p : prod2) {
+    W.sum2.ktot[p.out] += p.k;
+    W.sum2.max_ld = std::max(W.sum2.max_ld, std::max(p.lda, p.ldb));
     GemmSeg& g = S2[at[p.out]++];
     g.a_rel = p.ident ? 1 : 2;
     g.a_off = p.a_off;
@@ -2237,11 +2265,11 @@ static std::unique_ptr<SigmaPlan> plan_sigma_sets(lrt_ctx* c, const OpSet& X, co
     }
     g.a_vs = p.ident ? nelem : toff;
   }
-  for (GemmSeg& g : s1) g.b_vs = nelem;
+  W.sum1.max_vs = W.sum2.max_vs = std::max(nelem, toff);
   set_vectors(o1, o1.size(), O2, O2.size(), nvec, nelem, toff);
-  build_gemm(plan->p1, o1, s1, c->st, c->kernels, GemmMath::DIGITS);
+  build_gemm(plan->p1, o1, s1, c->st, c->kernels, GemmMath::DIGITS, false, nullptr, &W.sum1);
   // kept relative plans (first-order sets) are replayed over instances: no K parts
-  build_gemm(plan->p2, O2, S2, c->st, c->kernels, GemmMath::DIGITS, !rel_ops);
+  build_gemm(plan->p2, O2, S2, c->st, c->kernels, GemmMath::DIGITS, !rel_ops, nullptr, &W.sum2);
   // tensor-core twin: phase-2 outputs, one per (y block, column group)
   plan->has_tc = tc;
   for (size_t w = 0; w < wb.size() && tc; ++w)
@@ -2307,8 +2335,8 @@ static std::unique_ptr<SigmaPlan> plan_vectors(lrt_ctx* c, const SigmaPlan& P, i
   set_vectors(W.o1, (size_t)P.p1.nbase, W.o2, (size_t)P.p2.nbase, nvec, P.nelem, toff);
   // the kernels are P's too, unless a vector stride is beyond what one of them takes
   const bool same = std::max(P.nelem, toff) < (int64_t)1 << 29;
-  build_gemm(plan->p1, W.o1, W.s1, c->st, c->kernels, GemmMath::DIGITS, false, same ? &P.p1.kind : nullptr);
-  build_gemm(plan->p2, W.o2, W.s2, c->st, c->kernels, GemmMath::DIGITS, true, same ? &P.p2.kind : nullptr);
+  build_gemm(plan->p1, W.o1, W.s1, c->st, c->kernels, GemmMath::DIGITS, false, same ? &P.p1.kind : nullptr, &W.sum1);
+  build_gemm(plan->p2, W.o2, W.s2, c->st, c->kernels, GemmMath::DIGITS, true, same ? &P.p2.kind : nullptr, &W.sum2);
   CK(cudaStreamSynchronize(c->st));
   return plan;
 }
