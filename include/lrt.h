@@ -340,7 +340,8 @@ int mps_get_site(lrt_t ctx, int site, double* host_out, int64_t* nelem);
  * phase: the instances' block products are merged into one task list (FP64) or one
  * persistent tensor-core work stream (LRT_MIXED) with tiles dealt longest-first over
  * the SMs.  Instance j uses (sites[j], nsite, nvec) like sigma() and x_dev[j], y_dev[j]
- * in its wfn_layout.  The launch runs on ctxs[0]'s stream; the other contexts must be
+ * in its wfn_layout.  LRT_MIXED: every instance by its own size, smaller ones in FP64 (from a
+ * lower line than sigma()'s).  The launch runs on ctxs[0]'s stream; the other contexts must be
  * idle (or use the same stream).  The merged plan is cached in ctxs[0] and rebuilt when
  * an instance's plan changes (after renormalize); from the second call with the same
  * x/y pointers on, the whole call is replayed from a captured CUDA graph.  Errors are

@@ -2907,10 +2907,15 @@ static SigmaPlan& get_plan(lrt_ctx* c, int site, int nsite, int nvec, bool tc = 
 //   25   k = 12, M = 256, two sites 1.4 / 1.7    4.2 / 4.9
 //   100  k = 24, M = 400, one site  2.6 / 4.4    5.3 / 11.1
 //   260  k = 24, M = 500, one site  3.2 / 5.6    6.6 / 16.3
-// It is the position's, so that a vector's precision depends neither on the other vectors of
+// It is the position's own, so that a vector's precision depends neither on the other vectors of
 // the call nor on the other molecules of a batch.  A pending stall (lrt_set_wait_limit) is for the
 // next tensor-core launch, so such a call keeps it.
-constexpr double MIXED_MIN_WORK = 1.15e7;
+// In a batch the merged work stream fills the SMs and the host waits once for all instances.  Line
+// at 0.3 / 2 / 4 / 11.5 / nothing in split TF32, ms, 4 vectors: 32 molecules of k = 10 .. 16, M = 128 .. 384
+// 16.5 / 17.5 / 18.3 / 25.5 / 31.3, the first eight of them 4.8 / 5.3 / 6.0 / 7.8 / 8.9; eight of k = 8 ..
+// 12, M = 96 .. 174 1.47 / 1.07 / 1.07 / 1.07 / 1.07; four of k = 11, M = 200 .. 290 0.95 / 0.95 / 1.8 /
+// 1.8 / 1.8.
+constexpr double MIXED_MIN_WORK = 1.15e7, MIXED_MIN_WORK_BATCH = 2e6;
 static double tile_work(double macs, double padded) { return padded > 0.0 ? macs * (macs / padded) * (macs / padded) : 0.0; }
 static bool mixed_in_fp64(lrt_ctx* c, double work) {
   return !c->tc_stall && !c->kernels.mixed_always && work < MIXED_MIN_WORK;
@@ -5797,7 +5802,7 @@ static void sigma_batched_impl(lrt_ctx* const* ctxs, int n, const int* sites, in
   int ntc = 0;
   for (int j = 0; j < n && precision == LRT_MIXED; ++j) {
     PoolScope ps(&ctxs[j]->pool);
-    tc[j] = c0->tc_stall || c0->kernels.mixed_always || position_work(ctxs[j], sites[j], nsite) >= MIXED_MIN_WORK;
+    tc[j] = c0->tc_stall || c0->kernels.mixed_always || position_work(ctxs[j], sites[j], nsite) >= MIXED_MIN_WORK_BATCH;
     ntc += tc[j];
   }
   std::string key = std::to_string(nsite) + ":" + std::to_string(nvec) + ":" + std::to_string(precision);
