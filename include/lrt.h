@@ -337,7 +337,7 @@ int mps_get_site(lrt_t ctx, int site, double* host_out, int64_t* nelem);
 
 /* sigma_batched: y_j = H_eff^(j) x_j for n_inst independent instances, each its own
  * context (its own Hamiltonian and MPS, on the same device), in one grouped launch per
- * phase: the instances' block products are merged into one task list (FP64) or one
+ * phase: the instances' block products are merged into a task list per kernel (FP64) and one
  * persistent tensor-core work stream (LRT_MIXED) with tiles dealt longest-first over
  * the SMs.  Instance j uses (sites[j], nsite, nvec) like sigma() and x_dev[j], y_dev[j]
  * in its wfn_layout.  LRT_MIXED: every instance by its own size, smaller ones in FP64 (from a
